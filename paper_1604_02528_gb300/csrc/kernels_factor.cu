@@ -9,9 +9,11 @@
 //               parent J: entries whose column is one of J's columns go to
 //               J's panel, the rest into U_J (one launch per child rank, so
 //               no two writers meet; fixed order: deterministic)
-//   k_fdiag     dense LDL^T of J's diagonal block in place (one CTA)
-//   k_ftrsm     L(C,J) = A(C,J) L_JJ^{-T} D_J^{-1}, one thread per row
-//   k_fupd      U_J -= L_CJ D_J L_CJ^T (lower c x c, 64 x 64 tiles)
+//   k_fsmall    a whole narrow supernode: the next three steps at once
+//   k_fdiag     dense LDL^T of J's diagonal block in place (a cluster of CTAs)
+//   k_ftrsm     L(C,J) = A(C,J) L_JJ^{-T} D_J^{-1}, row tiles
+//   k_fupd      U_J -= L_CJ D_J L_CJ^T (lower c x c, tiles)
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,7 +27,10 @@
 
 namespace selinv {
 
-constexpr int kFT = 64;  // rows per factor tile
+namespace cg = cooperative_groups;
+
+constexpr int kFSmallS = 16;        // widest supernode of k_fsmall
+constexpr int kFSmallElems = 3400;  // ... and its largest panel (both copies of a complex one in 109 KB)
 
 template <typename T>
 __global__ void k_assemble(const int64_t *__restrict__ pos, const T *__restrict__ vals, int64_t nnz,
@@ -69,12 +74,12 @@ __global__ void __launch_bounds__(256) k_fasm(const FactorDesc *__restrict__ fd,
     }
 }
 
-// U_J -= L_CJ D_J L_CJ^T on one 64 x 64 tile of the lower c x c triangle
-template <typename T>
+// U_J -= L_CJ D_J L_CJ^T on one B x B tile of the lower c x c triangle
+template <typename T, int B>
 __global__ void __launch_bounds__(256) k_fupd(const FactorDesc *__restrict__ fd, const int4 *__restrict__ items,
                                               int nitems) {
     grid_dep_wait();
-    __shared__ SegSmem<T> sm;
+    __shared__ SegSmem<T, B> sm;
     const int w = blockIdx.x;
     if (w >= nitems) return;
     const FactorDesc &F = *fd;
@@ -85,23 +90,66 @@ __global__ void __launch_bounds__(256) k_fupd(const FactorDesc *__restrict__ fd,
     const T *LC = static_cast<const T *>(F.L) + F.panel_off[J] + sJ;   // L(p, k) = LC[k*ld + p]
     const T *DJ = static_cast<const T *>(F.D) + F.super_ptr[J];
     T *UJ = static_cast<T *>(F.U) + F.u_off[J];
-    const int pa = ti * kSegB, st = tj * kSegB;
-    const int np = c - pa < kSegB ? c - pa : kSegB, nq = c - st < kSegB ? c - st : kSegB;
+    const int pa = ti * B, st = tj * B;
+    const int np = c - pa < B ? c - pa : B, nq = c - st < B ? c - st : B;
     auto x = [&](int pl, int k) { return mul(LC[(int64_t)k * ld + pa + pl], DJ[k]); };
     auto y = [&](int ql, int k) { return cjif(LC[(int64_t)k * ld + st + ql], F.herm != 0); };
     auto out = [&](int pl, int ql, T v) {
         T *dst = UJ + (int64_t)(st + ql) * c + pa + pl;
         *dst = sub(*dst, v);
     };
-    seg_update<T>(pa, np, st, nq, sJ, x, y, out, sm);
+    seg_update<T, decltype(x), decltype(y), decltype(out), B>(pa, np, st, nq, sJ, x, y, out, sm);
+}
+
+// ---------------------------------------------------------------------------
+// k_fdiag: dense LDL^T of J's diagonal block (s > kFSmallS) by one thread-
+// block cluster.  GB300 issues one FP64 instruction per SM sub-partition in
+// 64 clocks (2 lanes per clock and SM), so the s^3 / 6 products of a 128-
+// column block alone take 85 us on one SM, and the levels near the root hold
+// one to eight such blocks: the cluster (8 CTAs there, 1 where a level has
+// blocks enough for every SM) holds the rows cyclically, four at a time, in
+// its CTAs' shared memory.  Per panel of 8 columns every CTA reads the panel
+// from the owners (distributed shared memory), factors it on all rows by
+// itself -- the chain reciprocal, scale, update per column is what bounds the
+// kernel, and repeating it costs less than exchanging it -- and updates its
+// own rows of the trailing block; one cluster barrier per panel.
+// ---------------------------------------------------------------------------
+constexpr int kFdThreads = 128;
+constexpr int kFdNB = 8;           // columns per panel
+constexpr int kFdLd = kFdNB + 1;   // panel row stride in shared memory
+
+// 1 / d: the hardware's approximate reciprocal r0 (relative error below
+// 2^-19), then one step of the third-order iteration r0 (1 + e + e^2),
+// e = 1 - d r0: three dependent FP64 operations (240 clocks with the seed)
+// where the division takes 385.  Magnitudes near the ends of the exponent
+// range (and zero, infinities, NaN) go through the division.
+__device__ __forceinline__ double fast_recip(double d) {
+    const int e = (int)((__double_as_longlong(d) >> 52) & 0x7FF);
+    if (e < 64 || e > 1982) return 1.0 / d;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double x = fma(-d, r, 1.0);
+    return fma(fma(x, x, x), r, r);
+}
+__device__ __forceinline__ zd fast_recip(zd d) { return recip(d); }
+
+// elements of a CTA's row store for s columns, clusters of cl CTAs: groups of
+// four rows, group g as 4 rows of 4 (g + 1) entries
+__host__ __device__ inline int fd_rows_elems(int s, int cl) {
+    const int groups = (s + 3) / 4, mine = (groups + cl - 1) / cl;   // at most, rank cl - 1
+    return 16 * (cl * (mine * (mine - 1) / 2) + mine * cl);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_fdiag(const FactorDesc *__restrict__ fd,
-                                               const int *__restrict__ js, int nj) {
+__global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restrict__ fd, const int *__restrict__ js,
+                                                      int nj) {
     grid_dep_wait();
-    const int w = blockIdx.x;
-    if (w >= nj) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T Ys[kFdNB][kFdNB];
+    cg::cluster_group cl = cg::this_cluster();
+    const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int w = blockIdx.x / CL;
+    if (w >= nj) return;                     // the grid is nj clusters: never taken by a part of one
     const FactorDesc &F = *fd;
     const int J = js[w];
     const int fc = F.super_ptr[J];
@@ -109,57 +157,273 @@ __global__ void __launch_bounds__(256) k_fdiag(const FactorDesc *__restrict__ fd
     const int64_t ld = F.rowptr[J + 1] - F.rowptr[J];
     T *P = static_cast<T *>(F.L) + F.panel_off[J];
     T *D = static_cast<T *>(F.D) + fc;
-    __shared__ T s_d;
-    for (int j = 0; j < s; j++) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const T d = P[(int64_t)j * ld + j];
-            if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
-            s_d = d;
-            D[j] = d;
+    const bool herm = F.herm != 0;
+    T *Yp = reinterpret_cast<T *>(smem_raw);          // [128][kFdLd] undivided panel columns y = l d
+    T *Lp = Yp + 128 * kFdLd;                         // [128][kFdLd] panel columns of L
+    T *A = Lp + 128 * kFdLd;                          // this CTA's rows
+    const int tid = threadIdx.x;
+    // row i = 4 g + u lives in rank g % CL at (local group g / CL)
+    auto off = [&](int i) {
+        const int g = i >> 2, lg = g / CL, r = g % CL;
+        return 16 * (CL * (lg * (lg - 1) / 2) + lg * (r + 1)) + (i & 3) * 4 * (g + 1);
+    };
+    const int groups = (s + 3) / 4;
+    const int myg = groups > rank ? (groups - rank + CL - 1) / CL : 0;   // row groups of this CTA
+    auto row_of = [&](int lr) { return ((lr >> 2) * CL + rank) * 4 + (lr & 3); };
+    for (int k = tid / 32; k < s; k += kFdThreads / 32)
+        for (int lr = tid % 32; lr < 4 * myg; lr += 32) {
+            const int i = row_of(lr);
+            if (i < s && k <= i) A[off(i) + k] = P[(int64_t)k * ld + i];
+        }
+    for (int b0 = 0; b0 < s; b0 += kFdNB) {
+        const int nb = s - b0 < kFdNB ? s - b0 : kFdNB;
+        cl.sync();
+        const int i = b0 + tid;                        // this thread's row of the panel
+        T a[kFdNB];
+        if (i < s) {
+            const T *src = cl.map_shared_rank(A, (i >> 2) % CL) + off(i) + b0;
+#pragma unroll
+            for (int j = 0; j < kFdNB; j++) a[j] = (j < nb && j <= tid) ? src[j] : Sc<T>::zero();
+        }
+#pragma unroll
+        for (int j = 0; j < kFdNB; j++) {
+            if (j < nb) {
+                if (tid >= j && tid < nb) Ys[j][tid] = a[j];
+                __syncthreads();
+                const T d = Ys[j][j];
+                if (i < s) {
+                    if (tid == j && rank == 0) {
+                        if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
+                        D[b0 + j] = d;
+                    }
+                    const T l = mul(a[j], fast_recip(d));
+                    Yp[tid * kFdLd + j] = a[j];
+                    Lp[tid * kFdLd + j] = l;
+#pragma unroll
+                    for (int k = j + 1; k < kFdNB; k++)
+                        if (k < nb) msub(a[k], l, cjif(Ys[j][k], herm));
+                }
+            }
         }
         __syncthreads();
-        const T rd = recip(s_d);
-        for (int i = j + 1 + threadIdx.x; i < s; i += blockDim.x) P[(int64_t)j * ld + i] = mul(P[(int64_t)j * ld + i], rd);
-        __syncthreads();
-        // a_ik -= L_ij d L_kj for j < k <= i < s
-        const int m = s - j - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            const int i = j + 1 + e % m, k = j + 1 + e / m;
-            if (k > i) continue;
-            T *a = P + (int64_t)k * ld + i;
-            *a = sub(*a, mul(mul(P[(int64_t)j * ld + i], s_d), cjif(P[(int64_t)j * ld + k], F.herm != 0)));
+        // L's columns of the panel, each row by its owner
+        for (int e = tid; e < 4 * myg * nb; e += kFdThreads) {
+            const int r = row_of(e % (4 * myg)), j = e / (4 * myg);
+            if (r >= s) continue;
+            P[(int64_t)(b0 + j) * ld + r] = r > b0 + j ? Lp[(r - b0) * kFdLd + j] : (r == b0 + j ? Sc<T>::one() : Sc<T>::zero());
+        }
+        // own rows of the trailing block: a_ik -= l_i y_k, columns b1 .. i of row i
+        const int b1 = b0 + kFdNB;
+        int lr = 0, q = tid;                           // q-th column of local row lr
+        while (lr < 4 * myg) {
+            const int r = row_of(lr);
+            const int cnt = r < s && r >= b1 ? r - b1 + 1 : 0;
+            if (q >= cnt) {
+                q -= cnt;
+                lr++;
+                continue;
+            }
+            T *dst = A + off(r) + b1 + q;
+            T acc = *dst;
+            const T *lrow = Lp + (r - b0) * kFdLd, *yrow = Yp + (b1 + q - b0) * kFdLd;
+#pragma unroll
+            for (int j = 0; j < kFdNB; j++) msub(acc, lrow[j], cjif(yrow[j], herm));   // a full panel: b1 <= s - 1
+            *dst = acc;
+            q += kFdThreads;
         }
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < s * s; e += blockDim.x) {
-        const int i = e % s, k = e / s;
-        if (i == k) P[(int64_t)k * ld + i] = Sc<T>::one();
-        else if (i < k) P[(int64_t)k * ld + i] = Sc<T>::zero();
+    cl.sync();   // no CTA leaves while another may still read its rows
+}
+
+// ---------------------------------------------------------------------------
+// k_ftrsm: X D L_JJ^T = A for the rows of C (D L_JJ^H for a Hermitian matrix),
+// a warp for R rows at a time, lanes over the columns: with y = x D, step j
+// broadcasts y_j and every later column subtracts y_j L(k, j); the rows are
+// scaled by 1 / D once at the end.  L_JJ's lower triangle waits in shared
+// memory (columns from their 32-block's first row on, zeros above the
+// diagonal), so each step is one broadcast and at most four FP64
+// instructions per row: the FP64 pipe bounds it, and the row tiles are made
+// small enough that every SM gets one.
+// items {J, first row of C, rows}
+// ---------------------------------------------------------------------------
+constexpr int kFtThreads = 128;
+
+// elements of L_JJ's store: nc blocks of 32 columns, block b with 32 (nc - b) rows
+__host__ __device__ inline int ft_store_elems(int s) {
+    const int nc = (s + 31) / 32;
+    return 32 * 32 * (nc * (nc + 1) / 2);
+}
+template <typename T> __device__ __forceinline__ T shfl_elem(T v, int src);
+template <> __device__ __forceinline__ double shfl_elem(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+template <> __device__ __forceinline__ zd shfl_elem(zd v, int src) {
+    return make_zd(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+template <typename T, int NC, int R>
+__device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, int row0, int nrows) {
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    for (int g = warp * R; g < nrows; g += kFtThreads / 32 * R) {
+        T a[R][NC];
+#pragma unroll
+        for (int r = 0; r < R; r++)
+#pragma unroll
+            for (int t = 0; t < NC; t++) {
+                const int k = lane + 32 * t;
+                a[r][t] = (g + r < nrows && k < s) ? P[(int64_t)k * ld + row0 + g + r] : Sc<T>::zero();
+            }
+        const T *Lb = Ls;
+#pragma unroll
+        for (int b = 0; b < NC; b++) {
+#pragma unroll 2
+            for (int jj = 0; jj < 32; jj++) {
+                T l[NC];
+#pragma unroll
+                for (int t = b; t < NC; t++) l[t] = Lb[jj * 32 * (NC - b) + lane + 32 * (t - b)];
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const T y = shfl_elem(a[r][b], jj);
+#pragma unroll
+                    for (int t = b; t < NC; t++)
+                        if (t > b || lane > jj) msub(a[r][t], y, l[t]);   // finished columns stay as they are
+                }
+            }
+            Lb += 32 * 32 * (NC - b);
+        }
+#pragma unroll
+        for (int r = 0; r < R; r++)
+#pragma unroll
+            for (int t = 0; t < NC; t++) {
+                const int k = lane + 32 * t;
+                if (g + r < nrows && k < s) P[(int64_t)k * ld + row0 + g + r] = mul(a[r][t], rD[k]);
+            }
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(64) k_ftrsm(const FactorDesc *__restrict__ fd,
-                                              const int2 *__restrict__ tiles, int ntiles) {
+__global__ void __launch_bounds__(kFtThreads) k_ftrsm(const FactorDesc *__restrict__ fd,
+                                                      const int4 *__restrict__ items, int nitems) {
     grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T rD[128];
+    T *Ls = reinterpret_cast<T *>(smem_raw);
     const int w = blockIdx.x;
-    if (w >= ntiles) return;
+    if (w >= nitems) return;
     const FactorDesc &F = *fd;
-    const int J = tiles[w].x;
+    const int4 it = items[w];
+    const int J = it.x;
     const int fc = F.super_ptr[J];
     const int s = F.super_ptr[J + 1] - fc;
     const int64_t ld = F.rowptr[J + 1] - F.rowptr[J];
-    const int64_t r = (int64_t)tiles[w].y * kFT + threadIdx.x;  // panel row
-    if (r < s || r >= ld) return;
     T *P = static_cast<T *>(F.L) + F.panel_off[J];
     const T *D = static_cast<const T *>(F.D) + fc;
-    // x (D L_JJ^T) = a : x_j = (a_j - sum_{k<j} x_k D_k L_jk) / D_j, in place (conj(L_jk): Hermitian)
     const bool h = F.herm != 0;
+    const int nc = (s + 31) / 32;
+    for (int k = threadIdx.x; k < s; k += kFtThreads) rD[k] = recip(D[k]);
+    {
+        T *dst = Ls;
+        for (int b = 0; b < nc; b++) {
+            const int rows = 32 * (nc - b);
+            for (int e = threadIdx.x; e < 32 * rows; e += kFtThreads) {
+                const int j = 32 * b + e / rows, k = 32 * b + e % rows;
+                dst[e] = (k < s && k > j) ? cjif(P[(int64_t)j * ld + k], h) : Sc<T>::zero();
+            }
+            dst += 32 * rows;
+        }
+    }
+    __syncthreads();
+    T *Pc = P + s;
+    // two rows at a time share the loads of L's column (one where a tile has no second row per warp)
+    constexpr int R = 2;
+    if (it.z <= kFtThreads / 32) {
+        if (nc == 1) ftrsm_rows<T, 1, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
+        else if (nc == 2) ftrsm_rows<T, 2, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
+        else if (nc == 3) ftrsm_rows<T, 3, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
+        else ftrsm_rows<T, 4, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
+    } else {
+        if (nc == 1) ftrsm_rows<T, 1, R>(Ls, rD, Pc, ld, s, it.y, it.z);
+        else if (nc == 2) ftrsm_rows<T, 2, R>(Ls, rD, Pc, ld, s, it.y, it.z);
+        else if (nc == 3) ftrsm_rows<T, 3, R>(Ls, rD, Pc, ld, s, it.y, it.z);
+        else ftrsm_rows<T, 4, R>(Ls, rD, Pc, ld, s, it.y, it.z);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_fsmall: a whole narrow supernode (s <= kFSmallS columns, its panel twice
+// in shared memory): LDL^T of the diagonal block and the rows of C together,
+// column by column (one barrier each), then U_J -= (L D) L^T over exactly the
+// entries of the lower triangle, 2 x 2 per thread.  One launch where the
+// blocks' own kernels would each be launch-bound, and no 64 x 64 x 16 tile
+// for a 20 x 20 x 3 product.
+// ---------------------------------------------------------------------------
+constexpr int kFsThreads = 128;
+
+template <typename T>
+__global__ void __launch_bounds__(kFsThreads) k_fsmall(const FactorDesc *__restrict__ fd, const int *__restrict__ js,
+                                                       int nj) {
+    grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int w = blockIdx.x;
+    if (w >= nj) return;
+    const FactorDesc &F = *fd;
+    const int J = js[w];
+    const int fc = F.super_ptr[J];
+    const int s = F.super_ptr[J + 1] - fc;
+    const int ld = (int)(F.rowptr[J + 1] - F.rowptr[J]);
+    const int c = ld - s;
+    T *P = static_cast<T *>(F.L) + F.panel_off[J];
+    T *D = static_cast<T *>(F.D) + fc;
+    const bool herm = F.herm != 0;
+    T *Y = reinterpret_cast<T *>(smem_raw);   // [s][ld] columns: the panel, then y = l d
+    T *Lp = Y + s * ld;                       // [s][ld] columns of L
+    const int tid = threadIdx.x;
+    for (int e = tid; e < s * ld; e += kFsThreads) Y[e] = P[e];
     for (int j = 0; j < s; j++) {
-        T acc = P[(int64_t)j * ld + r];
-        for (int k = 0; k < j; k++) msub(acc, mul(P[(int64_t)k * ld + r], D[k]), cjif(P[(int64_t)k * ld + j], h));
-        P[(int64_t)j * ld + r] = mul(acc, recip(D[j]));
+        __syncthreads();                      // column j is final on the rows of the diagonal block
+        const T d = Y[j * ld + j];
+        const T r = recip(d);
+        if (tid == 0) {
+            if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
+            D[j] = d;
+        }
+        for (int i = j + 1 + tid; i < ld; i += kFsThreads) {
+            const T l = mul(Y[j * ld + i], r);
+            Lp[j * ld + i] = l;
+            for (int k = j + 1; k < s && k <= i; k++) msub(Y[k * ld + i], l, cjif(Y[j * ld + k], herm));
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < s * ld; e += kFsThreads) {
+        const int j = e / ld, i = e % ld;
+        P[e] = i > j ? Lp[e] : (i == j ? Sc<T>::one() : Sc<T>::zero());
+    }
+    // U_J(p, q) -= sum_k y_p l_q, p >= q, in 2 x 2 blocks of the lower triangle
+    T *UJ = static_cast<T *>(F.U) + F.u_off[J];
+    const int nt = (c + 1) / 2;
+    int tj = 0, ti = tid;                     // block row ti (from the diagonal on) of block column tj
+    while (tj < nt) {
+        if (ti >= nt - tj) {
+            ti -= nt - tj;
+            tj++;
+            continue;
+        }
+        const int p = 2 * (tj + ti), q = 2 * tj;
+        const bool p1 = p + 1 < c, q1 = q + 1 < c;
+        T a00 = Sc<T>::zero(), a10 = Sc<T>::zero(), a01 = Sc<T>::zero(), a11 = Sc<T>::zero();
+        for (int k = 0; k < s; k++) {
+            const T *yk = Y + k * ld + s, *lk = Lp + k * ld + s;
+            const T y0 = yk[p], y1 = p1 ? yk[p + 1] : Sc<T>::zero();
+            const T l0 = cjif(lk[q], herm), l1 = q1 ? cjif(lk[q + 1], herm) : Sc<T>::zero();
+            madd(a00, y0, l0);
+            madd(a10, y1, l0);
+            madd(a01, y0, l1);
+            madd(a11, y1, l1);
+        }
+        T *u = UJ + (int64_t)q * c + p;
+        u[0] = sub(u[0], a00);
+        if (p1) u[1] = sub(u[1], a10);
+        if (q1 && p > q) u[c] = sub(u[c], a01);
+        if (p1 && q1) u[c + 1] = sub(u[c + 1], a11);
+        ti += kFsThreads;
     }
 }
 
@@ -194,18 +458,68 @@ int factor_tables(selinv_plan_s *plan) {
     const PlanData &p = plan->data;
     int rc = ensure_device(plan->data);
     if (rc) return rc;
-    // per-level launch lists, leaves first
-    f->h_tiles.clear(); f->h_js.clear();
-    f->tile_lptr.assign(1, 0); f->j_lptr.assign(1, 0);
+    // per-level launch lists, leaves first: the narrow supernodes, then the
+    // others' diagonal blocks and row tiles
+    f->lev.clear();
+    std::vector<int> js;
+    std::vector<int4> tiles, uitems;
+    auto width = [&](int32_t J) { return p.super_ptr[J + 1] - p.super_ptr[J]; };
+    auto below = [&](int32_t J) { return (int)(p.rowptr[J + 1] - p.rowptr[J]) - width(J); };
     for (int l = p.nlevels - 1; l >= 0; l--) {
+        FactorLevel v;
+        std::vector<int32_t> wide;
+        v.small0 = (int64_t)js.size();
         for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
             const int32_t J = p.level_list[e];
-            const int64_t ld = p.rowptr[J + 1] - p.rowptr[J];
-            for (int64_t t = 0; t < (ld + kFT - 1) / kFT; t++) f->h_tiles.push_back(make_int2(J, (int)t));
-            f->h_js.push_back(J);
+            const int s = width(J), elems = s * (s + below(J));
+            if (s <= kFSmallS && elems <= kFSmallElems) {
+                js.push_back(J);
+                v.small_elems = std::max(v.small_elems, elems);
+            } else {
+                wide.push_back(J);
+            }
         }
-        f->tile_lptr.push_back((int64_t)f->h_tiles.size());
-        f->j_lptr.push_back((int64_t)f->h_js.size());
+        v.wide0 = (int64_t)js.size();
+        v.wide1 = v.wide0 + (int64_t)wide.size();
+        js.insert(js.end(), wide.begin(), wide.end());
+        int64_t rows = 0;
+        for (int32_t J : wide) {
+            v.wide_s = std::max(v.wide_s, width(J));
+            rows += below(J);
+        }
+        // a cluster of 8 CTAs per diagonal block while all of them find an SM
+        // (one 128-column block: 54 us on 8 SMs, 127 on one); wide levels
+        // have blocks enough by themselves
+        const int64_t nw = (int64_t)wide.size();
+        v.cl = v.wide_s <= 32 ? 1 : (nw * 8 <= 152 ? 8 : (nw * 4 <= 152 ? 4 : (nw * 2 <= 152 ? 2 : 1)));
+        // row tiles: 4 rows (a row per warp) and more as the level's rows cover every SM
+        const int rt = (int)std::min<int64_t>(64, std::max<int64_t>(4, (rows / 152 + 3) / 4 * 4));
+        v.tile0 = (int64_t)tiles.size();
+        for (int32_t J : wide)
+            for (int r = 0, c = below(J); r < c; r += rt) tiles.push_back(make_int4(J, r, std::min(rt, c - r), 0));
+        v.tile1 = (int64_t)tiles.size();
+        // update tiles: the side (64, 32, 16) whose waves over the SMs multiply least
+        int64_t best = INT64_MAX;
+        for (int B : {64, 32, 16}) {
+            int64_t nt = 0;
+            for (int32_t J : wide) {
+                const int64_t t = (below(J) + B - 1) / B;
+                nt += t * (t + 1) / 2;
+            }
+            const int64_t cost = (nt + 151) / 152 * (B * B + 4 * B);
+            if (cost < best) {
+                best = cost;
+                v.ub = B;
+            }
+        }
+        v.u0 = (int64_t)uitems.size();
+        for (int32_t J : wide) {
+            const int nt = (below(J) + v.ub - 1) / v.ub;
+            for (int ti = 0; ti < nt; ti++)
+                for (int tj = 0; tj <= ti; tj++) uitems.push_back(make_int4(J, ti, tj, 0));
+        }
+        v.u1 = (int64_t)uitems.size();
+        f->lev.push_back(v);
     }
     // update matrices: offsets; the position of every C_K entry in its
     // parent's row list (closure: C_K lies inside rows(parent)); children by rank
@@ -236,9 +550,8 @@ int factor_tables(selinv_plan_s *plan) {
     std::vector<int32_t> kids(std::max<int64_t>(kid_ptr[p.ns], 1));
     for (int32_t K = 0; K < p.ns; K++)
         if (p.sparent[K] >= 0) kids[kid_ptr[p.sparent[K]] + rank[K]] = K;
-    f->asm_items.clear(); f->uitems.clear();
+    f->asm_items.clear();
     f->asm_lptr.assign(1, 0);
-    f->u_lptr.assign(1, 0);
     for (int l = p.nlevels - 1; l >= 0; l--) {
         for (int r = 0; r < f->npass; r++) {
             for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
@@ -250,19 +563,11 @@ int factor_tables(selinv_plan_s *plan) {
             }
             f->asm_lptr.push_back((int64_t)f->asm_items.size());
         }
-        for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
-            const int32_t K = p.level_list[e];
-            const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - (p.super_ptr[K + 1] - p.super_ptr[K]);
-            const int nt = (int)((c + kSegB - 1) / kSegB);
-            for (int ti = 0; ti < nt; ti++)
-                for (int tj = 0; tj <= ti; tj++) f->uitems.push_back(make_int4(K, ti, tj, 0));
-        }
-        f->u_lptr.push_back((int64_t)f->uitems.size());
     }
-    if ((rc = up(&f->d_tiles, f->h_tiles))) return rc;
-    if ((rc = up(&f->d_js, f->h_js))) return rc;
+    if ((rc = up(&f->d_tiles, tiles))) return rc;
+    if ((rc = up(&f->d_js, js))) return rc;
     if ((rc = up(&f->d_asm, f->asm_items))) return rc;
-    if ((rc = up(&f->d_uitems, f->uitems))) return rc;
+    if ((rc = up(&f->d_uitems, uitems))) return rc;
     if ((rc = up(&f->d_uoff, f->u_off))) return rc;
     if ((rc = up(&f->d_chpos, f->chpos))) return rc;
     if (cudaMalloc((void **)&f->d_desc, sizeof(FactorDesc)) != cudaSuccess) return SELINV_ERR_OOM;
@@ -289,6 +594,16 @@ FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, 
     return f->d_desc;
 }
 
+// the dynamic shared memory of the widest blocks, on the plan's device
+template <typename T> static cudaError_t configure_factor_kernels() {
+    const int diag = (int)(sizeof(T) * (size_t)(2 * 128 * kFdLd + fd_rows_elems(128, 1)));
+    const int trsm = (int)(sizeof(T) * (size_t)ft_store_elems(128)), small = (int)(2 * sizeof(T) * kFSmallElems);
+    cudaError_t e = cudaFuncSetAttribute(k_fdiag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, diag);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ftrsm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, trsm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fsmall<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
+    return e;
+}
+
 template <typename T>
 static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaStream_t st, int herm) {
     FactorData *f = plan->factor;
@@ -309,20 +624,51 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         k_assemble<T><<<blocks, 256, 0, st>>>(f->d_a_pos, static_cast<const T *>(A), f->nnzA, static_cast<T *>(L));
         note_launch();
     }
-    const int nl = (int)f->tile_lptr.size() - 1;
-    for (int l = 0; l < nl; l++) {
+    if (!f->configured[sizeof(T) > 8]) {
+        if (configure_factor_kernels<T>() != cudaSuccess) return SELINV_ERR_CUDA;
+        f->configured[sizeof(T) > 8] = true;
+    }
+    for (size_t l = 0; l < f->lev.size(); l++) {
         // the children's update matrices complete J's panel and start U_J
         for (int r = 0; r < f->npass; r++) {
             const int64_t x0 = f->asm_lptr[l * f->npass + r], x1 = f->asm_lptr[l * f->npass + r + 1];
             if (x1 > x0) { k_fasm<T><<<(int)(x1 - x0), 256, 0, st>>>(fd, f->d_asm + x0, (int)(x1 - x0)); note_launch(); }
         }
-        const int64_t t0 = f->tile_lptr[l], t1 = f->tile_lptr[l + 1];
-        const int64_t j0 = f->j_lptr[l], j1 = f->j_lptr[l + 1];
-        const int64_t u0 = f->u_lptr[l], u1 = f->u_lptr[l + 1];
-        if (j1 > j0) k_fdiag<T><<<(int)(j1 - j0), 256, 0, st>>>(fd, f->d_js + j0, (int)(j1 - j0));
-        if (t1 > t0) k_ftrsm<T><<<(int)(t1 - t0), kFT, 0, st>>>(fd, f->d_tiles + t0, (int)(t1 - t0));
-        if (u1 > u0) k_fupd<T><<<(int)(u1 - u0), 256, 0, st>>>(fd, f->d_uitems + u0, (int)(u1 - u0));
-        note_launch(3);
+        const FactorLevel &v = f->lev[l];
+        if (v.wide0 > v.small0) {
+            k_fsmall<T><<<(int)(v.wide0 - v.small0), kFsThreads, 2 * sizeof(T) * (size_t)v.small_elems, st>>>(
+                fd, f->d_js + v.small0, (int)(v.wide0 - v.small0));
+            note_launch();
+        }
+        if (v.wide1 > v.wide0) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)((v.wide1 - v.wide0) * v.cl));
+            cfg.blockDim = dim3(kFdThreads);
+            cfg.dynamicSmemBytes = sizeof(T) * (size_t)(2 * 128 * kFdLd + fd_rows_elems(v.wide_s, v.cl));
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)v.cl;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            if (cudaLaunchKernelEx(&cfg, k_fdiag<T>, (const FactorDesc *)fd, (const int *)(f->d_js + v.wide0),
+                                   (int)(v.wide1 - v.wide0)) != cudaSuccess)
+                return SELINV_ERR_CUDA;
+            note_launch();
+        }
+        if (v.tile1 > v.tile0) {
+            k_ftrsm<T><<<(int)(v.tile1 - v.tile0), kFtThreads, sizeof(T) * (size_t)ft_store_elems(v.wide_s), st>>>(
+                fd, f->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
+            note_launch();
+        }
+        if (v.u1 > v.u0) {
+            const int nu = (int)(v.u1 - v.u0);
+            if (v.ub == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, f->d_uitems + v.u0, nu);
+            else if (v.ub == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, f->d_uitems + v.u0, nu);
+            else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, f->d_uitems + v.u0, nu);
+            note_launch();
+        }
     }
     return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
 }

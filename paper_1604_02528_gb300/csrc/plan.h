@@ -230,16 +230,26 @@ struct FactorDesc {
     int herm;                 // complex Hermitian: A = L D L^H
 };
 
+// Launch lists of one level of the factorization (ranges into the device lists).
+struct FactorLevel {
+    int64_t small0 = 0, wide0 = 0, wide1 = 0;   // narrow supernodes [small0, wide0), the others [wide0, wide1)
+    int64_t tile0 = 0, tile1 = 0;               // row tiles of the others
+    int64_t u0 = 0, u1 = 0;                     // update tiles of the others
+    int small_elems = 0;                        // largest panel of the narrow ones
+    int wide_s = 0;                             // widest of the others
+    int cl = 1;                                 // CTAs per diagonal block
+    int ub = 64;                                // side of an update tile
+};
+
 struct FactorData {
     int32_t n = -1;
     int64_t nnzA = 0;
     std::vector<int64_t> a_pos;       // panel position of every stored entry of A
     int64_t *d_a_pos = nullptr;
     // launch lists, leaves first
-    std::vector<int2> h_tiles;        // (J, row tile) per level
-    std::vector<int> h_js;            // J per level
-    std::vector<int64_t> tile_lptr, j_lptr;
-    int2 *d_tiles = nullptr;
+    std::vector<FactorLevel> lev;
+    bool configured[2] = {false, false};   // kernel attributes set (real, complex)
+    int4 *d_tiles = nullptr;          // (J, first row of C, rows)
     int *d_js = nullptr;
     // update matrices (multifrontal hand-off from child to parent; shared
     // with the selected-inversion adjoint)
@@ -248,10 +258,8 @@ struct FactorData {
     std::vector<int2> asm_items;      // (child, kAsmChunk-entry chunk) per level and child rank
     std::vector<int64_t> asm_lptr;    // [level * npass + rank]
     int npass = 1;
-    std::vector<int4> uitems;         // (K, row tile, column tile) of the lower c x c, per level
-    std::vector<int64_t> u_lptr;
     int2 *d_asm = nullptr;
-    int4 *d_uitems = nullptr;
+    int4 *d_uitems = nullptr;         // (K, row tile, column tile) of the lower c x c
     int64_t *d_uoff = nullptr;
     int32_t *d_chpos = nullptr;
     void *U = nullptr;

@@ -1,0 +1,62 @@
+"""The factorization's kernels at the edges of their ranges: supernode widths
+around the narrow kernel's limit, the 8-column panels and the 32-column
+blocks, and levels with few to many diagonal blocks (clusters of 8 to 1 CTAs).
+
+Tolerance: the matrices are diagonally dominant, so the entries of L are at
+most 1 and an entry's error is a sum of at most n = 300 rounded products,
+n 2^-53 = 3e-14 of the largest; 1e-12 leaves room for the oracle's own."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _blocks(count, size, kind, seed):
+    """`count` dense diagonal blocks of `size` columns."""
+    rng = np.random.default_rng(seed)
+    colptr, rows, vals = [0], [], []
+    for b in range(count):
+        g = rng.standard_normal((size, size)) + (1j * rng.standard_normal((size, size)) if kind != "f64" else 0)
+        a = (g + (g.conj().T if kind == "c128h" else g.T)) / 2
+        np.fill_diagonal(a, np.abs(a).sum(axis=1) + 1.0)
+        for j in range(size):
+            rows.append(np.arange(b * size + j, (b + 1) * size))
+            vals.append(a[j:, j])
+            colptr.append(colptr[-1] + size - j)
+    return synth.Problem(f"blocks{count}x{size}", count * size, np.array(colptr, np.int64),
+                         np.concatenate(rows).astype(np.int32), np.concatenate(vals), np.arange(count * size),
+                         dict(synth.problems.RELAXED_128), {"hermitian": kind == "c128h"})
+
+
+def _check(p):
+    import torch
+    from paper_1604_02528_gb300.api import SelInvContext
+    ctx = SelInvContext.from_problem(p)
+    sym = oracle.symbolic_for(p)
+    L0, D0 = oracle.ldlt(p, sym)
+    L, D = ctx.factor(torch.from_numpy(p.values).cuda())
+    torch.cuda.synchronize()
+    assert ctx.status() == 0
+    r, c, _ = oracle.panel_entries(sym)
+    Lg = L.cpu().numpy()
+    assert np.abs(D.cpu().numpy() - D0).max() <= 1e-12 * np.abs(D0).max()
+    assert np.abs(np.where(r > c, Lg - L0, 0)).max() <= 1e-12
+    assert np.all(Lg[r == c] == 1) and np.all(Lg[r < c] == 0)
+
+
+@pytest.mark.parametrize("kind", ["f64", "c128", "c128h"])
+@pytest.mark.parametrize("width", [1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 65, 100, 127, 128])
+def test_widths(native, cuda_device, width, kind):
+    p = _blocks(1, 2 * width + 5, kind, width)
+    p.supernodes = {"kind": "fundamental", "cap": width, "fill": 0.0}
+    _check(p)
+
+
+@pytest.mark.parametrize("count,size", [(1, 40), (19, 40), (20, 40), (39, 33), (77, 40), (160, 33)])
+def test_levels_of_many_blocks(native, cuda_device, count, size):
+    _check(_blocks(count, size, "f64", count))
+    if count in (1, 160):
+        _check(_blocks(count, size, "c128", count))
