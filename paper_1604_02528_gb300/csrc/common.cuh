@@ -176,6 +176,16 @@ __device__ __forceinline__ GatherCheck gather_check(const ProbDesc &P) {
     return g;
 }
 
+// one element copied to shared memory without passing a register
+template <typename T>
+__device__ __forceinline__ void cp_async_elem(T *smem, const T *g) {
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+    if constexpr (sizeof(T) == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(g));
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(g));
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
+
 // atomicMax on a shared slot that every active lane of the warp targets: one
 // atomic per warp instead of one per lane (the lanes would serialize on it)
 __device__ __forceinline__ void warp_uniform_atomic_max(int *slot, int v) {

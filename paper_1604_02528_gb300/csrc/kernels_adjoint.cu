@@ -34,6 +34,7 @@
 #include "launch.h"
 #include "nvtx.h"
 #include "plan.h"
+#include "digit_rows.cuh"
 #include "fixedpoint.cuh"
 #include "tile_gemm.cuh"
 #include "seg_update.cuh"
@@ -470,62 +471,22 @@ __global__ void __launch_bounds__(256) k_small_digits(const AdjDesc *__restrict_
 }
 
 // Digit planes of [Ybar, Lhat] (rows p of C, the 2s columns k) for the SYRK
-// update of the transposed tcgen05 kernel: per block of 128 rows, per
-// 16-step of k the 7 planes of 128 x 16 one after the other (K-major 8 x 8
-// core matrices), one exponent per row (at its row position in syexp).  One
-// CTA per 32 rows: a warp per 4 rows finds their exponents, then each thread
-// cuts 8 consecutive k of one row, a 16-byte store per plane.
-// work: (K, 32-row block).
+// update of the transposed tcgen05 kernel (digit_rows).  work: (K, 32-row block).
 __global__ void __launch_bounds__(256) k_syrk_digits(const AdjDesc *__restrict__ ad, const int2 *__restrict__ work,
                                                      int nwork, uint16_t *__restrict__ sy,
                                                      const int64_t *__restrict__ sy_off, int *__restrict__ syexp) {
     grid_dep_wait();
-    __shared__ int rowE[32];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int w = blockIdx.x;
     if (w >= nwork) return;
     const AdjDesc &A = *ad;
     const int K = work[w].x, b = work[w].y;
     const int s = A.super_ptr[K + 1] - A.super_ptr[K];
     const int64_t ld = A.rowptr[K + 1] - A.rowptr[K];
-    const int c = (int)(ld - s);
     const int64_t off = A.panel_off[K];
-    const int kw = 2 * s, k16 = (kw + 15) / 16 * 16, nst = k16 / 16;
     auto x = [&](int p, int k) -> double {   // [Ybar, Lhat](p, k)
         return k < s ? A.YB[off + (int64_t)k * ld + s + p] : A.LD[off + (int64_t)(k - s) * ld + s + p];
     };
-    for (int rr = 0; rr < 4; rr++) {
-        const int r = warp * 4 + rr, p = b * 32 + r;
-        int E = 0;
-        if (p < c)
-            for (int k = lane; k < kw; k += 32) E = max(E, bexp(x(p, k)));
-#pragma unroll
-        for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-        if (lane == 0) {
-            rowE[r] = E;
-            if (p < c) syexp[A.rowptr[K] + s + p] = E;
-        }
-    }
-    __syncthreads();
-    uint16_t *base = sy + sy_off[K];
-    for (int e = threadIdx.x; e < 32 * (k16 / 8); e += 256) {
-        const int r = e % 32, k0 = (e / 32) * 8, p = b * 32 + r;
-        if (p >= c) continue;
-        uint32_t h[kDig][4];
-#pragma unroll
-        for (int t = 0; t < 8; t += 2) {
-            int d0[kDig], d1[kDig];
-            digits7(k0 + t < kw ? x(p, k0 + t) : 0.0, rowE[r], d0);
-            digits7(k0 + t + 1 < kw ? x(p, k0 + t + 1) : 0.0, rowE[r], d1);
-#pragma unroll
-            for (int i = 0; i < kDig; i++) h[i][t / 2] = f16_of_int(d0[i]) | (f16_of_int(d1[i]) << 16);
-        }
-        const int t1 = p / 128, r128 = p % 128, st = k0 / 16;
-        const int64_t ub = ((int64_t)(t1 * nst + st) * kDig) * 128 * 16 + (r128 / 8) * 128 + ((k0 % 16) / 8) * 64 + (r128 % 8) * 8;
-#pragma unroll
-        for (int i = 0; i < kDig; i++)
-            *reinterpret_cast<uint4 *>(base + ub + (int64_t)i * 128 * 16) = make_uint4(h[i][0], h[i][1], h[i][2], h[i][3]);
-    }
+    digit_rows(x, 2 * s, (int)(ld - s), b, sy + sy_off[K], syexp + A.rowptr[K] + s);
 }
 
 // The k16 stage of a row-product block: thread (tx, ty) adds rows ty + 16 i
@@ -1815,7 +1776,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
             }
             const int64_t z0 = a->sy_lptr[li], z1 = a->sy_lptr[li + 1];
             if (z1 > z0) {
-                launch_syrk_tcw(a->d_sydesc, a->d_sy + z0, (int)(z1 - z0), a->tcs.spin_limit, st);
+                launch_syrk_tcw(1, a->d_sydesc, a->d_sy + z0, (int)(z1 - z0), a->tcs.spin_limit, st);
                 note_launch();
             }
             const int d0 = (int)a->dig_lptr[li], d1 = (int)a->dig_lptr[li + 1];

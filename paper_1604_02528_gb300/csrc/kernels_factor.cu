@@ -12,7 +12,9 @@
 //   k_fsmall    a whole narrow supernode: the next three steps at once
 //   k_fdiag     dense LDL^T of J's diagonal block in place (a cluster of CTAs)
 //   k_ftrsm     L(C,J) = A(C,J) L_JJ^{-T} D_J^{-1}, row tiles
-//   k_fupd      U_J -= L_CJ D_J L_CJ^T (lower c x c, tiles)
+//   k_fupd      U_J -= L_CJ D_J L_CJ^T (lower c x c, tiles); large real ones
+//               on the tensor cores: k_fupd_digits (digit planes of L_CJ D_J)
+//               and the SYRK mode of the transposed tcgen05 kernel
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -20,6 +22,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "digit_rows.cuh"
 #include "launch.h"
 #include "nvtx.h"
 #include "plan.h"
@@ -31,6 +34,10 @@ namespace cg = cooperative_groups;
 
 constexpr int kFSmallS = 16;        // widest supernode of k_fsmall
 constexpr int kFSmallElems = 3400;  // ... and its largest panel (both copies of a complex one in 109 KB)
+// narrowest supernode and shortest C of the tcgen05 update: one of its
+// CTAs takes about as long as the FP64 pipe of an SM needs for 16 columns of
+// a 128 x 64 tile, and below 96 rows most of that tile is padding
+constexpr int kFTcS = 17, kFTcC = 96;
 
 template <typename T>
 __global__ void k_assemble(const int64_t *__restrict__ pos, const T *__restrict__ vals, int64_t nnz,
@@ -99,6 +106,23 @@ __global__ void __launch_bounds__(256) k_fupd(const FactorDesc *__restrict__ fd,
         *dst = sub(*dst, v);
     };
     seg_update<T, decltype(x), decltype(y), decltype(out), B>(pa, np, st, nq, sJ, x, y, out, sm);
+}
+
+// Digit planes of the rows of L_CJ D_J (undivided rows of the panel solve, up
+// to rounding) for the tcgen05 form of the update.  work: (J, 32-row block).
+__global__ void __launch_bounds__(256) k_fupd_digits(const FactorDesc *__restrict__ fd, const int2 *__restrict__ work,
+                                                     int nwork) {
+    grid_dep_wait();
+    const int w = blockIdx.x;
+    if (w >= nwork) return;
+    const FactorDesc &F = *fd;
+    const int J = work[w].x, b = work[w].y;
+    const int s = F.super_ptr[J + 1] - F.super_ptr[J];
+    const int64_t ld = F.rowptr[J + 1] - F.rowptr[J];
+    const double *LC = static_cast<const double *>(F.L) + F.panel_off[J] + s;
+    const double *DJ = static_cast<const double *>(F.D) + F.super_ptr[J];
+    auto x = [&](int p, int k) -> double { return LC[(int64_t)k * ld + p] * DJ[k]; };
+    digit_rows(x, s, (int)(ld - s), b, F.up.linvd + F.up.linvd_off[J], F.up.linvexp + F.rowptr[J] + s);
 }
 
 // ---------------------------------------------------------------------------
@@ -173,8 +197,10 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
     for (int k = tid / 32; k < s; k += kFdThreads / 32)
         for (int lr = tid % 32; lr < 4 * myg; lr += 32) {
             const int i = row_of(lr);
-            if (i < s && k <= i) A[off(i) + k] = P[(int64_t)k * ld + i];
+            if (i < s && k <= i) cp_async_elem(A + off(i) + k, P + (int64_t)k * ld + i);
         }
+    cp_async_commit();
+    cp_async_wait<0>();
     for (int b0 = 0; b0 < s; b0 += kFdNB) {
         const int nb = s - b0 < kFdNB ? s - b0 : kFdNB;
         cl.sync();
@@ -214,15 +240,22 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
         }
         // own rows of the trailing block: a_ik -= l_i y_k, columns b1 .. i of row i
         const int b1 = b0 + kFdNB;
-        int lr = 0, q = tid;                           // q-th column of local row lr
-        while (lr < 4 * myg) {
+        // -- entries dealt to the threads one by one (the FP64 pipe bounds the
+        // update, and an idle lane costs as much as a busy one), all lanes of a
+        // warp brought to their entry before the products start
+        int total = 0;
+        for (int lr = 0; lr < 4 * myg; lr++) {
             const int r = row_of(lr);
-            const int cnt = r < s && r >= b1 ? r - b1 + 1 : 0;
-            if (q >= cnt) {
+            total += r < s && r >= b1 ? r - b1 + 1 : 0;
+        }
+        int lr = 0, q = tid, r = row_of(0), cnt = r < s && r >= b1 ? r - b1 + 1 : 0;
+        for (int e = tid; e < total; e += kFdThreads) {
+            while (q >= cnt) {                         // to the q-th column of local row lr
                 q -= cnt;
-                lr++;
-                continue;
+                r = row_of(++lr);
+                cnt = r < s && r >= b1 ? r - b1 + 1 : 0;
             }
+            __syncwarp(__activemask());
             T *dst = A + off(r) + b1 + q;
             T acc = *dst;
             const T *lrow = Lp + (r - b0) * kFdLd, *yrow = Yp + (b1 + q - b0) * kFdLd;
@@ -260,7 +293,7 @@ template <> __device__ __forceinline__ zd shfl_elem(zd v, int src) {
 }
 
 template <typename T, int NC, int R>
-__device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, int row0, int nrows) {
+__device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, int row0, int nrows, bool herm) {
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
     for (int g = warp * R; g < nrows; g += kFtThreads / 32 * R) {
         T a[R][NC];
@@ -278,7 +311,7 @@ __device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, in
             for (int jj = 0; jj < 32; jj++) {
                 T l[NC];
 #pragma unroll
-                for (int t = b; t < NC; t++) l[t] = Lb[jj * 32 * (NC - b) + lane + 32 * (t - b)];
+                for (int t = b; t < NC; t++) l[t] = cjif(Lb[jj * 32 * (NC - b) + lane + 32 * (t - b)], herm);
 #pragma unroll
                 for (int r = 0; r < R; r++) {
                     const T y = shfl_elem(a[r][b], jj);
@@ -325,25 +358,28 @@ __global__ void __launch_bounds__(kFtThreads) k_ftrsm(const FactorDesc *__restri
             const int rows = 32 * (nc - b);
             for (int e = threadIdx.x; e < 32 * rows; e += kFtThreads) {
                 const int j = 32 * b + e / rows, k = 32 * b + e % rows;
-                dst[e] = (k < s && k > j) ? cjif(P[(int64_t)j * ld + k], h) : Sc<T>::zero();
+                if (k < s && k > j) cp_async_elem(dst + e, P + (int64_t)j * ld + k);
+                else dst[e] = Sc<T>::zero();
             }
             dst += 32 * rows;
         }
+        cp_async_commit();
+        cp_async_wait<0>();
     }
     __syncthreads();
     T *Pc = P + s;
     // two rows at a time share the loads of L's column (one where a tile has no second row per warp)
     constexpr int R = 2;
     if (it.z <= kFtThreads / 32) {
-        if (nc == 1) ftrsm_rows<T, 1, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
-        else if (nc == 2) ftrsm_rows<T, 2, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
-        else if (nc == 3) ftrsm_rows<T, 3, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
-        else ftrsm_rows<T, 4, 1>(Ls, rD, Pc, ld, s, it.y, it.z);
+        if (nc == 1) ftrsm_rows<T, 1, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+        else if (nc == 2) ftrsm_rows<T, 2, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+        else if (nc == 3) ftrsm_rows<T, 3, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+        else ftrsm_rows<T, 4, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
     } else {
-        if (nc == 1) ftrsm_rows<T, 1, R>(Ls, rD, Pc, ld, s, it.y, it.z);
-        else if (nc == 2) ftrsm_rows<T, 2, R>(Ls, rD, Pc, ld, s, it.y, it.z);
-        else if (nc == 3) ftrsm_rows<T, 3, R>(Ls, rD, Pc, ld, s, it.y, it.z);
-        else ftrsm_rows<T, 4, R>(Ls, rD, Pc, ld, s, it.y, it.z);
+        if (nc == 1) ftrsm_rows<T, 1, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+        else if (nc == 2) ftrsm_rows<T, 2, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+        else if (nc == 3) ftrsm_rows<T, 3, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+        else ftrsm_rows<T, 4, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
     }
 }
 
@@ -400,12 +436,12 @@ __global__ void __launch_bounds__(kFsThreads) k_fsmall(const FactorDesc *__restr
     T *UJ = static_cast<T *>(F.U) + F.u_off[J];
     const int nt = (c + 1) / 2;
     int tj = 0, ti = tid;                     // block row ti (from the diagonal on) of block column tj
-    while (tj < nt) {
-        if (ti >= nt - tj) {
+    for (int e = tid; e < nt * (nt + 1) / 2; e += kFsThreads) {
+        while (ti >= nt - tj) {
             ti -= nt - tj;
             tj++;
-            continue;
         }
+        __syncwarp(__activemask());           // all lanes at their block before the products start
         const int p = 2 * (tj + ti), q = 2 * tj;
         const bool p1 = p + 1 < c, q1 = q + 1 < c;
         T a00 = Sc<T>::zero(), a10 = Sc<T>::zero(), a01 = Sc<T>::zero(), a11 = Sc<T>::zero();
@@ -436,6 +472,7 @@ void factor_release(selinv_plan_s *plan) {
     auto fr = [](void *p) { if (p) cudaFree(p); };
     fr(f->d_a_pos); fr(f->d_tiles); fr(f->d_js); fr(f->d_desc);
     fr(f->d_asm); fr(f->d_uitems); fr(f->d_uoff); fr(f->d_chpos); fr(f->U);
+    fr(f->d_tcitems); fr(f->d_tcwork); fr(f->d_digoff); fr(f->digits); fr(f->digexp);
     adjoint_release(f->adj);
     delete f;
     plan->factor = nullptr;
@@ -463,6 +500,9 @@ int factor_tables(selinv_plan_s *plan) {
     f->lev.clear();
     std::vector<int> js;
     std::vector<int4> tiles, uitems;
+    std::vector<Item> tcitems;
+    std::vector<int2> tcwork;
+    std::vector<int64_t> digoff(std::max(p.ns, 1), 0);
     auto width = [&](int32_t J) { return p.super_ptr[J + 1] - p.super_ptr[J]; };
     auto below = [&](int32_t J) { return (int)(p.rowptr[J + 1] - p.rowptr[J]) - width(J); };
     for (int l = p.nlevels - 1; l >= 0; l--) {
@@ -498,27 +538,50 @@ int factor_tables(selinv_plan_s *plan) {
         for (int32_t J : wide)
             for (int r = 0, c = below(J); r < c; r += rt) tiles.push_back(make_int4(J, r, std::min(rt, c - r), 0));
         v.tile1 = (int64_t)tiles.size();
-        // update tiles: the side (64, 32, 16) whose waves over the SMs multiply least
-        int64_t best = INT64_MAX;
-        for (int B : {64, 32, 16}) {
-            int64_t nt = 0;
+        // update tiles: the side (64, 32, 16) whose waves over the SMs multiply
+        // least, for all of them and for those that the tcgen05 form leaves
+        auto tc = [&](int32_t J) { return width(J) >= kFTcS && below(J) >= kFTcC; };
+        for (int part = 0; part < 2; part++) {
+            FactorLevel::Upd &u = v.upd[part];
+            int64_t best = INT64_MAX;
+            for (int B : {64, 32, 16}) {
+                int64_t nt = 0;
+                for (int32_t J : wide) {
+                    const int64_t t = part && tc(J) ? 0 : (below(J) + B - 1) / B;
+                    nt += t * (t + 1) / 2;
+                }
+                const int64_t cost = (nt + 151) / 152 * (B * B + 4 * B);
+                if (cost < best) {
+                    best = cost;
+                    u.b = B;
+                }
+            }
+            u.i0 = (int64_t)uitems.size();
             for (int32_t J : wide) {
-                const int64_t t = (below(J) + B - 1) / B;
-                nt += t * (t + 1) / 2;
+                if (part && tc(J)) continue;
+                const int nt = (below(J) + u.b - 1) / u.b;
+                for (int ti = 0; ti < nt; ti++)
+                    for (int tj = 0; tj <= ti; tj++) uitems.push_back(make_int4(J, ti, tj, 0));
             }
-            const int64_t cost = (nt + 151) / 152 * (B * B + 4 * B);
-            if (cost < best) {
-                best = cost;
-                v.ub = B;
-            }
+            u.i1 = (int64_t)uitems.size();
         }
-        v.u0 = (int64_t)uitems.size();
+        // tcgen05 form: 128 x 64 tiles on or below the diagonal, the digit
+        // planes of a level one after the other in one buffer
+        v.tc0 = (int64_t)tcitems.size();
+        v.tw0 = (int64_t)tcwork.size();
+        int64_t dig = 0;
         for (int32_t J : wide) {
-            const int nt = (below(J) + v.ub - 1) / v.ub;
-            for (int ti = 0; ti < nt; ti++)
-                for (int tj = 0; tj <= ti; tj++) uitems.push_back(make_int4(J, ti, tj, 0));
+            if (!tc(J)) continue;
+            const int c = below(J), n2 = (c + 63) / 64;
+            for (int m = 0; m < (c + 127) / 128; m++)
+                for (int t = 0; t < n2 && 64 * t <= 128 * m + 127; t++) tcitems.push_back(Item{0, J, m * n2 + t, 1});
+            for (int b = 0; b < (c + 31) / 32; b++) tcwork.push_back(make_int2(J, b));
+            digoff[J] = dig;
+            dig += (int64_t)((c + 127) / 128) * 7 * 128 * ((width(J) + 15) / 16 * 16);
         }
-        v.u1 = (int64_t)uitems.size();
+        v.tc1 = (int64_t)tcitems.size();
+        v.tw1 = (int64_t)tcwork.size();
+        f->dig_total = std::max(f->dig_total, dig);
         f->lev.push_back(v);
     }
     // update matrices: offsets; the position of every C_K entry in its
@@ -568,6 +631,9 @@ int factor_tables(selinv_plan_s *plan) {
     if ((rc = up(&f->d_js, js))) return rc;
     if ((rc = up(&f->d_asm, f->asm_items))) return rc;
     if ((rc = up(&f->d_uitems, uitems))) return rc;
+    if ((rc = up(&f->d_tcitems, tcitems))) return rc;
+    if ((rc = up(&f->d_tcwork, tcwork))) return rc;
+    if ((rc = up(&f->d_digoff, digoff))) return rc;
     if ((rc = up(&f->d_uoff, f->u_off))) return rc;
     if ((rc = up(&f->d_chpos, f->chpos))) return rc;
     if (cudaMalloc((void **)&f->d_desc, sizeof(FactorDesc)) != cudaSuccess) return SELINV_ERR_OOM;
@@ -577,7 +643,18 @@ int factor_tables(selinv_plan_s *plan) {
 FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, int herm) {
     FactorData *f = plan->factor;
     const PlanData &p = plan->data;
-    FactorDesc h;
+    FactorDesc h = {};
+    // the tcgen05 update's view: L's panels, digit planes of L D, the update matrices
+    h.up.super_ptr = p.d_super_ptr;
+    h.up.rowptr = p.d_rowptr;
+    h.up.panel_off = p.d_panel_off;
+    h.up.L = L;
+    h.up.linvd = f->digits;
+    h.up.linvd_off = f->d_digoff;
+    h.up.linvexp = f->digexp;
+    h.up.Yout = f->U;
+    h.up.part_off = f->d_uoff;
+    h.up.status = p.d_status;
     h.super_ptr = p.d_super_ptr;
     h.sparent = p.d_sparent;
     h.rowptr = p.d_rowptr;
@@ -615,6 +692,12 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         f->U_bytes = 0;
         if (cudaMalloc(&f->U, ubytes) != cudaSuccess) return SELINV_ERR_OOM;
         f->U_bytes = ubytes;
+    }
+    // real updates on the tensor cores unless the plan asks for FP64 FMA
+    const bool tc = sizeof(T) == 8 && p.opts.fast_contraction == 1 && f->dig_total > 0;
+    if (tc && !f->digits) {
+        if (cudaMalloc(&f->digexp, sizeof(int) * (size_t)p.rowptr[p.ns]) != cudaSuccess) return SELINV_ERR_OOM;
+        if (cudaMalloc(&f->digits, sizeof(uint16_t) * (size_t)f->dig_total) != cudaSuccess) return SELINV_ERR_OOM;
     }
     FactorDesc *fd = factor_desc(plan, L, D, st, herm);
     if (cudaMemsetAsync(L, 0, sizeof(T) * (size_t)p.nnz, st) != cudaSuccess) return SELINV_ERR_CUDA;
@@ -662,12 +745,19 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
                 fd, f->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
             note_launch();
         }
-        if (v.u1 > v.u0) {
-            const int nu = (int)(v.u1 - v.u0);
-            if (v.ub == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, f->d_uitems + v.u0, nu);
-            else if (v.ub == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, f->d_uitems + v.u0, nu);
-            else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, f->d_uitems + v.u0, nu);
+        const FactorLevel::Upd &u = v.upd[tc];
+        if (u.i1 > u.i0) {
+            const int nu = (int)(u.i1 - u.i0);
+            if (u.b == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
+            else if (u.b == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
+            else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
             note_launch();
+        }
+        if (tc && v.tc1 > v.tc0) {
+            const int nw = (int)(v.tw1 - v.tw0);
+            k_fupd_digits<<<nw, 256, 0, st>>>(fd, f->d_tcwork + v.tw0, nw);
+            launch_syrk_tcw(2, &fd->up, f->d_tcitems + v.tc0, (int)(v.tc1 - v.tc0), p.opts.spin_limit, st);
+            note_launch(2);
         }
     }
     return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;

@@ -39,15 +39,6 @@ __device__ inline void latch_status(int *status, int code) {
 constexpr int kLinvThreads = 256;
 constexpr size_t kLinvSmemMax = (128 * 129 + 128 + 64 * 128) * sizeof(double);
 
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T *smem, const T *g) {
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
-    if constexpr (sizeof(T) == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(g));
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(g));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
-
 // LU form of the normalisation (Alg. 1 first loop with U kept separately):
 // X = L_KK^{-1} and V = (U_KK^T)^{-1} (U_KK^T is the lower diagonal block of
 // Ut, non-unit diagonal) by row-oriented forward substitution, row k of V

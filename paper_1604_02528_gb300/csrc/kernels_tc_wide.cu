@@ -92,12 +92,16 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[kTcDig][8], int 
 // items: tile = (row tile * nmt + m tile) * nsplit + k-range, ntiles = nsplit;
 // nmt = ceil(rows of A / 128) (1 for real supernodes of <= 128 columns).
 //
-// SYRK: the update that the reverse pass of the gather hands to the
+// SYRK 1: the update that the reverse pass of the gather hands to the
 // ancestors, V_K -= [Ybar, Lhat] [Lhat, Ybar]^T over the 2s columns (lower
 // triangle of the c x c update matrix, its diagonal halved): A = digit
 // planes of [Ybar, Lhat] for 128 rows of C (k_syrk_digits, one exponent per
 // row), B = 64 rows of [Lhat, Ybar] sliced here; items (K, 128-row block *
 // number of 64-row blocks + 64-row block) on or below the diagonal.
+// SYRK 2: the factorization's Schur update U_K -= (L_CK D_K) L_CK^T over the s
+// columns, the same with A = digit planes of L_CK D_K and B = L_CK; a row
+// that holds an infinity or a NaN makes its results NaN (the digits cannot
+// carry it), so that a later pivot reports it.
 //
 // LHAT: the same machinery forms products of a panel's rows with an s x s
 // matrix, out(p, j) = sum_k X(p, k) B(k, j) for the rows p of C: A = digit
@@ -107,7 +111,7 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[kTcDig][8], int 
 // a single chunk, no k-split.  The forward's Lhat_{C,K} = L_{C,K} L_KK^{-1}
 // (Alg. 1, first loop; digits by k_linv_digits) goes to Lhat's slots of the
 // LD panel; the reverse passes' row products use the other prod_op modes.
-template <bool CPLX, bool LHAT = false, bool SYRK = false>
+template <bool CPLX, bool LHAT = false, int SYRK = 0>
 __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__restrict__ descs,
                                                               const Item *__restrict__ items, int nitems,
                                                               long long *__restrict__ slab, long long wait_limit) {
@@ -144,7 +148,8 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
     const int c = (int)(ld - s);
     constexpr bool DENSE = LHAT || SYRK;                 // B from dense panels
-    const int kw = SYRK ? 2 * s : (LHAT ? s : (CPLX ? 2 * c : c));   // k extent
+    constexpr bool PAIR = SYRK == 1;                     // B's k runs over two panels
+    const int kw = PAIR ? 2 * s : (DENSE ? s : (CPLX ? 2 * c : c));   // k extent
     const int mrows = SYRK ? c : (CPLX ? 2 * s : s);     // rows of A (output rows)
     // operand rows of a stored digit block (SYRK: blocks of exactly 128 rows)
     const int s64 = SYRK ? kTcM : (mrows + 63) / 64 * 64;
@@ -229,8 +234,8 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         int e = 0;
         if (p0 + r < c)
             for (int k = tid / kTwN; k < kw; k += kTwThreads / kTwN) {
-                const double *src = static_cast<const double *>(SYRK && k >= s ? P.Z : P.L);
-                e = max(e, bexp(src[P.panel_off[K] + (int64_t)(SYRK && k >= s ? k - s : k) * ld + s + p0 + r]));
+                const double *src = static_cast<const double *>(PAIR && k >= s ? P.Z : P.L);
+                e = max(e, bexp(src[P.panel_off[K] + (int64_t)(PAIR && k >= s ? k - s : k) * ld + s + p0 + r]));
             }
         if (e) atomicMax(&rowE[r], e);
     } else {
@@ -321,13 +326,13 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         };
         // DENSE: the 4 values of step i_ straight from the dense panel(s)
         const double *Lc = static_cast<const double *>(P.L) + P.panel_off[K] + s + p0 + r;   // X(p0 + r, k) = Lc[k ld]
-        const double *Zc2 = static_cast<const double *>(P.Z) + P.panel_off[K] + s + p0 + r;  // SYRK: k >= s
+        const double *Zc2 = static_cast<const double *>(P.Z) + P.panel_off[K] + s + p0 + r;  // PAIR: k >= s
         const bool rok = p0 + r < c;
         auto load_dense = [&](int i_) {
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const int k = (st0 + i_) * 16 + kq * 4 + u;
-                v[u] = (rok && i_ < n && k < kw) ? (SYRK && k >= s ? Zc2[(int64_t)(k - s) * ld] : Lc[(int64_t)k * ld]) : 0.0;
+                v[u] = (rok && i_ < n && k < kw) ? (PAIR && k >= s ? Zc2[(int64_t)(k - s) * ld] : Lc[(int64_t)k * ld]) : 0.0;
             }
         };
         auto parts = [&](int i_) {
@@ -494,11 +499,15 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         // V_K(p1, p2) -= the product, p1 >= p2, the diagonal halved (exactly:
         // one less in the scale); A's rows carry their own exponents
         double *V = static_cast<double *>(P.Yout) + P.part_off[K];
+        // lanes along p1: contiguous in V's columns (and in the sums)
         for (int e = tid; e < kTwN * kTcM; e += kTwThreads) {
-            const int p = e % kTwN, mm = e / kTwN, p1 = m0 + mm, p2 = p0 + p;
+            const int mm = e % kTcM, p = e / kTcM, p1 = m0 + mm, p2 = p0 + p;
             if (p1 >= c || p2 >= c || p1 < p2) continue;
-            const int sc = (rowE[p] - 1022) + (P.linvexp[pos0 + p1] - 1022) - 13 - (p1 == p2 ? 1 : 0);
-            V[(int64_t)p2 * c + p1] -= fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
+            const int e1 = P.linvexp[pos0 + p1], e2 = rowE[p];
+            const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0);
+            const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
+            if (SYRK == 2 && (e1 == 0x7FF || e2 == 0x7FF)) V[(int64_t)p2 * c + p1] = __longlong_as_double(0x7FF8000000000000ll);
+            else V[(int64_t)p2 * c + p1] -= y;
         }
         return;
     }
@@ -616,7 +625,10 @@ cudaError_t configure_tcw_kernels() {
         e = cudaFuncSetAttribute(k_selinv_tcw<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)TwCfg::SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_selinv_tcw<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_selinv_tcw<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TwCfg::SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_selinv_tcw<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)TwCfg::SMEM);
     return e;
 }
@@ -635,9 +647,11 @@ cudaError_t launch_lhat_tcw(const ProbDesc *d, const Item *items, int n, long lo
     return cudaGetLastError();
 }
 
-cudaError_t launch_syrk_tcw(const ProbDesc *d, const Item *items, int n, long long wait_limit, cudaStream_t st) {
+cudaError_t launch_syrk_tcw(int mode, const ProbDesc *d, const Item *items, int n, long long wait_limit,
+                            cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_selinv_tcw<false, false, true><<<n, kTwThreads, TwCfg::SMEM, st>>>(d, items, n, nullptr, wait_limit);
+    if (mode == 1) k_selinv_tcw<false, false, 1><<<n, kTwThreads, TwCfg::SMEM, st>>>(d, items, n, nullptr, wait_limit);
+    else k_selinv_tcw<false, false, 2><<<n, kTwThreads, TwCfg::SMEM, st>>>(d, items, n, nullptr, wait_limit);
     return cudaGetLastError();
 }
 

@@ -228,17 +228,19 @@ struct FactorDesc {
     void *D;
     int *status;
     int herm;                 // complex Hermitian: A = L D L^H
+    ProbDesc up;              // what the tcgen05 form of the update reads
 };
 
 // Launch lists of one level of the factorization (ranges into the device lists).
 struct FactorLevel {
     int64_t small0 = 0, wide0 = 0, wide1 = 0;   // narrow supernodes [small0, wide0), the others [wide0, wide1)
     int64_t tile0 = 0, tile1 = 0;               // row tiles of the others
-    int64_t u0 = 0, u1 = 0;                     // update tiles of the others
+    struct Upd { int64_t i0 = 0, i1 = 0; int b = 64; };   // update tiles and their side
+    Upd upd[2];                                 // of all the others / of those that the tcgen05 form leaves
+    int64_t tc0 = 0, tc1 = 0, tw0 = 0, tw1 = 0; // tcgen05 form: its tiles, the row blocks of its digit planes
     int small_elems = 0;                        // largest panel of the narrow ones
     int wide_s = 0;                             // widest of the others
     int cl = 1;                                 // CTAs per diagonal block
-    int ub = 64;                                // side of an update tile
 };
 
 struct FactorData {
@@ -260,6 +262,12 @@ struct FactorData {
     int npass = 1;
     int2 *d_asm = nullptr;
     int4 *d_uitems = nullptr;         // (K, row tile, column tile) of the lower c x c
+    Item *d_tcitems = nullptr;        // tcgen05 form of the update
+    int2 *d_tcwork = nullptr;         // (K, 32-row block) of its digit planes
+    int64_t *d_digoff = nullptr;      // [ns] where K's digit planes start (per level, one buffer)
+    int64_t dig_total = 0;
+    uint16_t *digits = nullptr;
+    int *digexp = nullptr;            // row exponents, by row-list position
     int64_t *d_uoff = nullptr;
     int32_t *d_chpos = nullptr;
     void *U = nullptr;

@@ -60,3 +60,30 @@ def test_levels_of_many_blocks(native, cuda_device, count, size):
     _check(_blocks(count, size, "f64", count))
     if count in (1, 160):
         _check(_blocks(count, size, "c128", count))
+
+
+# the update matrix on the tensor cores: C from just below its shortest, one
+# and several 128 x 64 tiles, remainders of the 16-column steps
+@pytest.mark.parametrize("cap,n", [(17, 112), (17, 113), (17, 114), (24, 153), (32, 160), (33, 290), (128, 256), (128, 449)])
+def test_update_on_tensor_cores(native, cuda_device, cap, n):
+    p = _blocks(1, n, "f64", n)
+    p.supernodes = {"kind": "fundamental", "cap": cap, "fill": 0.0}
+    _check(p)
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_nonfinite_entry_reaches_a_pivot(native, cuda_device, bad):
+    """A non-finite entry below the diagonal blocks is reported by a later
+    pivot, through the digit planes as through FP64 products."""
+    import torch
+    from paper_1604_02528_gb300.api import SelInvContext
+    p = _blocks(1, 300, "f64", 3)
+    p.supernodes = {"kind": "fundamental", "cap": 64, "fill": 0.0}
+    ctx = SelInvContext.from_problem(p)
+    v = p.values.copy()
+    v[int(p.colptr[5]) + 200] = bad
+    for fast in (1, 0):
+        ctx.set_options(fast_contraction=fast)
+        ctx.factor(torch.from_numpy(v).cuda())
+        torch.cuda.synchronize()
+        assert ctx.status() == native.SELINV_ERR_ZERO_PIVOT
