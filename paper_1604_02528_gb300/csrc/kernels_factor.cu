@@ -27,6 +27,7 @@
 #include "nvtx.h"
 #include "plan.h"
 #include "seg_update.cuh"
+#include "tri_rows.cuh"
 
 namespace selinv {
 
@@ -138,7 +139,8 @@ __global__ void __launch_bounds__(256) k_fupd_digits(const FactorDesc *__restric
 // kernel, and repeating it costs less than exchanging it -- and updates its
 // own rows of the trailing block; one cluster barrier per panel.
 // ---------------------------------------------------------------------------
-constexpr int kFdThreads = 128;
+constexpr int kFdThreads = 256;   // the panel's 128 rows, and as many again for the trailing block
+constexpr int kFdRows = 128;
 constexpr int kFdNB = 8;           // columns per panel
 constexpr int kFdLd = kFdNB + 1;   // panel row stride in shared memory
 
@@ -155,7 +157,14 @@ __device__ __forceinline__ double fast_recip(double d) {
     const double x = fma(-d, r, 1.0);
     return fma(fma(x, x, x), r, r);
 }
-__device__ __forceinline__ zd fast_recip(zd d) { return recip(d); }
+// complex: conj(d) / |d|^2 while |d|^2 and its reciprocal stay in range
+__device__ __forceinline__ zd fast_recip(zd d) {
+    const int ex = (int)((__double_as_longlong(d.x) >> 52) & 0x7FF), ey = (int)((__double_as_longlong(d.y) >> 52) & 0x7FF);
+    const int e = ex > ey ? ex : ey;
+    if (e < 623 || e > 1423) return recip(d);
+    const double r = fast_recip(fma(d.x, d.x, d.y * d.y));
+    return make_zd(d.x * r, -d.y * r);
+}
 
 // elements of a CTA's row store for s columns, clusters of cl CTAs: groups of
 // four rows, group g as 4 rows of 4 (g + 1) entries
@@ -183,8 +192,8 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
     T *D = static_cast<T *>(F.D) + fc;
     const bool herm = F.herm != 0;
     T *Yp = reinterpret_cast<T *>(smem_raw);          // [128][kFdLd] undivided panel columns y = l d
-    T *Lp = Yp + 128 * kFdLd;                         // [128][kFdLd] panel columns of L
-    T *A = Lp + 128 * kFdLd;                          // this CTA's rows
+    T *Lp = Yp + kFdRows * kFdLd;                     // 2 x [128][kFdLd] columns of L: this panel and the last
+    T *A = Lp + 2 * kFdRows * kFdLd;                  // this CTA's rows
     const int tid = threadIdx.x;
     // row i = 4 g + u lives in rank g % CL at (local group g / CL)
     auto off = [&](int i) {
@@ -201,48 +210,57 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
         }
     cp_async_commit();
     cp_async_wait<0>();
-    for (int b0 = 0; b0 < s; b0 += kFdNB) {
+    // a finished panel's columns of L into the row store (the owners read it
+    // no more once every CTA has passed the next barrier); global memory gets
+    // the block at the end, so that no barrier waits for stores to reach it
+    auto keep = [&](int b0, const T *Lq) {
         const int nb = s - b0 < kFdNB ? s - b0 : kFdNB;
-        cl.sync();
-        const int i = b0 + tid;                        // this thread's row of the panel
-        T a[kFdNB];
-        if (i < s) {
-            const T *src = cl.map_shared_rank(A, (i >> 2) % CL) + off(i) + b0;
-#pragma unroll
-            for (int j = 0; j < kFdNB; j++) a[j] = (j < nb && j <= tid) ? src[j] : Sc<T>::zero();
+        for (int e = tid; e < 4 * myg * nb; e += kFdThreads) {
+            const int r = row_of(e % (4 * myg)), j = e / (4 * myg);
+            if (r < s && r > b0 + j) A[off(r) + b0 + j] = Lq[(r - b0) * kFdLd + j];
         }
+    };
+    int pb = 0;
+    for (int b0 = 0; b0 < s; b0 += kFdNB, pb ^= 1) {
+        const int nb = s - b0 < kFdNB ? s - b0 : kFdNB;
+        T *Lq = Lp + pb * kFdRows * kFdLd;
+        cl.sync();
+        if (b0) keep(b0 - kFdNB, Lp + (pb ^ 1) * kFdRows * kFdLd);
+        const int i = b0 + tid;                        // this thread's row of the panel
+        if (tid < kFdRows) {
+            T a[kFdNB];
+            if (i < s) {
+                const T *src = cl.map_shared_rank(A, (i >> 2) % CL) + off(i) + b0;
 #pragma unroll
-        for (int j = 0; j < kFdNB; j++) {
-            if (j < nb) {
-                if (tid >= j && tid < nb) Ys[j][tid] = a[j];
-                __syncthreads();
-                const T d = Ys[j][j];
-                if (i < s) {
-                    if (tid == j && rank == 0) {
-                        if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
-                        D[b0 + j] = d;
+                for (int j = 0; j < kFdNB; j++) a[j] = (j < nb && j <= tid) ? src[j] : Sc<T>::zero();
+            }
+#pragma unroll
+            for (int j = 0; j < kFdNB; j++) {
+                if (j < nb) {
+                    if (tid >= j && tid < nb) Ys[j][tid] = a[j];
+                    asm volatile("bar.sync 1, 128;\n" ::: "memory");
+                    const T d = Ys[j][j];
+                    if (i < s) {
+                        if (tid == j && rank == 0) {
+                            if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
+                            D[b0 + j] = d;
+                        }
+                        const T l = mul(a[j], fast_recip(d));
+                        Yp[tid * kFdLd + j] = a[j];
+                        Lq[tid * kFdLd + j] = l;
+#pragma unroll
+                        for (int k = j + 1; k < kFdNB; k++)
+                            if (k < nb) msub(a[k], l, cjif(Ys[j][k], herm));
                     }
-                    const T l = mul(a[j], fast_recip(d));
-                    Yp[tid * kFdLd + j] = a[j];
-                    Lp[tid * kFdLd + j] = l;
-#pragma unroll
-                    for (int k = j + 1; k < kFdNB; k++)
-                        if (k < nb) msub(a[k], l, cjif(Ys[j][k], herm));
                 }
             }
         }
         __syncthreads();
-        // L's columns of the panel, each row by its owner
-        for (int e = tid; e < 4 * myg * nb; e += kFdThreads) {
-            const int r = row_of(e % (4 * myg)), j = e / (4 * myg);
-            if (r >= s) continue;
-            P[(int64_t)(b0 + j) * ld + r] = r > b0 + j ? Lp[(r - b0) * kFdLd + j] : (r == b0 + j ? Sc<T>::one() : Sc<T>::zero());
-        }
         // own rows of the trailing block: a_ik -= l_i y_k, columns b1 .. i of row i
-        const int b1 = b0 + kFdNB;
         // -- entries dealt to the threads one by one (the FP64 pipe bounds the
         // update, and an idle lane costs as much as a busy one), all lanes of a
         // warp brought to their entry before the products start
+        const int b1 = b0 + kFdNB;
         int total = 0;
         for (int lr = 0; lr < 4 * myg; lr++) {
             const int r = row_of(lr);
@@ -258,14 +276,21 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
             __syncwarp(__activemask());
             T *dst = A + off(r) + b1 + q;
             T acc = *dst;
-            const T *lrow = Lp + (r - b0) * kFdLd, *yrow = Yp + (b1 + q - b0) * kFdLd;
+            const T *lrow = Lq + (r - b0) * kFdLd, *yrow = Yp + (b1 + q - b0) * kFdLd;
 #pragma unroll
             for (int j = 0; j < kFdNB; j++) msub(acc, lrow[j], cjif(yrow[j], herm));   // a full panel: b1 <= s - 1
             *dst = acc;
             q += kFdThreads;
         }
     }
-    cl.sync();   // no CTA leaves while another may still read its rows
+    cl.sync();   // the last panel is read no more, and no CTA leaves while another may still read its rows
+    keep((s - 1) / kFdNB * kFdNB, Lp + (pb ^ 1) * kFdRows * kFdLd);
+    __syncthreads();
+    for (int k = tid / 32; k < s; k += kFdThreads / 32)
+        for (int lr = tid % 32; lr < 4 * myg; lr += 32) {
+            const int i = row_of(lr);
+            if (i < s) P[(int64_t)k * ld + i] = i > k ? A[off(i) + k] : (i == k ? Sc<T>::one() : Sc<T>::zero());
+        }
 }
 
 // ---------------------------------------------------------------------------
@@ -279,18 +304,7 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
 // small enough that every SM gets one.
 // items {J, first row of C, rows}
 // ---------------------------------------------------------------------------
-constexpr int kFtThreads = 128;
-
-// elements of L_JJ's store: nc blocks of 32 columns, block b with 32 (nc - b) rows
-__host__ __device__ inline int ft_store_elems(int s) {
-    const int nc = (s + 31) / 32;
-    return 32 * 32 * (nc * (nc + 1) / 2);
-}
-template <typename T> __device__ __forceinline__ T shfl_elem(T v, int src);
-template <> __device__ __forceinline__ double shfl_elem(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-template <> __device__ __forceinline__ zd shfl_elem(zd v, int src) {
-    return make_zd(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
+constexpr int kFtThreads = kTriThreads;
 
 template <typename T, int NC, int R>
 __device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, int row0, int nrows, bool herm) {
@@ -304,24 +318,7 @@ __device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, in
                 const int k = lane + 32 * t;
                 a[r][t] = (g + r < nrows && k < s) ? P[(int64_t)k * ld + row0 + g + r] : Sc<T>::zero();
             }
-        const T *Lb = Ls;
-#pragma unroll
-        for (int b = 0; b < NC; b++) {
-#pragma unroll 2
-            for (int jj = 0; jj < 32; jj++) {
-                T l[NC];
-#pragma unroll
-                for (int t = b; t < NC; t++) l[t] = cjif(Lb[jj * 32 * (NC - b) + lane + 32 * (t - b)], herm);
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const T y = shfl_elem(a[r][b], jj);
-#pragma unroll
-                    for (int t = b; t < NC; t++)
-                        if (t > b || lane > jj) msub(a[r][t], y, l[t]);   // finished columns stay as they are
-                }
-            }
-            Lb += 32 * 32 * (NC - b);
-        }
+        tri_rows<T, NC, R, false>(a, Ls, nullptr, 0, herm);
 #pragma unroll
         for (int r = 0; r < R; r++)
 #pragma unroll
@@ -352,20 +349,7 @@ __global__ void __launch_bounds__(kFtThreads) k_ftrsm(const FactorDesc *__restri
     const bool h = F.herm != 0;
     const int nc = (s + 31) / 32;
     for (int k = threadIdx.x; k < s; k += kFtThreads) rD[k] = recip(D[k]);
-    {
-        T *dst = Ls;
-        for (int b = 0; b < nc; b++) {
-            const int rows = 32 * (nc - b);
-            for (int e = threadIdx.x; e < 32 * rows; e += kFtThreads) {
-                const int j = 32 * b + e / rows, k = 32 * b + e % rows;
-                if (k < s && k > j) cp_async_elem(dst + e, P + (int64_t)j * ld + k);
-                else dst[e] = Sc<T>::zero();
-            }
-            dst += 32 * rows;
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-    }
+    tri_store(Ls, P, ld, s, 0);
     __syncthreads();
     T *Pc = P + s;
     // two rows at a time share the loads of L's column (one where a tile has no second row per warp)
@@ -532,8 +516,9 @@ int factor_tables(selinv_plan_s *plan) {
         // have blocks enough by themselves
         const int64_t nw = (int64_t)wide.size();
         v.cl = v.wide_s <= 32 ? 1 : (nw * 8 <= 152 ? 8 : (nw * 4 <= 152 ? 4 : (nw * 2 <= 152 ? 2 : 1)));
-        // row tiles: 4 rows (a row per warp) and more as the level's rows cover every SM
-        const int rt = (int)std::min<int64_t>(64, std::max<int64_t>(4, (rows / 152 + 3) / 4 * 4));
+        // row tiles: 4 rows (a row per warp), up to 16 as the level's rows cover every
+        // SM (64-row tiles left a third of the SMs idle in the last wave)
+        const int rt = (int)std::min<int64_t>(16, std::max<int64_t>(4, (rows / 152 + 3) / 4 * 4));
         v.tile0 = (int64_t)tiles.size();
         for (int32_t J : wide)
             for (int r = 0, c = below(J); r < c; r += rt) tiles.push_back(make_int4(J, r, std::min(rt, c - r), 0));
@@ -673,8 +658,8 @@ FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, 
 
 // the dynamic shared memory of the widest blocks, on the plan's device
 template <typename T> static cudaError_t configure_factor_kernels() {
-    const int diag = (int)(sizeof(T) * (size_t)(2 * 128 * kFdLd + fd_rows_elems(128, 1)));
-    const int trsm = (int)(sizeof(T) * (size_t)ft_store_elems(128)), small = (int)(2 * sizeof(T) * kFSmallElems);
+    const int diag = (int)(sizeof(T) * (size_t)(3 * kFdRows * kFdLd + fd_rows_elems(128, 1)));
+    const int trsm = (int)(sizeof(T) * (size_t)tri_store_elems(128)), small = (int)(2 * sizeof(T) * kFSmallElems);
     cudaError_t e = cudaFuncSetAttribute(k_fdiag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, diag);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ftrsm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, trsm);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fsmall<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
@@ -727,7 +712,7 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)((v.wide1 - v.wide0) * v.cl));
             cfg.blockDim = dim3(kFdThreads);
-            cfg.dynamicSmemBytes = sizeof(T) * (size_t)(2 * 128 * kFdLd + fd_rows_elems(v.wide_s, v.cl));
+            cfg.dynamicSmemBytes = sizeof(T) * (size_t)(3 * kFdRows * kFdLd + fd_rows_elems(v.wide_s, v.cl));
             cfg.stream = st;
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
@@ -741,7 +726,7 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
             note_launch();
         }
         if (v.tile1 > v.tile0) {
-            k_ftrsm<T><<<(int)(v.tile1 - v.tile0), kFtThreads, sizeof(T) * (size_t)ft_store_elems(v.wide_s), st>>>(
+            k_ftrsm<T><<<(int)(v.tile1 - v.tile0), kFtThreads, sizeof(T) * (size_t)tri_store_elems(v.wide_s), st>>>(
                 fd, f->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
             note_launch();
         }

@@ -16,6 +16,7 @@
 #include "common.cuh"
 #include "launch.h"
 #include "tile_gemm.cuh"
+#include "tri_rows.cuh"
 
 namespace selinv {
 
@@ -164,16 +165,62 @@ __global__ void __launch_bounds__(kLinvThreads) k_linv(const ProbDesc *__restric
 }
 
 // ---------------------------------------------------------------------------
-// k_dinv: Dinv_K = X^T D_K^{-1} X (X^H for a Hermitian problem), X = L_KK^{-1}
-// from k_linv, for the wide supernodes: one 32 x 32 tile (i0 >= j0) of the
-// lower triangle per CTA, mirrored; k runs from i0 (X is lower triangular).
-// work (problem, K << 8 | tile), tiles row-major over the lower triangle.
+// k_linv_cols: L_KK^{-1} of the supernodes wider than 32 columns, 8 columns
+// per CTA (the columns of an inverse are independent: 16 CTAs share the 128-
+// column blocks at the top of the tree, whose one CTA took 190 us real and
+// 590 us complex).  work (problem, K << 8 | side << 7 | column block); side 1
+// (LU form): (U_KK^T)^{-1}, whose diagonal is not one, into Vt.
 // ---------------------------------------------------------------------------
+template <typename T>
+__global__ void __launch_bounds__(kTriThreads) k_linv_cols(const ProbDesc *__restrict__ descs,
+                                                           const int2 *__restrict__ work, int nwork) {
+    grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T rd[128];
+    T *Ls = reinterpret_cast<T *>(smem_raw);
+    const int w = blockIdx.x;
+    if (w >= nwork) return;
+    const ProbDesc &P = descs[work[w].x];
+    const int K = work[w].y >> 8, side = (work[w].y >> 7) & 1, j0 = (work[w].y & 0x7F) * kTriCols;
+    const int fc = P.super_ptr[K];
+    const int s = P.super_ptr[K + 1] - fc;
+    const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
+    const T *L = static_cast<const T *>(side ? P.Ut : P.L) + P.panel_off[K];
+    if (side) {
+        for (int k = threadIdx.x; k < s; k += kTriThreads) {
+            const T u = L[(int64_t)k * ld + k];
+            if (j0 == 0 && (is_zero(u) || !finite_val(u))) latch_status(P.status, SELINV_ERR_ZERO_PIVOT);
+            rd[k] = recip(u);
+        }
+    } else if (j0 == 0 && !P.lu) {
+        const T *D = static_cast<const T *>(P.D) + fc;
+        for (int k = threadIdx.x; k < s; k += kTriThreads)
+            if (is_zero(D[k]) || !finite_val(D[k])) latch_status(P.status, SELINV_ERR_ZERO_PIVOT);
+    }
+    tri_store(Ls, L, ld, s, j0 / 32);
+    __syncthreads();
+    if (side) tri_inverse<T, true>(Ls, rd, static_cast<T *>(P.Vt) + P.linv_off[K], s, s, j0);
+    else tri_inverse<T, false>(Ls, nullptr, static_cast<T *>(P.Linv) + P.linv_off[K], s, s, j0);
+}
+
+// ---------------------------------------------------------------------------
+// k_dinv: Dinv_K = X^T D_K^{-1} X (X^H for a Hermitian problem), X = L_KK^{-1}
+// from k_linv_cols, for the wide supernodes: one 16 x 16 tile (i0 >= j0) of the
+// lower triangle per CTA, mirrored; k runs from i0 (X is lower triangular).
+// LU form: U_KK^{-1} L_KK^{-1} = V^T X, every tile (not symmetric), k from
+// max(i0, j0).  work (problem, K << 8 | tile), tiles row-major over the lower
+// triangle (LU: over the square).  16 x 16: the FP64 pipe bounds a tile, and
+// the top levels have a few blocks only (32 x 32 tiles: 43 us real, 143 us
+// complex for 16 blocks of 128 columns).
+// ---------------------------------------------------------------------------
+constexpr int kDinvT = kDinvTile;
+static_assert(kTriCols == kLinvCols, "the planner counts k_linv_cols' work entries");
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_dinv(const ProbDesc *__restrict__ descs, const int2 *__restrict__ work,
                                               int nwork) {
     grid_dep_wait();
-    __shared__ T As[32][33], Bs[32][33];
+    __shared__ T As[32][kDinvT + 1], Bs[32][kDinvT + 1];
     __shared__ T rD[128];
     const int w = blockIdx.x;
     if (w >= nwork) return;
@@ -182,42 +229,43 @@ __global__ void __launch_bounds__(256) k_dinv(const ProbDesc *__restrict__ descs
     const int fc = P.super_ptr[K];
     const int s = P.super_ptr[K + 1] - fc;
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
+    const bool lu = P.lu != 0;
     int ti = 0, r = t;
-    while (r > ti) { r -= ti + 1; ti++; }            // tile t -> (ti, tj), tj <= ti
-    const int i0 = ti * 32, j0 = r * 32;
+    if (lu) {
+        const int nt = (s + kDinvT - 1) / kDinvT;
+        ti = t / nt;
+        r = t % nt;
+    } else {
+        while (r > ti) { r -= ti + 1; ti++; }        // tile t -> (ti, tj), tj <= ti
+    }
+    const int i0 = ti * kDinvT, j0 = r * kDinvT;
     const T *X = static_cast<const T *>(P.Linv) + P.linv_off[K];   // X(k, j) = X[j*s + k]
-    const T *D = static_cast<const T *>(P.D) + fc;
+    const T *V = lu ? static_cast<const T *>(P.Vt) + P.linv_off[K] : X;
+    const T *D = lu ? nullptr : static_cast<const T *>(P.D) + fc;
     T *LD = static_cast<T *>(P.LD) + P.panel_off[K];
     const bool h = P.herm != 0;
-    for (int k = threadIdx.x; k < s; k += 256) rD[k] = recip(D[k]);
+    for (int k = threadIdx.x; k < s; k += 256) rD[k] = lu ? Sc<T>::one() : recip(D[k]);
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    T acc[2][2] = {{Sc<T>::zero(), Sc<T>::zero()}, {Sc<T>::zero(), Sc<T>::zero()}};
-    for (int k0 = i0; k0 < s; k0 += 32) {
+    T acc = Sc<T>::zero();
+    for (int k0 = max(i0, j0); k0 < s; k0 += 32) {
         __syncthreads();
-        for (int e = threadIdx.x; e < 32 * 32; e += 256) {
+#pragma unroll
+        for (int e = threadIdx.x; e < 32 * kDinvT; e += 256) {
             const int q = e % 32, rr = e / 32, k = k0 + q;   // k fastest: contiguous in X's columns
-            As[q][rr] = (k < s && i0 + rr < s) ? mul(cjif(X[(int64_t)(i0 + rr) * s + k], h), rD[k]) : Sc<T>::zero();
+            T a = (k < s && i0 + rr < s) ? cjif(V[(int64_t)(i0 + rr) * s + k], h) : Sc<T>::zero();
+            if (!lu && k < s) a = mul(a, rD[k]);
+            As[q][rr] = a;
             Bs[q][rr] = (k < s && j0 + rr < s) ? X[(int64_t)(j0 + rr) * s + k] : Sc<T>::zero();
         }
         __syncthreads();
+        const int kk = s - k0 < 32 ? s - k0 : 32;
 #pragma unroll 8
-        for (int q = 0; q < 32; q++) {
-            const T a0 = As[q][ty], a1 = As[q][ty + 16], b0 = Bs[q][tx], b1 = Bs[q][tx + 16];
-            madd(acc[0][0], a0, b0);
-            madd(acc[0][1], a0, b1);
-            madd(acc[1][0], a1, b0);
-            madd(acc[1][1], a1, b1);
-        }
+        for (int q = 0; q < kk; q++) madd(acc, As[q][ty], Bs[q][tx]);
     }
-#pragma unroll
-    for (int u = 0; u < 2; u++)
-#pragma unroll
-        for (int v = 0; v < 2; v++) {
-            const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
-            if (i >= s || j >= s || i < j) continue;
-            LD[(int64_t)j * ld + i] = acc[u][v];
-            LD[(int64_t)i * ld + j] = cjif(acc[u][v], h);
-        }
+    const int i = i0 + ty, j = j0 + tx;
+    if (i >= s || j >= s || (!lu && i < j)) return;
+    LD[(int64_t)j * ld + i] = acc;
+    if (!lu) LD[(int64_t)i * ld + j] = cjif(acc, h);
 }
 
 // ---------------------------------------------------------------------------
@@ -813,6 +861,15 @@ cudaError_t launch_linv(int dtype, const ProbDesc *d, const int2 *work, int nwor
                                 : launch_linv_t<double>(d, work, nwork, large, with_dinv, st);
 }
 
+cudaError_t launch_linv_cols(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st) {
+    if (nwork <= 0) return cudaSuccess;
+    if (dtype == SELINV_C128)
+        k_linv_cols<zd><<<nwork, kTriThreads, sizeof(zd) * tri_store_elems(128), st>>>(d, work, nwork);
+    else
+        k_linv_cols<double><<<nwork, kTriThreads, sizeof(double) * tri_store_elems(128), st>>>(d, work, nwork);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_dinv(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st) {
     if (nwork <= 0) return cudaSuccess;
     if (dtype == SELINV_C128) k_dinv<zd><<<nwork, 256, 0, st>>>(d, work, nwork);
@@ -880,6 +937,12 @@ cudaError_t configure_selinv_kernels() {
     cudaError_t e = cudaFuncSetAttribute(k_linv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLinvSmemMax);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_linv<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLinvSmemMax);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_linv_cols<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(double) * tri_store_elems(128));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_linv_cols<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(zd) * tri_store_elems(128));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_selinv_persist<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist_smem<double>());
     if (e == cudaSuccess)

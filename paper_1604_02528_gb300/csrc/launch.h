@@ -11,9 +11,13 @@ namespace selinv {
 void note_launch(int n = 1);
 
 cudaError_t configure_selinv_kernels();
-// large = 1 for supernodes with s > 32 (128 KB of shared memory), 0 otherwise
+// L_KK^{-1} (and Dinv_K) by one CTA per supernode; large = 1: any width (128 KB of shared memory), 0: s <= 32
 cudaError_t launch_linv(int dtype, const ProbDesc *d, const int2 *work, int nwork, int large, cudaStream_t st,
                         int with_dinv = 1);
+// L_KK^{-1} of supernodes wider than 32 columns, kLinvCols columns per work entry
+constexpr int kLinvCols = 8;
+cudaError_t launch_linv_cols(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);
+constexpr int kDinvTile = 16;
 cudaError_t launch_dinv(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);
 cudaError_t launch_lhat(int dtype, int bucket, const ProbDesc *d, const Item *items, int n,
                         cudaStream_t st);

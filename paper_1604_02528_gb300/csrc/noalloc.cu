@@ -1,4 +1,4 @@
-// Allocation-free variant of the diagonal-block kernel k_linv:
+// Allocation-free variant of the diagonal-block step:
 // Dinv = L_KK^{-T} D_K^{-1} L_KK^{-1} for one unit-lower diagonal block.
 //
 // Some callers cannot allocate device memory: code in a latency-critical
@@ -15,8 +15,11 @@
 #include <mutex>
 
 #include "selinv.h"
+#include "tri_rows.cuh"
 
 namespace {
+
+using namespace selinv;
 
 constexpr int kMaxS = SELINV_NOALLOC_MAX_S;
 constexpr int kMaxDevices = 64;
@@ -25,6 +28,45 @@ constexpr int kMaxDevices = 64;
 // the library holds this array (kMaxS^2 doubles = 128 KB) until the process
 // exits.  All calls share it.
 static __device__ __align__(256) double g_linv_scratch[kMaxS * kMaxS];
+
+// Two kernels, both spread over SMs (one CTA walking the block in global
+// memory took 1325 us at s = 96).  First the columns of L_KK^{-1}, 8 per CTA
+// (they are independent), into the scratch block: every entry is written, so
+// nothing needs clearing between calls.
+__global__ void __launch_bounds__(kTriThreads) k_noalloc_linv(int s, const double *__restrict__ L, int64_t ld,
+                                                              double *__restrict__ X) {
+    grid_dep_wait();   // the previous call's k_noalloc_dinv may still read the scratch block
+    extern __shared__ __align__(16) double Ls[];
+    const int j0 = blockIdx.x * kTriCols;
+    tri_store(Ls, L, ld, s, j0 / 32);
+    __syncthreads();
+    tri_inverse<double, false>(Ls, nullptr, X, s, s, j0);
+}
+
+// Then Dinv(i, j) = sum_{k >= max(i, j)} X(k, i) X(k, j) / D_k, one 16 x 16 tile
+// (i0 >= j0) of the lower triangle per CTA, mirrored: k over 16 lanes at a time.
+__global__ void __launch_bounds__(256) k_noalloc_dinv(int s, const double *__restrict__ X, const double *__restrict__ D,
+                                                      double *__restrict__ Dinv, int64_t ldo) {
+    grid_dep_wait();
+    __shared__ double As[128][17], Bs[128][17], rd[128];
+    int ti = 0, tj = blockIdx.x;
+    while (tj > ti) { tj -= ti + 1; ti++; }
+    const int i0 = ti * 16, j0 = tj * 16, n = s - i0;
+    for (int q = threadIdx.x; q < n; q += 256) rd[q] = 1.0 / D[i0 + q];
+    __syncthreads();
+    for (int e = threadIdx.x; e < 16 * n; e += 256) {
+        const int q = e % n, r = e / n, k = i0 + q;   // k fastest: contiguous in X's columns
+        As[q][r] = i0 + r < s ? X[(int64_t)(i0 + r) * s + k] * rd[q] : 0.0;
+        Bs[q][r] = j0 + r < s ? X[(int64_t)(j0 + r) * s + k] : 0.0;
+    }
+    __syncthreads();
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, i = i0 + ty, j = j0 + tx;
+    double acc = 0.0;
+    for (int q = 0; q < n; q++) acc = fma(As[q][ty], Bs[q][tx], acc);
+    if (i >= s || j >= s || i < j) return;
+    Dinv[(int64_t)j * ldo + i] = acc;
+    Dinv[(int64_t)i * ldo + j] = acc;
+}
 
 // Device address of g_linv_scratch per device ordinal, looked up once per
 // device (in host code the symbol is only a host-side stand-in).  The
@@ -41,38 +83,14 @@ int scratch_address(double **out) {
     if (!g_addr[dev]) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_linv_scratch) != cudaSuccess || !p) return SELINV_ERR_CUDA;
+        // (with the first call's address goes the kernel's shared-memory opt-in)
+        if (cudaFuncSetAttribute(k_noalloc_linv, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(double) * tri_store_elems(kMaxS)) != cudaSuccess)
+            return SELINV_ERR_CUDA;
         g_addr[dev] = static_cast<double *>(p);
     }
     *out = g_addr[dev];
     return SELINV_OK;
-}
-
-// One CTA: columns of L_KK^{-1} by forward substitution (thread per column),
-// then Dinv(i, j) = sum_{k >= max(i,j)} Linv(k, i) Linv(k, j) / D_k.  Every
-// entry of the scratch block that is read is written first in this call, so
-// nothing needs clearing between calls.
-__global__ void __launch_bounds__(128) k_dinv_noalloc(int s, const double *__restrict__ L, int64_t ld,
-                                                      const double *__restrict__ D,
-                                                      double *__restrict__ Dinv, int64_t ldo,
-                                                      double *__restrict__ Li) {
-    for (int j = threadIdx.x; j < s; j += blockDim.x) {
-        double *x = Li + (int64_t)j * s;
-        for (int i = 0; i < j; i++) x[i] = 0.0;
-        x[j] = 1.0;
-        for (int i = j + 1; i < s; i++) {
-            double acc = 0.0;
-            for (int k = j; k < i; k++) acc = fma(L[(int64_t)k * ld + i], x[k], acc);
-            x[i] = -acc;
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < s * s; e += blockDim.x) {
-        const int i = e % s, j = e / s;
-        double acc = 0.0;
-        for (int k = (i > j ? i : j); k < s; k++)
-            acc = fma(Li[(int64_t)i * s + k] / D[k], Li[(int64_t)j * s + k], acc);
-        Dinv[(int64_t)j * ldo + i] = acc;
-    }
 }
 
 }  // namespace
@@ -85,6 +103,9 @@ extern "C" int selinv_dinv_noalloc(int32_t s, const double *Lkk, int64_t ld, con
     double *scratch = nullptr;
     int rc = scratch_address(&scratch);
     if (rc) return rc;
-    k_dinv_noalloc<<<1, 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(s, Lkk, ld, D, Dinv, ldo, scratch);
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    const int nt = (s + 15) / 16;
+    k_noalloc_linv<<<(s + kTriCols - 1) / kTriCols, kTriThreads, sizeof(double) * tri_store_elems(s), st>>>(s, Lkk, ld, scratch);
+    k_noalloc_dinv<<<nt * (nt + 1) / 2, 256, 0, st>>>(s, scratch, D, Dinv, ldo);
     return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
 }
