@@ -13,7 +13,8 @@ namespace selinv {
 // one after the other (K-major 8 x 8 core matrices), one exponent per row
 // (exps[row]).  A warp per 4 rows finds their exponents, then each thread
 // cuts 8 consecutive k of one row, a 16-byte store per plane.
-template <class X>
+// ROUND: to the nearest point of the row's grid instead of toward zero.
+template <bool ROUND, class X>
 __device__ __forceinline__ void digit_rows(const X &x, int kw, int c, int b, uint16_t *base, int *exps) {
     __shared__ int rowE[32];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -38,8 +39,8 @@ __device__ __forceinline__ void digit_rows(const X &x, int kw, int c, int b, uin
 #pragma unroll
         for (int t = 0; t < 8; t += 2) {
             int d0[kDig], d1[kDig];
-            digits7(k0 + t < kw ? x(p, k0 + t) : 0.0, rowE[r], d0);
-            digits7(k0 + t + 1 < kw ? x(p, k0 + t + 1) : 0.0, rowE[r], d1);
+            digits7<ROUND>(k0 + t < kw ? x(p, k0 + t) : 0.0, rowE[r], d0);
+            digits7<ROUND>(k0 + t + 1 < kw ? x(p, k0 + t + 1) : 0.0, rowE[r], d1);
 #pragma unroll
             for (int i = 0; i < kDig; i++) h[i][t / 2] = f16_of_int(d0[i]) | (f16_of_int(d1[i]) << 16);
         }

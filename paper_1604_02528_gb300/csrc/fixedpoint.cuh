@@ -16,12 +16,15 @@ __device__ __forceinline__ uint32_t f16_of_int(int v) {
 }
 
 // 7 balanced base-256 digits (most significant first) of x on the grid of
-// biased exponent E (E >= exponent of x): x ~= sum_i d_i 2^(E-1022-7-8i).
+// biased exponent E (E >= exponent of x): x ~= sum_i d_i 2^(E-1022-7-8i), cut
+// toward zero (ROUND: to nearest, half away from zero).
+template <bool ROUND = false>
 __device__ __forceinline__ void digits7(double x, int E, int d[kDig]) {
     const long long b = __double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7FF);
     unsigned long long mant = ex ? ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) : 0ull;
     const int sh = E - ex - 2;                       // M = mant * 2^(2 - (E - ex)) < 2^55
+    if (ROUND && sh > 0 && sh < 55) mant += 1ull << (sh - 1);
     unsigned long long M = sh < 0 ? (mant << (-sh)) : (sh < 64 ? (mant >> sh) : 0ull);
 #pragma unroll
     for (int i = kDig - 1; i >= 1; i--) {

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) k_fupd_digits(const FactorDesc *__restric
     const double *LC = static_cast<const double *>(F.L) + F.panel_off[J] + s;
     const double *DJ = static_cast<const double *>(F.D) + F.super_ptr[J];
     auto x = [&](int p, int k) -> double { return LC[(int64_t)k * ld + p] * DJ[k]; };
-    digit_rows(x, s, (int)(ld - s), b, F.up.linvd + F.up.linvd_off[J], F.up.linvexp + F.rowptr[J] + s);
+    digit_rows<true>(x, s, (int)(ld - s), b, F.up.linvd + F.up.linvd_off[J], F.up.linvexp + F.rowptr[J] + s);
 }
 
 // ---------------------------------------------------------------------------

@@ -73,17 +73,18 @@ static_assert(TwCfg::SMEM + 2048 <= 232448, "dynamic + static shared memory with
 // g5 2^8 + g6 (|l| < 2^48), and what lo cannot hold is carried into hi.
 // Groups 0 and 1 (one and two digit pairs: |g| <= 2^22) are converted by the
 // exact magic-number addition on the FP32 pipe, the others by F2I, whose
-// unit is the epilogue's bottleneck.
-__device__ __forceinline__ void add_chunk(const uint32_t (&acc)[kTcDig][8], int jj, bool first, long long &hi,
+// unit is the epilogue's bottleneck.  NG 8: group 7, worth g7 2^-8, rounded.
+template <int NG>
+__device__ __forceinline__ void add_chunk(const uint32_t (&acc)[NG][8], int jj, bool first, long long &hi,
                                           uint32_t &lo) {
-    long long gv[kTcDig];
+    long long gv[NG];
 #pragma unroll
     for (int gq = 0; gq < 2; gq++)
         gv[gq] = (long long)(__float_as_int(__fadd_rn(__uint_as_float(acc[gq][jj]), 12582912.0f)) - 0x4B400000);
 #pragma unroll
-    for (int gq = 2; gq < kTcDig; gq++) gv[gq] = (long long)__float2int_rn(__uint_as_float(acc[gq][jj]));
+    for (int gq = 2; gq < NG; gq++) gv[gq] = (long long)__float2int_rn(__uint_as_float(acc[gq][jj]));
     const long long h = (gv[0] << 16) + (gv[1] << 8) + gv[2];
-    const long long l = (gv[3] << 24) + (gv[4] << 16) + (gv[5] << 8) + gv[6];
+    const long long l = (gv[3] << 24) + (gv[4] << 16) + (gv[5] << 8) + gv[6] + (NG == 8 ? (gv[NG - 1] + 128) >> 8 : 0ll);
     const long long t = (first ? 0ll : (long long)lo) + l;
     hi = (first ? 0ll : hi) + h + (t >> 32);
     lo = (uint32_t)t;
@@ -99,9 +100,12 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[kTcDig][8], int 
 // row), B = 64 rows of [Lhat, Ybar] sliced here; items (K, 128-row block *
 // number of 64-row blocks + 64-row block) on or below the diagonal.
 // SYRK 2: the factorization's Schur update U_K -= (L_CK D_K) L_CK^T over the s
-// columns, the same with A = digit planes of L_CK D_K and B = L_CK; a row
-// that holds an infinity or a NaN makes its results NaN (the digits cannot
-// carry it), so that a later pivot reports it.
+// columns, the same with A = digit planes of L_CK D_K and B = L_CK.  Rows are
+// rounded to their grid, not cut (the entries of L mostly share a sign, and
+// cut products would all err to one side), and the digit pairs i + j = 7
+// count too: L's error against 64-bit arithmetic is then that of FP64 FMA.
+// A row that holds an infinity or a NaN makes its results NaN (the digits
+// cannot carry it), so that a later pivot reports it.
 //
 // LHAT: the same machinery forms products of a panel's rows with an s x s
 // matrix, out(p, j) = sum_k X(p, k) B(k, j) for the rows p of C: A = digit
@@ -148,6 +152,10 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
     const int c = (int)(ld - s);
     constexpr bool DENSE = LHAT || SYRK;                 // B from dense panels
+    // digit groups: 7, or 8 for the factorization, whose error would otherwise
+    // be the dropped pairs' (2^-53 of the rows' largest per step) rather than
+    // the rounding of U
+    constexpr int NG = SYRK == 2 ? 8 : kTcDig;
     constexpr bool PAIR = SYRK == 1;                     // B's k runs over two panels
     const int kw = PAIR ? 2 * s : (DENSE ? s : (CPLX ? 2 * c : c));   // k extent
     const int mrows = SYRK ? c : (CPLX ? 2 * s : s);     // rows of A (output rows)
@@ -368,7 +376,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 uint32_t lo[4], hi[4];
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
-                    const unsigned long long wv = (unsigned long long)(fixed54(v[u], E) + 0x80808080808080ll);
+                    const unsigned long long wv = (unsigned long long)(fixed54<SYRK == 2>(v[u], E) + 0x80808080808080ll);
                     lo[u] = (uint32_t)wv;
                     hi[u] = (uint32_t)(wv >> 32);
                 }
@@ -412,7 +420,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 umma::fence_after_sync();
                 const uint64_t ad0 = umma::smem_desc(umma::smem_u32(As + sa * Cfg::A_STAGE), 128, 256);
                 const uint64_t bd0 = umma::smem_desc(umma::smem_u32(Bs + sb * Cfg::B_STAGE), 128, 256);
-                digit_products<kTwN, Cfg::A_PLANE, Cfg::B_PLANE>(tmem, ad0, bd0, first);
+                digit_products<kTwN, Cfg::A_PLANE, Cfg::B_PLANE, NG>(tmem, ad0, bd0, first);
                 umma::commit(&aempty[sa]);
                 umma::commit(&bempty[sb]);
                 if (i_ % kTcFlush == kTcFlush - 1 || i_ == n - 1) umma::commit(&acc_full);
@@ -451,15 +459,15 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             umma::fence_after_sync();
 #pragma unroll 1
             for (int cb = 0; cb < 4; cb++) {
-                uint32_t acc[kTcDig][8];
+                uint32_t acc[NG][8];
 #pragma unroll
-                for (int gq = 0; gq < kTcDig; gq++)
+                for (int gq = 0; gq < NG; gq++)
                     umma::tmem_ld8(tmem + ((uint32_t)lb << 16) + (uint32_t)(gq * kTwN + half * 32 + cb * 8), acc[gq]);
                 umma::tmem_wait_ld();
 #pragma unroll
                 for (int jj = 0; jj < 8; jj++) {   // the first chunk writes, the later ones add
                     const int e = (half * 32 + cb * 8 + jj) * kTwHS + m;
-                    add_chunk(acc, jj, f == 0, Hi[e], Lo[e]);
+                    add_chunk<NG>(acc, jj, f == 0, Hi[e], Lo[e]);
                 }
             }
             umma::fence_before_sync();

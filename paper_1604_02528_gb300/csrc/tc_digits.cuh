@@ -21,12 +21,15 @@ static_assert(kTcFlush == 8, "the planner sizes k-ranges in whole chunks of 8 st
 constexpr long long kMbarMinPolls = 1ll << 22;
 
 // x = M * 2^(E - 1076) with |M| < 2^54 (E >= the biased exponent of x),
-// truncated toward zero; integer operations only.
+// truncated toward zero (ROUND: to nearest, half away from zero); integer
+// operations only.
+template <bool ROUND = false>
 __device__ __forceinline__ long long fixed54(double x, int E) {
     const long long b = __double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7FF);
-    const long long mant = ex ? ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) : 0ll;
+    long long mant = ex ? ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) : 0ll;
     const int sh = E - ex - 1;
+    if (ROUND && sh > 0 && sh < 55) mant += 1ll << (sh - 1);
     const long long M = sh < 0 ? (mant << 1) : (sh < 63 ? (mant >> sh) : 0ll);
     return b < 0 ? -M : M;
 }
@@ -53,19 +56,30 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
 // (i + j0) TN computes A_i B_j0 .. A_i B_{j0+m-1} into groups i + j0 ..
 // i + j0 + m - 1.  Per step 10 MMAs for TN = 64, 7 for TN <= 32 (against 28
 // of N = TN).  A group starts from zero at the first step of a chunk, with
-// the products of A plane 0.
-template <int TN, int A_PLANE, int B_PLANE>
+// the products of A plane 0.  NG 8: the six pairs with i + j = 7 as well, in
+// group 7 (its first products are those of A plane 1).
+template <int TN, int A_PLANE, int B_PLANE, int NG = kTcDig>
 __device__ __forceinline__ void digit_products(uint32_t tmem, uint64_t ad0, uint64_t bd0, bool first) {
     constexpr int kPer = 256 / TN;   // B planes per MMA (N <= 256)
 #pragma unroll
     for (int i = 0; i < kTcDig; i++) {
         const uint64_t ad = ad0 + (uint64_t)(i * A_PLANE * 2 / 16);
 #pragma unroll
-        for (int j0 = 0; j0 < kTcDig - i; j0 += kPer) {
-            const int m = kTcDig - i - j0 < kPer ? kTcDig - i - j0 : kPer;
+        for (int j0 = 0; j0 < (NG - i < kTcDig ? NG - i : kTcDig); j0 += kPer) {
+            constexpr int kAll = kTcDig;
+            const int nj = NG - i < kAll ? NG - i : kAll;
+            const int m = nj - j0 < kPer ? nj - j0 : kPer;
             const uint64_t bd = bd0 + (uint64_t)(j0 * B_PLANE * 2 / 16);
-            umma::mma_f16kind(tmem + (uint32_t)((i + j0) * TN), ad, bd, umma::idesc_f16_f32(kTcM, m * TN),
-                              (first && i == 0) ? 0u : 1u);
+            // plane pair (1, 6) opens group 7: an MMA of its own, so that the
+            // groups before it in the same plane run keep accumulating
+            const bool opens = NG == 8 && i == 1 && j0 + m == kAll;
+            const int m1 = opens ? m - 1 : m;
+            if (m1)
+                umma::mma_f16kind(tmem + (uint32_t)((i + j0) * TN), ad, bd, umma::idesc_f16_f32(kTcM, m1 * TN),
+                                  (first && i == 0) ? 0u : 1u);
+            if (opens)
+                umma::mma_f16kind(tmem + (uint32_t)(7 * TN), ad, bd0 + (uint64_t)(6 * B_PLANE * 2 / 16),
+                                  umma::idesc_f16_f32(kTcM, TN), first ? 0u : 1u);
         }
     }
 }
