@@ -1639,7 +1639,7 @@ static void row_product(AdjData *a, int pd, int li, cudaStream_t st) {
     }
     const int t0 = (int)a->pr_lptr[li], t1 = (int)a->pr_lptr[li + 1];
     if (t1 > t0) {
-        launch_lhat_tcw(a->d_pdp + pd, a->d_pr + t0, t1 - t0, a->tcs.spin_limit, st);
+        launch_lhat_tcw(0, a->d_pdp + pd, a->d_pr + t0, t1 - t0, a->tcs.spin_limit, st);
         note_launch();
     }
 }

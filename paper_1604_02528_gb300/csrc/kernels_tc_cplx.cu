@@ -24,16 +24,24 @@ namespace selinv {
 
 
 // ---------------------------------------------------------------------------
-// k_lhat_digits_z: the left operand above for X = Lhat (complex), as fp16
-// digit planes in the tcgen05 operand layout: per 16-step of k' and plane
-// (the 7 planes of a step one after the other) a block of roundup(2s, 64)
-// rows x 16, K-major 8 x 8 core matrices.  One exponent per column j of
-// Lhat over both parts (shared by rows j and s + j).  One warp per column;
+// k_digits_z: the left operand above for X = Lhat (complex), or (LINV) for
+// X = L_KK^{-1} over its s rows, the operand of Lhat_{C,K} = L_{C,K} L_KK^{-1} on
+// tcgen05, as fp16 digit planes in the tcgen05 operand layout: per 16-step
+// of k' and plane (the 7 planes of a step one after the other) a block of
+// roundup(2s, 64) rows x 16, K-major 8 x 8 core matrices.  One exponent per
+// column j of X over both parts (shared by rows j and s + j); L_KK^{-1} is
+// rounded to its grid.  One CTA per 8 columns: a warp finds a column's
+// exponent, then each thread cuts 4 entries of one column -- 8 consecutive k'
+// of both rows, whose digits differ in order and sign only -- and stores 16
+// bytes per plane and row (2-byte stores of one k' at a time: 542 us for the
+// 64-column supernodes of a 1024-atom sheet).
 // work = (problem, (K << 8) | block of 8 columns).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_lhat_digits_z(const ProbDesc *__restrict__ descs,
-                                                       const int2 *__restrict__ work, int nwork) {
+template <bool LINV>
+__global__ void __launch_bounds__(256) k_digits_z(const ProbDesc *__restrict__ descs, const int2 *__restrict__ work,
+                                                  int nwork) {
     grid_dep_wait();
+    __shared__ int colE[8];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int w = blockIdx.x;
     if (w >= nwork) return;
@@ -43,39 +51,54 @@ __global__ void __launch_bounds__(256) k_lhat_digits_z(const ProbDesc *__restric
     const int fc = P.super_ptr[K];
     const int s = P.super_ptr[K + 1] - fc;
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
-    const int c = (int)(ld - s);
-    const int j = jb * 8 + warp;
-    if (j >= s) return;
-    const double2 *Lh = static_cast<const double2 *>(P.LD) + P.panel_off[K] + (int64_t)j * ld + s;
-    int E = 0;
-    for (int q = lane; q < c; q += 32) {
-        const double2 v = Lh[q];
-        E = max(E, max(bexp(v.x), bexp(v.y)));
-    }
+    const int len = LINV ? s : (int)(ld - s);               // entries of a column
+    const int64_t ldx = LINV ? s : ld;
+    const double2 *X = LINV ? static_cast<const double2 *>(P.Linv) + P.linv_off[K]
+                            : static_cast<const double2 *>(P.LD) + P.panel_off[K] + s;
+    {
+        const int j = jb * 8 + warp;
+        int E = 0;
+        if (j < s)
+            for (int q = lane; q < len; q += 32) {
+                const double2 v = X[(int64_t)j * ldx + q];
+                E = max(E, max(bexp(v.x), bexp(v.y)));
+            }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-    if (lane == 0) P.colexp[fc + j] = E;
-    const int64_t s64 = (2 * s + 63) / 64 * 64;
-    const int k16 = (2 * c + 15) / 16 * 16;
-    uint16_t *pu = P.lhsu + P.lhsu_off[K];
-    for (int kp = lane; kp < k16; kp += 32) {
-        const int q = kp >> 1, part = kp & 1;
-        double re = 0.0, im = 0.0;
-        if (q < c) {
-            const double2 v = Lh[q];
-            re = part ? -v.y : v.x;   // row j:     (Re, -Im)
-            im = part ? v.x : v.y;    // row s + j: (Im,  Re)
+        for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+        if (lane == 0) {
+            colE[warp] = E;
+            if (j < s) (LINV ? P.linvexp : P.colexp)[fc + j] = E;
         }
-        int dr[kDig], di[kDig];
-        digits7(re, E, dr);
-        digits7(im, E, di);
-        const int64_t base = (int64_t)(kp / 16) * kDig * s64 * 16 + ((kp % 16) / 8) * 64 + kp % 8;
-        const int r1 = j, r2 = s + j;
-        const int64_t o1 = base + (r1 / 8) * 128 + (r1 % 8) * 8, o2 = base + (r2 / 8) * 128 + (r2 % 8) * 8;
+    }
+    __syncthreads();
+    const int64_t s64 = (2 * s + 63) / 64 * 64;
+    const int k16 = (2 * len + 15) / 16 * 16;
+    uint16_t *pu = LINV ? P.linvd + P.linvd_off[K] : P.lhsu + P.lhsu_off[K];
+    for (int e = threadIdx.x; e < k16; e += 256) {            // (column, 8 k' = 4 entries)
+        const int jj = e % 8, k8 = e / 8, j = jb * 8 + jj, E = colE[jj];
+        if (j >= s) continue;
+        uint32_t h1[kDig][4], h2[kDig][4];                     // rows j and s + j, a (2q, 2q + 1) pair per word
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int q = 4 * k8 + u;
+            const double2 v = q < len ? X[(int64_t)j * ldx + q] : make_double2(0.0, 0.0);
+            int dr[kDig], di[kDig];
+            digits7<LINV>(v.x, E, dr);
+            digits7<LINV>(v.y, E, di);
+#pragma unroll
+            for (int i = 0; i < kDig; i++) {
+                const uint32_t r = f16_of_int(dr[i]), m = f16_of_int(di[i]);
+                h1[i][u] = r | ((m ^ 0x8000u) << 16);          // (Re, -Im)
+                h2[i][u] = m | (r << 16);                      // (Im,  Re)
+            }
+        }
+        const int64_t base = (int64_t)(k8 / 2) * kDig * s64 * 16 + (k8 % 2) * 64;
+        const int r2 = s + j;
+        const int64_t o1 = base + (j / 8) * 128 + (j % 8) * 8, o2 = base + (r2 / 8) * 128 + (r2 % 8) * 8;
 #pragma unroll
         for (int i = 0; i < kDig; i++) {
-            pu[i * s64 * 16 + o1] = f16_of_int(dr[i]);
-            pu[i * s64 * 16 + o2] = f16_of_int(di[i]);
+            *reinterpret_cast<uint4 *>(pu + i * s64 * 16 + o1) = make_uint4(h1[i][0], h1[i][1], h1[i][2], h1[i][3]);
+            *reinterpret_cast<uint4 *>(pu + i * s64 * 16 + o2) = make_uint4(h2[i][0], h2[i][1], h2[i][2], h2[i][3]);
         }
     }
 }
@@ -95,9 +118,10 @@ __global__ void __launch_bounds__(256) k_diag_fin_z(const ProbDesc *__restrict__
     diag_fin_pair<true>(descs[it.prob], it.K, 2 * it.tile, 1);
 }
 
-cudaError_t launch_lhat_digits_z(const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st) {
+cudaError_t launch_digits_z(int linv, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st) {
     if (nwork <= 0) return cudaSuccess;
-    k_lhat_digits_z<<<nwork, 256, 0, st>>>(d, work, nwork);
+    if (linv) k_digits_z<true><<<nwork, 256, 0, st>>>(d, work, nwork);
+    else k_digits_z<false><<<nwork, 256, 0, st>>>(d, work, nwork);
     return cudaGetLastError();
 }
 

@@ -115,6 +115,8 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[NG][8], int jj, 
 // a single chunk, no k-split.  The forward's Lhat_{C,K} = L_{C,K} L_KK^{-1}
 // (Alg. 1, first loop; digits by k_linv_digits) goes to Lhat's slots of the
 // LD panel; the reverse passes' row products use the other prod_op modes.
+// Complex (CPLX and LHAT): the operand of 2s rows over k' = 2k + part
+// (k_digits_z), (64-row tile, m tile) items, Lhat only.
 template <bool CPLX, bool LHAT = false, int SYRK = 0>
 __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__restrict__ descs,
                                                               const Item *__restrict__ items, int nitems,
@@ -152,12 +154,12 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
     const int c = (int)(ld - s);
     constexpr bool DENSE = LHAT || SYRK;                 // B from dense panels
-    // digit groups: 7, or 8 for the factorization, whose error would otherwise
-    // be the dropped pairs' (2^-53 of the rows' largest per step) rather than
-    // the rounding of U
-    constexpr int NG = SYRK == 2 ? 8 : kTcDig;
+    // digit groups: 7, or 8 for the factorization and the complex Lhat, whose
+    // error would otherwise be the dropped pairs' (2^-53 of the rows' largest
+    // per step) rather than FP64 rounding
+    constexpr int NG = SYRK == 2 || (LHAT && CPLX) ? 8 : kTcDig;
     constexpr bool PAIR = SYRK == 1;                     // B's k runs over two panels
-    const int kw = PAIR ? 2 * s : (DENSE ? s : (CPLX ? 2 * c : c));   // k extent
+    const int kw = PAIR ? 2 * s : ((DENSE ? s : c) * (CPLX ? 2 : 1));   // k extent
     const int mrows = SYRK ? c : (CPLX ? 2 * s : s);     // rows of A (output rows)
     // operand rows of a stored digit block (SYRK: blocks of exactly 128 rows)
     const int s64 = SYRK ? kTcM : (mrows + 63) / 64 * 64;
@@ -242,6 +244,10 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         int e = 0;
         if (p0 + r < c)
             for (int k = tid / kTwN; k < kw; k += kTwThreads / kTwN) {
+                if (CPLX) {   // k = 2q + part: the parts of one entry share the exponent
+                    e = max(e, bexp(static_cast<const double *>(P.L)[2 * (P.panel_off[K] + (int64_t)(k >> 1) * ld + s + p0 + r) + (k & 1)]));
+                    continue;
+                }
                 const double *src = static_cast<const double *>(PAIR && k >= s ? P.Z : P.L);
                 e = max(e, bexp(src[P.panel_off[K] + (int64_t)(PAIR && k >= s ? k - s : k) * ld + s + p0 + r]));
             }
@@ -336,7 +342,18 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         const double *Lc = static_cast<const double *>(P.L) + P.panel_off[K] + s + p0 + r;   // X(p0 + r, k) = Lc[k ld]
         const double *Zc2 = static_cast<const double *>(P.Z) + P.panel_off[K] + s + p0 + r;  // PAIR: k >= s
         const bool rok = p0 + r < c;
+        const double2 *Lz = static_cast<const double2 *>(P.L) + P.panel_off[K] + s + p0 + r;   // complex X(p0 + r, q)
         auto load_dense = [&](int i_) {
+            if (CPLX) {
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const int q = (st0 + i_) * 8 + kq * 2 + u;
+                    const double2 z = (rok && i_ < n && q < s) ? Lz[(int64_t)q * ld] : make_double2(0.0, 0.0);
+                    v[2 * u] = z.x;
+                    v[2 * u + 1] = z.y;
+                }
+                return;
+            }
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const int k = (st0 + i_) * 16 + kq * 4 + u;
@@ -376,7 +393,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 uint32_t lo[4], hi[4];
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
-                    const unsigned long long wv = (unsigned long long)(fixed54<SYRK == 2>(v[u], E) + 0x80808080808080ll);
+                    const unsigned long long wv = (unsigned long long)(fixed54<NG == 8>(v[u], E) + 0x80808080808080ll);
                     lo[u] = (uint32_t)wv;
                     hi[u] = (uint32_t)(wv >> 32);
                 }
@@ -522,6 +539,20 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     if constexpr (LHAT) {
         double *Lh = static_cast<double *>(P.LD) + P.panel_off[K];
         const double *Ad = static_cast<const double *>(P.Yout) + P.panel_off[K];
+        if (CPLX) {   // rows j: real parts, rows s + j: imaginary parts
+            double *Lz = static_cast<double *>(P.LD) + 2 * P.panel_off[K];
+            for (int e = tid; e < kTwN * kTcM; e += kTwThreads) {
+                const int p = e % kTwN, mm = e / kTwN, jr = m0 + mm;
+                if (p0 + p >= c || jr >= mrows) continue;
+                const int j = jr >= s ? jr - s : jr;
+                const int e1 = rowE[p], e2 = P.linvexp[fc + j];
+                const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], e1 - 1022 + e2 - 1022 - 13);
+                // an infinity or a NaN in the row or the column: NaN, as FP64 products give
+                Lz[2 * ((int64_t)j * ld + s + p0 + p) + (jr >= s ? 1 : 0)] =
+                    e1 == 0x7FF || e2 == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll) : y;
+            }
+            return;
+        }
         const int op = P.prod_op;
         for (int e = tid; e < kTwN * kTcM; e += kTwThreads) {
             const int p = e % kTwN, j = e / kTwN;
@@ -633,6 +664,9 @@ cudaError_t configure_tcw_kernels() {
         e = cudaFuncSetAttribute(k_selinv_tcw<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)TwCfg::SMEM);
     if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_selinv_tcw<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TwCfg::SMEM);
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_selinv_tcw<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)TwCfg::SMEM);
     if (e == cudaSuccess)
@@ -649,9 +683,11 @@ cudaError_t launch_selinv_tcw(int cplx, const ProbDesc *d, const Item *items, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_lhat_tcw(const ProbDesc *d, const Item *items, int n, long long wait_limit, cudaStream_t st) {
+cudaError_t launch_lhat_tcw(int cplx, const ProbDesc *d, const Item *items, int n, long long wait_limit,
+                            cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_selinv_tcw<false, true><<<n, kTwThreads, TwCfg::SMEM, st>>>(d, items, n, nullptr, wait_limit);
+    if (cplx) k_selinv_tcw<true, true><<<n, kTwThreads, TwCfg::SMEM, st>>>(d, items, n, nullptr, wait_limit);
+    else k_selinv_tcw<false, true><<<n, kTwThreads, TwCfg::SMEM, st>>>(d, items, n, nullptr, wait_limit);
     return cudaGetLastError();
 }
 

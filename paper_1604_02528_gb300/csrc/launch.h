@@ -32,7 +32,7 @@ cudaError_t launch_tc_reduce(int tn, const ProbDesc *d, const Item *items, const
 cudaError_t configure_tcw_kernels();
 cudaError_t launch_selinv_tcw(int cplx, const ProbDesc *d, const Item *items, int n, long long *slab,
                               long long wait_limit, cudaStream_t st);
-cudaError_t launch_lhat_tcw(const ProbDesc *d, const Item *items, int n, long long wait_limit, cudaStream_t st);
+cudaError_t launch_lhat_tcw(int cplx, const ProbDesc *d, const Item *items, int n, long long wait_limit, cudaStream_t st);
 // mode 1: the reverse pass' update matrix, 2: the factorization's
 cudaError_t launch_syrk_tcw(int mode, const ProbDesc *d, const Item *items, int n, long long wait_limit,
                             cudaStream_t st);
@@ -41,7 +41,8 @@ cudaError_t launch_tcw_reduce(int cplx, const ProbDesc *d, const Item *items, co
 cudaError_t launch_diag_fin(const ProbDesc *d, const Item *items, int n, cudaStream_t st);
 cudaError_t launch_diag_tc(int tn, int cplx, const ProbDesc *d, const Item *items, int n, long long wait_limit,
                            cudaStream_t st);
-cudaError_t launch_lhat_digits_z(const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);
+// complex left operands: of Lhat, or (linv) of L_KK^{-1}
+cudaError_t launch_digits_z(int linv, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);
 cudaError_t launch_diag_fin_z(const ProbDesc *d, const Item *items, int n, cudaStream_t st);
 cudaError_t launch_check_finite(const void *x, int64_t n_doubles, int *status, cudaStream_t st);
 cudaError_t launch_selinv_persist(int dtype, const ProbDesc *d, const Item *items, const int8_t *buckets,

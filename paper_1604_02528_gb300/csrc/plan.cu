@@ -103,9 +103,9 @@ int Workspace::ensure(const PlanData &p, int dtype) {
     if (!wget(*this, &dacc, sizeof(long long) * dwords)) return SELINV_ERR_OOM;
     if (!wget(*this, &colexpZ, sizeof(int) * (size_t)std::max(p.n, 1))) return SELINV_ERR_OOM;
     if (!wget(*this, &linvexp, sizeof(int) * (size_t)std::max(p.n, 1))) return SELINV_ERR_OOM;
-    if (!wget(*this, &linvd, sizeof(uint16_t) * (size_t)std::max<int64_t>(p.linvd_total, 8)))
-        return SELINV_ERR_OOM;
-    cudaMemset(linvd, 0, sizeof(uint16_t) * (size_t)std::max<int64_t>(p.linvd_total, 8));   // padding rows stay zero
+    const int64_t nlinvd = std::max<int64_t>(dtype == SELINV_F64 ? p.linvd_total : std::max(p.linvd_total, p.linvdz_total), 8);
+    if (!wget(*this, &linvd, sizeof(uint16_t) * (size_t)nlinvd)) return SELINV_ERR_OOM;
+    cudaMemset(linvd, 0, sizeof(uint16_t) * (size_t)nlinvd);   // padding rows stay zero
     cudaMemset(colexpZ, 0, sizeof(int) * (size_t)std::max(p.n, 1));
     const size_t ny = (dtype == SELINV_F64 && p.lhs_total > 0) ? 2 * (size_t)p.nnz : 2;
     if (!wget(*this, &yacc, sizeof(long long) * ny)) return SELINV_ERR_OOM;
@@ -337,6 +337,12 @@ static int build_plan(PlanData &p, int32_t n, int32_t ns, const int32_t *super_p
         p.linvd_off[K + 1] = p.linvd_off[K] + (s >= kOzMinS ? 7 * rows * ((s + 15) / 16 * 16) : 0);
     }
     p.linvd_total = p.linvd_off[ns];
+    p.linvdz_off.assign(ns + 1, 0);
+    for (int32_t K = 0; K < ns; K++) {
+        const int64_t s = super_ptr[K + 1] - super_ptr[K];
+        p.linvdz_off[K + 1] = p.linvdz_off[K] + (s >= kZLhatS ? 7 * ((2 * s + 63) / 64 * 64) * ((2 * s + 15) / 16 * 16) : 0);
+    }
+    p.linvdz_total = p.linvdz_off[ns];
     p.tile_base.assign(ns + 1, 0);
     for (int32_t K = 0; K < ns; K++) p.tile_base[K + 1] = p.tile_base[K] + p.ntiles[K];
     p.tile_total = p.tile_base[ns];
@@ -392,6 +398,7 @@ int ensure_device(PlanData &p) {
     if ((rc = upload(&p.d_lhsuz_off, p.lhsuz_off))) return rc;
     if ((rc = upload(&p.d_tile_base, p.tile_base))) return rc;
     if ((rc = upload(&p.d_linvd_off, p.linvd_off))) return rc;
+    if ((rc = upload(&p.d_linvdz_off, p.linvdz_off))) return rc;
     if ((rc = upload(&p.d_seg_ptr, p.seg_ptr))) return rc;
     if ((rc = upload(&p.d_seg_start, p.seg_start))) return rc;
     int *st = nullptr;
@@ -404,9 +411,9 @@ int ensure_device(PlanData &p) {
 void PlanData::release_device() {
     dfree(d_super_ptr); dfree(d_sparent); dfree(d_rowptr); dfree(d_rows); dfree(d_panel_off);
     dfree(d_colbase); dfree(d_relbase); dfree(d_relidx); dfree(d_linv_off); dfree(d_part_off); dfree(d_part_off_all);
-    dfree(d_lhs_off); dfree(d_lhsu_off); dfree(d_lhsuz_off); dfree(d_tile_base); dfree(d_linvd_off); dfree(d_status); dfree(d_sel_pos);
+    dfree(d_lhs_off); dfree(d_lhsu_off); dfree(d_lhsuz_off); dfree(d_tile_base); dfree(d_linvd_off); dfree(d_linvdz_off); dfree(d_status); dfree(d_sel_pos);
     dfree(d_seg_ptr); dfree(d_seg_start);
-    d_lhs_off = d_lhsu_off = d_lhsuz_off = d_tile_base = d_linvd_off = d_sel_pos = d_seg_ptr = nullptr;
+    d_lhs_off = d_lhsu_off = d_lhsuz_off = d_tile_base = d_linvd_off = d_linvdz_off = d_sel_pos = d_seg_ptr = nullptr;
     d_seg_start = nullptr;
     d_super_ptr = d_sparent = d_rows = d_relidx = nullptr;
     d_rowptr = d_panel_off = d_colbase = d_relbase = d_linv_off = d_part_off = d_part_off_all = nullptr;
@@ -448,7 +455,7 @@ ProbDesc make_desc(const PlanData &p, Workspace &w, int dtype, const void *L, co
     d.dacc = w.dacc;
     d.colexpZ = w.colexpZ;
     d.linvd = w.linvd;
-    d.linvd_off = p.d_linvd_off;
+    d.linvd_off = dtype == SELINV_F64 ? p.d_linvd_off : p.d_linvdz_off;
     d.linvexp = w.linvexp;
     d.yacc = w.yacc;
     d.tcount = w.tcount;
@@ -502,12 +509,15 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
     auto lhat_tc = [&](int i, int s) { return plans[i]->opts.fast_contraction == 1 && s > 64; };
     // complex supernodes (symmetric or Hermitian) on tcgen05 (the transposed
     // gather-GEMM and the diagonal block over the real 2c-long contraction;
-    // level and plain schedules, not the LU form; their Lhat stays on the FP64 pipe)
+    // level and plain schedules, not the LU form)
     auto zok = [&](int i, int s) {
         const selinv_opts &o = plans[i]->opts;
         return !descs[i].lu && descs[i].dtype == SELINV_C128 && o.fast_contraction == 1 &&
                s >= std::max(kOzMinS, o.oz_min_s) && (mode == SELINV_SCHED_LEVEL || mode == SELINV_SCHED_PLAIN);
     };
+    // ... whose Lhat runs there too: from 17 columns on (a CTA's 64 rows take
+    // about 15 us on tcgen05; on the FP64 pipe 9 us at 16 columns, 34 at 32)
+    auto zlhat = [&](int i, int s) { return zok(i, s) && s >= kZLhatS; };
     // DFMA supernodes small enough for a warp each (k_selinv_tiny; not the LU form)
     auto tiny = [&](int i, int32_t K) {
         const PlanData &p = *plans[i];
@@ -602,6 +612,17 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             }
             const int cnt = (int)(S.h_work.size() - off);
             if (cnt) S.launches.push_back({KL_LINV_DIGITS, SELINV_F64, 0, off, cnt, -1});
+            const int64_t offz = (int64_t)S.h_work.size();
+            for (int i = 0; i < np; i++) {
+                const PlanData &p = *plans[i];
+                for (int32_t K = 0; K < p.ns; K++) {
+                    const int s = p.super_ptr[K + 1] - p.super_ptr[K];
+                    if (p.rowptr[K + 1] - p.rowptr[K] == s || !actn(i, K) || !zlhat(i, s)) continue;
+                    for (int jb = 0; jb < (s + 7) / 8; jb++) S.h_work.push_back(make_int2(i, (K << 8) | jb));
+                }
+            }
+            const int cntz = (int)(S.h_work.size() - offz);
+            if (cntz) S.launches.push_back({KL_LINV_DIGITS, SELINV_C128, 0, offz, cntz, -1});
         }
         {
             // Lhat of the supernodes wider than 64 columns on tcgen05: (K, 64-row tile) items
@@ -617,6 +638,20 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             }
             const int cnt = (int)(S.h_items.size() - off);
             if (cnt) S.launches.push_back({KL_LHAT_OZ, SELINV_F64, kTcWide, off, cnt, -1});
+            // the complex ones: (K, 64-row tile, 128 of the 2s output rows) items
+            const int64_t offz = (int64_t)S.h_items.size();
+            for (int i = 0; i < np; i++) {
+                const PlanData &p = *plans[i];
+                for (int32_t K = 0; K < p.ns; K++) {
+                    const int s = p.super_ptr[K + 1] - p.super_ptr[K];
+                    const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s;
+                    if (c == 0 || !actn(i, K) || !zlhat(i, s)) continue;
+                    const int64_t nt = (c + kTcWideRows - 1) / kTcWideRows * ((2 * s + kTcRows - 1) / kTcRows);
+                    for (int64_t t = 0; t < nt; t++) S.h_items.push_back({i, K, (int)t, 1});
+                }
+            }
+            const int cntz = (int)(S.h_items.size() - offz);
+            if (cntz) S.launches.push_back({KL_LHAT_OZ, SELINV_C128, kTcWide, offz, cntz, -1});
         }
         for (int tn : {64, 32, 16}) {
             const int64_t off = (int64_t)S.h_items.size();
@@ -645,7 +680,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                     for (int32_t K = 0; K < p.ns; K++) {
                         const int s = p.super_ptr[K + 1] - p.super_ptr[K];
                         const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s;
-                        if (c == 0 || !actn(i, K) || bucket_of(s) != b || ozok(i, s)) continue;
+                        if (c == 0 || !actn(i, K) || bucket_of(s) != b || ozok(i, s) || zlhat(i, s)) continue;
                         for (int t = 0; t < p.ntiles[K]; t++) S.h_items.push_back({i, K, t, p.ntiles[K]});
                     }
                 }
@@ -1227,13 +1262,15 @@ cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, c
     case KL_LHAT: return launch_lhat(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_SELINV: return launch_selinv(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_DIGITS:
-        if (L.dtype != SELINV_F64) return launch_lhat_digits_z(d, S.d_work + L.off, L.count, st);
+        if (L.dtype != SELINV_F64) return launch_digits_z(0, d, S.d_work + L.off, L.count, st);
         return launch_lhat_digits(d, S.d_work + L.off, L.count, st);
     case KL_SELINV_OZ: return launch_selinv_oz(L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_DIAG: return launch_diag_oz(d, S.d_items + L.off, L.count, st);
-    case KL_LINV_DIGITS: return launch_linv_digits(d, S.d_work + L.off, L.count, st);
+    case KL_LINV_DIGITS:
+        if (L.dtype != SELINV_F64) return launch_digits_z(1, d, S.d_work + L.off, L.count, st);
+        return launch_linv_digits(d, S.d_work + L.off, L.count, st);
     case KL_LHAT_OZ:
-        if (L.bucket == kTcWide) return launch_lhat_tcw(d, S.d_items + L.off, L.count, S.spin_limit, st);
+        if (L.bucket == kTcWide) return launch_lhat_tcw(L.dtype != SELINV_F64, d, S.d_items + L.off, L.count, S.spin_limit, st);
         return launch_lhat_oz(L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_SELINV_TC:
         if (L.bucket == kTcWide)

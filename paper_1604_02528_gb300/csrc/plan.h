@@ -45,6 +45,7 @@ struct PlanData {
     std::vector<int64_t> lhsuz_off;         // complex Lhat operand (2s rows, 2c k) in that layout
     std::vector<int64_t> tile_base;         // prefix sums of the 64-row tiles of each supernode
     std::vector<int64_t> linvd_off;         // digit planes of L_KK^{-1} (tensor-core path)
+    std::vector<int64_t> linvdz_off;        // complex operand of L_KK^{-1} (2s rows, 2s k)
     // subset selection: the supernodes that run (empty: all) and the panel
     // positions of the selected entries
     std::vector<uint8_t> active;
@@ -53,13 +54,13 @@ struct PlanData {
     int64_t *d_sel_pos = nullptr;
     int nlevels = 0;
     int64_t nnz = 0, linv_total = 0, part_max = 1, part_all = 1, lhs_total = 0, lhsu_total = 0, tile_total = 0, linvd_total = 0,
-            lhsuz_total = 0;
+            lhsuz_total = 0, linvdz_total = 0;
     // device copies
     int32_t *d_super_ptr = nullptr, *d_sparent = nullptr, *d_rows = nullptr, *d_relidx = nullptr;
     int64_t *d_rowptr = nullptr, *d_panel_off = nullptr, *d_colbase = nullptr, *d_relbase = nullptr;
     int64_t *d_linv_off = nullptr, *d_part_off = nullptr, *d_part_off_all = nullptr, *d_lhs_off = nullptr, *d_lhsu_off = nullptr, *d_tile_base = nullptr,
             *d_lhsuz_off = nullptr;
-    int64_t *d_linvd_off = nullptr;
+    int64_t *d_linvd_off = nullptr, *d_linvdz_off = nullptr;
     int64_t *d_seg_ptr = nullptr;      // owner segments (push schedule)
     int32_t *d_seg_start = nullptr;
     int *d_status = nullptr;
@@ -129,6 +130,7 @@ inline bool oz_eligible(int dtype, int s, const selinv_opts &o) {
     return o.fast_contraction && dtype == SELINV_F64 && s >= std::max(kOzMinS, o.oz_min_s);
 }
 constexpr int kTcRows = 128;   // rows of C per tcgen05 item
+constexpr int kZLhatS = 17;    // narrowest complex tensor-core supernode whose Lhat runs on tcgen05 (FP64 tiles below)
 constexpr int kTcChunkSteps = 8;   // k16 steps per exact fp32 chunk of the tensor-core kernels (k-ranges are whole chunks)
 constexpr int kTcWide = 128;   // launch bucket of the transposed tcgen05 kernel (supernodes wider than 64)
 constexpr int kTcWideRows = 64;   // rows of C per item of that kernel

@@ -70,3 +70,27 @@ def test_noalloc_widths(native, cuda_device, s):
     ref = np.linalg.inv(a)
     assert np.linalg.norm(got[:, :s] - ref) <= 1e-12 * np.linalg.norm(ref)
     assert np.all(got[:, s:] == -7.0)                # nothing past the block's rows
+
+
+# complex Lhat on the tensor cores: the widths around its narrowest, one and
+# two 128-row tiles of the 2s output rows, odd remainders of the 16-step k,
+# C of one to several 64-row tiles, and values spread over decades by rows.
+# The digits carry 54 bits below a row's largest entry and the dropped pairs
+# 2^-61 of it, so Lhat errs by s 2^-54 of row times column maxima: 1e-12
+# normwise with room.
+@pytest.mark.parametrize("kind", ["c128", "c128h"])
+@pytest.mark.parametrize("width,n", [(16, 90), (17, 81), (18, 82), (31, 96), (32, 97), (33, 290), (63, 128), (64, 200), (65, 194), (127, 300)])
+def test_complex_lhat_widths(native, cuda_device, width, n, kind):
+    import torch
+    from paper_1604_02528_gb300.api import SelInvContext
+    make = synth.random_sparse_hpd if kind == "c128h" else synth.random_sparse_spd
+    kw = {"complex_values": True} if kind == "c128" else {}
+    p = make(n, 1.0, n, supernodes={"kind": "fundamental", "cap": width, "fill": 0.0}, **kw)
+    ctx = SelInvContext.from_problem(p)
+    ctx.set_options(oz_min_s=1)
+    sym = oracle.symbolic_for(p)
+    L0, D0 = oracle.ldlt(p, sym)
+    Z = ctx.selinv(torch.from_numpy(L0).cuda(), torch.from_numpy(D0).cuda())
+    torch.cuda.synchronize()
+    assert ctx.status() == 0
+    assert oracle.block_errors(sym, Z.cpu().numpy(), oracle.selinv(sym, L0, D0, hermitian=kind == "c128h")).max() <= 1e-12
