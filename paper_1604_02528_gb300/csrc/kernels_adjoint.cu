@@ -132,10 +132,7 @@ struct AdjData {
     // the per-level loops of the two passes as CUDA graphs (captured on first
     // use, rebuilt when the lists or the workspace change)
     int gen = 0;                              // bumped whenever the lists are rebuilt
-    cudaGraphExec_t g_sel = nullptr, g_fac = nullptr;
-    int g_sel_n = 0, g_fac_n = 0;             // launches in each graph
-    long long g_sel_key = -1, g_fac_key = -1;
-    const void *g_sel_ws = nullptr, *g_fac_ws = nullptr;
+    CapturedLoop g_sel, g_fac;
     // row products of the wide supernodes on the transposed tcgen05 kernel:
     // (K, 64-row tile) items and (K, 8-column block) digit work per level, the
     // digit planes of the s x s factor (7 x roundup(s, 64) x roundup(s, 16) per
@@ -1266,8 +1263,8 @@ void adjoint_release(void *p) {
     fr(a->d_sm); fr(a->d_wd); fr(a->d_row); fr(a->d_rg); fr(a->d_mbp); fr(a->d_dig); fr(a->d_tcdesc); fr(a->cy);
     fr(a->d_pr); fr(a->d_sdw); fr(a->sd); fr(a->d_sd_off); fr(a->sdexp); fr(a->d_pdp);
     fr(a->d_syw); fr(a->d_sy); fr(a->d_vn); fr(a->sy); fr(a->d_sy_off); fr(a->syexp); fr(a->d_sydesc);
-    if (a->g_sel) cudaGraphExecDestroy(a->g_sel);
-    if (a->g_fac) cudaGraphExecDestroy(a->g_fac);
+    a->g_sel.release();
+    a->g_fac.release();
     a->tcs.release();
     a->tcn.release();
     delete a;
@@ -1644,53 +1641,6 @@ static void row_product(AdjData *a, int pd, int li, cudaStream_t st) {
     }
 }
 
-// Issues body(st) through a CUDA graph captured on the first call and replayed
-// afterwards.  The per-level launches of the reverse passes take only the
-// plan's own device buffers as arguments (the caller's pointers reach them
-// through descriptors uploaded before the graph runs), so one capture serves
-// every call until the lists (key) or the workspace (ws) change.  A stream
-// that cannot be captured -- the legacy default stream, or one the caller is
-// capturing already -- runs body(st) directly.
-template <class F>
-static int run_captured(cudaGraphExec_t &exec, int &nlaunch, long long &key, const void *&ws, long long want_key,
-                        const void *want_ws, cudaStream_t st, F body) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (st == nullptr || st == cudaStreamLegacy || cudaStreamIsCapturing(st, &cs) != cudaSuccess ||
-        cs != cudaStreamCaptureStatusNone) {
-        body(st);
-        return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
-    }
-    if (!exec || key != want_key || ws != want_ws) {
-        if (exec) cudaGraphExecDestroy(exec);
-        exec = nullptr;
-        const int64_t n0 = selinv_launch_count();
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
-        body(st);
-        cudaError_t e = cudaStreamEndCapture(st, &g);
-        nlaunch = (int)(selinv_launch_count() - n0);
-        note_launch(-nlaunch);   // captured, not yet issued
-        if (e != cudaSuccess || !g) {
-            if (g) cudaGraphDestroy(g);
-            return SELINV_ERR_CUDA;
-        }
-        if (programmatic_edges(g) != cudaSuccess) {
-            cudaGraphDestroy(g);
-            return SELINV_ERR_CUDA;
-        }
-        e = cudaGraphInstantiate(&exec, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) {
-            exec = nullptr;
-            return SELINV_ERR_CUDA;
-        }
-        key = want_key;
-        ws = want_ws;
-    }
-    note_launch(nlaunch);
-    return cudaGraphLaunch(exec, st) == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
-}
-
 extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *L, const void *D,
                               const void *Z, const void *Zbar, void *Lbar, void *Dbar, void *stream) {
     NvtxRange nvtx_range("selinv_adjoint");
@@ -1808,7 +1758,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
             if (j1 > j0) { k_adj_sel_dbar<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0)); note_launch(); }
         }
     };
-    return run_captured(a->g_sel, a->g_sel_n, a->g_sel_key, a->g_sel_ws, a->gen, w.colexpZ, st, levels);
+    return a->g_sel.run(a->gen, w.colexpZ, st, levels);
 }
 
 extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const void *L, const void *D,
@@ -1908,7 +1858,7 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
             }
         }
     };
-    if ((rc = run_captured(a->g_fac, a->g_fac_n, a->g_fac_key, a->g_fac_ws, a->gen, w.colexpZ, st, levels))) return rc;
+    if ((rc = a->g_fac.run(a->gen, w.colexpZ, st, levels))) return rc;
     if (f->nnzA > 0) {
         const int blocks = (int)std::min<int64_t>((f->nnzA + 255) / 256, 152 * 8);
         k_gather_vals<<<blocks, 256, 0, st>>>(f->d_a_pos, a->Ab, f->nnzA, static_cast<double *>(Abar_vals));

@@ -457,6 +457,7 @@ void factor_release(selinv_plan_s *plan) {
     fr(f->d_a_pos); fr(f->d_tiles); fr(f->d_js); fr(f->d_desc);
     fr(f->d_asm); fr(f->d_uitems); fr(f->d_uoff); fr(f->d_chpos); fr(f->U);
     fr(f->d_tcitems); fr(f->d_tcwork); fr(f->d_digoff); fr(f->digits); fr(f->digexp);
+    for (CapturedLoop &g : f->loop) g.release();
     adjoint_release(f->adj);
     delete f;
     plan->factor = nullptr;
@@ -696,56 +697,58 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         if (configure_factor_kernels<T>() != cudaSuccess) return SELINV_ERR_CUDA;
         f->configured[sizeof(T) > 8] = true;
     }
-    for (size_t l = 0; l < f->lev.size(); l++) {
-        // the children's update matrices complete J's panel and start U_J
-        for (int r = 0; r < f->npass; r++) {
-            const int64_t x0 = f->asm_lptr[l * f->npass + r], x1 = f->asm_lptr[l * f->npass + r + 1];
-            if (x1 > x0) { k_fasm<T><<<(int)(x1 - x0), 256, 0, st>>>(fd, f->d_asm + x0, (int)(x1 - x0)); note_launch(); }
+    auto levels = [&](cudaStream_t st) {
+        for (size_t l = 0; l < f->lev.size(); l++) {
+            // the children's update matrices complete J's panel and start U_J
+            for (int r = 0; r < f->npass; r++) {
+                const int64_t x0 = f->asm_lptr[l * f->npass + r], x1 = f->asm_lptr[l * f->npass + r + 1];
+                if (x1 > x0) { k_fasm<T><<<(int)(x1 - x0), 256, 0, st>>>(fd, f->d_asm + x0, (int)(x1 - x0)); note_launch(); }
+            }
+            const FactorLevel &v = f->lev[l];
+            if (v.wide0 > v.small0) {
+                k_fsmall<T><<<(int)(v.wide0 - v.small0), kFsThreads, 2 * sizeof(T) * (size_t)v.small_elems, st>>>(
+                    fd, f->d_js + v.small0, (int)(v.wide0 - v.small0));
+                note_launch();
+            }
+            if (v.wide1 > v.wide0) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)((v.wide1 - v.wide0) * v.cl));
+                cfg.blockDim = dim3(kFdThreads);
+                cfg.dynamicSmemBytes = sizeof(T) * (size_t)(3 * kFdRows * kFdLd + fd_rows_elems(v.wide_s, v.cl));
+                cfg.stream = st;
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = (unsigned)v.cl;
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                cudaLaunchKernelEx(&cfg, k_fdiag<T>, (const FactorDesc *)fd, (const int *)(f->d_js + v.wide0),
+                                   (int)(v.wide1 - v.wide0));   // (an error stays for cudaGetLastError)
+                note_launch();
+            }
+            if (v.tile1 > v.tile0) {
+                k_ftrsm<T><<<(int)(v.tile1 - v.tile0), kFtThreads, sizeof(T) * (size_t)tri_store_elems(v.wide_s), st>>>(
+                    fd, f->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
+                note_launch();
+            }
+            const FactorLevel::Upd &u = v.upd[tc];
+            if (u.i1 > u.i0) {
+                const int nu = (int)(u.i1 - u.i0);
+                if (u.b == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
+                else if (u.b == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
+                else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
+                note_launch();
+            }
+            if (tc && v.tc1 > v.tc0) {
+                const int nw = (int)(v.tw1 - v.tw0);
+                k_fupd_digits<<<nw, 256, 0, st>>>(fd, f->d_tcwork + v.tw0, nw);
+                launch_syrk_tcw(2, &fd->up, f->d_tcitems + v.tc0, (int)(v.tc1 - v.tc0), p.opts.spin_limit, st);
+                note_launch(2);
+            }
         }
-        const FactorLevel &v = f->lev[l];
-        if (v.wide0 > v.small0) {
-            k_fsmall<T><<<(int)(v.wide0 - v.small0), kFsThreads, 2 * sizeof(T) * (size_t)v.small_elems, st>>>(
-                fd, f->d_js + v.small0, (int)(v.wide0 - v.small0));
-            note_launch();
-        }
-        if (v.wide1 > v.wide0) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)((v.wide1 - v.wide0) * v.cl));
-            cfg.blockDim = dim3(kFdThreads);
-            cfg.dynamicSmemBytes = sizeof(T) * (size_t)(3 * kFdRows * kFdLd + fd_rows_elems(v.wide_s, v.cl));
-            cfg.stream = st;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = (unsigned)v.cl;
-            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            if (cudaLaunchKernelEx(&cfg, k_fdiag<T>, (const FactorDesc *)fd, (const int *)(f->d_js + v.wide0),
-                                   (int)(v.wide1 - v.wide0)) != cudaSuccess)
-                return SELINV_ERR_CUDA;
-            note_launch();
-        }
-        if (v.tile1 > v.tile0) {
-            k_ftrsm<T><<<(int)(v.tile1 - v.tile0), kFtThreads, sizeof(T) * (size_t)tri_store_elems(v.wide_s), st>>>(
-                fd, f->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
-            note_launch();
-        }
-        const FactorLevel::Upd &u = v.upd[tc];
-        if (u.i1 > u.i0) {
-            const int nu = (int)(u.i1 - u.i0);
-            if (u.b == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
-            else if (u.b == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
-            else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
-            note_launch();
-        }
-        if (tc && v.tc1 > v.tc0) {
-            const int nw = (int)(v.tw1 - v.tw0);
-            k_fupd_digits<<<nw, 256, 0, st>>>(fd, f->d_tcwork + v.tw0, nw);
-            launch_syrk_tcw(2, &fd->up, f->d_tcitems + v.tc0, (int)(v.tc1 - v.tc0), p.opts.spin_limit, st);
-            note_launch(2);
-        }
-    }
-    return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
+    };
+    if (cudaGetLastError() != cudaSuccess) return SELINV_ERR_CUDA;
+    return f->loop[sizeof(T) > 8].run(2 * p.opts.spin_limit + tc, f->d_js, st, levels);
 }
 
 }  // namespace selinv

@@ -476,6 +476,9 @@ ProbDesc make_desc(const PlanData &p, Workspace &w, int dtype, const void *L, co
 void Schedule::release() {
     if (graph) cudaGraphExecDestroy(graph);
     graph = nullptr;
+    if (cap) cudaStreamDestroy(cap);
+    cap = nullptr;
+    issued = false;
     if (graph_host) cudaGraphExecDestroy(graph_host);
     graph_host = nullptr;
     host_key.fill(nullptr);
@@ -1432,14 +1435,68 @@ cudaError_t programmatic_edges(cudaGraph_t g) {
     return cudaSuccess;
 }
 
+int CapturedLoop::run(long long want_key, const void *want_ws, cudaStream_t st,
+                      const std::function<void(cudaStream_t)> &body) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool legacy = st == nullptr || st == cudaStreamLegacy;
+    const bool capturing = !legacy && (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
+    const bool known = key == want_key && ws == want_ws;
+    if (capturing || !known) {
+        if (!capturing) {
+            if (exec) cudaGraphExecDestroy(exec);
+            exec = nullptr;
+            key = want_key;
+            ws = want_ws;
+        }
+        body(st);
+        return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
+    }
+    if (!exec) {
+        if (!cap && cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return SELINV_ERR_CUDA;
+        const int64_t n0 = selinv_launch_count();
+        cudaGraph_t g = nullptr;
+        if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
+        body(cap);
+        cudaError_t e = cudaStreamEndCapture(cap, &g);
+        nlaunch = (int)(selinv_launch_count() - n0);
+        note_launch(-nlaunch);   // captured, not yet issued
+        if (e == cudaSuccess && g) e = programmatic_edges(g);
+        if (e == cudaSuccess && g) e = cudaGraphInstantiate(&exec, g, 0);
+        if (g) cudaGraphDestroy(g);
+        if (e != cudaSuccess || !g) {
+            exec = nullptr;
+            return SELINV_ERR_CUDA;
+        }
+    }
+    note_launch(nlaunch);
+    return cudaGraphLaunch(exec, st) == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
+}
+
+void CapturedLoop::release() {
+    if (exec) cudaGraphExecDestroy(exec);
+    if (cap) cudaStreamDestroy(cap);
+    exec = nullptr;
+    cap = nullptr;
+    key = -1;
+    ws = nullptr;
+}
+
 int run_schedule(Schedule &S, cudaStream_t st, bool use_graph) {
-    // graphs need a capturable stream (not the legacy default stream)
-    if (use_graph && st != nullptr && st != cudaStreamLegacy) {
+    // a graph captured on the first call, or -- for the legacy default stream,
+    // which cannot be captured -- on a stream of its own on the second
+    // (launch by launch a 63 x 63 grid's 72 kernels leave gaps of 2 us each)
+    const bool legacy = st == nullptr || st == cudaStreamLegacy;
+    const bool first = !S.issued;
+    S.issued = true;
+    if (use_graph && (S.graph || !legacy || !first)) {
         if (!S.graph) {
             cudaGraph_t g = nullptr;
-            if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
-            cudaError_t e = issue(S, st, false);
-            cudaError_t e2 = cudaStreamEndCapture(st, &g);
+            if (legacy && !S.cap && cudaStreamCreateWithFlags(&S.cap, cudaStreamNonBlocking) != cudaSuccess)
+                return SELINV_ERR_CUDA;
+            cudaStream_t cs = legacy ? S.cap : st;
+            if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
+            cudaError_t e = issue(S, cs, false);
+            cudaError_t e2 = cudaStreamEndCapture(cs, &g);
             if (e != cudaSuccess || e2 != cudaSuccess) {
                 if (g) cudaGraphDestroy(g);
                 return SELINV_ERR_CUDA;

@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <algorithm>
 #include <array>
+#include <functional>
 #include <memory>
 #include <utility>
 #include <vector>
@@ -173,6 +174,11 @@ struct Schedule {
     long long spin_limit = 0;   // bound of every device wait of the schedule's kernels
     int wait_on_unset = 0;
     cudaGraphExec_t graph = nullptr;
+    // the legacy default stream cannot be captured: its graph is captured on a
+    // stream of the schedule's own, on the second call (the first is issued
+    // launch by launch, so that a single inversion does not pay for a graph)
+    cudaStream_t cap = nullptr;
+    bool issued = false;
     // selinv_numeric_host's captured call and the buffers it was captured for
     cudaGraphExec_t graph_host = nullptr;
     std::array<const void *, 6> host_key{};
@@ -214,6 +220,23 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
 int run_schedule(Schedule &S, cudaStream_t st, bool use_graph);
 // kernel-to-kernel edges of a captured graph -> programmatic (see plan.cu)
 cudaError_t programmatic_edges(cudaGraph_t g);
+
+// A loop of launches replayed as a CUDA graph: issued directly on the first
+// call, captured on the second (on a stream of its own, so the caller's may be
+// the legacy default stream) and replayed from then on.  The launches take
+// only the plan's own device buffers as arguments (the caller's pointers reach
+// the kernels through descriptors uploaded before), so one capture serves
+// every call until the lists (key) or the workspace (ws) change.  A stream
+// that the caller is capturing gets the launches themselves.
+struct CapturedLoop {
+    cudaGraphExec_t exec = nullptr;
+    cudaStream_t cap = nullptr;
+    int nlaunch = 0;
+    long long key = -1;
+    const void *ws = nullptr;
+    int run(long long want_key, const void *want_ws, cudaStream_t st, const std::function<void(cudaStream_t)> &body);
+    void release();
+};
 cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, cudaStream_t st);
 
 // factorization / adjoint state
@@ -274,6 +297,7 @@ struct FactorData {
     int32_t *d_chpos = nullptr;
     void *U = nullptr;
     size_t U_bytes = 0;
+    CapturedLoop loop[2];             // the level loops (real, complex)
     FactorDesc *d_desc = nullptr;
     const void *key_L = nullptr, *key_D = nullptr;
     int key_dtype = -1;
