@@ -13,9 +13,10 @@ namespace selinv {
 // one after the other (K-major 8 x 8 core matrices), one exponent per row
 // (exps[row]).  A warp per 4 rows finds their exponents, then each thread
 // cuts 8 consecutive k of one row, a 16-byte store per plane.
-// ROUND: to the nearest point of the row's grid instead of toward zero.
-template <bool ROUND, class X>
-__device__ __forceinline__ void digit_rows(const X &x, int kw, int c, int b, uint16_t *base, int *exps) {
+// ROUND: to the nearest point of the row's grid instead of toward zero, the
+// columns' exponents shifted by add(k) (balanced rows; else add gives 0).
+template <bool ROUND, class X, class S>
+__device__ __forceinline__ void digit_rows(const X &x, const S &add, int kw, int c, int b, uint16_t *base, int *exps) {
     __shared__ int rowE[32];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int k16 = (kw + 15) / 16 * 16, nst = k16 / 16;
@@ -23,7 +24,7 @@ __device__ __forceinline__ void digit_rows(const X &x, int kw, int c, int b, uin
         const int r = warp * 4 + rr, p = b * 32 + r;
         int E = 0;
         if (p < c)
-            for (int k = lane; k < kw; k += 32) E = max(E, bexp(x(p, k)));
+            for (int k = lane; k < kw; k += 32) E = max(E, ROUND ? bal_exp(bexp(x(p, k)), add(k)) : bexp(x(p, k)));
 #pragma unroll
         for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
         if (lane == 0) {
@@ -39,8 +40,8 @@ __device__ __forceinline__ void digit_rows(const X &x, int kw, int c, int b, uin
 #pragma unroll
         for (int t = 0; t < 8; t += 2) {
             int d0[kDig], d1[kDig];
-            digits7<ROUND>(k0 + t < kw ? x(p, k0 + t) : 0.0, rowE[r], d0);
-            digits7<ROUND>(k0 + t + 1 < kw ? x(p, k0 + t + 1) : 0.0, rowE[r], d1);
+            digits7<ROUND>(k0 + t < kw ? x(p, k0 + t) : 0.0, rowE[r], d0, k0 + t < kw ? add(k0 + t) : 0);
+            digits7<ROUND>(k0 + t + 1 < kw ? x(p, k0 + t + 1) : 0.0, rowE[r], d1, k0 + t + 1 < kw ? add(k0 + t + 1) : 0);
 #pragma unroll
             for (int i = 0; i < kDig; i++) h[i][t / 2] = f16_of_int(d0[i]) | (f16_of_int(d1[i]) << 16);
         }

@@ -15,15 +15,31 @@ __device__ __forceinline__ uint32_t f16_of_int(int v) {
     return (uint32_t)__half_as_ushort(__float2half_rn(f));
 }
 
+// Balanced operands of a product over the columns k of a supernode, sum_k
+// X(p, k) Y(k, j) with X(p, k) growing like 1 / sqrt(D_k) and Y like sqrt(D_k)
+// (rows of L against rows of L D, or against columns of L_KK^{-1}): in a badly
+// scaled matrix D spans many decades within one supernode, and digits on one
+// grid per row would lose what the grid's largest entry hides.  With e_k half
+// of D_k's exponent, X 2^{e_k} and Y 2^{-e_k} have rows of even size and the
+// same product, exactly.  k_balance(D_k) is e_k + kBalBias, the shift of X's
+// exponents; 2 kBalBias - k_balance that of Y's; exponents on the biased scale
+// stay positive, and kBalBad marks an infinity or a NaN.
+constexpr int kBalBias = 1024, kBalBad = 1 << 20;
+__device__ __forceinline__ int k_balance(int dexp) {   // dexp: biased exponent of D_k (its larger part)
+    return ((dexp - 1023) >> 1) + kBalBias;
+}
+__device__ __forceinline__ int bal_exp(int e, int add) { return e == 0x7FF ? kBalBad : (e ? e + add : 0); }
+
 // 7 balanced base-256 digits (most significant first) of x on the grid of
 // biased exponent E (E >= exponent of x): x ~= sum_i d_i 2^(E-1022-7-8i), cut
-// toward zero (ROUND: to nearest, half away from zero).
+// toward zero (ROUND: to nearest, half away from zero); add: x taken as
+// x 2^add (E on that scale).
 template <bool ROUND = false>
-__device__ __forceinline__ void digits7(double x, int E, int d[kDig]) {
+__device__ __forceinline__ void digits7(double x, int E, int d[kDig], int add = 0) {
     const long long b = __double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7FF);
     unsigned long long mant = ex ? ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) : 0ull;
-    const int sh = E - ex - 2;                       // M = mant * 2^(2 - (E - ex)) < 2^55
+    const int sh = E - (ex + add) - 2;               // M = mant * 2^(2 - (E - ex)) < 2^55
     if (ROUND && sh > 0 && sh < 55) mant += 1ull << (sh - 1);
     unsigned long long M = sh < 0 ? (mant << (-sh)) : (sh < 64 ? (mant >> sh) : 0ull);
 #pragma unroll

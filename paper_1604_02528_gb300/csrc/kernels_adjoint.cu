@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(256) k_syrk_digits(const AdjDesc *__restrict__
     auto x = [&](int p, int k) -> double {   // [Ybar, Lhat](p, k)
         return k < s ? A.YB[off + (int64_t)k * ld + s + p] : A.LD[off + (int64_t)(k - s) * ld + s + p];
     };
-    digit_rows<false>(x, 2 * s, (int)(ld - s), b, sy + sy_off[K], syexp + A.rowptr[K] + s);
+    digit_rows<false>(x, [](int) { return 0; }, 2 * s, (int)(ld - s), b, sy + sy_off[K], syexp + A.rowptr[K] + s);
 }
 
 // The k16 stage of a row-product block: thread (tx, ty) adds rows ty + 16 i

@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(256) k_fupd_digits(const FactorDesc *__restric
     const double *LC = static_cast<const double *>(F.L) + F.panel_off[J] + s;
     const double *DJ = static_cast<const double *>(F.D) + F.super_ptr[J];
     auto x = [&](int p, int k) -> double { return LC[(int64_t)k * ld + p] * DJ[k]; };
-    digit_rows<true>(x, s, (int)(ld - s), b, F.up.linvd + F.up.linvd_off[J], F.up.linvexp + F.rowptr[J] + s);
+    auto add = [&](int k) { return 2 * kBalBias - k_balance(bexp(DJ[k])); };
+    digit_rows<true>(x, add, s, (int)(ld - s), b, F.up.linvd + F.up.linvd_off[J], F.up.linvexp + F.rowptr[J] + s);
 }
 
 // ---------------------------------------------------------------------------
@@ -635,6 +636,7 @@ FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, 
     h.up.rowptr = p.d_rowptr;
     h.up.panel_off = p.d_panel_off;
     h.up.L = L;
+    h.up.D = D;
     h.up.linvd = f->digits;
     h.up.linvd_off = f->d_digoff;
     h.up.linvexp = f->digexp;

@@ -30,7 +30,7 @@ namespace selinv {
 // of k' and plane (the 7 planes of a step one after the other) a block of
 // roundup(2s, 64) rows x 16, K-major 8 x 8 core matrices.  One exponent per
 // column j of X over both parts (shared by rows j and s + j); L_KK^{-1} is
-// rounded to its grid.  One CTA per 8 columns: a warp finds a column's
+// balanced by D and rounded to its grid.  One CTA per 8 columns: a warp finds a column's
 // exponent, then each thread cuts 4 entries of one column -- 8 consecutive k'
 // of both rows, whose digits differ in order and sign only -- and stores 16
 // bytes per plane and row (2-byte stores of one k' at a time: 542 us for the
@@ -55,13 +55,17 @@ __global__ void __launch_bounds__(256) k_digits_z(const ProbDesc *__restrict__ d
     const int64_t ldx = LINV ? s : ld;
     const double2 *X = LINV ? static_cast<const double2 *>(P.Linv) + P.linv_off[K]
                             : static_cast<const double2 *>(P.LD) + P.panel_off[K] + s;
+    // L_KK^{-1}'s rows k are balanced against L's columns (k_balance)
+    const zd *D = static_cast<const zd *>(P.D) + fc;
+    auto add = [&](int q) { return LINV ? 2 * kBalBias - k_balance(bexp(D[q])) : 0; };
     {
         const int j = jb * 8 + warp;
         int E = 0;
         if (j < s)
             for (int q = lane; q < len; q += 32) {
                 const double2 v = X[(int64_t)j * ldx + q];
-                E = max(E, max(bexp(v.x), bexp(v.y)));
+                const int ev = max(bexp(v.x), bexp(v.y));
+                E = max(E, LINV ? bal_exp(ev, add(q)) : ev);
             }
 #pragma unroll
         for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
@@ -83,8 +87,9 @@ __global__ void __launch_bounds__(256) k_digits_z(const ProbDesc *__restrict__ d
             const int q = 4 * k8 + u;
             const double2 v = q < len ? X[(int64_t)j * ldx + q] : make_double2(0.0, 0.0);
             int dr[kDig], di[kDig];
-            digits7<LINV>(v.x, E, dr);
-            digits7<LINV>(v.y, E, di);
+            const int sh = q < len ? add(q) : 0;
+            digits7<LINV>(v.x, E, dr, sh);
+            digits7<LINV>(v.y, E, di, sh);
 #pragma unroll
             for (int i = 0; i < kDig; i++) {
                 const uint32_t r = f16_of_int(dr[i]), m = f16_of_int(di[i]);

@@ -101,9 +101,10 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[NG][8], int jj, 
 // number of 64-row blocks + 64-row block) on or below the diagonal.
 // SYRK 2: the factorization's Schur update U_K -= (L_CK D_K) L_CK^T over the s
 // columns, the same with A = digit planes of L_CK D_K and B = L_CK.  Rows are
-// rounded to their grid, not cut (the entries of L mostly share a sign, and
-// cut products would all err to one side), and the digit pairs i + j = 7
-// count too: L's error against 64-bit arithmetic is then that of FP64 FMA.
+// balanced by D (k_balance) and rounded to their grid, not cut (the entries
+// of L mostly share a sign, and cut products would all err to one side), and
+// the digit pairs i + j = 7 count too: L's error against 64-bit arithmetic is
+// then that of FP64 FMA.
 // A row that holds an infinity or a NaN makes its results NaN (the digits
 // cannot carry it), so that a later pivot reports it.
 //
@@ -116,13 +117,19 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[NG][8], int jj, 
 // (Alg. 1, first loop; digits by k_linv_digits) goes to Lhat's slots of the
 // LD panel; the reverse passes' row products use the other prod_op modes.
 // Complex (CPLX and LHAT): the operand of 2s rows over k' = 2k + part
-// (k_digits_z), (64-row tile, m tile) items, Lhat only.
+// (k_digits_z), (64-row tile, m tile) items, Lhat only; balanced, rounded and
+// with the eighth digit group like SYRK 2.
 template <bool CPLX, bool LHAT = false, int SYRK = 0>
 __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__restrict__ descs,
                                                               const Item *__restrict__ items, int nitems,
                                                               long long *__restrict__ slab, long long wait_limit) {
     grid_dep_wait();
     using Cfg = TwCfg;
+    // digit groups: 7, or 8 for the factorization and the complex Lhat, whose
+    // error would otherwise be the dropped pairs' (2^-53 of the rows' largest
+    // per step) rather than FP64 rounding
+    constexpr int NG = SYRK == 2 || (LHAT && CPLX) ? 8 : kTcDig;
+    constexpr bool BAL = NG == 8;                        // operands balanced by D over k
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint16_t *As = reinterpret_cast<uint16_t *>(smem_raw);                    // [kTwAS][7][A_PLANE] Lhat^T digits
     uint16_t *Bs = As + kTwAS * Cfg::A_STAGE;                                  // [kTwBS][7][B_PLANE] gathered digits
@@ -141,6 +148,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     __shared__ int s_pre;
     __shared__ volatile int s_abort;
     __shared__ int ymax[kTcM];
+    __shared__ int ksh[BAL ? kTcM : 1];   // shift of the exponents of B's column k
 
     const int w = blockIdx.x;
     if (w >= nitems) return;
@@ -154,10 +162,6 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
     const int c = (int)(ld - s);
     constexpr bool DENSE = LHAT || SYRK;                 // B from dense panels
-    // digit groups: 7, or 8 for the factorization and the complex Lhat, whose
-    // error would otherwise be the dropped pairs' (2^-53 of the rows' largest
-    // per step) rather than FP64 rounding
-    constexpr int NG = SYRK == 2 || (LHAT && CPLX) ? 8 : kTcDig;
     constexpr bool PAIR = SYRK == 1;                     // B's k runs over two panels
     const int kw = PAIR ? 2 * s : ((DENSE ? s : c) * (CPLX ? 2 : 1));   // k extent
     const int mrows = SYRK ? c : (CPLX ? 2 * s : s);     // rows of A (output rows)
@@ -226,6 +230,9 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                     *reinterpret_cast<uint4 *>(As + st * Cfg::A_STAGE + pl * Cfg::A_PLANE + e) = make_uint4(0, 0, 0, 0);
     if (DENSE)
         for (int e = tid; e < kTwN; e += kTwThreads) rowE[e] = 0;
+    if (BAL)
+        for (int k = tid; k < s; k += kTwThreads)
+            ksh[k] = k_balance(CPLX ? bexp(static_cast<const zd *>(P.D)[fc + k]) : bexp(static_cast<const double *>(P.D)[fc + k]));
     umma::fence_proxy_async();   // zeroed A rows are seen by the tensor cores
     __syncthreads();
     // the first copies (one per stage) go out before the rest of the set-up;
@@ -245,11 +252,13 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         if (p0 + r < c)
             for (int k = tid / kTwN; k < kw; k += kTwThreads / kTwN) {
                 if (CPLX) {   // k = 2q + part: the parts of one entry share the exponent
-                    e = max(e, bexp(static_cast<const double *>(P.L)[2 * (P.panel_off[K] + (int64_t)(k >> 1) * ld + s + p0 + r) + (k & 1)]));
+                    e = max(e, bal_exp(bexp(static_cast<const double *>(P.L)[2 * (P.panel_off[K] + (int64_t)(k >> 1) * ld + s + p0 + r) + (k & 1)]),
+                                       ksh[BAL ? k >> 1 : 0]));
                     continue;
                 }
                 const double *src = static_cast<const double *>(PAIR && k >= s ? P.Z : P.L);
-                e = max(e, bexp(src[P.panel_off[K] + (int64_t)(PAIR && k >= s ? k - s : k) * ld + s + p0 + r]));
+                const int ev = bexp(src[P.panel_off[K] + (int64_t)(PAIR && k >= s ? k - s : k) * ld + s + p0 + r]);
+                e = max(e, BAL ? bal_exp(ev, ksh[BAL ? k : 0]) : ev);
             }
         if (e) atomicMax(&rowE[r], e);
     } else {
@@ -393,7 +402,12 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 uint32_t lo[4], hi[4];
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
-                    const unsigned long long wv = (unsigned long long)(fixed54<NG == 8>(v[u], E) + 0x80808080808080ll);
+                    int add = 0;
+                    if (BAL) {
+                        const int k = (st0 + i_) * 16 + kq * 4 + u;
+                        add = k < kw ? ksh[BAL ? (CPLX ? k >> 1 : k) : 0] : 0;
+                    }
+                    const unsigned long long wv = (unsigned long long)(fixed54<BAL>(v[u], E, add) + 0x80808080808080ll);
                     lo[u] = (uint32_t)wv;
                     hi[u] = (uint32_t)(wv >> 32);
                 }
@@ -529,9 +543,9 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             const int mm = e % kTcM, p = e / kTcM, p1 = m0 + mm, p2 = p0 + p;
             if (p1 >= c || p2 >= c || p1 < p2) continue;
             const int e1 = P.linvexp[pos0 + p1], e2 = rowE[p];
-            const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0);
+            const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0) - (BAL ? 2 * kBalBias : 0);
             const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
-            if (SYRK == 2 && (e1 == 0x7FF || e2 == 0x7FF)) V[(int64_t)p2 * c + p1] = __longlong_as_double(0x7FF8000000000000ll);
+            if (SYRK == 2 && max(e1, e2) >= kBalBad) V[(int64_t)p2 * c + p1] = __longlong_as_double(0x7FF8000000000000ll);
             else V[(int64_t)p2 * c + p1] -= y;
         }
         return;
@@ -546,10 +560,10 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 if (p0 + p >= c || jr >= mrows) continue;
                 const int j = jr >= s ? jr - s : jr;
                 const int e1 = rowE[p], e2 = P.linvexp[fc + j];
-                const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], e1 - 1022 + e2 - 1022 - 13);
+                const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], e1 - 1022 + e2 - 1022 - 13 - 2 * kBalBias);
                 // an infinity or a NaN in the row or the column: NaN, as FP64 products give
                 Lz[2 * ((int64_t)j * ld + s + p0 + p) + (jr >= s ? 1 : 0)] =
-                    e1 == 0x7FF || e2 == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll) : y;
+                    max(e1, e2) >= kBalBad ? __longlong_as_double(0x7FF8000000000000ll) : y;
             }
             return;
         }

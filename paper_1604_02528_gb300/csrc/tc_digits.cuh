@@ -23,12 +23,13 @@ constexpr long long kMbarMinPolls = 1ll << 22;
 // x = M * 2^(E - 1076) with |M| < 2^54 (E >= the biased exponent of x),
 // truncated toward zero (ROUND: to nearest, half away from zero); integer
 // operations only.
+// add: x taken as x 2^add (E on that scale).
 template <bool ROUND = false>
-__device__ __forceinline__ long long fixed54(double x, int E) {
+__device__ __forceinline__ long long fixed54(double x, int E, int add = 0) {
     const long long b = __double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7FF);
     long long mant = ex ? ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) : 0ll;
-    const int sh = E - ex - 1;
+    const int sh = E - (ex + add) - 1;
     if (ROUND && sh > 0 && sh < 55) mant += 1ll << (sh - 1);
     const long long M = sh < 0 ? (mant << 1) : (sh < 63 ? (mant >> sh) : 0ll);
     return b < 0 ? -M : M;

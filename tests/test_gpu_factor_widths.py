@@ -87,3 +87,24 @@ def test_nonfinite_entry_reaches_a_pivot(native, cuda_device, bad):
         ctx.factor(torch.from_numpy(v).cuda())
         torch.cuda.synchronize()
         assert ctx.status() == native.SELINV_ERR_ZERO_PIVOT
+
+
+@pytest.mark.parametrize("cap", [17, 64, 128])
+def test_badly_scaled_matrix(native, cuda_device, cap):
+    """S A S with S over six decades: D spans twelve within a supernode, rows
+    of L as many the other way.  Row p of L times sqrt(D), over S_p, is of even
+    size (at most 1), and its error the unscaled factorization's: 1e-12."""
+    import torch
+    from paper_1604_02528_gb300.api import SelInvContext
+    p = synth.symmetric_scaling(_blocks(1, 300, "f64", 5), 12.0, 7)
+    p.supernodes = {"kind": "fundamental", "cap": cap, "fill": 0.0}
+    ctx = SelInvContext.from_problem(p)
+    sym = oracle.symbolic_for(p)
+    L0, D0 = oracle.ldlt(p, sym)
+    L, D = ctx.factor(torch.from_numpy(p.values).cuda())
+    torch.cuda.synchronize()
+    assert ctx.status() == 0
+    r, c, _ = oracle.panel_entries(sym)
+    scale = np.sqrt(np.abs(D0))[c] / np.sqrt(p.values[p.diag_positions()])[r]
+    assert np.abs(np.where(r > c, (L.cpu().numpy() - L0) * scale, 0)).max() <= 1e-12
+    assert np.abs(D.cpu().numpy() / D0 - 1).max() <= 1e-12
