@@ -588,189 +588,6 @@ __global__ void __launch_bounds__(kThreads) k_push(const ProbDesc *__restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// k_selinv_tiny: the whole of Alg. 1's second loop for a supernode with s <= 8
-// columns and c <= 64 rows below them, one warp per supernode (eight per CTA):
-// the deep levels of a nested-dissection tree hold thousands of these, for
-// which a CTA per row tile is mostly synchronisation.  Lane l owns rows l and
-// l + 32 of A^{-1}_{C,K} = -A^{-1}_{C,C} Lhat (the gather as in k_selinv,
-// 16 columns of C at a time with all their loads in flight -- the kernel is
-// bound by the latency of the gathers' dependent loads --, Lhat rows
-// broadcast); each entry of the s x s diagonal
-// block Dinv - Lhat^T A^{-1}_{C,K} is a warp sum over the lanes' own rows,
-// symmetrized through shared memory.  Writes the whole-column exponents for
-// the row bounds of later tensor-core gathers.
-// ---------------------------------------------------------------------------
-constexpr int kTinyS = 8, kTinyC = 64;
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ zd warp_sum(zd v) { return make_zd(warp_sum(v.x), warp_sum(v.y)); }
-
-// The supernode's work with its width S known at compile time, and nr = 1
-// or 2 row groups of 32 (c <= 32 or c <= 64): no product term is spent on
-// columns past s or rows past c (the kernel is bound by the FP64 pipe).
-template <typename T, int S>
-__device__ __forceinline__ void tiny_one(const ProbDesc &P, const int K, const int lane, T *Xw) {
-    const int fc = P.super_ptr[K];
-    const int s = S;
-    const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
-    const int c = (int)(ld - s);
-    const int nr = c > 32 ? 2 : 1;
-    const int64_t pos0 = P.rowptr[K] + s;
-    const bool h = P.herm != 0;
-    const T *Zc = static_cast<const T *>(P.Z);
-    T *Zk = static_cast<T *>(P.Z) + P.panel_off[K];
-    const T *LDk = static_cast<const T *>(P.LD) + P.panel_off[K];
-    const int64_t *pcb = P.colbase + pos0, *prb = P.relbase + pos0;
-    T acc[2][S];
-#pragma unroll
-    for (int r = 0; r < 2; r++)
-#pragma unroll
-        for (int j = 0; j < S; j++) acc[r][j] = Sc<T>::zero();
-    // the column data of C, lane l holding positions l and l + 32 (the lanes'
-    // own rows p use theirs for the entries above the diagonal); then QB
-    // columns q at a time: all their relative rows in flight together, then
-    // all their values
-    const GatherCheck chk = gather_check(P);
-    int64_t cbq[2] = {0, 0}, rbq[2] = {0, 0};
-#pragma unroll
-    for (int r = 0; r < 2; r++)
-        if (lane + 32 * r < c) {
-            cbq[r] = pcb[lane + 32 * r];
-            rbq[r] = prb[lane + 32 * r];
-        }
-    constexpr int QB = sizeof(T) == sizeof(double) ? 16 : 4;
-    for (int q0 = 0; q0 < c; q0 += QB) {
-        int32_t rel[2][QB];
-#pragma unroll
-        for (int u = 0; u < QB; u++) {
-            const int q = q0 + u;   // the same in every lane
-            const int64_t rq = __shfl_sync(0xffffffffu, q < 32 ? rbq[0] : rbq[1], q & 31);
-#pragma unroll
-            for (int r = 0; r < 2; r++) {
-                const int p = lane + 32 * r;
-                // entry (p, q) of A^{-1}_{C,C}: stored at (max, min)
-                rel[r][u] = (p < c && q < c) ? P.relidx[p >= q ? rq + p : rbq[r] + q] : 0;
-            }
-        }
-        T v[2][QB];
-#pragma unroll
-        for (int u = 0; u < QB; u++) {
-            const int q = q0 + u;
-            const int64_t cq = __shfl_sync(0xffffffffu, q < 32 ? cbq[0] : cbq[1], q & 31);
-#pragma unroll
-            for (int r = 0; r < 2; r++) {
-                const int p = lane + 32 * r;
-                v[r][u] = Sc<T>::zero();
-                if (p >= c || q >= c) continue;
-                const int64_t addr = (p >= q ? cq : cbq[r]) + rel[r][u];
-                if (chk.ok(addr)) v[r][u] = Zc[addr];
-                if (p < q) v[r][u] = cjif(v[r][u], h);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < QB; u++) {
-            const int q = q0 + u;
-            if (q >= c) break;
-            T lh[S];
-#pragma unroll
-            for (int j = 0; j < S; j++) lh[j] = LDk[(int64_t)j * ld + s + q];
-#pragma unroll
-            for (int r = 0; r < 2; r++) {
-                if (r >= nr) break;
-#pragma unroll
-                for (int j = 0; j < S; j++) madd(acc[r][j], v[r][u], lh[j]);
-            }
-        }
-    }
-    // A^{-1}_{C,K} = -acc, written; the lanes' own Lhat rows for the diagonal block
-    T own[2][S];
-    int ye[S];
-#pragma unroll
-    for (int j = 0; j < S; j++) {
-        int e = 0;
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
-            const int p = lane + 32 * r;
-            const bool ok = p < c;
-            acc[r][j] = ok ? neg(acc[r][j]) : Sc<T>::zero();
-            own[r][j] = ok ? cjif(LDk[(int64_t)j * ld + s + p], h) : Sc<T>::zero();
-            if (ok) {
-                Zk[(int64_t)j * ld + s + p] = acc[r][j];
-                e = max(e, bexp(acc[r][j]));
-            }
-        }
-        ye[j] = __reduce_max_sync(0xffffffffu, e);
-    }
-    // X(i, j) = Dinv(i, j) - sum_p Lhat(p, i) A^{-1}_{C,K}(p, j)  (Lhat conjugated: Hermitian)
-#pragma unroll
-    for (int i = 0; i < S; i++)
-#pragma unroll
-        for (int j = 0; j < S; j++) {
-            T part = Sc<T>::zero();
-#pragma unroll
-            for (int r = 0; r < 2; r++) {
-                if (r >= nr) break;
-                madd(part, own[r][i], acc[r][j]);
-            }
-            part = warp_sum(part);
-            if (lane == 0) Xw[j * kTinyS + i] = sub(LDk[(int64_t)j * ld + i], part);
-        }
-    __syncwarp();
-    int ze = 0;
-    for (int e = lane; e < s * s; e += 32) {
-        const int i = e % s, j = e / s;
-        T x = Xw[j * kTinyS + i];
-        if (P.symmetrize) x = half(add(x, cjif(Xw[i * kTinyS + j], h)));
-        Zk[(int64_t)j * ld + i] = x;
-        ze = max(ze, bexp(x));
-    }
-    // one bound for the whole block and the rows below each column (a column's
-    // own maximum would do; a larger bound keeps the gathers exact as well)
-    ze = __reduce_max_sync(0xffffffffu, ze);
-    if (lane < s) {
-        int y = 0;
-#pragma unroll
-        for (int j = 0; j < S; j++)
-            if (j == lane) y = ye[j];
-        P.colexpZ[fc + lane] = max(ze, y);
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_selinv_tiny(const ProbDesc *__restrict__ descs,
-                                                     const Item *__restrict__ items, int nitems) {
-    grid_dep_wait();
-    __shared__ T Xs[8][kTinyS * kTinyS];   // per warp: the unsymmetrized diagonal block
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int w = blockIdx.x * 8 + warp;
-    if (w >= nitems) return;               // the whole warp
-    const Item it = items[w];
-    const ProbDesc &P = descs[it.prob];
-    const int K = it.K;
-    switch (P.super_ptr[K + 1] - P.super_ptr[K]) {
-    case 1: tiny_one<T, 1>(P, K, lane, Xs[warp]); break;
-    case 2: tiny_one<T, 2>(P, K, lane, Xs[warp]); break;
-    case 3: tiny_one<T, 3>(P, K, lane, Xs[warp]); break;
-    case 4: tiny_one<T, 4>(P, K, lane, Xs[warp]); break;
-    case 5: tiny_one<T, 5>(P, K, lane, Xs[warp]); break;
-    case 6: tiny_one<T, 6>(P, K, lane, Xs[warp]); break;
-    case 7: tiny_one<T, 7>(P, K, lane, Xs[warp]); break;
-    default: tiny_one<T, 8>(P, K, lane, Xs[warp]); break;
-    }
-}
-
-cudaError_t launch_selinv_tiny(int dtype, const ProbDesc *d, const Item *items, int n, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    if (dtype == SELINV_C128) k_selinv_tiny<zd><<<(n + 7) / 8, 256, 0, st>>>(d, items, n);
-    else k_selinv_tiny<double><<<(n + 7) / 8, 256, 0, st>>>(d, items, n);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
 // k_selinv_persist: the whole traversal in one launch.  Work items are listed
 // root level first; each CTA claims the next item from a global ticket and,
 // before working on supernode K, waits for the completion flag of K's parent

@@ -379,6 +379,7 @@ int ensure_device(PlanData &p) {
         if (configure_ozaki_kernels() != cudaSuccess) return SELINV_ERR_CUDA;
         if (configure_tc_kernels() != cudaSuccess) return SELINV_ERR_CUDA;
         if (configure_tcw_kernels() != cudaSuccess) return SELINV_ERR_CUDA;
+        if (configure_narrow_kernels() != cudaSuccess) return SELINV_ERR_CUDA;
         configured = true;
     }
     int rc;
@@ -521,13 +522,20 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
     // ... whose Lhat runs there too: from 17 columns on (a CTA's 64 rows take
     // about 15 us on tcgen05; on the FP64 pipe 9 us at 16 columns, 34 at 32)
     auto zlhat = [&](int i, int s) { return zok(i, s) && s >= kZLhatS; };
-    // DFMA supernodes small enough for a warp each (k_selinv_tiny; not the LU form)
-    auto tiny = [&](int i, int32_t K) {
-        const PlanData &p = *plans[i];
-        const int s = p.super_ptr[K + 1] - p.super_ptr[K];
-        const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s;
-        return !descs[i].lu && s <= 8 && c <= 64 && !ozok(i, s) && !zok(i, s);
-    };
+    // supernodes off the tensor cores that are narrow enough for k_selinv_narrow
+    std::vector<std::vector<uint8_t>> narrow_k(np);
+    if (mode == SELINV_SCHED_LEVEL)
+        for (int i = 0; i < np; i++) {
+            const PlanData &p = *plans[i];
+            narrow_k[i].assign(p.ns, 0);
+            for (int32_t K = 0; K < p.ns; K++) {
+                const int s = p.super_ptr[K + 1] - p.super_ptr[K];
+                const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s;
+                narrow_k[i][K] = s <= kNarrowS && c <= 256 && !ozok(i, s) && !zok(i, s) &&
+                                 narrow_elems(s, (int)c, 1, descs[i].lu) * (int64_t)elem_size(descs[i].dtype) <= kNarrowSmem;
+            }
+        }
+    auto narrow = [&](int i, int32_t K) { return narrow_k[i][K] != 0; };
     // Level schedule: the normalization (steps 1, 2, 2b) runs in up to three
     // phases.  The supernodes of the first `ltop` levels -- the top of the
     // tree, a few large supernodes per level whose launches leave most SMs
@@ -1179,21 +1187,46 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 }
                 add_diag_fin(fins);
             }
-            // fused DFMA kernel for everything else: a warp per tiny supernode,
-            // a CTA per row tile for the rest
+            // fused FP64 kernels for everything else: narrow supernodes, then a
+            // CTA per row tile of the rest
             for (int dt = 0; dt < 2; dt++) {
                 const int64_t off = (int64_t)S.h_items.size();
+                std::vector<std::pair<int64_t, Item>> list;   // (work, supernode)
+                int64_t cmax = 0;
                 for (int i = 0; i < np; i++) {
                     if (descs[i].dtype != dt) continue;
                     const PlanData &p = *plans[i];
                     if (l >= p.nlevels) continue;
                     for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
                         const int32_t K = p.level_list[e];
-                        if (act(i, K) && tiny(i, K)) S.h_items.push_back({i, K, 0, 1});
+                        if (!act(i, K) || !narrow(i, K)) continue;
+                        const int64_t s = p.super_ptr[K + 1] - p.super_ptr[K], c = p.rowptr[K + 1] - p.rowptr[K] - s;
+                        list.push_back({c * c * s, {i, K, 0, 1}});
+                        cmax = std::max(cmax, c);
                     }
                 }
-                const int cnt = (int)(S.h_items.size() - off);
-                if (cnt) S.launches.push_back({KL_SELINV_TINY, dt, 0, off, cnt, l});
+                if (list.empty()) continue;
+                // CTAs per supernode: up to 8 while they all find an SM and each keeps
+                // 8 rows of C (shorter ones lose more to the cluster's barriers than
+                // the split saves); the supernodes in order of their work, longest first,
+                // where the SMs hold few of them (longer levels even out by themselves)
+                int cl = 8;
+                while (cl > 1 && ((int64_t)list.size() * cl > 152 || cmax < 8 * cl)) cl /= 2;
+                if (list.size() <= 512)
+                    std::stable_sort(list.begin(), list.end(), [](const std::pair<int64_t, Item> &a, const std::pair<int64_t, Item> &b) {
+                        return a.first > b.first;
+                    });
+                int smem = 0;
+                for (const auto &x : list) {
+                    const PlanData &p = *plans[x.second.prob];
+                    const int32_t K = x.second.K;
+                    const int s = p.super_ptr[K + 1] - p.super_ptr[K], c = (int)(p.rowptr[K + 1] - p.rowptr[K]) - s;
+                    smem = std::max(smem, narrow_elems(s, c, cl, descs[x.second.prob].lu) * (int)elem_size(dt));
+                    S.h_items.push_back(x.second);
+                }
+                Launch nl{KL_SELINV_TINY, dt, cl, off, (int)list.size(), l};
+                nl.smem = smem;
+                S.launches.push_back(nl);
             }
             for (int dt = 0; dt < 2; dt++)
                 for (int b = kNumBuckets - 1; b >= 0; b--) {
@@ -1205,7 +1238,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                         for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
                             const int32_t K = p.level_list[e];
                             const int s = p.super_ptr[K + 1] - p.super_ptr[K];
-                            if (act(i, K) && bucket_of(s) == b && !ozok(i, s) && !zok(i, s) && !tiny(i, K))
+                            if (act(i, K) && bucket_of(s) == b && !ozok(i, s) && !zok(i, s) && !narrow(i, K))
                                 push_items(i, K);
                         }
                     }
@@ -1288,7 +1321,8 @@ cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, c
         return launch_diag_fin(d, S.d_items + L.off, L.count, st);
     case KL_DIAG_TC:
         return launch_diag_tc(L.bucket, L.dtype != SELINV_F64, d, S.d_items + L.off, L.count, S.spin_limit, st);
-    case KL_SELINV_TINY: return launch_selinv_tiny(L.dtype, d, S.d_items + L.off, L.count, st);
+    case KL_SELINV_TINY:
+        return launch_selinv_narrow(L.dtype, L.bucket, L.smem, d, S.d_items + L.off, L.count, st);
     case KL_PUSH_DIAG: return launch_push(L.dtype, 0, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_PUSH: return launch_push(L.dtype, 1, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_PERSIST: {

@@ -146,6 +146,7 @@ struct Launch {
     int64_t off;
     int count;
     int level;
+    int smem = 0;   // dynamic shared memory (narrow supernodes)
     int side = 0;   // 1, 2: issued on the schedule's side stream (normalization phases of the lower levels)
 };
 
