@@ -1324,12 +1324,14 @@ static int adj_build(selinv_plan_s *plan) {
     }
     for (int32_t K = 0; K < p.ns; K++) a->linv_work.push_back(make_int2(0, K));
     a->lhat_bptr.push_back(0);
-    for (int b = 0; b < kNumBuckets; b++) {
+    for (int nar = 0; nar < 2; nar++) {   // the wide ones, then the narrow ones (launch_fma_lhat)
         for (int32_t K = 0; K < p.ns; K++) {
             const int s = p.super_ptr[K + 1] - p.super_ptr[K];
             const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s;
-            if (c == 0 || bucket_of(s) != b) continue;
-            for (int t = 0; t < p.ntiles[K]; t++) a->lhat_items.push_back({0, K, t, p.ntiles[K]});
+            if (c == 0 || (s <= kNarrowS) != (nar == 1)) continue;
+            const int rows = nar ? kFmaNarrowRows : kFmaLhatRows, ncol = nar ? 1 : (s + kFmaCols - 1) / kFmaCols;
+            for (int t = 0; t < (c + rows - 1) / rows; t++)
+                for (int ct = 0; ct < ncol; ct++) a->lhat_items.push_back({0, K, t, ct << 1});
         }
         a->lhat_bptr.push_back((int)a->lhat_items.size());
     }
@@ -1398,10 +1400,10 @@ static int adj_normalize(selinv_plan_s *plan, const void *L, const void *D, cuda
     }
     launch_linv(SELINV_F64, a->d_pdesc, a->d_linv, (int)a->linv_work.size(), 1, st);
     note_launch();
-    for (int b = 0; b < kNumBuckets; b++) {
+    for (int b = 0; b < 2; b++) {
         const int n = a->lhat_bptr[b + 1] - a->lhat_bptr[b];
         if (n > 0) {
-            launch_lhat(SELINV_F64, b, a->d_pdesc, a->d_lhat + a->lhat_bptr[b], n, st);
+            launch_fma_lhat(SELINV_F64, b, a->d_pdesc, a->d_lhat + a->lhat_bptr[b], n, st);
             note_launch();
         }
     }

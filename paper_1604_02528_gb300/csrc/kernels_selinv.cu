@@ -1,7 +1,6 @@
 // sm_103a kernels of the selected-inversion traversal (Alg. 1 of the paper):
 //   k_linv    L_KK^{-1} and Dinv_K = L_KK^{-T} D_K^{-1} L_KK^{-1}       (Alg. 1 loop 1)
 //             (L_KK^{-H} for a Hermitian problem, Sec. II-C; likewise Lhat^H below)
-//   k_lhat    Lhat_{C,K} = L_{C,K} L_KK^{-1}, tiled over rows of C       (Alg. 1 loop 1)
 //   k_selinv  A^{-1}_{C,K} = -A^{-1}_{C,C} Lhat_{C,K} with the gather of
 //             A^{-1}_{C,C} from the ancestors' panels fused into the GEMM,
 //             then the split contribution Lhat^T A^{-1}_{C,K} of every row
@@ -268,66 +267,9 @@ __global__ void __launch_bounds__(256) k_dinv(const ProbDesc *__restrict__ descs
     if (!lu) LD[(int64_t)i * ld + j] = cjif(acc, h);
 }
 
-// ---------------------------------------------------------------------------
-// k_lhat: Lhat(p, :) = L(s + p, :) L_KK^{-1} for the TM rows of one item.
-// ---------------------------------------------------------------------------
-template <typename T, int TN> struct LoadPanelRows {  // A = L rows s+p0.., k = column of K
-    const T *L;
-    int64_t ld;
-    int s, p0, c;
-    __device__ void operator()(int k0, T *As) const {
-        for (int e = threadIdx.x; e < kTK * kTM; e += kThreads) {
-            const int p = e % kTM, kk = e / kTM;
-            const int k = k0 + kk, pr = p0 + p;
-            As[kk * kTM + p] = (k < s && pr < c) ? L[(int64_t)k * ld + s + pr] : Sc<T>::zero();
-        }
-    }
-};
-
 template <typename T, int TN> __host__ __device__ constexpr int smem_a_elems() { return kTK * (kTM > TN ? kTM : TN); }
 template <typename T, int TN> __host__ __device__ constexpr size_t smem_bytes() {
     return sizeof(T) * (size_t)(smem_a_elems<T, TN>() + kTK * TN);
-}
-
-template <typename T, int TN>
-__global__ void __launch_bounds__(kThreads) k_lhat(const ProbDesc *__restrict__ descs,
-                                                   const Item *__restrict__ items, int nitems) {
-    grid_dep_wait();
-    using S = Shape<TN>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *As = reinterpret_cast<T *>(smem_raw);
-    T *Bs = As + smem_a_elems<T, TN>();
-    const int w = blockIdx.x;
-    if (w >= nitems) return;
-    const Item it = items[w];
-    const ProbDesc &P = descs[it.prob];
-    const int K = it.K;
-    const int s = P.super_ptr[K + 1] - P.super_ptr[K];
-    const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
-    const int c = (int)(ld - s);
-    const int p0 = it.tile * kTM;
-    // LU form: a second pass forms Uhat^T = U(K,C)^T (U_KK^T)^{-1}
-    for (int side = 0; side < (P.lu ? 2 : 1); side++) {
-        const T *L = static_cast<const T *>(side ? P.Ut : P.L) + P.panel_off[K];
-        const T *Li = static_cast<const T *>(side ? P.Vt : P.Linv) + P.linv_off[K];
-        T *LD = static_cast<T *>(side ? P.LDu : P.LD) + P.panel_off[K];
-        T acc[S::MI][S::NJ];
-#pragma unroll
-        for (int i = 0; i < S::MI; i++)
-#pragma unroll
-            for (int j = 0; j < S::NJ; j++) acc[i][j] = Sc<T>::zero();
-        LoadPanelRows<T, TN> la{L, ld, s, p0, c};
-        LoadColMajor<T, TN> lb{Li, (int64_t)s, s, s};
-        tile_gemm<T, TN>(s, la, lb, acc, As, Bs);
-        const int tx = threadIdx.x % S::TX, ty = threadIdx.x / S::TX;
-#pragma unroll
-        for (int i = 0; i < S::MI; i++)
-#pragma unroll
-            for (int j = 0; j < S::NJ; j++) {
-                const int p = p0 + ty + S::TY * i, col = tx + S::TX * j;
-                if (p < c && col < s) LD[(int64_t)col * ld + s + p] = acc[i][j];
-            }
-    }
 }
 
 // Split contribution of one row tile to the diagonal block,
@@ -699,9 +641,8 @@ static cudaError_t launch_items_t(int kernel, const ProbDesc *d, const Item *ite
                                   cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     constexpr size_t smem = smem_bytes<T, TN>();
-    if (kernel == 0) k_lhat<T, TN><<<n, kThreads, smem, st>>>(d, items, n);
-    else if (kernel == 1) k_selinv<T, TN><<<n, kThreads, smem, st>>>(d, items, n);
-    else if (kernel == 2) k_push_diag<T, TN><<<n, kThreads, smem, st>>>(d, items, n);
+    if (kernel == 0) k_selinv<T, TN><<<n, kThreads, smem, st>>>(d, items, n);
+    else if (kernel == 1) k_push_diag<T, TN><<<n, kThreads, smem, st>>>(d, items, n);
     else k_push<T, TN><<<n, kThreads, smem, st>>>(d, items, n);
     return cudaGetLastError();
 }
@@ -709,9 +650,7 @@ static cudaError_t launch_items_t(int kernel, const ProbDesc *d, const Item *ite
 template <typename T, int TN>
 static cudaError_t configure_t() {
     constexpr int smem = (int)smem_bytes<T, TN>();
-    cudaError_t e = cudaFuncSetAttribute(k_lhat<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_selinv<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_selinv<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_push_diag<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_push<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -781,23 +720,17 @@ static cudaError_t launch_items_dt(int kernel, int bucket, const ProbDesc *d, co
     }
 }
 
-cudaError_t launch_lhat(int dtype, int bucket, const ProbDesc *d, const Item *items, int n,
-                        cudaStream_t st) {
-    return dtype == SELINV_C128 ? launch_items_dt<zd>(0, bucket, d, items, n, st)
-                                : launch_items_dt<double>(0, bucket, d, items, n, st);
-}
-
 cudaError_t launch_selinv(int dtype, int bucket, const ProbDesc *d, const Item *items, int n,
                           cudaStream_t st) {
-    return dtype == SELINV_C128 ? launch_items_dt<zd>(1, bucket, d, items, n, st)
-                                : launch_items_dt<double>(1, bucket, d, items, n, st);
+    return dtype == SELINV_C128 ? launch_items_dt<zd>(0, bucket, d, items, n, st)
+                                : launch_items_dt<double>(0, bucket, d, items, n, st);
 }
 
 // push schedule: kind 0 = diagonal blocks, 1 = the pushes (bucket of the target's width)
 cudaError_t launch_push(int dtype, int kind, int bucket, const ProbDesc *d, const Item *items, int n,
                         cudaStream_t st) {
-    return dtype == SELINV_C128 ? launch_items_dt<zd>(2 + kind, bucket, d, items, n, st)
-                                : launch_items_dt<double>(2 + kind, bucket, d, items, n, st);
+    return dtype == SELINV_C128 ? launch_items_dt<zd>(1 + kind, bucket, d, items, n, st)
+                                : launch_items_dt<double>(1 + kind, bucket, d, items, n, st);
 }
 
 

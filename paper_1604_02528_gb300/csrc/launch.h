@@ -19,10 +19,16 @@ constexpr int kLinvCols = 8;
 cudaError_t launch_linv_cols(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);
 constexpr int kDinvTile = 16;
 cudaError_t launch_dinv(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);
-cudaError_t launch_lhat(int dtype, int bucket, const ProbDesc *d, const Item *items, int n,
-                        cudaStream_t st);
 cudaError_t launch_selinv(int dtype, int bucket, const ProbDesc *d, const Item *items, int n,
                           cudaStream_t st);
+// FP64 products of the level schedule (kernels_fma.cu): Lhat (narrow: s <= 16,
+// tiles of kFmaNarrowRows rows; else of kFmaLhatRows), A^{-1}_{C,K} by tiles of
+// `rows` (16 or 32) rows, columns by kFmaCols, and the diagonal block by 16 x 16
+// tiles, cl CTAs each
+constexpr int kFmaCols = 32, kFmaLhatRows = 32, kFmaNarrowRows = 128;
+cudaError_t launch_fma_lhat(int dtype, int narrow, const ProbDesc *d, const Item *items, int n, cudaStream_t st);
+cudaError_t launch_fma_rows(int dtype, int rows, const ProbDesc *d, const Item *items, int n, cudaStream_t st);
+cudaError_t launch_fma_diag(int dtype, int cl, const ProbDesc *d, const Item *items, int n, cudaStream_t st);
 cudaError_t configure_ozaki_kernels();
 cudaError_t configure_tc_kernels();
 cudaError_t launch_selinv_tc(int tn, const ProbDesc *d, const Item *items, int n, long long *slab,

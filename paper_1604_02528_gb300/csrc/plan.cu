@@ -683,7 +683,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             if (cnt) S.launches.push_back({KL_LHAT_OZ, SELINV_F64, tn, off, cnt, -1});
         }
         for (int dt = 0; dt < 2; dt++)
-            for (int b = 0; b < kNumBuckets; b++) {
+            for (int nar = 0; nar < 2; nar++) {
                 const int64_t off = (int64_t)S.h_items.size();
                 for (int i = 0; i < np; i++) {
                     if (descs[i].dtype != dt) continue;
@@ -691,12 +691,15 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                     for (int32_t K = 0; K < p.ns; K++) {
                         const int s = p.super_ptr[K + 1] - p.super_ptr[K];
                         const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s;
-                        if (c == 0 || !actn(i, K) || bucket_of(s) != b || ozok(i, s) || zlhat(i, s)) continue;
-                        for (int t = 0; t < p.ntiles[K]; t++) S.h_items.push_back({i, K, t, p.ntiles[K]});
+                        if (c == 0 || (s <= kNarrowS) != (nar == 1) || !actn(i, K) || ozok(i, s) || zlhat(i, s)) continue;
+                        const int rows = nar ? kFmaNarrowRows : kFmaLhatRows, ncol = nar ? 1 : (s + kFmaCols - 1) / kFmaCols;
+                        for (int side = 0; side <= (descs[i].lu ? 1 : 0); side++)
+                            for (int64_t t = 0; t < (c + rows - 1) / rows; t++)
+                                for (int ct = 0; ct < ncol; ct++) S.h_items.push_back({i, K, (int)t, (ct << 1) | side});
                     }
                 }
                 const int cnt = (int)(S.h_items.size() - off);
-                if (cnt) S.launches.push_back({1, dt, b, off, cnt, -1});
+                if (cnt) S.launches.push_back({KL_LHAT, dt, nar, off, cnt, -1});
             }
         // 2b) bf16 digit planes of Lhat for the tensor-core contraction
         {
@@ -1228,23 +1231,51 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 nl.smem = smem;
                 S.launches.push_back(nl);
             }
-            for (int dt = 0; dt < 2; dt++)
-                for (int b = kNumBuckets - 1; b >= 0; b--) {
-                    const int64_t off = (int64_t)S.h_items.size();
-                    for (int i = 0; i < np; i++) {
-                        if (descs[i].dtype != dt) continue;
-                        const PlanData &p = *plans[i];
-                        if (l >= p.nlevels) continue;
-                        for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
-                            const int32_t K = p.level_list[e];
-                            const int s = p.super_ptr[K + 1] - p.super_ptr[K];
-                            if (act(i, K) && bucket_of(s) == b && !ozok(i, s) && !zok(i, s) && !narrow(i, K))
-                                push_items(i, K);
-                        }
+            for (int dt = 0; dt < 2; dt++) {
+                std::vector<std::pair<int, int32_t>> ks;   // (problem, K)
+                int64_t ctas = 0, tiles = 0, cmax = 0;     // row tiles of 32, diagonal tiles
+                for (int i = 0; i < np; i++) {
+                    if (descs[i].dtype != dt) continue;
+                    const PlanData &p = *plans[i];
+                    if (l >= p.nlevels) continue;
+                    for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
+                        const int32_t K = p.level_list[e];
+                        const int s = p.super_ptr[K + 1] - p.super_ptr[K];
+                        if (!act(i, K) || ozok(i, s) || zok(i, s) || narrow(i, K)) continue;
+                        ks.push_back({i, K});
+                        const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s, nt = (s + 15) / 16, two = descs[i].lu ? 2 : 1;
+                        ctas += two * ((c + 31) / 32) * ((s + kFmaCols - 1) / kFmaCols);
+                        tiles += descs[i].lu ? nt * nt : nt * (nt + 1) / 2;
+                        cmax = std::max(cmax, c);
                     }
-                    const int cnt = (int)(S.h_items.size() - off);
-                    if (cnt) S.launches.push_back({KL_SELINV, dt, b, off, cnt, l});
                 }
+                if (ks.empty()) continue;
+                // rows of a tile: 32, or 16 where that leaves SMs without three CTAs
+                // (what hides a stage's gather)
+                const int rows = ctas < 3 * 152 ? 16 : 32;
+                const int64_t off = (int64_t)S.h_items.size();
+                for (auto &ik : ks) {
+                    const PlanData &p = *plans[ik.first];
+                    const int s = p.super_ptr[ik.second + 1] - p.super_ptr[ik.second];
+                    const int64_t c = p.rowptr[ik.second + 1] - p.rowptr[ik.second] - s;
+                    for (int64_t t = 0; t < (c + rows - 1) / rows; t++)
+                        for (int ct = 0; ct < (s + kFmaCols - 1) / kFmaCols; ct++)
+                            for (int side = 0; side <= (descs[ik.first].lu ? 1 : 0); side++)
+                                S.h_items.push_back({ik.first, ik.second, (int)t, (ct << 1) | side});
+                }
+                const int cnt = (int)(S.h_items.size() - off);
+                if (cnt) S.launches.push_back({KL_SELINV, dt, kFmaRows + rows, off, cnt, l});
+                const int64_t off2 = (int64_t)S.h_items.size();
+                for (auto &ik : ks) {
+                    const PlanData &p = *plans[ik.first];
+                    const int nt = (p.super_ptr[ik.second + 1] - p.super_ptr[ik.second] + 15) / 16;
+                    for (int t = 0; t < (descs[ik.first].lu ? nt * nt : nt * (nt + 1) / 2); t++)
+                        S.h_items.push_back({ik.first, ik.second, t, 1});
+                }
+                int cl = 8;   // CTAs per diagonal tile: two per SM over the level, 64 rows of C each
+                while (cl > 1 && (tiles * cl > 2 * 152 || cmax < 64 * cl)) cl /= 2;
+                S.launches.push_back({KL_SELINV, dt, kFmaDiag + cl, off2, (int)(S.h_items.size() - off2), l});
+            }
         }
     }
     S.h_descs = descs;
@@ -1260,6 +1291,16 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
         for (const Launch &L : S.launches)
             if (L.kind == KL_DIAG || L.kind == KL_DIAG_TC)
                 for (int64_t e = L.off; e < L.off + L.count; e++) has[S.h_items[e].prob] = 1;
+        // ... and so do the whole-column maxima that the FP64 tiles raise
+        std::vector<char> fma(np, 0);
+        for (const Launch &L : S.launches)
+            if (L.kind == KL_SELINV && L.bucket >= kFmaRows)
+                for (int64_t e = L.off; e < L.off + L.count; e++) fma[S.h_items[e].prob] = 1;
+        for (int i = 0; i < np; i++)
+            if (fma[i]) {
+                S.pre_ptr.push_back(descs[i].colexpZ);
+                S.pre_bytes.push_back(sizeof(int) * (size_t)std::max(plans[i]->n, 1));
+            }
         for (int i = 0; i < np; i++) {
             if (!has[i]) continue;
             S.pre_ptr.push_back(descs[i].dacc);
@@ -1295,8 +1336,11 @@ cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, c
         return L.bucket ? launch_linv_cols(L.dtype, d, S.d_work + L.off, L.count, st)
                         : launch_linv(L.dtype, d, S.d_work + L.off, L.count, 0, st);
     case KL_DINV: return launch_dinv(L.dtype, d, S.d_work + L.off, L.count, st);
-    case KL_LHAT: return launch_lhat(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
-    case KL_SELINV: return launch_selinv(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
+    case KL_LHAT: return launch_fma_lhat(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
+    case KL_SELINV:
+        if (L.bucket >= kFmaDiag) return launch_fma_diag(L.dtype, L.bucket - kFmaDiag, d, S.d_items + L.off, L.count, st);
+        if (L.bucket >= kFmaRows) return launch_fma_rows(L.dtype, L.bucket - kFmaRows, d, S.d_items + L.off, L.count, st);
+        return launch_selinv(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_DIGITS:
         if (L.dtype != SELINV_F64) return launch_digits_z(0, d, S.d_work + L.off, L.count, st);
         return launch_lhat_digits(d, S.d_work + L.off, L.count, st);

@@ -139,6 +139,9 @@ constexpr int kAsmChunk = 1024;   // entries of an update matrix per extend-add 
 constexpr int kTopSupernodes = 16;   // level schedule: the top levels (up to this many supernodes) normalized first
 constexpr int kMidSupernodes = 256;  // ... and the levels up to this many normalized in the side stream's first phase
 
+// KL_SELINV launches of the level schedule: bucket kFmaRows + rows of a tile, kFmaDiag + CTAs per tile
+constexpr int kFmaRows = 1000, kFmaDiag = 2000;
+
 struct Launch {
     int kind;    // KL_*
     int dtype;
