@@ -128,41 +128,52 @@ __global__ void __launch_bounds__(256) k_fupd_digits(const FactorDesc *__restric
 }
 
 // ---------------------------------------------------------------------------
-// k_fdiag: dense LDL^T of J's diagonal block (s > kFSmallS) by one thread-
-// block cluster.  GB300 issues one FP64 instruction per SM sub-partition in
-// 64 clocks (2 lanes per clock and SM), so the s^3 / 6 products of a 128-
-// column block alone take 85 us on one SM, and the levels near the root hold
-// one to eight such blocks: the cluster (8 CTAs there, 1 where a level has
-// blocks enough for every SM) holds the rows cyclically, four at a time, in
-// its CTAs' shared memory.  Per panel of 8 columns every CTA reads the panel
-// from the owners (distributed shared memory), factors it on all rows by
-// itself -- the chain reciprocal, scale, update per column is what bounds the
-// kernel, and repeating it costs less than exchanging it -- and updates its
-// own rows of the trailing block; one cluster barrier per panel.
+// k_fdiag: dense LDL^T of J's diagonal block by one thread-block cluster.
+// GB300 issues one FP64 instruction per SM sub-partition in 64 clocks, and a
+// dependent one no later, so two things bound it: the s^3 / 6 products (85 us
+// for 128 columns on one SM), and the chain pivot, reciprocal, scale, update
+// of every column (5 instructions at least, 20 us).  The levels near the root
+// hold one to eight such blocks: a cluster (8 CTAs there, 1 where a level has
+// blocks enough for every SM) keeps the rows cyclically, four at a time, in
+// its CTAs' shared memory.  Per block of 32 columns:
+//   - every CTA reads the 32 x 32 diagonal block from the owners (distributed
+//     shared memory) and factors it by itself, the triangle's entries dealt to
+//     four warps (no lane idle, little else on the pipe than the chain);
+//   - its own rows below are solved against it, a warp per two rows;
+//   - the solved rows are exchanged and the CTA's rows of the trailing block
+//     updated.
+// Two cluster barriers per block.  (Panels of 8 columns factored on all rows
+// by every CTA put 3.5 more instructions per column on the chain: 114 us for
+// 128 columns, against 600 us for one CTA in global memory.)
 // ---------------------------------------------------------------------------
-constexpr int kFdThreads = 256;   // the panel's 128 rows, and as many again for the trailing block
-constexpr int kFdRows = 128;
-constexpr int kFdNB = 8;           // columns per panel
-constexpr int kFdLd = kFdNB + 1;   // panel row stride in shared memory
+constexpr int kFdThreads = 256;
+constexpr int kFdChain = 128;      // threads that factor the diagonal block
+constexpr int kFdNB = 32;          // columns per block
+constexpr int kFdLd = kFdNB + 1;   // row stride of the exchanged rows
+constexpr int kFdSlots = (kFdNB * (kFdNB + 1) / 2 + kFdChain - 1) / kFdChain;   // entries per chain thread
 
 // 1 / d: the hardware's approximate reciprocal r0 (relative error below
 // 2^-19), then one step of the third-order iteration r0 (1 + e + e^2),
 // e = 1 - d r0: three dependent FP64 operations (240 clocks with the seed)
 // where the division takes 385.  Magnitudes near the ends of the exponent
 // range (and zero, infinities, NaN) go through the division.
+// The division is a call: inlined, its own FP64 operations would run beside
+// the others in every lane.
+__device__ __noinline__ double full_recip(double d) { return 1.0 / d; }
 __device__ __forceinline__ double fast_recip(double d) {
     const int e = (int)((__double_as_longlong(d) >> 52) & 0x7FF);
-    if (e < 64 || e > 1982) return 1.0 / d;
+    if (e < 64 || e > 1982) return full_recip(d);
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     const double x = fma(-d, r, 1.0);
     return fma(fma(x, x, x), r, r);
 }
+__device__ __noinline__ zd full_recip(zd d) { return recip(d); }
 // complex: conj(d) / |d|^2 while |d|^2 and its reciprocal stay in range
 __device__ __forceinline__ zd fast_recip(zd d) {
     const int ex = (int)((__double_as_longlong(d.x) >> 52) & 0x7FF), ey = (int)((__double_as_longlong(d.y) >> 52) & 0x7FF);
     const int e = ex > ey ? ex : ey;
-    if (e < 623 || e > 1423) return recip(d);
+    if (e < 623 || e > 1423) return full_recip(d);
     const double r = fast_recip(fma(d.x, d.x, d.y * d.y));
     return make_zd(d.x * r, -d.y * r);
 }
@@ -173,16 +184,21 @@ __host__ __device__ inline int fd_rows_elems(int s, int cl) {
     const int groups = (s + 3) / 4, mine = (groups + cl - 1) / cl;   // at most, rank cl - 1
     return 16 * (cl * (mine * (mine - 1) / 2) + mine * cl);
 }
+// ... and of everything: the rows below a block, the block's columns (y and L), the row store
+__host__ __device__ inline int fd_elems(int s, int cl) {
+    return (s > kFdNB ? s - kFdNB : 0) * kFdLd + 2 * kFdNB * kFdLd + fd_rows_elems(s, cl);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restrict__ fd, const int *__restrict__ js,
                                                       int nj) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ T Ys[kFdNB][kFdNB];
+    __shared__ T rD[kFdNB];
     cg::cluster_group cl = cg::this_cluster();
     const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    const int w = blockIdx.x / CL;
+    const int lc = 31 - __clz(CL);           // CL = 1 << lc
+    const int w = blockIdx.x >> lc;
     if (w >= nj) return;                     // the grid is nj clusters: never taken by a part of one
     const FactorDesc &F = *fd;
     const int J = js[w];
@@ -192,76 +208,128 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
     T *P = static_cast<T *>(F.L) + F.panel_off[J];
     T *D = static_cast<T *>(F.D) + fc;
     const bool herm = F.herm != 0;
-    T *Yp = reinterpret_cast<T *>(smem_raw);          // [128][kFdLd] undivided panel columns y = l d
-    T *Lp = Yp + kFdRows * kFdLd;                     // 2 x [128][kFdLd] columns of L: this panel and the last
-    T *A = Lp + 2 * kFdRows * kFdLd;                  // this CTA's rows
-    const int tid = threadIdx.x;
+    T *Yd = reinterpret_cast<T *>(smem_raw);            // [column][row] of the diagonal block, undivided (y = l d)
+    T *Ld = Yd + kFdNB * kFdLd;                         // [column][row] of its L
+    T *Yp = Ld + kFdNB * kFdLd;                         // [row below the block][column] undivided
+    T *A = Yp + (s > kFdNB ? s - kFdNB : 0) * kFdLd;    // this CTA's rows
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     // row i = 4 g + u lives in rank g % CL at (local group g / CL)
     auto off = [&](int i) {
-        const int g = i >> 2, lg = g / CL, r = g % CL;
-        return 16 * (CL * (lg * (lg - 1) / 2) + lg * (r + 1)) + (i & 3) * 4 * (g + 1);
+        const int g = i >> 2, lg = g >> lc, r = g & (CL - 1);
+        return 16 * (((lg * (lg - 1) / 2) << lc) + lg * (r + 1)) + (i & 3) * 4 * (g + 1);
     };
     const int groups = (s + 3) / 4;
-    const int myg = groups > rank ? (groups - rank + CL - 1) / CL : 0;   // row groups of this CTA
-    auto row_of = [&](int lr) { return ((lr >> 2) * CL + rank) * 4 + (lr & 3); };
-    for (int k = tid / 32; k < s; k += kFdThreads / 32)
-        for (int lr = tid % 32; lr < 4 * myg; lr += 32) {
+    const int myg = groups > rank ? (groups - rank + CL - 1) >> lc : 0;   // row groups of this CTA
+    auto row_of = [&](int lr) { return (((lr >> 2) << lc) + rank) * 4 + (lr & 3); };
+    auto owner = [&](int i) { return (i >> 2) & (CL - 1); };
+    for (int k = warp; k < s; k += kFdThreads / 32)
+        for (int lr = lane; lr < 4 * myg; lr += 32) {
             const int i = row_of(lr);
             if (i < s && k <= i) cp_async_elem(A + off(i) + k, P + (int64_t)k * ld + i);
         }
     cp_async_commit();
     cp_async_wait<0>();
-    // a finished panel's columns of L into the row store (the owners read it
-    // no more once every CTA has passed the next barrier); global memory gets
-    // the block at the end, so that no barrier waits for stores to reach it
-    auto keep = [&](int b0, const T *Lq) {
+    // the block's rows of L into the row store, when every CTA has read them
+    auto keep = [&](int b0) {
         const int nb = s - b0 < kFdNB ? s - b0 : kFdNB;
-        for (int e = tid; e < 4 * myg * nb; e += kFdThreads) {
-            const int r = row_of(e % (4 * myg)), j = e / (4 * myg);
-            if (r < s && r > b0 + j) A[off(r) + b0 + j] = Lq[(r - b0) * kFdLd + j];
+        for (int e = tid; e < nb * nb; e += kFdThreads) {
+            const int i = e % nb, j = e / nb;
+            if (i > j && owner(b0 + i) == rank) A[off(b0 + i) + b0 + j] = Ld[j * kFdLd + i];
         }
     };
-    int pb = 0;
-    for (int b0 = 0; b0 < s; b0 += kFdNB, pb ^= 1) {
+    // the chain threads' entries of a block's triangle, column after column
+    // (as the chain moves on, whole slots fall done): row and column, and the
+    // last column in the warp's slot
+    T a[kFdSlots];
+    int ei[kFdSlots], ek[kFdSlots], last[kFdSlots];
+    auto deal = [&](int nb) {
+        const int ne = nb * (nb + 1) / 2;
+        int k = 0, q = tid;
+#pragma unroll
+        for (int u = 0; u < kFdSlots; u++) {
+            const bool on = tid + u * kFdChain < ne;
+            while (on && q >= nb - k) q -= nb - k++;
+            ek[u] = on ? k : -1;
+            ei[u] = on ? k + q : 0;
+            last[u] = __reduce_max_sync(0xffffffffu, ek[u]);
+            q += kFdChain;
+        }
+    };
+    if (tid < kFdChain) deal(s < kFdNB ? s : kFdNB);
+    for (int b0 = 0; b0 < s; b0 += kFdNB) {
         const int nb = s - b0 < kFdNB ? s - b0 : kFdNB;
-        T *Lq = Lp + pb * kFdRows * kFdLd;
-        cl.sync();
-        if (b0) keep(b0 - kFdNB, Lp + (pb ^ 1) * kFdRows * kFdLd);
-        const int i = b0 + tid;                        // this thread's row of the panel
-        if (tid < kFdRows) {
-            T a[kFdNB];
-            if (i < s) {
-                const T *src = cl.map_shared_rank(A, (i >> 2) % CL) + off(i) + b0;
+        if (CL > 1) cl.sync();
+        else __syncthreads();
+        if (tid < kFdChain) {
+            if (b0 && nb < kFdNB) deal(nb);
 #pragma unroll
-                for (int j = 0; j < kFdNB; j++) a[j] = (j < nb && j <= tid) ? src[j] : Sc<T>::zero();
+            for (int u = 0; u < kFdSlots; u++) {
+                const int i = b0 + ei[u];
+                a[u] = ek[u] >= 0 ? (CL > 1 ? cl.map_shared_rank(A, owner(i)) : A)[off(i) + b0 + ek[u]] : Sc<T>::zero();
             }
+            for (int j = 0; j < nb; j++) {
 #pragma unroll
-            for (int j = 0; j < kFdNB; j++) {
-                if (j < nb) {
-                    if (tid >= j && tid < nb) Ys[j][tid] = a[j];
-                    asm volatile("bar.sync 1, 128;\n" ::: "memory");
-                    const T d = Ys[j][j];
-                    if (i < s) {
-                        if (tid == j && rank == 0) {
-                            if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
-                            D[b0 + j] = d;
-                        }
-                        const T l = mul(a[j], fast_recip(d));
-                        Yp[tid * kFdLd + j] = a[j];
-                        Lq[tid * kFdLd + j] = l;
+                for (int u = 0; u < kFdSlots; u++)
+                    if (ek[u] == j) Yd[j * kFdLd + ei[u]] = a[u];
+                asm volatile("bar.sync 1, 128;\n" ::: "memory");
+                const T dj = Yd[j * kFdLd + j], r = fast_recip(dj);
+                const T l = mul(Yd[j * kFdLd + (lane > j && lane < nb ? lane : j)], r);   // row `lane` of L's column
 #pragma unroll
-                        for (int k = j + 1; k < kFdNB; k++)
-                            if (k < nb) msub(a[k], l, cjif(Ys[j][k], herm));
-                    }
+                for (int u = 0; u < kFdSlots; u++) {
+                    if (last[u] <= j) continue;                  // the whole warp's slot is done
+                    const T li = shfl_elem(l, ei[u]);
+                    if (ek[u] > j) msub(a[u], li, cjif(Yd[j * kFdLd + ek[u]], herm));
+                }
+                if (warp == 3 && lane >= j && lane < nb) {
+                    if (lane > j) Ld[j * kFdLd + lane] = l;
+                    else rD[j] = r;
                 }
             }
         }
         __syncthreads();
+        if (rank == 0 && warp == 7 && lane < nb) {               // the pivots, off the chain
+            const T d = Yd[lane * kFdLd + lane];
+            if (is_zero(d) || !finite_val(d)) atomicCAS(F.status, 0, SELINV_ERR_ZERO_PIVOT);
+            D[b0 + lane] = d;
+        }
+        const int b1 = b0 + kFdNB, below = s - b1;
+        if (below <= 0) break;                                   // (a full block otherwise: nb = 32)
+        // own rows below the block: y L^T = a, lanes over the block's columns, two rows per warp
+        for (int lr = 2 * warp; lr < 4 * myg; lr += 2 * (kFdThreads / 32)) {
+            const int i0 = row_of(lr), i1 = row_of(lr + 1);      // (of one group of four)
+            if (i1 < b1 || i0 >= s) continue;
+            const bool second = i1 < s;
+            T y0 = A[off(i0) + b0 + lane], y1 = second ? A[off(i1) + b0 + lane] : Sc<T>::zero();
+#pragma unroll 4
+            for (int j = 0; j < kFdNB; j++) {
+                const T v0 = shfl_elem(y0, j), v1 = shfl_elem(y1, j);
+                if (lane > j) {
+                    const T l = cjif(Ld[j * kFdLd + lane], herm);
+                    msub(y0, v0, l);
+                    msub(y1, v1, l);
+                }
+            }
+            const T r = rD[lane];
+            Yp[(i0 - b1) * kFdLd + lane] = y0;
+            A[off(i0) + b0 + lane] = mul(y0, r);
+            if (second) {
+                Yp[(i1 - b1) * kFdLd + lane] = y1;
+                A[off(i1) + b0 + lane] = mul(y1, r);
+            }
+        }
+        if (CL > 1) {
+            cl.sync();
+            for (int i = b1 + warp; i < s; i += kFdThreads / 32) {
+                const int o = owner(i);
+                if (o != rank) Yp[(i - b1) * kFdLd + lane] = cl.map_shared_rank(Yp, o)[(i - b1) * kFdLd + lane];
+            }
+        }
+        __syncthreads();
+        keep(b0);
         // own rows of the trailing block: a_ik -= l_i y_k, columns b1 .. i of row i
-        // -- entries dealt to the threads one by one (the FP64 pipe bounds the
-        // update, and an idle lane costs as much as a busy one), all lanes of a
-        // warp brought to their entry before the products start
-        const int b1 = b0 + kFdNB;
+        // -- entries dealt to the threads one by one (an idle lane costs as much
+        // as a busy one), all lanes of a warp brought to their entry before the
+        // products start
         int total = 0;
         for (int lr = 0; lr < 4 * myg; lr++) {
             const int r = row_of(lr);
@@ -275,20 +343,20 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
                 cnt = r < s && r >= b1 ? r - b1 + 1 : 0;
             }
             __syncwarp(__activemask());
-            T *dst = A + off(r) + b1 + q;
-            T acc = *dst;
-            const T *lrow = Lq + (r - b0) * kFdLd, *yrow = Yp + (b1 + q - b0) * kFdLd;
-#pragma unroll
-            for (int j = 0; j < kFdNB; j++) msub(acc, lrow[j], cjif(yrow[j], herm));   // a full panel: b1 <= s - 1
-            *dst = acc;
+            T *row = A + off(r);
+            T acc = row[b1 + q];
+            const T *lrow = row + b0, *yrow = Yp + q * kFdLd;
+#pragma unroll 8
+            for (int j = 0; j < kFdNB; j++) msub(acc, lrow[j], cjif(yrow[j], herm));
+            row[b1 + q] = acc;
             q += kFdThreads;
         }
     }
-    cl.sync();   // the last panel is read no more, and no CTA leaves while another may still read its rows
-    keep((s - 1) / kFdNB * kFdNB, Lp + (pb ^ 1) * kFdRows * kFdLd);
+    if (CL > 1) cl.sync();   // the last block is read no more, and no CTA leaves while another may still read its rows
+    keep((s - 1) / kFdNB * kFdNB);
     __syncthreads();
-    for (int k = tid / 32; k < s; k += kFdThreads / 32)
-        for (int lr = tid % 32; lr < 4 * myg; lr += 32) {
+    for (int k = warp; k < s; k += kFdThreads / 32)
+        for (int lr = lane; lr < 4 * myg; lr += 32) {
             const int i = row_of(lr);
             if (i < s) P[(int64_t)k * ld + i] = i > k ? A[off(i) + k] : (i == k ? Sc<T>::one() : Sc<T>::zero());
         }
@@ -495,10 +563,15 @@ int factor_tables(selinv_plan_s *plan) {
         FactorLevel v;
         std::vector<int32_t> wide;
         v.small0 = (int64_t)js.size();
+        // one CTA for a whole supernode while its update's c^2 s / 2 products take
+        // under 10 us of an SM (c = 64, s = 16), or up to twice that where the
+        // level has supernodes for two CTAs on every SM
+        const int64_t small_prod = p.level_ptr[l + 1] - p.level_ptr[l] >= 304 ? 150000 : 65536;
         for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
             const int32_t J = p.level_list[e];
             const int s = width(J), elems = s * (s + below(J));
-            if (s <= kFSmallS && elems <= kFSmallElems) {
+            const int64_t prod = (int64_t)s * below(J) * below(J);
+            if (s <= kFSmallS && elems <= kFSmallElems && prod <= small_prod) {
                 js.push_back(J);
                 v.small_elems = std::max(v.small_elems, elems);
             } else {
@@ -518,9 +591,20 @@ int factor_tables(selinv_plan_s *plan) {
         // have blocks enough by themselves
         const int64_t nw = (int64_t)wide.size();
         v.cl = v.wide_s <= 32 ? 1 : (nw * 8 <= 152 ? 8 : (nw * 4 <= 152 ? 4 : (nw * 2 <= 152 ? 2 : 1)));
-        // row tiles: 4 rows (a row per warp), up to 16 as the level's rows cover every
-        // SM (64-row tiles left a third of the SMs idle in the last wave)
-        const int rt = (int)std::min<int64_t>(16, std::max<int64_t>(4, (rows / 152 + 3) / 4 * 4));
+        // rows per tile: the number whose tiles, dealt to the SMs, take least --
+        // a row per warp costs about 10 us of an SM sub-partition at 128
+        // columns, a tile's L_JJ 5 us more for each of the two CTAs in flight
+        int rt = 4;
+        int64_t least = INT64_MAX;
+        for (int t = 4; t <= 64; t += 4) {
+            int64_t nt = 0;
+            for (int32_t J : wide) nt += (below(J) + t - 1) / t;
+            const int64_t per = (nt + 151) / 152, cost = per * (t / 4) * 10 + (per + 1) / 2 * 5;
+            if (cost < least) {
+                least = cost;
+                rt = t;
+            }
+        }
         v.tile0 = (int64_t)tiles.size();
         for (int32_t J : wide)
             for (int r = 0, c = below(J); r < c; r += rt) tiles.push_back(make_int4(J, r, std::min(rt, c - r), 0));
@@ -661,7 +745,7 @@ FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, 
 
 // the dynamic shared memory of the widest blocks, on the plan's device
 template <typename T> static cudaError_t configure_factor_kernels() {
-    const int diag = (int)(sizeof(T) * (size_t)(3 * kFdRows * kFdLd + fd_rows_elems(128, 1)));
+    const int diag = (int)(sizeof(T) * (size_t)fd_elems(128, 1));
     const int trsm = (int)(sizeof(T) * (size_t)tri_store_elems(128)), small = (int)(2 * sizeof(T) * kFSmallElems);
     cudaError_t e = cudaFuncSetAttribute(k_fdiag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, diag);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ftrsm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, trsm);
@@ -716,7 +800,7 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3((unsigned)((v.wide1 - v.wide0) * v.cl));
                 cfg.blockDim = dim3(kFdThreads);
-                cfg.dynamicSmemBytes = sizeof(T) * (size_t)(3 * kFdRows * kFdLd + fd_rows_elems(v.wide_s, v.cl));
+                cfg.dynamicSmemBytes = sizeof(T) * (size_t)fd_elems(v.wide_s, v.cl);
                 cfg.stream = st;
                 cudaLaunchAttribute at[1];
                 at[0].id = cudaLaunchAttributeClusterDimension;

@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         const int r = tid % kTwN;
         int e = 0;
         if (p0 + r < c)
+#pragma unroll 8
             for (int k = tid / kTwN; k < kw; k += kTwThreads / kTwN) {
                 if (CPLX) {   // k = 2q + part: the parts of one entry share the exponent
                     e = max(e, bal_exp(bexp(static_cast<const double *>(P.L)[2 * (P.panel_off[K] + (int64_t)(k >> 1) * ld + s + p0 + r) + (k & 1)]),
@@ -538,15 +539,25 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         // V_K(p1, p2) -= the product, p1 >= p2, the diagonal halved (exactly:
         // one less in the scale); A's rows carry their own exponents
         double *V = static_cast<double *>(P.Yout) + P.part_off[K];
-        // lanes along p1: contiguous in V's columns (and in the sums)
-        for (int e = tid; e < kTwN * kTcM; e += kTwThreads) {
-            const int mm = e % kTcM, p = e / kTcM, p1 = m0 + mm, p2 = p0 + p;
-            if (p1 >= c || p2 >= c || p1 < p2) continue;
-            const int e1 = P.linvexp[pos0 + p1], e2 = rowE[p];
-            const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0) - (BAL ? 2 * kBalBias : 0);
-            const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
-            if (SYRK == 2 && max(e1, e2) >= kBalBad) V[(int64_t)p2 * c + p1] = __longlong_as_double(0x7FF8000000000000ll);
-            else V[(int64_t)p2 * c + p1] -= y;
+        // lanes along p1: contiguous in V's columns (and in the sums); the old
+        // values of several entries on their way before the first is needed
+        constexpr int NV = 5;
+        for (int e0 = tid; e0 < kTwN * kTcM; e0 += NV * kTwThreads) {
+            double old[NV];
+#pragma unroll
+            for (int u = 0; u < NV; u++) {
+                const int e = e0 + u * kTwThreads, p1 = m0 + e % kTcM, p2 = p0 + e / kTcM;
+                old[u] = e < kTwN * kTcM && p1 < c && p1 >= p2 ? V[(int64_t)p2 * c + p1] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < NV; u++) {
+                const int e = e0 + u * kTwThreads, mm = e % kTcM, p = e / kTcM, p1 = m0 + mm, p2 = p0 + p;
+                if (e >= kTwN * kTcM || p1 >= c || p1 < p2) continue;
+                const int e1 = P.linvexp[pos0 + p1], e2 = rowE[p];
+                const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0) - (BAL ? 2 * kBalBias : 0);
+                const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
+                V[(int64_t)p2 * c + p1] = SYRK == 2 && max(e1, e2) >= kBalBad ? __longlong_as_double(0x7FF8000000000000ll) : old[u] - y;
+            }
         }
         return;
     }
