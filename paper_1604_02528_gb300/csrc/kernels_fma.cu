@@ -26,41 +26,47 @@ namespace cg = cooperative_groups;
 
 constexpr int kFmThreads = 128;
 constexpr int kFmK = 32;                     // k per stage
-static_assert(kFmaCols == 32, "the column tiles below are two groups of 16");
+static_assert(kFmaCols == 32, "the widest column tile below");
 
-// acc += A(R x 32) B(32 x 32) from shared memory; thread (tx, ty): rows
+// acc += A(R x 32) B(32 x TN) from shared memory; thread (tx, ty): rows
 // tx + 16 i, columns ty + 8 j
-template <typename T, int R>
-__device__ __forceinline__ void fma_stage(const T (&As)[kFmK][R + 1], const T (&Bs)[kFmK][kFmaCols + 1], int kk,
-                                          T (&acc)[R / 16][4]) {
+template <typename T, int R, int TN>
+__device__ __forceinline__ void fma_stage(const T (&As)[kFmK][R + 1], const T (&Bs)[kFmK][TN + 1], int kk,
+                                          T (&acc)[R / 16][TN / 8]) {
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll 4
     for (int k = 0; k < kk; k++) {
-        T a[R / 16], b[4];
+        T a[R / 16], b[TN / 8];
 #pragma unroll
         for (int i = 0; i < R / 16; i++) a[i] = As[k][tx + 16 * i];
 #pragma unroll
-        for (int j = 0; j < 4; j++) b[j] = Bs[k][ty + 8 * j];
+        for (int j = 0; j < TN / 8; j++) b[j] = Bs[k][ty + 8 * j];
 #pragma unroll
         for (int i = 0; i < R / 16; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) madd(acc[i][j], a[i], b[j]);
+            for (int j = 0; j < TN / 8; j++) madd(acc[i][j], a[i], b[j]);
     }
 }
 
-// items: tile = row tile of R rows, ntiles = (column tile of 32) << 1 | side
-template <typename T, int R>
+// items: tile = row tile of R rows, ntiles = (column tile of TN) << 1 | side; a
+// cluster shares the rows q of C, the partial sums meeting in its first CTA
+// (where a level has a few narrow supernodes with a long C: 34 tiles of
+// c = 500 took 123 us)
+template <typename T, int R, int TN>
 __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restrict__ descs,
                                                          const Item *__restrict__ items, int nitems) {
     grid_dep_wait();
-    __shared__ T As[kFmK][R + 1], Bs[kFmK][kFmaCols + 1];
+    __shared__ T As[kFmK][R + 1], Bs[kFmK][TN + 1];
+    static_assert(kFmK * (R + 1) >= R * TN || kFmK * (TN + 1) >= R * TN, "a tile's sums fit a stage");
     __shared__ int64_t tile_cb[R], tile_rb[R];
-    __shared__ int ymax[kFmaCols];
-    const int w = blockIdx.x;
-    if (w >= nitems) return;
+    __shared__ int ymax[TN];
+    cg::cluster_group cl = cg::this_cluster();
+    const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int w = blockIdx.x / CL;
+    if (w >= nitems) return;                 // the grid is nitems clusters: never taken by a part of one
     const Item it = items[w];
     const ProbDesc &P = descs[it.prob];
-    const int K = it.K, side = it.ntiles & 1, j0 = (it.ntiles >> 1) * kFmaCols, p0 = it.tile * R;
+    const int K = it.K, side = it.ntiles & 1, j0 = (it.ntiles >> 1) * TN, p0 = it.tile * R;
     const int fc = P.super_ptr[K];
     const int s = P.super_ptr[K + 1] - fc;
     const int64_t ld = P.rowptr[K + 1] - P.rowptr[K];
@@ -77,13 +83,13 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restr
         tile_cb[r] = p0 + r < c ? P.colbase[pos0 + p0 + r] : 0;
         tile_rb[r] = p0 + r < c ? P.relbase[pos0 + p0 + r] : 0;
     }
-    if (tid < kFmaCols) ymax[tid] = 0;
-    T acc[R / 16][4];
+    if (tid < TN) ymax[tid] = 0;
+    T acc[R / 16][TN / 8];
 #pragma unroll
     for (int i = 0; i < R / 16; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = Sc<T>::zero();
-    constexpr int NA = R * kFmK / kFmThreads, NB = kFmaCols * kFmK / kFmThreads;
+        for (int j = 0; j < TN / 8; j++) acc[i][j] = Sc<T>::zero();
+    constexpr int NA = R * kFmK / kFmThreads, NB = TN * kFmK / kFmThreads;
     // entry u of this thread in the stage at k0: contiguous down the stored
     // columns, rows fastest below the diagonal, k fastest above it
     auto place = [&](int k0, int u, int &r, int &kk) {
@@ -91,6 +97,8 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restr
         if (k0 >= p0 + R) { kk = e % kFmK; r = e / kFmK; }
         else { r = e % R; kk = e / R; }
     };
+    const int per = ((c + CL - 1) / CL + kFmK - 1) / kFmK * kFmK;     // this CTA's range of q
+    const int ka = rank * per, kb = c < ka + per ? c : ka + per;
     __syncthreads();
     int64_t addr[NA];            // of the next stage
     auto find = [&](int k0) {
@@ -100,7 +108,7 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restr
             place(k0, u, r, kk);
             const int p = p0 + r, q = k0 + kk;
             addr[u] = -1;
-            if (p < c && q < c) {
+            if (p < c && q < kb) {
                 const int64_t a = p >= q ? pcb[q] + P.relidx[prb[q] + p] : tile_cb[r] + P.relidx[tile_rb[r] + q];
                 if (chk.ok(a)) addr[u] = a;
             }
@@ -119,13 +127,13 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restr
 #pragma unroll
         for (int u = 0; u < NB; u++) {
             const int e = tid + kFmThreads * u, kk = e % kFmK, j = e / kFmK;
-            vb[u] = k0 + kk < c && j0 + j < s ? B[(int64_t)(j0 + j) * ld + k0 + kk] : Sc<T>::zero();
+            vb[u] = k0 + kk < kb && j0 + j < s ? B[(int64_t)(j0 + j) * ld + k0 + kk] : Sc<T>::zero();
         }
     };
-    find(0);
-    load(0);
-    find(kFmK);
-    for (int k0 = 0; k0 < c; k0 += kFmK) {
+    find(ka);
+    load(ka);
+    find(ka + kFmK);
+    for (int k0 = ka; k0 < kb; k0 += kFmK) {
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < NA; u++) {
@@ -139,16 +147,35 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restr
             Bs[e % kFmK][e / kFmK] = vb[u];
         }
         __syncthreads();
-        if (k0 + kFmK < c) {     // the next stage's values and the addresses after them, under the products
+        if (k0 + kFmK < kb) {    // the next stage's values and the addresses after them, under the products
             load(k0 + kFmK);
             find(k0 + 2 * kFmK);
         }
-        fma_stage<T, R>(As, Bs, c - k0 < kFmK ? c - k0 : kFmK, acc);
+        fma_stage<T, R, TN>(As, Bs, kb - k0 < kFmK ? kb - k0 : kFmK, acc);
     }
     T *out = static_cast<T *>(side ? P.Zu : P.Z) + off + s;
     const int tx = tid % 16, ty = tid / 16;
+    if (CL > 1) {                // the partial sums through shared memory, added in rank order
+        T *Pt = kFmK * (R + 1) >= R * TN ? &As[0][0] : &Bs[0][0];
+        __syncthreads();
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
+        for (int i = 0; i < R / 16; i++)
+#pragma unroll
+            for (int j = 0; j < TN / 8; j++) Pt[(ty + 8 * j) * R + tx + 16 * i] = acc[i][j];
+        cl.sync();
+        if (rank == 0)
+            for (int q = 1; q < CL; q++) {
+                const T *pq = cl.map_shared_rank(Pt, q);
+#pragma unroll
+                for (int i = 0; i < R / 16; i++)
+#pragma unroll
+                    for (int j = 0; j < TN / 8; j++) acc[i][j] = add(acc[i][j], pq[(ty + 8 * j) * R + tx + 16 * i]);
+            }
+        cl.sync();
+        if (rank) return;
+    }
+#pragma unroll
+    for (int j = 0; j < TN / 8; j++) {
         const int col = j0 + ty + 8 * j;
         int e = 0;
 #pragma unroll
@@ -164,7 +191,7 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_rows(const ProbDesc *__restr
     if (side) return;
     __syncthreads();
     // whole-column exponents for the row bounds of later tensor-core gathers (zeroed at the start of the call)
-    if (tid < kFmaCols && ymax[tid]) atomicMax(&P.colexpZ[fc + j0 + tid], ymax[tid]);
+    if (tid < TN && ymax[tid]) atomicMax(&P.colexpZ[fc + j0 + tid], ymax[tid]);
 }
 
 // items: tile = row tile of 32 rows, ntiles = (column tile of 32) << 1 | side
@@ -204,7 +231,7 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_lhat(const ProbDesc *__restr
             Bs[kk][j] = k0 + kk < s && j0 + j < s ? X[(int64_t)(j0 + j) * s + k0 + kk] : Sc<T>::zero();
         }
         __syncthreads();
-        fma_stage<T, R>(As, Bs, s - k0 < kFmK ? s - k0 : kFmK, acc);
+        fma_stage<T, R, kFmaCols>(As, Bs, s - k0 < kFmK ? s - k0 : kFmK, acc);
     }
     const int tx = tid % 16, ty = tid / 16;
 #pragma unroll
@@ -345,16 +372,34 @@ __global__ void __launch_bounds__(kFmThreads) k_fma_diag(const ProbDesc *__restr
     if (CL > 1) cl.sync();   // no CTA leaves while the first may still read its sums
 }
 
-cudaError_t launch_fma_rows(int dtype, int rows, const ProbDesc *d, const Item *items, int n, cudaStream_t st) {
+template <typename... A>
+static cudaError_t launch_cluster(void (*kernel)(A...), int n, int cl, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n * cl));
+    cfg.blockDim = dim3(kFmThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename T>
+static cudaError_t launch_fma_rows_t(int rows, int cols, int cl, const ProbDesc *d, const Item *items, int n, cudaStream_t st) {
+    if (rows == 16)
+        return cols == 16 ? launch_cluster(k_fma_rows<T, 16, 16>, n, cl, st, d, items, n)
+                          : launch_cluster(k_fma_rows<T, 16, 32>, n, cl, st, d, items, n);
+    return cols == 16 ? launch_cluster(k_fma_rows<T, 32, 16>, n, cl, st, d, items, n)
+                      : launch_cluster(k_fma_rows<T, 32, 32>, n, cl, st, d, items, n);
+}
+
+cudaError_t launch_fma_rows(int dtype, int rows, int cols, int cl, const ProbDesc *d, const Item *items, int n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (dtype == SELINV_C128) {
-        if (rows == 16) k_fma_rows<zd, 16><<<n, kFmThreads, 0, st>>>(d, items, n);
-        else k_fma_rows<zd, 32><<<n, kFmThreads, 0, st>>>(d, items, n);
-    } else {
-        if (rows == 16) k_fma_rows<double, 16><<<n, kFmThreads, 0, st>>>(d, items, n);
-        else k_fma_rows<double, 32><<<n, kFmThreads, 0, st>>>(d, items, n);
-    }
-    return cudaGetLastError();
+    return dtype == SELINV_C128 ? launch_fma_rows_t<zd>(rows, cols, cl, d, items, n, st)
+                                : launch_fma_rows_t<double>(rows, cols, cl, d, items, n, st);
 }
 
 cudaError_t launch_fma_lhat(int dtype, int narrow, const ProbDesc *d, const Item *items, int n, cudaStream_t st) {
@@ -371,18 +416,8 @@ cudaError_t launch_fma_lhat(int dtype, int narrow, const ProbDesc *d, const Item
 
 cudaError_t launch_fma_diag(int dtype, int cl, const ProbDesc *d, const Item *items, int n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n * cl));
-    cfg.blockDim = dim3(kFmThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cl;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return dtype == SELINV_C128 ? cudaLaunchKernelEx(&cfg, k_fma_diag<zd>, d, items, n)
-                                : cudaLaunchKernelEx(&cfg, k_fma_diag<double>, d, items, n);
+    return dtype == SELINV_C128 ? launch_cluster(k_fma_diag<zd>, n, cl, st, d, items, n)
+                                : launch_cluster(k_fma_diag<double>, n, cl, st, d, items, n);
 }
 
 }  // namespace selinv

@@ -22,12 +22,13 @@ cudaError_t launch_dinv(int dtype, const ProbDesc *d, const int2 *work, int nwor
 cudaError_t launch_selinv(int dtype, int bucket, const ProbDesc *d, const Item *items, int n,
                           cudaStream_t st);
 // FP64 products of the level schedule (kernels_fma.cu): Lhat (narrow: s <= 16,
-// tiles of kFmaNarrowRows rows; else of kFmaLhatRows), A^{-1}_{C,K} by tiles of
-// `rows` (16 or 32) rows, columns by kFmaCols, and the diagonal block by 16 x 16
-// tiles, cl CTAs each
+// tiles of kFmaNarrowRows rows; else of kFmaLhatRows, columns by kFmaCols),
+// A^{-1}_{C,K} by tiles of `rows` rows x `cols` columns (16 or 32), and the
+// diagonal block by 16 x 16 tiles; cl CTAs each
 constexpr int kFmaCols = 32, kFmaLhatRows = 32, kFmaNarrowRows = 128;
 cudaError_t launch_fma_lhat(int dtype, int narrow, const ProbDesc *d, const Item *items, int n, cudaStream_t st);
-cudaError_t launch_fma_rows(int dtype, int rows, const ProbDesc *d, const Item *items, int n, cudaStream_t st);
+cudaError_t launch_fma_rows(int dtype, int rows, int cols, int cl, const ProbDesc *d, const Item *items, int n,
+                            cudaStream_t st);
 cudaError_t launch_fma_diag(int dtype, int cl, const ProbDesc *d, const Item *items, int n, cudaStream_t st);
 cudaError_t configure_ozaki_kernels();
 cudaError_t configure_tc_kernels();

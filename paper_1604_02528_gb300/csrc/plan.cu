@@ -483,6 +483,13 @@ void Schedule::release() {
     if (graph_host) cudaGraphExecDestroy(graph_host);
     graph_host = nullptr;
     host_key.fill(nullptr);
+    for (int b = 1; b < kBranches; b++) {
+        if (br[b]) cudaStreamDestroy(br[b]);
+        if (ev_bf[b]) cudaEventDestroy(ev_bf[b]);
+        if (ev_bj[b]) cudaEventDestroy(ev_bj[b]);
+        br[b] = nullptr;
+        ev_bf[b] = ev_bj[b] = nullptr;
+    }
     if (side) cudaStreamDestroy(side);
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
@@ -735,6 +742,25 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             if (cntz) S.launches.push_back({KL_DIGITS, SELINV_C128, 0, offz, cntz, -1});
         }
         for (size_t q = ph_first; q < S.launches.size(); q++) S.launches[q].side = ph;
+        if (ph == 0) continue;
+        // the side stream's long launches of one CTA per SM, in pieces: a grid
+        // of many waves would keep the main stream's few CTAs waiting to its
+        // end (320 us for the Lhat of 40^3's middle levels, 460 for a sheet's)
+        std::vector<Launch> cut(S.launches.begin() + ph_first, S.launches.end());
+        S.launches.resize(ph_first);
+        for (const Launch &L : cut) {
+            const bool fills = (L.kind == KL_LHAT_OZ && L.bucket == kTcWide) || (L.kind == KL_LINV && L.bucket == 1);
+            if (!fills || L.count < 2 * 152) {
+                S.launches.push_back(L);
+                continue;
+            }
+            for (int o = 0; o < L.count; o += kSideCtas) {
+                Launch piece = L;
+                piece.off = L.off + o;
+                piece.count = std::min(kSideCtas, L.count - o);
+                S.launches.push_back(piece);
+            }
+        }
     }
     // 3) the traversal, root to leaves
     auto push_items = [&](int i, int32_t K) {
@@ -867,7 +893,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             const int tn = s <= 32 ? 32 : 64;
             units += (int64_t)((s + tn - 1) / tn) * z_nmt(s);
         }
-        for (int tn : {64, 32}) {
+        for (int tn : {32, 64}) {   // (the narrow ones beside the wide ones in a level: group())
             const int64_t off2 = (int64_t)S.h_items.size();
             for (auto &ik : zs) {
                 const int s = plans[ik.first]->super_ptr[ik.second + 1] - plans[ik.first]->super_ptr[ik.second];
@@ -1135,7 +1161,16 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             }
             int64_t level_ctas = 0;
             for (auto &ik : oz) level_ctas += oz_ctas(ik.first, ik.second);
+            // The launches of a level in groups that do not depend on one another
+            // (every one reads the levels above): the contraction of each width
+            // class with its split-k sums, the diagonal blocks after it, complex
+            // supernodes, FP64 tiles, narrow supernodes.  Each fills a part of the
+            // chip only, so they run on branches of the main stream.
+            const size_t lev0 = S.launches.size();
+            struct Group { size_t lo, hi; };
+            auto group = [&](size_t lo) { return Group{lo, S.launches.size()}; };
             launch_z(zs, l, level_ctas);
+            const Group g_z = group(lev0);
             // the level's split, and its supernodes in the order of their items'
             // length, longest first (the CTAs that start last are short ones)
             const int sig = level_split(oz, level_ctas);
@@ -1143,8 +1178,8 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 return oz_chunk(a.first, a.second, oz_split(a.first, a.second, level_ctas, sig)) >
                        oz_chunk(b.first, b.second, oz_split(b.first, b.second, level_ctas, sig));
             });
-            for (int tc = 1; tc >= 0; tc--)
-                for (int tn : {kTcWide, 64, 32, 16}) {
+            auto gemm = [&](int tn) {
+                for (int tc = 1; tc >= 0; tc--) {
                     const int64_t off = (int64_t)S.h_items.size();
                     for (auto &ik : oz) {
                         const PlanData &p = *plans[ik.first];
@@ -1158,38 +1193,59 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                         if (tc) add_tc_reduce(S.launches.back());
                     }
                 }
+            };
+            size_t at = S.launches.size();
+            gemm(kTcWide);
+            const Group g_wide = group(at);
+            at = S.launches.size();
+            gemm(64);
+            const Group g_64 = group(at);
+            at = S.launches.size();
+            gemm(32);
+            gemm(16);
+            // diagonal blocks: tcgen05 (per column-tile width) or mma.sync
+            int64_t diag_units = 0;
+            for (auto &ik : oz) {
+                const int s = plans[ik.first]->super_ptr[ik.second + 1] - plans[ik.first]->super_ptr[ik.second];
+                if (diag_tc(ik.first, s)) diag_units += (s + dtc_tn(s) - 1) / dtc_tn(s);
+            }
+            std::vector<std::pair<Launch, int>> fins;
+            // those of at most 32 columns on the mma.sync kernel; wider ones of a
+            // problem off tcgen05 there too, after every contraction
+            bool oz_wide = false;
             {
-                // diagonal blocks: tcgen05 (per column-tile width) or mma.sync
-                int64_t diag_units = 0;
-                for (auto &ik : oz) {
-                    const int s = plans[ik.first]->super_ptr[ik.second + 1] - plans[ik.first]->super_ptr[ik.second];
-                    if (diag_tc(ik.first, s)) diag_units += (s + dtc_tn(s) - 1) / dtc_tn(s);
-                }
-                std::vector<std::pair<Launch, int>> fins;
-                for (int tn : {64, 32}) {
-                    const int64_t off = (int64_t)S.h_items.size();
-                    for (auto &ik : oz) {
-                        const int s = plans[ik.first]->super_ptr[ik.second + 1] - plans[ik.first]->super_ptr[ik.second];
-                        if (diag_tc(ik.first, s) && dtc_tn(s) == tn) push_diag_tc(ik.first, ik.second, diag_units);
-                    }
-                    const int cnt = (int)(S.h_items.size() - off);
-                    if (cnt) {
-                        S.launches.push_back({KL_DIAG_TC, SELINV_F64, tn, off, cnt, l});
-                        fins.push_back({S.launches.back(), 1});
-                    }
-                }
                 const int64_t off = (int64_t)S.h_items.size();
                 for (auto &ik : oz) {
                     const int s = plans[ik.first]->super_ptr[ik.second + 1] - plans[ik.first]->super_ptr[ik.second];
-                    if (!diag_tc(ik.first, s)) push_diag(ik.first, ik.second);
+                    if (diag_tc(ik.first, s)) continue;
+                    push_diag(ik.first, ik.second);
+                    oz_wide = oz_wide || s > 32;
                 }
                 const int cnt = (int)(S.h_items.size() - off);
                 if (cnt) {
                     S.launches.push_back({KL_DIAG, SELINV_F64, 0, off, cnt, l});
                     fins.push_back({S.launches.back(), 0});
                 }
-                add_diag_fin(fins);
             }
+            const Group g_small = group(at);
+            at = S.launches.size();
+            for (int tn : {64, 32}) {
+                const int64_t off = (int64_t)S.h_items.size();
+                for (auto &ik : oz) {
+                    const int s = plans[ik.first]->super_ptr[ik.second + 1] - plans[ik.first]->super_ptr[ik.second];
+                    if (diag_tc(ik.first, s) && dtc_tn(s) == tn) push_diag_tc(ik.first, ik.second, diag_units);
+                }
+                const int cnt = (int)(S.h_items.size() - off);
+                if (cnt) {
+                    S.launches.push_back({KL_DIAG_TC, SELINV_F64, tn, off, cnt, l});
+                    fins.push_back({S.launches.back(), 1});
+                }
+            }
+            const Group g_diag = group(at);
+            at = S.launches.size();
+            add_diag_fin(fins);
+            const Group g_fin = group(at);
+            at = S.launches.size();
             // fused FP64 kernels for everything else: narrow supernodes, then a
             // CTA per row tile of the rest
             for (int dt = 0; dt < 2; dt++) {
@@ -1231,9 +1287,12 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 nl.smem = smem;
                 S.launches.push_back(nl);
             }
+            const Group g_narrow = group(at);
+            at = S.launches.size();
             for (int dt = 0; dt < 2; dt++) {
                 std::vector<std::pair<int, int32_t>> ks;   // (problem, K)
                 int64_t ctas = 0, tiles = 0, cmax = 0;     // row tiles of 32, diagonal tiles
+                int smax = 0;
                 for (int i = 0; i < np; i++) {
                     if (descs[i].dtype != dt) continue;
                     const PlanData &p = *plans[i];
@@ -1245,26 +1304,34 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                         ks.push_back({i, K});
                         const int64_t c = p.rowptr[K + 1] - p.rowptr[K] - s, nt = (s + 15) / 16, two = descs[i].lu ? 2 : 1;
                         ctas += two * ((c + 31) / 32) * ((s + kFmaCols - 1) / kFmaCols);
+                        smax = std::max(smax, s);
                         tiles += descs[i].lu ? nt * nt : nt * (nt + 1) / 2;
                         cmax = std::max(cmax, c);
                     }
                 }
                 if (ks.empty()) continue;
                 // rows of a tile: 32, or 16 where that leaves SMs without three CTAs
-                // (what hides a stage's gather)
-                const int rows = ctas < 3 * 152 ? 16 : 32;
+                // (what hides a stage's gather); 16 columns when no supernode has
+                // more; then a cluster per tile, 64 rows of C each, up to two CTAs per SM
+                const int rows = ctas < 3 * 152 ? 16 : 32, cols = smax <= 16 ? 16 : kFmaCols;
                 const int64_t off = (int64_t)S.h_items.size();
                 for (auto &ik : ks) {
                     const PlanData &p = *plans[ik.first];
                     const int s = p.super_ptr[ik.second + 1] - p.super_ptr[ik.second];
                     const int64_t c = p.rowptr[ik.second + 1] - p.rowptr[ik.second] - s;
                     for (int64_t t = 0; t < (c + rows - 1) / rows; t++)
-                        for (int ct = 0; ct < (s + kFmaCols - 1) / kFmaCols; ct++)
+                        for (int ct = 0; ct < (s + cols - 1) / cols; ct++)
                             for (int side = 0; side <= (descs[ik.first].lu ? 1 : 0); side++)
                                 S.h_items.push_back({ik.first, ik.second, (int)t, (ct << 1) | side});
                 }
                 const int cnt = (int)(S.h_items.size() - off);
-                if (cnt) S.launches.push_back({KL_SELINV, dt, kFmaRows + rows, off, cnt, l});
+                int ksp = 8;
+                while (ksp > 1 && ((int64_t)cnt * ksp > 2 * 152 || cmax < 64 * ksp)) ksp /= 2;
+                if (cnt) {
+                    Launch nl{KL_SELINV, dt, kFmaRows + rows + (cols == 16 ? 1 : 0), off, cnt, l};
+                    nl.smem = ksp;
+                    S.launches.push_back(nl);
+                }
                 const int64_t off2 = (int64_t)S.h_items.size();
                 for (auto &ik : ks) {
                     const PlanData &p = *plans[ik.first];
@@ -1274,8 +1341,81 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 }
                 int cl = 8;   // CTAs per diagonal tile: two per SM over the level, 64 rows of C each
                 while (cl > 1 && (tiles * cl > 2 * 152 || cmax < 64 * cl)) cl /= 2;
-                S.launches.push_back({KL_SELINV, dt, kFmaDiag + cl, off2, (int)(S.h_items.size() - off2), l});
+                Launch nl{KL_SELINV, dt, kFmaDiag, off2, (int)(S.h_items.size() - off2), l};
+                nl.smem = cl;
+                S.launches.push_back(nl);
             }
+            const Group g_fma = group(at);
+            // the groups in order, the main stream's last (a branch forks where its
+            // first launch stands in the list): the branches of the level's
+            // contractions, then the main chain with the joins that it needs
+            std::vector<Launch> all(S.launches.begin() + lev0, S.launches.end());
+            S.launches.resize(lev0);
+            auto put = [&](const Group &g, int branch, unsigned join) {
+                for (size_t q = g.lo; q < g.hi; q++) {
+                    Launch L = all[q - lev0];
+                    L.branch = branch;
+                    L.join = q == g.lo ? join : 0;
+                    S.launches.push_back(L);
+                }
+            };
+            auto some = [](const Group &g) { return g.hi > g.lo; };
+            const bool any_oz = some(g_wide) || some(g_64) || some(g_small) || some(g_diag);
+            // the chain that keeps the main stream: real tensor-core supernodes,
+            // else the complex ones, else the FP64 tiles, else the narrow ones
+            const bool z_main = !any_oz, fma_main = z_main && !some(g_z), nar_main = fma_main && !some(g_fma);
+            if (!nar_main) put(g_narrow, 5, 0);
+            if (!fma_main) put(g_fma, 3, 0);
+            if (!z_main) put(g_z, 4, 0);
+            const bool b64 = some(g_64) && some(g_wide);
+            // (a wide supernode's diagonal block on mma.sync waits for its contraction: no branch then)
+            const bool bsm = some(g_small) && (some(g_wide) || some(g_64)) && !oz_wide;
+            if (bsm) put(g_small, 2, 0);
+            if (b64) put(g_64, 1, 0);
+            put(g_wide, 0, 0);
+            if (!b64) put(g_64, 0, 0);
+            if (!bsm) put(g_small, 0, b64 ? 1u << 1 : 0);
+            put(g_diag, 0, b64 && bsm ? 1u << 1 : (b64 ? 1u << 1 : 0));
+            put(g_fin, 0, (b64 ? 1u << 1 : 0) | (bsm ? 1u << 2 : 0));
+            if (z_main && some(g_z)) {
+                // complex: after the contraction and its sums, the diagonal blocks of
+                // the narrow class (the first of the two) beside those of the wide one
+                std::vector<size_t> dg;
+                for (size_t q = g_z.lo; q < g_z.hi; q++)
+                    if (all[q - lev0].kind == KL_DIAG_TC) dg.push_back(q);
+                if (dg.size() == 2) {
+                    put(Group{g_z.lo, dg[0]}, 0, 0);
+                    put(Group{dg[0], dg[1]}, 2, 0);
+                    put(Group{dg[1], g_z.hi}, 0, 0);
+                } else {
+                    put(g_z, 0, 0);
+                }
+            }
+            if (fma_main) put(g_fma, 0, 0);
+            if (nar_main) put(g_narrow, 0, 0);
+        }
+    }
+    // split-k slots: the launches of a level may run side by side
+    int64_t slab_slots = 0;
+    {
+        int level = -2;
+        int64_t next = 0, last[2][kTcWide + 1] = {};   // per type and bucket: the level's latest contraction
+        for (Launch &L : S.launches) {
+            if (L.kind != KL_SELINV_TC && L.kind != KL_TC_REDUCE) continue;
+            if (L.level != level || mode == SELINV_SCHED_PLAIN) {
+                if (L.kind == KL_SELINV_TC) next = 0;
+                level = L.level;
+            }
+            int64_t &mine = last[L.dtype != SELINV_F64][L.bucket];
+            if (L.kind == KL_TC_REDUCE) {
+                L.slab = mine;
+                continue;
+            }
+            bool split = false;
+            for (int64_t e = L.off; e < L.off + L.count && !split; e++) split = S.h_items[e].ntiles > 1;
+            L.slab = mine = next;
+            if (split) next += L.count;
+            slab_slots = std::max(slab_slots, next);
         }
     }
     S.h_descs = descs;
@@ -1316,12 +1456,9 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             S.pre_ptr.push_back(descs[i].Z);
             S.pre_bytes.push_back(elem_size(descs[i].dtype) * (size_t)std::max<int64_t>(plans[i]->nnz, 1));
         }
-    // one partial (hi, lo) tile of 128 x 64 per CTA of the widest tcgen05 launch
-    int64_t tc_ctas = 0;
-    for (const Launch &L : S.launches)
-        if (L.kind == KL_SELINV_TC) tc_ctas = std::max<int64_t>(tc_ctas, L.count);
-    if (tc_ctas > 0 &&
-        cudaMalloc((void **)&S.tcslab, sizeof(long long) * (size_t)kTcSlotWords * (size_t)tc_ctas) != cudaSuccess)
+    // one partial (hi, lo) tile of 128 x 64 per CTA of a level's k-split tcgen05 launches
+    if (slab_slots > 0 &&
+        cudaMalloc((void **)&S.tcslab, sizeof(long long) * (size_t)kTcSlotWords * (size_t)slab_slots) != cudaSuccess)
         return SELINV_ERR_OOM;
 
     if (!S.h_red.empty() && (rc = upload(&S.d_red, S.h_red))) return rc;
@@ -1330,6 +1467,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
 
 // one launch of a schedule with the problem descriptors at `d`
 cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, cudaStream_t st) {
+    long long *slab = S.tcslab ? S.tcslab + L.slab * kTcSlotWords : nullptr;
     switch (L.kind) {
     // the wide supernodes' Dinv follows in KL_DINV launches
     case KL_LINV:
@@ -1338,8 +1476,10 @@ cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, c
     case KL_DINV: return launch_dinv(L.dtype, d, S.d_work + L.off, L.count, st);
     case KL_LHAT: return launch_fma_lhat(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_SELINV:
-        if (L.bucket >= kFmaDiag) return launch_fma_diag(L.dtype, L.bucket - kFmaDiag, d, S.d_items + L.off, L.count, st);
-        if (L.bucket >= kFmaRows) return launch_fma_rows(L.dtype, L.bucket - kFmaRows, d, S.d_items + L.off, L.count, st);
+        if (L.bucket >= kFmaDiag) return launch_fma_diag(L.dtype, L.smem, d, S.d_items + L.off, L.count, st);
+        if (L.bucket >= kFmaRows)
+            return launch_fma_rows(L.dtype, (L.bucket - kFmaRows) & ~1, (L.bucket - kFmaRows) & 1 ? 16 : kFmaCols, L.smem, d,
+                                   S.d_items + L.off, L.count, st);
         return launch_selinv(L.dtype, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_DIGITS:
         if (L.dtype != SELINV_F64) return launch_digits_z(0, d, S.d_work + L.off, L.count, st);
@@ -1354,12 +1494,12 @@ cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, c
         return launch_lhat_oz(L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_SELINV_TC:
         if (L.bucket == kTcWide)
-            return launch_selinv_tcw(L.dtype != SELINV_F64, d, S.d_items + L.off, L.count, S.tcslab, S.spin_limit, st);
-        return launch_selinv_tc(L.bucket, d, S.d_items + L.off, L.count, S.tcslab, S.spin_limit, st);
+            return launch_selinv_tcw(L.dtype != SELINV_F64, d, S.d_items + L.off, L.count, slab, S.spin_limit, st);
+        return launch_selinv_tc(L.bucket, d, S.d_items + L.off, L.count, slab, S.spin_limit, st);
     case KL_TC_REDUCE:
         if (L.bucket == kTcWide)
-            return launch_tcw_reduce(L.dtype != SELINV_F64, d, S.d_items, S.d_red + L.off, L.count, S.tcslab, st);
-        return launch_tc_reduce(L.bucket, d, S.d_items, S.d_red + L.off, L.count, S.tcslab, st);
+            return launch_tcw_reduce(L.dtype != SELINV_F64, d, S.d_items, S.d_red + L.off, L.count, slab, st);
+        return launch_tc_reduce(L.bucket, d, S.d_items, S.d_red + L.off, L.count, slab, st);
     case KL_DIAG_FIN:
         if (L.dtype != SELINV_F64) return launch_diag_fin_z(d, S.d_items + L.off, L.count, st);
         return launch_diag_fin(d, S.d_items + L.off, L.count, st);
@@ -1430,10 +1570,26 @@ static cudaError_t issue(Schedule &S, cudaStream_t st, bool count, const IssueHo
         return cudaSuccess;
     };
     int side_phase = 0;   // phase of the side stream's last launch
+    unsigned out = 0;     // branches of the level that the main stream has not joined
+    auto join_branches = [&](unsigned which) -> cudaError_t {
+        for (int b = 1; b < kBranches; b++) {
+            if (!(out & which & (1u << b))) continue;
+            out &= ~(1u << b);
+            cudaError_t e = cudaEventRecord(S.ev_bj[b], S.br[b]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, S.ev_bj[b], 0);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
+    int level = -1;
     for (size_t i = 0; i < S.launches.size(); i++) {
         const Launch &L = S.launches[i];
-        cudaError_t e = marks(i);
-        if (e != cudaSuccess) return e;
+        cudaError_t e = cudaSuccess;
+        if (!L.side && L.level != level) {   // the next level reads all of this one
+            if ((e = join_branches(~0u)) != cudaSuccess) return e;
+            level = L.level;
+        }
+        if ((e = marks(i)) != cudaSuccess) return e;
         if (forked && (int)i == S.join_at) {
             if (S.join_at2 < 0) e = join();   // (two phases: the side stream's whole work)
             else e = cudaStreamWaitEvent(st, S.ev_mid, 0);
@@ -1457,12 +1613,27 @@ static cudaError_t issue(Schedule &S, cudaStream_t st, bool count, const IssueHo
                 side_phase = L.side;
             }
             ls = S.side;
+        } else if (L.branch) {
+            const int b = L.branch;
+            if (!(out & (1u << b))) {
+                if (!S.br[b] && (e = cudaStreamCreateWithFlags(&S.br[b], cudaStreamNonBlocking)) != cudaSuccess) return e;
+                for (cudaEvent_t *ev : {&S.ev_bf[b], &S.ev_bj[b]})
+                    if (!*ev && (e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return e;
+                if ((e = cudaEventRecord(S.ev_bf[b], st)) != cudaSuccess) return e;
+                if ((e = cudaStreamWaitEvent(S.br[b], S.ev_bf[b], 0)) != cudaSuccess) return e;
+                out |= 1u << b;
+            }
+            ls = S.br[b];
+        } else if (L.join && (e = join_branches(L.join)) != cudaSuccess) {
+            return e;
         }
         char name[48];
         std::snprintf(name, sizeof(name), "L%d %s", L.level, launch_kind_name(L.kind));
         NvtxRange r(name);
         if ((e = launch_one(S, L, ls)) != cudaSuccess) return e;
     }
+    const cudaError_t eb = join_branches(~0u);
+    if (eb != cudaSuccess) return eb;
     if (forked) {
         const cudaError_t e = join();
         if (e != cudaSuccess) return e;

@@ -139,7 +139,8 @@ constexpr int kAsmChunk = 1024;   // entries of an update matrix per extend-add 
 constexpr int kTopSupernodes = 16;   // level schedule: the top levels (up to this many supernodes) normalized first
 constexpr int kMidSupernodes = 256;  // ... and the levels up to this many normalized in the side stream's first phase
 
-// KL_SELINV launches of the level schedule: bucket kFmaRows + rows of a tile, kFmaDiag + CTAs per tile
+// KL_SELINV launches of the level schedule: bucket kFmaRows + rows of a tile
+// (+ 1 with 16 columns, else 32), kFmaDiag: diagonal tiles; smem: CTAs per tile
 constexpr int kFmaRows = 1000, kFmaDiag = 2000;
 
 struct Launch {
@@ -149,9 +150,18 @@ struct Launch {
     int64_t off;
     int count;
     int level;
-    int smem = 0;   // dynamic shared memory (narrow supernodes)
+    int smem = 0;   // dynamic shared memory (narrow supernodes); CTAs per tile (FP64 tiles)
+    int branch = 0;          // stream of the level that runs it: 0 the main one, else one of its side branches
+    unsigned join = 0;       // branches (bits) that the main stream waits for before it
+    int64_t slab = 0;        // first split-k slot of a tcgen05 gather-GEMM and of its reduction
     int side = 0;   // 1, 2: issued on the schedule's side stream (normalization phases of the lower levels)
 };
+
+constexpr int kBranches = 6;
+// CTAs of a launch on the side stream that would fill the chip for two waves
+// or more (one per SM): it goes out in pieces that leave the main stream the
+// other SMs
+constexpr int kSideCtas = 112;
 
 struct Schedule {
     bool valid = false;
@@ -190,6 +200,8 @@ struct Schedule {
     // supernodes while the main stream traverses the top levels, and the
     // launch before which the main stream waits for it (-1: none)
     int join_at = -1, join_at2 = -1;   // the second join: three phases
+    cudaStream_t br[kBranches] = {};   // branches of a level (index 0 unused)
+    cudaEvent_t ev_bf[kBranches] = {}, ev_bj[kBranches] = {};
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_mid = nullptr;
     void release();
