@@ -60,10 +60,10 @@ cudaError_t launch_lhat_oz(int tn, const ProbDesc *d, const Item *items, int n, 
 // Narrow supernodes (at most kNarrowS columns, narrow_elems of shared memory
 // within kNarrowSmem: two CTAs per SM): cl CTAs and smem bytes each
 constexpr int kNarrowS = 16;
-constexpr int kNarrowSmem = 110 * 1024;
+constexpr int kNarrowSmem = 110 * 1024, kNarrowAlone = 116 * 1024;
 int narrow_elems(int s, int c, int cl, int lu);
 cudaError_t configure_narrow_kernels();
-cudaError_t launch_selinv_narrow(int dtype, int cl, int smem, const ProbDesc *d, const Item *items, int n,
+cudaError_t launch_selinv_narrow(int dtype, int cl, int lu, int smem, const ProbDesc *d, const Item *items, int n,
                                  cudaStream_t st);
 cudaError_t launch_push(int dtype, int kind, int bucket, const ProbDesc *d, const Item *items, int n,
                         cudaStream_t st);

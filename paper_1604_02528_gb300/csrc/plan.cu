@@ -743,14 +743,13 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
         }
         for (size_t q = ph_first; q < S.launches.size(); q++) S.launches[q].side = ph;
         if (ph == 0) continue;
-        // the side stream's long launches of one CTA per SM, in pieces: a grid
-        // of many waves would keep the main stream's few CTAs waiting to its
-        // end (320 us for the Lhat of 40^3's middle levels, 460 for a sheet's)
+        // the side stream's long launches of one CTA per SM (Lhat), in pieces: a
+        // grid of many waves would keep the main stream's few CTAs waiting to
+        // its end (320 us for 40^3's middle levels, 460 for a sheet's)
         std::vector<Launch> cut(S.launches.begin() + ph_first, S.launches.end());
         S.launches.resize(ph_first);
         for (const Launch &L : cut) {
-            const bool fills = (L.kind == KL_LHAT_OZ && L.bucket == kTcWide) || (L.kind == KL_LINV && L.bucket == 1);
-            if (!fills || L.count < 2 * 152) {
+            if (L.kind != KL_LHAT_OZ || L.bucket != kTcWide || L.count < 2 * 152) {
                 S.launches.push_back(L);
                 continue;
             }
@@ -1267,8 +1266,12 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 if (list.empty()) continue;
                 // CTAs per supernode: up to 8 while they all find an SM and each keeps
                 // 8 rows of C (shorter ones lose more to the cluster's barriers than
-                // the split saves); the supernodes in order of their work, longest first,
-                // where the SMs hold few of them (longer levels even out by themselves)
+                // the split saves; so do clusters on more than the 152 SMs for levels
+                // whose largest supernode is far above the average: up to 304, 608 or
+                // 1216 CTAs the 12 poles took 12.16, 12.46 and 12.46 ms against 11.88,
+                // a batch of 24 matrices 3.59, 3.74 and 3.88 against 3.51); the
+                // supernodes in order of their work, longest first, where the SMs hold
+                // few of them (longer levels even out by themselves)
                 int cl = 8;
                 while (cl > 1 && ((int64_t)list.size() * cl > 152 || cmax < 8 * cl)) cl /= 2;
                 if (list.size() <= 512)
@@ -1276,6 +1279,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                         return a.first > b.first;
                     });
                 int smem = 0;
+                const bool lu_any = descs[list[0].second.prob].lu != 0;   // (an LU schedule holds one problem)
                 for (const auto &x : list) {
                     const PlanData &p = *plans[x.second.prob];
                     const int32_t K = x.second.K;
@@ -1283,11 +1287,11 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                     smem = std::max(smem, narrow_elems(s, c, cl, descs[x.second.prob].lu) * (int)elem_size(dt));
                     S.h_items.push_back(x.second);
                 }
-                Launch nl{KL_SELINV_TINY, dt, cl, off, (int)list.size(), l};
+                Launch nl{KL_SELINV_TINY, dt, cl | (lu_any ? 16 : 0), off, (int)list.size(), l};   // (CTAs each, LU form)
                 nl.smem = smem;
                 S.launches.push_back(nl);
             }
-            const Group g_narrow = group(at);
+            const Group g_narrow = group(at);   // (one launch per element type)
             at = S.launches.size();
             for (int dt = 0; dt < 2; dt++) {
                 std::vector<std::pair<int, int32_t>> ks;   // (problem, K)
@@ -1364,7 +1368,8 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             // the chain that keeps the main stream: real tensor-core supernodes,
             // else the complex ones, else the FP64 tiles, else the narrow ones
             const bool z_main = !any_oz, fma_main = z_main && !some(g_z), nar_main = fma_main && !some(g_fma);
-            if (!nar_main) put(g_narrow, 5, 0);
+            for (size_t q = g_narrow.lo; q < g_narrow.hi; q++)
+                if (!nar_main || q + 1 < g_narrow.hi) put(Group{q, q + 1}, q == g_narrow.lo ? 5 : 6, 0);
             if (!fma_main) put(g_fma, 3, 0);
             if (!z_main) put(g_z, 4, 0);
             const bool b64 = some(g_64) && some(g_wide);
@@ -1392,7 +1397,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 }
             }
             if (fma_main) put(g_fma, 0, 0);
-            if (nar_main) put(g_narrow, 0, 0);
+            if (nar_main && some(g_narrow)) put(Group{g_narrow.hi - 1, g_narrow.hi}, 0, 0);
         }
     }
     // split-k slots: the launches of a level may run side by side
@@ -1506,7 +1511,7 @@ cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, c
     case KL_DIAG_TC:
         return launch_diag_tc(L.bucket, L.dtype != SELINV_F64, d, S.d_items + L.off, L.count, S.spin_limit, st);
     case KL_SELINV_TINY:
-        return launch_selinv_narrow(L.dtype, L.bucket, L.smem, d, S.d_items + L.off, L.count, st);
+        return launch_selinv_narrow(L.dtype, L.bucket & 15, L.bucket >> 4, L.smem, d, S.d_items + L.off, L.count, st);
     case KL_PUSH_DIAG: return launch_push(L.dtype, 0, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_PUSH: return launch_push(L.dtype, 1, L.bucket, d, S.d_items + L.off, L.count, st);
     case KL_PERSIST: {

@@ -157,7 +157,7 @@ struct Launch {
     int side = 0;   // 1, 2: issued on the schedule's side stream (normalization phases of the lower levels)
 };
 
-constexpr int kBranches = 6;
+constexpr int kBranches = 7;
 // CTAs of a launch on the side stream that would fill the chip for two waves
 // or more (one per SM): it goes out in pieces that leave the main stream the
 // other SMs

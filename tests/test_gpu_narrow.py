@@ -67,3 +67,10 @@ def test_narrow_lu(native, cuda_device, cap, n, cplx):
     low = oracle.lower_mask(sym)
     assert oracle.block_errors(sym, Zl.cpu().numpy(), Zl0).max() <= 1e-12
     assert oracle.block_errors(sym, np.where(low, Zu.cpu().numpy(), 0), np.where(low, Zu0, 0)).max() <= 1e-12
+
+
+# more supernodes in a level than SMs: small CTAs on the packed triangle
+@pytest.mark.parametrize("make", [lambda: synth.laplacian_2d(63, 19), lambda: synth.laplacian_3d(14, 4),
+                                  lambda: synth.magnetic_laplacian_3d(13, 4)])
+def test_narrow_long_levels(native, cuda_device, make):
+    _selinv(make())
