@@ -363,38 +363,47 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
 }
 
 // ---------------------------------------------------------------------------
-// k_ftrsm: X D L_JJ^T = A for the rows of C (D L_JJ^H for a Hermitian matrix),
-// a warp for R rows at a time, lanes over the columns: with y = x D, step j
-// broadcasts y_j and every later column subtracts y_j L(k, j); the rows are
-// scaled by 1 / D once at the end.  L_JJ's lower triangle waits in shared
-// memory (columns from their 32-block's first row on, zeros above the
-// diagonal), so each step is one broadcast and at most four FP64
-// instructions per row: the FP64 pipe bounds it, and the row tiles are made
-// small enough that every SM gets one.
+// k_ftrsm: X D L_JJ^T = A for the rows of C (D L_JJ^H for a Hermitian matrix):
+// with y = x D, step j broadcasts y_j and every later column subtracts
+// y_j L(k, j); the rows are scaled by 1 / D once at the end.  L_JJ's lower
+// triangle waits in shared memory (columns from their 32-block's first row on,
+// zeros above the diagonal).  The FP64 pipe bounds it, so a warp packs four
+// rows of its share into its lanes, then two, then one (tri_rows), and the row
+// tiles are made small enough that every SM gets one.
 // items {J, first row of C, rows}
 // ---------------------------------------------------------------------------
 constexpr int kFtThreads = kTriThreads;
 
-template <typename T, int NC, int R>
+template <typename T, int W, int NC>
+__device__ __forceinline__ void ftrsm_group(const T *Ls, const T *rD, T *P, int64_t ld, int s, int row, int end, bool herm) {
+    constexpr int NT = NC * 32 / W;
+    const int c = threadIdx.x % W;
+    row += threadIdx.x % 32 / W;
+    T a[NT];
+#pragma unroll
+    for (int t = 0; t < NT; t++) {
+        const int k = c + W * t;
+        a[t] = row < end && k < s ? P[(int64_t)k * ld + row] : Sc<T>::zero();
+    }
+    tri_rows<T, W, NC, false>(a, Ls, nullptr, (s + W - 1) / W, 0, herm);
+#pragma unroll
+    for (int t = 0; t < NT; t++) {
+        const int k = c + W * t;
+        if (row < end && k < s) P[(int64_t)k * ld + row] = mul(a[t], rD[k]);
+    }
+}
+
+template <typename T, int NC>
 __device__ void ftrsm_rows(const T *Ls, const T *rD, T *P, int64_t ld, int s, int row0, int nrows, bool herm) {
-    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    for (int g = warp * R; g < nrows; g += kFtThreads / 32 * R) {
-        T a[R][NC];
-#pragma unroll
-        for (int r = 0; r < R; r++)
-#pragma unroll
-            for (int t = 0; t < NC; t++) {
-                const int k = lane + 32 * t;
-                a[r][t] = (g + r < nrows && k < s) ? P[(int64_t)k * ld + row0 + g + r] : Sc<T>::zero();
-            }
-        tri_rows<T, NC, R, false>(a, Ls, nullptr, 0, herm);
-#pragma unroll
-        for (int r = 0; r < R; r++)
-#pragma unroll
-            for (int t = 0; t < NC; t++) {
-                const int k = lane + 32 * t;
-                if (g + r < nrows && k < s) P[(int64_t)k * ld + row0 + g + r] = mul(a[r][t], rD[k]);
-            }
+    constexpr int kWarps = kFtThreads / 32;
+    const int share = (nrows + kWarps - 1) / kWarps, warp = threadIdx.x / 32;
+    const int end = row0 + min(nrows, (warp + 1) * share);
+    for (int row = row0 + warp * share; row < end;) {
+        const int left = end - row;
+        if (left > 2) ftrsm_group<T, 8, NC>(Ls, rD, P, ld, s, row, end, herm);
+        else if (left == 2) ftrsm_group<T, 16, NC>(Ls, rD, P, ld, s, row, end, herm);
+        else ftrsm_group<T, 32, NC>(Ls, rD, P, ld, s, row, end, herm);
+        row += left > 2 ? 4 : left;
     }
 }
 
@@ -421,19 +430,10 @@ __global__ void __launch_bounds__(kFtThreads) k_ftrsm(const FactorDesc *__restri
     tri_store(Ls, P, ld, s, 0);
     __syncthreads();
     T *Pc = P + s;
-    // two rows at a time share the loads of L's column (one where a tile has no second row per warp)
-    constexpr int R = 2;
-    if (it.z <= kFtThreads / 32) {
-        if (nc == 1) ftrsm_rows<T, 1, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-        else if (nc == 2) ftrsm_rows<T, 2, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-        else if (nc == 3) ftrsm_rows<T, 3, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-        else ftrsm_rows<T, 4, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-    } else {
-        if (nc == 1) ftrsm_rows<T, 1, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-        else if (nc == 2) ftrsm_rows<T, 2, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-        else if (nc == 3) ftrsm_rows<T, 3, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-        else ftrsm_rows<T, 4, R>(Ls, rD, Pc, ld, s, it.y, it.z, h);
-    }
+    if (nc == 1) ftrsm_rows<T, 1>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+    else if (nc == 2) ftrsm_rows<T, 2>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+    else if (nc == 3) ftrsm_rows<T, 3>(Ls, rD, Pc, ld, s, it.y, it.z, h);
+    else ftrsm_rows<T, 4>(Ls, rD, Pc, ld, s, it.y, it.z, h);
 }
 
 // ---------------------------------------------------------------------------
@@ -592,14 +592,16 @@ int factor_tables(selinv_plan_s *plan) {
         const int64_t nw = (int64_t)wide.size();
         v.cl = v.wide_s <= 32 ? 1 : (nw * 8 <= 152 ? 8 : (nw * 4 <= 152 ? 4 : (nw * 2 <= 152 ? 2 : 1)));
         // rows per tile: the number whose tiles, dealt to the SMs, take least --
-        // a row per warp costs about 10 us of an SM sub-partition at 128
-        // columns, a tile's L_JJ 5 us more for each of the two CTAs in flight
+        // a warp's groups of four, two and one row cost about 34, 18 and 10 us
+        // of an SM sub-partition at 128 columns, a tile's L_JJ 5 us more for
+        // each of the two CTAs in flight
         int rt = 4;
         int64_t least = INT64_MAX;
         for (int t = 4; t <= 64; t += 4) {
             int64_t nt = 0;
             for (int32_t J : wide) nt += (below(J) + t - 1) / t;
-            const int64_t per = (nt + 151) / 152, cost = per * (t / 4) * 10 + (per + 1) / 2 * 5;
+            constexpr int rest[4] = {0, 10, 18, 34};
+            const int64_t per = (nt + 151) / 152, cost = per * (t / 16 * 34 + rest[t / 4 % 4]) + (per + 1) / 2 * 5;
             if (cost < least) {
                 least = cost;
                 rt = t;

@@ -108,3 +108,12 @@ def test_badly_scaled_matrix(native, cuda_device, cap):
     scale = np.sqrt(np.abs(D0))[c] / np.sqrt(p.values[p.diag_positions()])[r]
     assert np.abs(np.where(r > c, (L.cpu().numpy() - L0) * scale, 0)).max() <= 1e-12
     assert np.abs(D.cpu().numpy() / D0 - 1).max() <= 1e-12
+
+
+# row tiles of 4 to 64 rows: groups of four, two and one row per warp, and ragged last tiles
+@pytest.mark.parametrize("kind", ["f64", "c128h"])
+@pytest.mark.parametrize("count,size,cap", [(6, 101, 34), (10, 143, 50), (16, 167, 33), (16, 230, 96), (24, 167, 33), (30, 201, 70)])
+def test_row_tiles(native, cuda_device, count, size, cap, kind):
+    p = _blocks(count, size, kind, size)
+    p.supernodes = {"kind": "fundamental", "cap": cap, "fill": 0.0}
+    _check(p)
