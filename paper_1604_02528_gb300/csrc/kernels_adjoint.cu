@@ -92,6 +92,7 @@ struct AdjData {
     int4 *d_vitems = nullptr;
     std::vector<int64_t> g_lptr, c_lptr, j_lptr;
     double *V = nullptr;  // update matrices (tables shared with the factorization)
+    double *part = nullptr;   // split partials of every supernode (at most two panels' worth: s^2 per 64 rows)
     Item *d_items = nullptr, *d_lhat = nullptr;
     int2 *d_linv = nullptr, *d_gitems = nullptr, *d_citems = nullptr;
     int *d_js = nullptr;
@@ -132,6 +133,14 @@ struct AdjData {
     // the per-level loops of the two passes as CUDA graphs (captured on first
     // use, rebuilt when the lists or the workspace change)
     int gen = 0;                              // bumped whenever the lists are rebuilt
+    // groups of levels of the selected inversion's adjoint, and the narrow
+    // supernodes' items by group and bucket, highest level first
+    std::vector<int> grp;
+    std::vector<Item> sg_items;
+    std::vector<int> sg_bptr;
+    Item *d_sg = nullptr;
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     CapturedLoop g_sel, g_fac;
     // row products of the wide supernodes on the transposed tcgen05 kernel:
     // (K, 64-row tile) items and (K, 8-column block) digit work per level, the
@@ -146,7 +155,7 @@ struct AdjData {
     uint16_t *sd = nullptr;
     int64_t *d_sd_off = nullptr;
     int *sdexp = nullptr;
-    ProbDesc *d_pdp = nullptr;               // [5]: YBAR, LHB, LBC, FAC, FABAR
+    ProbDesc *d_pdp = nullptr;               // [4]: YBAR, LHB, LBC, FABAR
     // the update V_K -= sym(Ybar Lhat^T) of the wide supernodes on the
     // transposed tcgen05 kernel (SYRK mode): digit work (K, 32-row block) and
     // items (K, 128 x 64 tile) per level, the digit planes of [Ybar, Lhat]
@@ -397,7 +406,7 @@ __global__ void __launch_bounds__(256) k_adj_colexpz(const AdjDesc *__restrict__
     if (lane == 0) colexpZ[fc + j] = e;
 }
 
-enum { RP_YBAR = 0, RP_LHB, RP_LBC, RP_MBP, RP_FAC, RP_FABAR, RP_FNBP };
+enum { RP_YBAR = 0, RP_LHB, RP_LBC, RP_MBP, RP_FABAR, RP_FUB };
 
 // One 32 x 32 block of
 //   RP_YBAR  Ybar = Zbar_{C,K} - Lhat S          (block 0 also stores S)
@@ -406,9 +415,9 @@ enum { RP_YBAR = 0, RP_LHB, RP_LBC, RP_MBP, RP_FAC, RP_FABAR, RP_FNBP };
 //   RP_MBP   partial of tile t: P_t(i, j) = sum_{p in t} L_C(p, i) Lhat_bar(p, j),
 //            rows i of the item's 32-row block of s
 // and of the factorization adjoint (Lb = the working Lbar)
-//   RP_FAC   G = A_C = L_C D L_KK^T
 //   RP_FABAR Abar_C = Lbar_C D^{-1} M,  M = L_KK^{-1}
-//   RP_FNBP  partial of tile t: N_t(i, j) = sum_{p in t} A_C(p, i) Lbar_C(p, j)
+//   RP_FUB   partial of tile t: U_t(i, j) = sum_{p in t} L_C(p, i) Abar_C(p, j),
+//            the 32 x 32 blocks with an entry i <= j
 // items (K, t, 32-column chunk of s, b): t is the 32-row block of C, or
 // for the partials the 64-row tile of C whose slot they fill; b is the
 // partials' 32-row block of s.
@@ -417,10 +426,8 @@ enum { RP_YBAR = 0, RP_LHB, RP_LBC, RP_MBP, RP_FAC, RP_FABAR, RP_FNBP };
 // of B, k in 16-steps, the 7 planes of a step one after the other, K-major
 // 8 x 8 core matrices), with one exponent per column j.  B by product:
 //   RP_YBAR  S, the symmetric cotangent of the diagonal block (also stored
-//            in YB's diagonal block, as the product RP_LHB reads it)
-//   RP_LHB   S from YB's diagonal block
+//            in YB's diagonal block); RP_LHB takes the same planes
 //   RP_LBC   M^T, M = L_KK^{-1}
-//   RP_FAC   D L_KK^T
 //   RP_FABAR D^{-1} M
 // One CTA per 8 columns, a warp per column; work: (0, K << 8 | column block).
 template <int OP>
@@ -445,9 +452,7 @@ __global__ void __launch_bounds__(256) k_small_digits(const AdjDesc *__restrict_
             if (k == j) return A.Zb[off + (int64_t)j * ld + j];
             return 0.5 * (k > j ? A.Zb[off + (int64_t)j * ld + k] : A.Zb[off + (int64_t)k * ld + j]);
         }
-        if (OP == RP_LHB) return A.YB[off + (int64_t)j * ld + k];
         if (OP == RP_LBC) return A.Linv[A.linv_off[K] + (int64_t)k * s + j];
-        if (OP == RP_FAC) return k == j ? A.D[fc + k] : (k < j ? A.D[fc + k] * A.L[off + (int64_t)k * ld + j] : 0.0);
         return k >= j ? A.Linv[A.linv_off[K] + (int64_t)j * s + k] / A.D[fc + k] : 0.0;
     };
     int E = 0;
@@ -508,7 +513,7 @@ template <int OP>
 __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restrict__ ad,
                                                           const int4 *__restrict__ items, int nitems) {
     grid_dep_wait();
-    constexpr bool kPart = OP == RP_MBP || OP == RP_FNBP;
+    constexpr bool kPart = OP == RP_MBP || OP == RP_FUB;
     constexpr int BM = 32;                  // rows of the output block
     constexpr int MI = BM / 16;
     __shared__ double As[kTK * BM], Bs[kTK * 32];
@@ -517,6 +522,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
     const AdjDesc &A = *ad;
     const int4 it = items[w];
     const int K = it.x, t = it.y, j0 = it.z * 32, i0 = it.w * 32;
+    if (OP == RP_FUB && i0 > j0) return;
     const int s = A.super_ptr[K + 1] - A.super_ptr[K];
     const int64_t ld = A.rowptr[K + 1] - A.rowptr[K];
     const int c = (int)(ld - s);
@@ -538,10 +544,8 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
         if (OP == RP_YBAR) return A.LD[off + (int64_t)k * ld + s + p0 + r];
         if (OP == RP_LHB) return A.Z[off + (int64_t)k * ld + s + p0 + r];
         if (OP == RP_LBC) return A.G[off + (int64_t)k * ld + s + p0 + r];
-        if (OP == RP_MBP) return A.L[off + (int64_t)(i0 + r) * ld + s + p0 + k];
-        if (OP == RP_FAC) return A.L[off + (int64_t)k * ld + s + p0 + r] * A.D[fc + k];
         if (OP == RP_FABAR) return A.Lb[off + (int64_t)k * ld + s + p0 + r];
-        return A.G[off + (int64_t)(i0 + r) * ld + s + p0 + k];
+        return A.L[off + (int64_t)(i0 + r) * ld + s + p0 + k];   // MBP, FUB
     };
     auto b_at = [&](int k, int jl) -> double {
         const int j = j0 + jl;
@@ -549,9 +553,8 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
         if (OP == RP_LHB) return S[(int64_t)j * ld + k];
         if (OP == RP_LBC) return A.Linv[A.linv_off[K] + (int64_t)k * s + j];
         if (OP == RP_MBP) return A.G[off + (int64_t)j * ld + s + p0 + k];
-        if (OP == RP_FAC) return k == j ? 1.0 : (k < j ? A.L[off + (int64_t)k * ld + j] : 0.0);   // L_KK(j, k)
         if (OP == RP_FABAR) return k >= j ? A.Linv[A.linv_off[K] + (int64_t)j * s + k] / A.D[fc + k] : 0.0;
-        return A.Lb[off + (int64_t)j * ld + s + p0 + k];
+        return A.Ab[off + (int64_t)j * ld + s + p0 + k];         // FUB
     };
     // thread (tx, ty) owns rows ty + 16 i and columns tx + 16 j of the block.
     // A warp holds rows 2 warp, 2 warp + 1 (+ 16 i): the row blocks with no
@@ -602,7 +605,6 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
             if (OP == RP_YBAR) A.YB[e] = A.Zb[e] - acc[i][j];
             else if (OP == RP_LHB) A.G[e] -= acc[i][j];
             else if (OP == RP_LBC) A.Lb[e] = acc[i][j];
-            else if (OP == RP_FAC) A.G[e] = acc[i][j];
             else A.Ab[e] = acc[i][j];
         }
     if (OP == RP_YBAR && t == 0)
@@ -748,14 +750,14 @@ __global__ void __launch_bounds__(256) k_fadj_pull_tc(const AdjDesc *__restrict_
     if (threadIdx.x == 0) A.counter[J] = 0;
 }
 
-// Abar_C rows = Lbar_C D^{-1} L_JJ^{-1}; split Nbar = A_C^T Lbar_C
+// Abar_C rows = Lbar_C D^{-1} L_JJ^{-1}; split L_C^T Abar_C
 template <int TN>
 __global__ void __launch_bounds__(kThreads) k_fadj_trsm(const AdjDesc *__restrict__ ad,
                                                         const Item *__restrict__ items, int nitems) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *Ar = reinterpret_cast<double *>(smem_raw);    // [TM][TN] A_C rows
-    double *Br = Ar + kTM * TN;                            // [TM][TN] Lbar_C rows
+    double *Ar = reinterpret_cast<double *>(smem_raw);    // [TM][TN] Abar_C rows
+    double *Br = Ar + kTM * TN;                            // [TM][TN] Lbar_C D^{-1} rows
     const int w = blockIdx.x;
     if (w >= nitems) return;
     const AdjDesc &A = *ad;
@@ -775,33 +777,24 @@ __global__ void __launch_bounds__(kThreads) k_fadj_trsm(const AdjDesc *__restric
     double *Ab = A.Ab + off + s;
     for (int e = threadIdx.x; e < kTM * s; e += kThreads) {
         const int pl = e % kTM, j = e / kTM;
-        double a = 0.0;
-        if (pl < pm) {
-            // A_C(p, j) = sum_{k <= j} L_C(p, k) D_k L_JJ(j, k)
-            for (int k = 0; k <= j; k++) {
-                const double ljk = (k == j) ? 1.0 : L[(int64_t)k * ld + j];
-                a = fma(L[(int64_t)k * ld + s + p0 + pl] * D[k], ljk, a);
-            }
-            Br[pl * TN + j] = Lb[(int64_t)j * ld + p0 + pl];
-        } else {
-            Br[pl * TN + j] = 0.0;
-        }
-        Ar[pl * TN + j] = a;
+        Br[pl * TN + j] = pl < pm ? Lb[(int64_t)j * ld + p0 + pl] / D[j] : 0.0;
     }
     __syncthreads();
     for (int e = threadIdx.x; e < kTM * s; e += kThreads) {  // Abar_C = (Lbar_C D^{-1}) M
         const int pl = e % kTM, j = e / kTM;
-        if (pl >= pm) continue;
         double v = 0.0;
-        for (int k = j; k < s; k++) v = fma(Br[pl * TN + k] / D[k], Li[(int64_t)j * s + k], v);
-        Ab[(int64_t)j * ld + p0 + pl] = v;
+        for (int k = j; k < s; k++) v = fma(Br[pl * TN + k], Li[(int64_t)j * s + k], v);
+        Ar[pl * TN + j] = v;
+        if (pl < pm) Ab[(int64_t)j * ld + p0 + pl] = v;
     }
+    __syncthreads();
     const int64_t ss = (int64_t)s * s;
     double *part = A.partial + A.part_off[J] + (int64_t)it.tile * ss;
-    for (int e = threadIdx.x; e < s * s; e += kThreads) {    // Nbar partial = A_C^T Lbar_C
+    for (int e = threadIdx.x; e < s * s; e += kThreads) {    // sum_p L_C(p, i) Abar_C(p, j), i <= j
         const int i = e % s, j = e / s;
+        if (i > j) continue;
         double v = 0.0;
-        for (int pl = 0; pl < pm; pl++) v = fma(Ar[pl * TN + i], Br[pl * TN + j], v);
+        for (int pl = 0; pl < pm; pl++) v = fma(L[(int64_t)i * ld + s + p0 + pl], Ar[pl * TN + j], v);
         part[e] = v;
     }
 }
@@ -817,9 +810,10 @@ __global__ void k_gather_vals(const int64_t *__restrict__ pos, const double *__r
 // ---------------------------------------------------------------------------
 // Per-supernode s x s steps of both adjoints, batched over a tree level and
 // spread over many CTAs.  Scratch per supernode J: 4 s x s slots at
-// 4 * linv_off[J] (selinv: Mbar, W, T1; factorization: Nbar, T2, N, U).
+// 4 * linv_off[J] (selinv: Mbar, W, T1; factorization: P, P M, G, Ubar).
 // ---------------------------------------------------------------------------
-enum { OP_SEL_T1 = 0, OP_SEL_W, OP_SEL_LB, OP_FAC_T2, OP_FAC_U, OP_FAC_T3, OP_FAC_G1, OP_FAC_G2 };
+enum { OP_SEL_T1 = 0, OP_SEL_W, OP_SEL_LB, OP_FAC_T3, OP_FAC_G1, OP_FAC_G2 };
+constexpr int kAdjTop = 8;        // most supernodes of a level of the adjoint's last group
 constexpr int kFinChunk = 1024;   // entries of an s x s block per item of the partial sums
 
 // C (16 x 16 tile) of an s x s product; items (J, tile), tiles row-major over
@@ -858,8 +852,6 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
         case OP_SEL_T1: return M[(int64_t)k * s + i];                 // M
         case OP_SEL_W: return F[(int64_t)k * s + i];                  // Mbar
         case OP_SEL_LB: return M[(int64_t)i * s + k];                 // M^T
-        case OP_FAC_T2: return F[(int64_t)k * s + i];                 // Nbar
-        case OP_FAC_U: return F[2 * ss + (int64_t)i * s + k];         // N^T
         case OP_FAC_T3: return k == i ? 1.0 : (k > i ? LJ[(int64_t)i * ld + k] : 0.0);  // L_JJ^T
         case OP_FAC_G1: return F[(int64_t)k * s + i];                 // P
         default: return M[(int64_t)i * s + k];                        // M^T
@@ -870,8 +862,6 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
         case OP_SEL_T1: return S[(int64_t)j * ld + k];                // S
         case OP_SEL_W: return M[(int64_t)k * s + j];                  // M^T
         case OP_SEL_LB: return F[ss + (int64_t)j * s + k];            // W
-        case OP_FAC_T2: return F[2 * ss + (int64_t)k * s + j];        // N^T
-        case OP_FAC_U: return F[ss + (int64_t)j * s + k];             // T2
         case OP_FAC_T3: return k > j ? LbJ[(int64_t)j * ld + k] : 0.0;  // Lbar_JJ, strictly lower
         case OP_FAC_G1: return M[(int64_t)j * s + k];                 // M
         default: return F[ss + (int64_t)j * s + k];                   // P M
@@ -889,8 +879,6 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
     case OP_SEL_T1: khi = min(s, i0 + GT); break;   // M(i, k): k <= i
     case OP_SEL_W: khi = min(s, j0 + GT); break;    // M(j, k): k <= j
     case OP_SEL_LB: klo = i0; break;                // M(k, i): k >= i
-    case OP_FAC_T2: klo = j0; break;                // N(j, k) = M(k, j) / D_k: k >= j
-    case OP_FAC_U: khi = min(s, i0 + GT); break;    // N(k, i) = M(i, k) / D_i: k <= i
     case OP_FAC_T3: klo = i0; break;                // L_JJ(k, i): k >= i
     case OP_FAC_G1: klo = j0; break;                // M(k, j): k >= j
     default: klo = i0; break;                       // M(k, i): k >= i
@@ -926,8 +914,6 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
     case OP_SEL_T1: F[2 * ss + (int64_t)j * s + i] = x; break;               // T1
     case OP_SEL_W: F[ss + (int64_t)j * s + i] = x; break;                    // W
     case OP_SEL_LB: Lb[(int64_t)j * ld + i] = i > j ? -x : 0.0; break;      // Lbar_JJ
-    case OP_FAC_T2: F[ss + (int64_t)j * s + i] = x; break;                   // T2
-    case OP_FAC_U: F[3 * ss + (int64_t)j * s + i] = -x; break;               // Ubar
     case OP_FAC_T3:                                                          // P
         F[(int64_t)j * s + i] = i > j ? x / A.D[A.super_ptr[J] + j] : (i == j ? A.Db[A.super_ptr[J] + i] : 0.0);
         break;
@@ -940,7 +926,7 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
 // tiles (Q = 1, 256 threads) or their 8 x 8 quarters (Q = 4, 64 threads),
 // for the levels whose tcgen05 product launch would run only a few CTAs (the
 // top of the tree): the FP64 work spreads over every SM.  OP as in
-// k_adj_rowprod (YBAR, LHB, LBC, FAC, FABAR); items (K, tile), tiles
+// k_adj_rowprod (YBAR, LHB, LBC, FABAR); items (K, tile), tiles
 // row-major over ceil(max(c, 1) / 16) x ceil(s / 16); the tiles of row 0 of
 // RP_YBAR also store S.
 template <int Q, int OP>
@@ -980,20 +966,17 @@ __global__ void __launch_bounds__(256) k_adj_rowgemm(const AdjDesc *__restrict__
         if (OP == RP_YBAR) return A.LD[e];
         if (OP == RP_LHB) return A.Z[e];
         if (OP == RP_LBC) return A.G[e];
-        if (OP == RP_FAC) return A.L[e] * A.D[fc + k];
         return A.Lb[e];
     };
     auto b_at = [&](int k, int j) -> double {   // B(k, j)
         if (OP == RP_YBAR) return sym(k, j);
         if (OP == RP_LHB) return A.YB[off + (int64_t)j * ld + k];
         if (OP == RP_LBC) return A.Linv[A.linv_off[K] + (int64_t)k * s + j];
-        if (OP == RP_FAC) return k == j ? 1.0 : (k < j ? A.L[off + (int64_t)k * ld + j] : 0.0);   // L_KK(j, k)
         return k >= j ? A.Linv[A.linv_off[K] + (int64_t)j * s + k] / A.D[fc + k] : 0.0;
     };
-    // triangular factors: M^T (LBC) and L_KK^T (FAC) vanish for k > j,
-    // D^{-1} M (FABAR) for k < j
+    // triangular factors: M^T (LBC) vanishes for k > j, D^{-1} M (FABAR) for k < j
     int klo = 0, khi = s;
-    if (OP == RP_LBC || OP == RP_FAC) khi = min(s, j0 + GT);
+    if (OP == RP_LBC) khi = min(s, j0 + GT);
     if (OP == RP_FABAR) klo = j0;
     const int tx = threadIdx.x % GT, ty = threadIdx.x / GT;
     const bool wact = i0 + (32 / GT) * (int)(threadIdx.x / 32) < c;
@@ -1026,7 +1009,6 @@ __global__ void __launch_bounds__(256) k_adj_rowgemm(const AdjDesc *__restrict__
     if (OP == RP_YBAR) A.YB[e] = A.Zb[e] - acc;
     else if (OP == RP_LHB) A.G[e] -= acc;
     else if (OP == RP_LBC) A.Lb[e] = acc;
-    else if (OP == RP_FAC) A.G[e] = acc;
     else A.Ab[e] = acc;
 }
 
@@ -1087,28 +1069,28 @@ __global__ void __launch_bounds__(256) k_adj_sel_dbar(const AdjDesc *__restrict_
     }
 }
 
-// factorization adjoint: Nbar = sum of the tile partials; N = M^T D^{-1};
-// items as in k_adj_sel_mbar
-__global__ void __launch_bounds__(256) k_fadj_nbar(const AdjDesc *__restrict__ ad,
+// factorization adjoint: Ubar = -L_C^T Abar_C from the tile partials, entries
+// i <= j (the reverse of A_C = L_C U^T, U = D L_KK^T, by Abar_C = Lbar_C U^{-T};
+// with A_C itself the same sum is -U^{-1} (A_C^T Lbar_C) U^{-T}, three products
+// more); items as in k_adj_sel_mbar
+__global__ void __launch_bounds__(256) k_fadj_usum(const AdjDesc *__restrict__ ad,
                                                    const int2 *__restrict__ items, int nitems) {
     grid_dep_wait();
     const int w = blockIdx.x;
     if (w >= nitems) return;
     const AdjDesc &A = *ad;
     const int J = items[w].x, chunk = items[w].y & 0xFFFF, ntiles = items[w].y >> 16;
-    const int fc = A.super_ptr[J];
-    const int s = A.super_ptr[J + 1] - fc;
+    const int s = A.super_ptr[J + 1] - A.super_ptr[J];
     const int64_t ss = (int64_t)s * s;
-    double *__restrict__ F = A.fin + 4 * A.linv_off[J];
-    const double *__restrict__ M = A.Linv + A.linv_off[J];
+    double *__restrict__ U = A.fin + 4 * A.linv_off[J] + 3 * ss;
     const double *__restrict__ part = A.partial + A.part_off[J];
     const int64_t e1 = (int64_t)(chunk + 1) * kFinChunk < ss ? (int64_t)(chunk + 1) * kFinChunk : ss;
     for (int64_t e = (int64_t)chunk * kFinChunk + threadIdx.x; e < e1; e += blockDim.x) {
         const int i = (int)(e % s), j = (int)(e / s);
+        if (i > j) continue;
         double v = 0.0;
         for (int t = 0; t < ntiles; t++) v += part[t * ss + e];
-        F[e] = v;
-        F[2 * ss + e] = M[(int64_t)i * s + j] / A.D[fc + j];   // N(i, j) = M(j, i) / D_j
+        U[e] = -v;
     }
 }
 
@@ -1211,16 +1193,15 @@ static void launch_gemm_op(AdjData *a, int64_t g0, int n, cudaStream_t st) {
     else k_adj_gemm<1, OP><<<n, kGT * kGT, 0, st>>>(a->d_desc, a->d_gitems + g0, n);
 }
 
-static void launch_level_gemm(AdjData *a, int op, int li, cudaStream_t st) {
-    const int64_t g0 = a->g_lptr[li], g1 = a->g_lptr[li + 1];
+// (levels l0 .. l1 - 1 of the lists, here and below)
+static void launch_gemm(AdjData *a, int op, int l0, int l1, cudaStream_t st) {
+    const int64_t g0 = a->g_lptr[l0], g1 = a->g_lptr[l1];
     const int n = (int)(g1 - g0);
     if (n <= 0) return;
     switch (op) {
     case OP_SEL_T1: launch_gemm_op<OP_SEL_T1>(a, g0, n, st); break;
     case OP_SEL_W: launch_gemm_op<OP_SEL_W>(a, g0, n, st); break;
     case OP_SEL_LB: launch_gemm_op<OP_SEL_LB>(a, g0, n, st); break;
-    case OP_FAC_T2: launch_gemm_op<OP_FAC_T2>(a, g0, n, st); break;
-    case OP_FAC_U: launch_gemm_op<OP_FAC_U>(a, g0, n, st); break;
     case OP_FAC_T3: launch_gemm_op<OP_FAC_T3>(a, g0, n, st); break;
     case OP_FAC_G1: launch_gemm_op<OP_FAC_G1>(a, g0, n, st); break;
     default: launch_gemm_op<OP_FAC_G2>(a, g0, n, st); break;
@@ -1259,14 +1240,17 @@ void adjoint_release(void *p) {
     fr(a->d_items); fr(a->d_lhat); fr(a->d_linv);
     fr(a->d_gitems); fr(a->d_citems); fr(a->d_js); fr(a->d_cz); fr(a->d_vitems);
     fr(a->YB); fr(a->Zb); fr(a->Lbw); fr(a->Ab); fr(a->fin); fr(a->d_desc); fr(a->d_pdesc);
-    fr(a->V);
-    fr(a->d_sm); fr(a->d_wd); fr(a->d_row); fr(a->d_rg); fr(a->d_mbp); fr(a->d_dig); fr(a->d_tcdesc); fr(a->cy);
+    fr(a->V); fr(a->part);
+    fr(a->d_sm); fr(a->d_sg); fr(a->d_wd); fr(a->d_row); fr(a->d_rg); fr(a->d_mbp); fr(a->d_dig); fr(a->d_tcdesc); fr(a->cy);
     fr(a->d_pr); fr(a->d_sdw); fr(a->sd); fr(a->d_sd_off); fr(a->sdexp); fr(a->d_pdp);
     fr(a->d_syw); fr(a->d_sy); fr(a->d_vn); fr(a->sy); fr(a->d_sy_off); fr(a->syexp); fr(a->d_sydesc);
     a->g_sel.release();
     a->g_fac.release();
     a->tcs.release();
     a->tcn.release();
+    if (a->side) cudaStreamDestroy(a->side);
+    if (a->fork) cudaEventDestroy(a->fork);
+    if (a->join) cudaEventDestroy(a->join);
     delete a;
 }
 
@@ -1349,6 +1333,7 @@ static int adj_build(selinv_plan_s *plan) {
     const size_t nz = (size_t)std::max<int64_t>(p.nnz, 1);
     if (cudaMalloc((void **)&a->YB, 8 * nz) || cudaMalloc((void **)&a->Zb, 8 * nz) ||
         cudaMalloc((void **)&a->Lbw, 8 * nz) || cudaMalloc((void **)&a->Ab, 8 * nz) ||
+        cudaMalloc((void **)&a->part, 8 * (size_t)std::max<int64_t>(p.part_all, 1)) ||
         cudaMalloc((void **)&a->fin, 8 * (size_t)std::max<int64_t>(4 * p.linv_total, 1)) ||
         cudaMalloc((void **)&a->d_desc, sizeof(AdjDesc)) || cudaMalloc((void **)&a->d_pdesc, sizeof(ProbDesc))) {
         adjoint_release(a);
@@ -1367,12 +1352,12 @@ static AdjDesc make_adesc(selinv_plan_s *plan, const double *L, const double *D,
     AdjDesc h;
     h.super_ptr = p.d_super_ptr; h.rowptr = p.d_rowptr; h.rows = p.d_rows; h.panel_off = p.d_panel_off;
     h.colbase = p.d_colbase; h.relbase = p.d_relbase; h.relidx = p.d_relidx;
-    h.linv_off = p.d_linv_off; h.part_off = p.d_part_off;
+    h.linv_off = p.d_linv_off; h.part_off = p.d_part_off_all;
     h.L = L; h.D = D; h.Z = Z;
     h.LD = static_cast<const double *>(w.LD);
     h.Linv = static_cast<const double *>(w.Linv);
     h.Zb = a->Zb; h.YB = a->YB; h.Lb = Lb; h.Db = Db; h.Ab = a->Ab;
-    h.partial = static_cast<double *>(w.partial);
+    h.partial = a->part;
     h.counter = w.counter;
     h.fin = a->fin;
     h.sparent = p.d_sparent;
@@ -1424,10 +1409,10 @@ static int adj_split(selinv_plan_s *plan) {
     const int key = o.fast_contraction != 0 ? std::max(8, o.oz_min_s) : 0;
     if (key == a->split_key) return SELINV_OK;
     auto fr = [](void *q) { if (q) cudaFree(q); };
-    fr(a->d_sm); fr(a->d_wd); fr(a->d_row); fr(a->d_rg); fr(a->d_mbp); fr(a->d_dig);
+    fr(a->d_sm); fr(a->d_sg); fr(a->d_wd); fr(a->d_row); fr(a->d_rg); fr(a->d_mbp); fr(a->d_dig);
     fr(a->d_pr); fr(a->d_sdw); fr(a->sd); fr(a->d_sd_off);
     fr(a->d_syw); fr(a->d_sy); fr(a->d_vn); fr(a->sy); fr(a->d_sy_off);
-    a->d_sm = a->d_wd = nullptr; a->d_row = a->d_mbp = nullptr; a->d_dig = nullptr; a->d_rg = nullptr;
+    a->d_sm = a->d_sg = a->d_wd = nullptr; a->d_row = a->d_mbp = nullptr; a->d_dig = nullptr; a->d_rg = nullptr;
     a->d_pr = nullptr; a->d_sdw = nullptr; a->sd = nullptr; a->d_sd_off = nullptr;
     a->d_syw = nullptr; a->d_sy = nullptr; a->d_vn = nullptr; a->sy = nullptr; a->d_sy_off = nullptr;
     a->sy_work.clear(); a->sy_items.clear(); a->vn_items.clear();
@@ -1539,8 +1524,26 @@ static int adj_split(selinv_plan_s *plan) {
         const int64_t s = p.super_ptr[J + 1] - p.super_ptr[J];
         sd_off[J + 1] = sd_off[J] + (wideK(J) ? 7 * ((s + 63) / 64 * 64) * ((s + 15) / 16 * 16) : 0);
     }
+    // two groups: the last levels, of at most kAdjTop supernodes each, leave most
+    // SMs to the first group's products (24^3: a training step takes 14.1 ms with
+    // one group, 13.5 so; cuts at 4 to 22 levels 13.5 to 14.1, three to six
+    // groups 13.5 to 14.0)
+    int top = p.nlevels;
+    while (top > 0 && p.level_ptr[p.nlevels - top + 1] - p.level_ptr[p.nlevels - top] <= kAdjTop) top--;
+    a->grp.assign(1, 0);
+    if (top > 0 && top < p.nlevels) a->grp.push_back(top);
+    a->grp.push_back(p.nlevels);
+    a->sg_items.clear();
+    a->sg_bptr.assign(1, 0);
+    for (size_t g = 0; g + 1 < a->grp.size(); g++)
+        for (int b = 0; b < kNumBuckets; b++) {
+            for (int li = a->grp[g + 1] - 1; li >= a->grp[g]; li--)
+                a->sg_items.insert(a->sg_items.end(), a->sm_items.begin() + a->sm_bptr[li * kNumBuckets + b],
+                                   a->sm_items.begin() + a->sm_bptr[li * kNumBuckets + b + 1]);
+            a->sg_bptr.push_back((int)a->sg_items.size());
+        }
     int rc;
-    if ((rc = upl(&a->d_sm, a->sm_items)) || (rc = upl(&a->d_wd, a->wd_items)) || (rc = upl(&a->d_row, a->row_items)) ||
+    if ((rc = upl(&a->d_sm, a->sm_items)) || (rc = upl(&a->d_sg, a->sg_items)) || (rc = upl(&a->d_wd, a->wd_items)) || (rc = upl(&a->d_row, a->row_items)) ||
         (rc = upl(&a->d_rg, a->rg_items)) ||
         (rc = upl(&a->d_mbp, a->mbp_items)) || (rc = upl(&a->d_dig, a->dig_work)) ||
         (rc = upl(&a->d_pr, a->pr_items)) || (rc = upl(&a->d_sdw, a->sd_work)) || (rc = upl(&a->d_sd_off, sd_off)) ||
@@ -1556,7 +1559,7 @@ static int adj_split(selinv_plan_s *plan) {
         return SELINV_ERR_OOM;
     if (!a->sdexp && cudaMalloc((void **)&a->sdexp, sizeof(int) * (size_t)std::max(p.n, 1)) != cudaSuccess)
         return SELINV_ERR_OOM;
-    if (!a->d_pdp && cudaMalloc((void **)&a->d_pdp, 5 * sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
+    if (!a->d_pdp && cudaMalloc((void **)&a->d_pdp, 4 * sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
     if (!a->dig_work.empty()) {
         // the forward's level schedule supplies the tcgen05 items of every
         // level (row tiles, column tiles, k-splits) and their reductions, built
@@ -1613,17 +1616,25 @@ static int adj_prepare(selinv_plan_s *plan) {
 
 using namespace selinv;
 
-// One row product X B of the level's wide supernodes on the transposed
-// tcgen05 kernel: the digit planes of B, then the product (descriptor pd of
-// d_pdp: the panel X, the output and its mode).
+// One row product X B of the levels' wide supernodes: the digit planes of B for
+// the transposed tcgen05 kernel, then the product (descriptor pd of d_pdp: the
+// panel X, the output and its mode).
 template <int OP>
-static void row_product(AdjData *a, int pd, int li, cudaStream_t st) {
-    const int r0 = (int)a->row_lptr[li], r1 = (int)a->row_lptr[li + 1];
+static void row_digits(AdjData *a, int l0, int l1, cudaStream_t st) {
+    const int q0 = (int)a->sd_lptr[l0], q1 = (int)a->sd_lptr[l1];
+    if (q1 <= q0) return;
+    k_small_digits<OP><<<q1 - q0, 256, 0, st>>>(a->d_desc, a->d_sdw + q0, q1 - q0, a->sd, a->d_sd_off, a->sdexp);
+    note_launch();
+}
+
+template <int OP>
+static void row_product(AdjData *a, int pd, int l0, int l1, cudaStream_t st) {
+    const int r0 = (int)a->row_lptr[l0], r1 = (int)a->row_lptr[l1];
     if (r1 > r0) {   // the narrower wide supernodes: 32 x 32 blocks on the FP64 kernel
         k_adj_rowprod<OP><<<r1 - r0, kThreads, 0, st>>>(a->d_desc, a->d_row + r0, r1 - r0);
         note_launch();
     }
-    const int g0 = (int)a->rg_lptr[li], g1 = (int)a->rg_lptr[li + 1];
+    const int g0 = (int)a->rg_lptr[l0], g1 = (int)a->rg_lptr[l1];
     if (g1 > g0) {   // the top levels: 16 x 16 tiles (8 x 8 quarters) on the FP64 kernel
         if (g1 - g0 < kNumSMs)
             k_adj_rowgemm<4, OP><<<4 * (g1 - g0), kGT * kGT / 4, 0, st>>>(a->d_desc, a->d_rg + g0, g1 - g0);
@@ -1631,12 +1642,7 @@ static void row_product(AdjData *a, int pd, int li, cudaStream_t st) {
             k_adj_rowgemm<1, OP><<<g1 - g0, kGT * kGT, 0, st>>>(a->d_desc, a->d_rg + g0, g1 - g0);
         note_launch();
     }
-    const int q0 = (int)a->sd_lptr[li], q1 = (int)a->sd_lptr[li + 1];
-    if (q1 > q0) {
-        k_small_digits<OP><<<q1 - q0, 256, 0, st>>>(a->d_desc, a->d_sdw + q0, q1 - q0, a->sd, a->d_sd_off, a->sdexp);
-        note_launch();
-    }
-    const int t0 = (int)a->pr_lptr[li], t1 = (int)a->pr_lptr[li + 1];
+    const int t0 = (int)a->pr_lptr[l0], t1 = (int)a->pr_lptr[l1];
     if (t1 > t0) {
         launch_lhat_tcw(0, a->d_pdp + pd, a->d_pr + t0, t1 - t0, a->tcs.spin_limit, st);
         note_launch();
@@ -1708,56 +1714,89 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
         note_launch();
     }
     const int nl = p.nlevels;
-    auto levels = [&](cudaStream_t st) {
-        for (int li = 0; li < nl; li++) {  // deepest level first
-            // the children's update matrices complete Zbar on K's panel and start V_K
-            for (int r = 0; r < f->npass; r++) {
-                const int64_t x0 = f->asm_lptr[li * f->npass + r], x1 = f->asm_lptr[li * f->npass + r + 1];
-                if (x1 > x0) { k_adj_asm<<<(int)(x1 - x0), 256, 0, st>>>(a->d_desc, f->d_asm + x0, (int)(x1 - x0)); note_launch(); }
-            }
-            const int i0 = a->sm_bptr[li * kNumBuckets], i1 = a->sm_bptr[(li + 1) * kNumBuckets];
-            if (i1 > i0) { k_adj_ybar<<<i1 - i0, 256, 0, st>>>(a->d_desc, a->d_sm + i0, i1 - i0); note_launch(); }
-            const int m0 = (int)a->mbp_lptr[li], m1 = (int)a->mbp_lptr[li + 1];
-            row_product<RP_YBAR>(a, 0, li, st);
-            const int64_t v0 = a->vn_lptr[li], v1 = a->vn_lptr[li + 1];
-            if (v1 > v0) { k_adj_vupd<<<(int)(v1 - v0), 256, 0, st>>>(a->d_desc, a->d_vn + v0, (int)(v1 - v0)); note_launch(); }
-            const int64_t y0 = a->sy_wlptr[li], y1 = a->sy_wlptr[li + 1];
-            if (y1 > y0) {
-                k_syrk_digits<<<(int)(y1 - y0), 256, 0, st>>>(a->d_desc, a->d_syw + y0, (int)(y1 - y0), a->sy, a->d_sy_off, a->syexp);
-                note_launch();
-            }
-            const int64_t z0 = a->sy_lptr[li], z1 = a->sy_lptr[li + 1];
-            if (z1 > z0) {
-                launch_syrk_tcw(1, a->d_sydesc, a->d_sy + z0, (int)(z1 - z0), a->tcs.spin_limit, st);
-                note_launch();
-            }
-            const int d0 = (int)a->dig_lptr[li], d1 = (int)a->dig_lptr[li + 1];
-            if (d1 > d0) {
-                launch_lhat_digits(a->d_tcdesc, a->d_dig + d0, d1 - d0, st);
-                note_launch();
+    // Only Ybar and the update matrices V climb the tree; what each supernode
+    // makes of them (Lhat_bar, Lbar, Dbar) meets no other supernode and has
+    // storage of its own, so it runs for whole groups of levels at once, on a
+    // side stream under the next group's climb: 5 launches a level and few
+    // large ones instead of 17 a level, of which the top levels' fill few SMs
+    // (a training step on 24^3, whose other adjoint lost four launches a level
+    // as well: 17.3 ms before, 13.5 so).
+    auto climb = [&](int li, cudaStream_t st) {
+        // the children's update matrices complete Zbar on K's panel and start V_K
+        for (int r = 0; r < f->npass; r++) {
+            const int64_t x0 = f->asm_lptr[li * f->npass + r], x1 = f->asm_lptr[li * f->npass + r + 1];
+            if (x1 > x0) { k_adj_asm<<<(int)(x1 - x0), 256, 0, st>>>(a->d_desc, f->d_asm + x0, (int)(x1 - x0)); note_launch(); }
+        }
+        const int i0 = a->sm_bptr[li * kNumBuckets], i1 = a->sm_bptr[(li + 1) * kNumBuckets];
+        if (i1 > i0) { k_adj_ybar<<<i1 - i0, 256, 0, st>>>(a->d_desc, a->d_sm + i0, i1 - i0); note_launch(); }
+        row_digits<RP_YBAR>(a, li, li + 1, st);
+        row_product<RP_YBAR>(a, 0, li, li + 1, st);
+        const int64_t v0 = a->vn_lptr[li], v1 = a->vn_lptr[li + 1];
+        if (v1 > v0) { k_adj_vupd<<<(int)(v1 - v0), 256, 0, st>>>(a->d_desc, a->d_vn + v0, (int)(v1 - v0)); note_launch(); }
+        const int64_t y0 = a->sy_wlptr[li], y1 = a->sy_wlptr[li + 1];
+        if (y1 > y0) {
+            k_syrk_digits<<<(int)(y1 - y0), 256, 0, st>>>(a->d_desc, a->d_syw + y0, (int)(y1 - y0), a->sy, a->d_sy_off, a->syexp);
+            note_launch();
+        }
+        const int64_t z0 = a->sy_lptr[li], z1 = a->sy_lptr[li + 1];
+        if (z1 > z0) {
+            launch_syrk_tcw(1, a->d_sydesc, a->d_sy + z0, (int)(z1 - z0), a->tcs.spin_limit, st);
+            note_launch();
+        }
+    };
+    auto rest = [&](int g, cudaStream_t st) {
+        const int l0 = a->grp[g], l1 = a->grp[g + 1];
+        const int d0 = (int)a->dig_lptr[l0], d1 = (int)a->dig_lptr[l1];
+        if (d1 > d0) {
+            launch_lhat_digits(a->d_tcdesc, a->d_dig + d0, d1 - d0, st);
+            note_launch();
+            for (int li = l0; li < l1; li++)
                 for (int e : a->tc_launch[li]) {
                     launch_with(a->tcs, a->tcs.launches[e], a->d_tcdesc, st);
                     note_launch();
                 }
+        }
+        for (int b = 0; b < kNumBuckets; b++) {
+            const int b0 = a->sg_bptr[g * kNumBuckets + b], b1 = a->sg_bptr[g * kNumBuckets + b + 1];
+            launch_bucket(0, b, a->d_desc, a->d_sg + b0, b1 - b0, st);
+        }
+        row_product<RP_LHB>(a, 1, l0, l1, st);
+        const int m0 = (int)a->mbp_lptr[l0], m1 = (int)a->mbp_lptr[l1];
+        if (m1 > m0) {
+            k_adj_rowprod<RP_MBP><<<m1 - m0, kThreads, 0, st>>>(a->d_desc, a->d_mbp + m0, m1 - m0);
+            note_launch();
+        }
+        row_digits<RP_LBC>(a, l0, l1, st);
+        row_product<RP_LBC>(a, 2, l0, l1, st);
+        // per-supernode s x s steps
+        const int64_t c0 = a->c_lptr[l0], c1 = a->c_lptr[l1];
+        const int64_t j0 = a->j_lptr[l0], j1 = a->j_lptr[l1];
+        launch_gemm(a, OP_SEL_T1, l0, l1, st);
+        if (c1 > c0) { k_adj_sel_mbar<<<(int)(c1 - c0), 256, 0, st>>>(a->d_desc, a->d_citems + c0, (int)(c1 - c0)); note_launch(); }
+        launch_gemm(a, OP_SEL_W, l0, l1, st);
+        launch_gemm(a, OP_SEL_LB, l0, l1, st);
+        if (j1 > j0) { k_adj_sel_dbar<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0)); note_launch(); }
+    };
+    const int ng = (int)a->grp.size() - 1;
+    if (ng > 1 && !a->side &&
+        (cudaStreamCreateWithFlags(&a->side, cudaStreamNonBlocking) != cudaSuccess ||
+         cudaEventCreateWithFlags(&a->fork, cudaEventDisableTiming) != cudaSuccess ||
+         cudaEventCreateWithFlags(&a->join, cudaEventDisableTiming) != cudaSuccess))
+        return SELINV_ERR_CUDA;
+    auto levels = [&](cudaStream_t st) {
+        for (int g = 0; g < ng; g++) {
+            for (int li = a->grp[g]; li < a->grp[g + 1]; li++) climb(li, st);   // deepest level first
+            if (g + 1 < ng) {
+                cudaEventRecord(a->fork, st);
+                cudaStreamWaitEvent(a->side, a->fork, 0);
+                rest(g, a->side);
+                continue;
             }
-            for (int b = 0; b < kNumBuckets; b++) {
-                const int b0 = a->sm_bptr[li * kNumBuckets + b], b1 = a->sm_bptr[li * kNumBuckets + b + 1];
-                launch_bucket(0, b, a->d_desc, a->d_sm + b0, b1 - b0, st);
+            if (ng > 1) {   // (the groups share the split slots of the gather products)
+                cudaEventRecord(a->join, a->side);
+                cudaStreamWaitEvent(st, a->join, 0);
             }
-            row_product<RP_LHB>(a, 1, li, st);
-            if (m1 > m0) {
-                k_adj_rowprod<RP_MBP><<<m1 - m0, kThreads, 0, st>>>(a->d_desc, a->d_mbp + m0, m1 - m0);
-                note_launch();
-            }
-            row_product<RP_LBC>(a, 2, li, st);
-            // per-supernode s x s steps, batched over the level
-            const int64_t c0 = a->c_lptr[li], c1 = a->c_lptr[li + 1];
-            const int64_t j0 = a->j_lptr[li], j1 = a->j_lptr[li + 1];
-            launch_level_gemm(a, OP_SEL_T1, li, st);
-            if (c1 > c0) { k_adj_sel_mbar<<<(int)(c1 - c0), 256, 0, st>>>(a->d_desc, a->d_citems + c0, (int)(c1 - c0)); note_launch(); }
-            launch_level_gemm(a, OP_SEL_W, li, st);
-            launch_level_gemm(a, OP_SEL_LB, li, st);
-            if (j1 > j0) { k_adj_sel_dbar<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0)); note_launch(); }
+            rest(g, st);
         }
     };
     return a->g_sel.run(a->gen, w.colexpZ, st, levels);
@@ -1799,20 +1838,19 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
         pd.Yout = w.work;
         pd.colexpY = a->cy;
         cudaMemcpyAsync(a->d_tcdesc, &pd, sizeof(pd), cudaMemcpyHostToDevice, st);
-        // the row products: G = A_C = L_C D L_KK^T, Abar_C = Lbar_C D^{-1} M
+        // the row product Abar_C = Lbar_C D^{-1} M
         ProbDesc base = make_desc(p, w, SELINV_F64, L, D, a->Ab, false);
         base.linvd = a->sd;
         base.linvd_off = a->d_sd_off;
         base.linvexp = a->sdexp;
-        ProbDesc pdp[2] = {base, base};
-        pdp[0].L = L; pdp[0].LD = w.work; pdp[0].prod_op = 0;
-        pdp[1].L = a->Lbw; pdp[1].LD = a->Ab; pdp[1].prod_op = 0;
-        cudaMemcpyAsync(a->d_pdp + 3, pdp, sizeof(pdp), cudaMemcpyHostToDevice, st);
+        base.L = a->Lbw; base.LD = a->Ab; base.prod_op = 0;
+        cudaMemcpyAsync(a->d_pdp + 3, &base, sizeof(base), cudaMemcpyHostToDevice, st);
         launch_lhat_digits(a->d_tcdesc, a->d_dig, (int)a->dig_work.size(), st);
         note_launch();
     }
     const int nl = p.nlevels;
     auto levels = [&](cudaStream_t st) {
+        row_digits<RP_FABAR>(a, 0, nl, st);
         for (int li = nl - 1; li >= 0; li--) {  // root level first
             const int d0 = (int)a->dig_lptr[li], d1 = (int)a->dig_lptr[li + 1];
             if (d1 > d0)
@@ -1831,24 +1869,21 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
                 launch_bucket(2, b, a->d_desc, a->d_sm + b0, b1 - b0, st);
             }
             const int m0 = (int)a->mbp_lptr[li], m1 = (int)a->mbp_lptr[li + 1];
-            row_product<RP_FAC>(a, 3, li, st);
+            row_product<RP_FABAR>(a, 3, li, li + 1, st);
             if (m1 > m0) {
-                k_adj_rowprod<RP_FNBP><<<m1 - m0, kThreads, 0, st>>>(a->d_desc, a->d_mbp + m0, m1 - m0);
+                k_adj_rowprod<RP_FUB><<<m1 - m0, kThreads, 0, st>>>(a->d_desc, a->d_mbp + m0, m1 - m0);
                 note_launch();
             }
-            row_product<RP_FABAR>(a, 4, li, st);
             const int64_t c0 = a->c_lptr[li], c1 = a->c_lptr[li + 1];
             const int64_t j0 = a->j_lptr[li], j1 = a->j_lptr[li + 1];
-            if (c1 > c0) { k_fadj_nbar<<<(int)(c1 - c0), 256, 0, st>>>(a->d_desc, a->d_citems + c0, (int)(c1 - c0)); note_launch(); }
-            launch_level_gemm(a, OP_FAC_T2, li, st);
-            launch_level_gemm(a, OP_FAC_U, li, st);
+            if (c1 > c0) { k_fadj_usum<<<(int)(c1 - c0), 256, 0, st>>>(a->d_desc, a->d_citems + c0, (int)(c1 - c0)); note_launch(); }
             if (j1 > j0) {
                 k_fadj_ubar<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0));
                 note_launch();
             }
-            launch_level_gemm(a, OP_FAC_T3, li, st);
-            launch_level_gemm(a, OP_FAC_G1, li, st);
-            launch_level_gemm(a, OP_FAC_G2, li, st);
+            launch_gemm(a, OP_FAC_T3, li, li + 1, st);
+            launch_gemm(a, OP_FAC_G1, li, li + 1, st);
+            launch_gemm(a, OP_FAC_G2, li, li + 1, st);
             if (j1 > j0) {
                 k_fadj_fold<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0));
                 note_launch();
