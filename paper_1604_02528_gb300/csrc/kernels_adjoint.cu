@@ -71,6 +71,7 @@ struct AdjDesc {
     const int64_t *v_off;   // update matrix of K: c x c column-major at V + v_off[K]
     const int32_t *chpos;   // row-list position p of C_K[q]: its position in rows(parent(K))
     double *V;              // update matrices: the part of Zbar(C,C) not yet handed to an owner
+    int *colexp;            // factorization adjoint: largest biased exponent of each column of Abar (null: not wanted)
     double *G;              // panels: -A^{-1}(C,C) Ybar, then Lhat_bar (supernodes on the split path)
 };
 
@@ -84,8 +85,7 @@ struct AdjData {
     std::vector<int> lhat_bptr;
     std::vector<int2> gitems, citems;  // per level: (J, 16x16 tile) and (J, chunk | ntiles << 16)
     std::vector<int> js;               // per level: supernodes
-    std::vector<int2> cz_work;         // per level: (J, 8-column block)
-    std::vector<int64_t> cz_lptr;
+    std::vector<int2> cz_work;         // (J, 8-column block)
     int2 *d_cz = nullptr;
     std::vector<int4> vitems;          // per level: (J, 32-row tile, 32-column tile) of the lower c x c
     std::vector<int64_t> v_lptr;
@@ -517,6 +517,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
     constexpr int BM = 32;                  // rows of the output block
     constexpr int MI = BM / 16;
     __shared__ double As[kTK * BM], Bs[kTK * 32];
+    __shared__ int cmax[32];   // RP_FUB, row block 0: largest exponent of each column of the tile's Abar_C
     const int w = blockIdx.x;
     if (w >= nitems) return;
     const AdjDesc &A = *ad;
@@ -567,6 +568,8 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
     double acc[MI][2];
 #pragma unroll
     for (int i = 0; i < MI; i++) acc[i][0] = acc[i][1] = 0.0;
+    const bool cexp = OP == RP_FUB && i0 == 0 && A.colexp;
+    if (cexp && threadIdx.x < 32) cmax[threadIdx.x] = 0;
     for (int k0 = 0; k0 < kdim; k0 += kTK) {
         __syncthreads();
         for (int e = threadIdx.x; e < kTK * BM; e += kThreads) {
@@ -575,7 +578,9 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
         }
         for (int e = threadIdx.x; e < kTK * 32; e += kThreads) {
             const int kk = e % kTK, jl = e / kTK, k = k0 + kk;
-            Bs[kk * 32 + jl] = (k < kdim && jl < nj) ? b_at(k, jl) : 0.0;
+            const double b = (k < kdim && jl < nj) ? b_at(k, jl) : 0.0;
+            Bs[kk * 32 + jl] = b;
+            if (cexp) atomicMax(&cmax[jl], bexp(b));
         }
         __syncthreads();
         switch (sel) {
@@ -607,6 +612,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_rowprod(const AdjDesc *__restr
             else if (OP == RP_LBC) A.Lb[e] = acc[i][j];
             else A.Ab[e] = acc[i][j];
         }
+    if (cexp && kdim > 0 && (int)threadIdx.x < nj) atomicMax(&A.colexp[fc + j0 + threadIdx.x], cmax[threadIdx.x]);
     if (OP == RP_YBAR && t == 0)
         for (int e = threadIdx.x; e < s * nj; e += kThreads) {
             const int k = e % s, j = j0 + e / s;
@@ -693,7 +699,10 @@ __global__ void __launch_bounds__(kThreads) k_fadj_pull(const AdjDesc *__restric
 
 // k_fadj_pull for a wide supernode whose gather-GEMM ran on the tensor
 // cores: G = -Abar(C,C) L_C with every gathered entry counted once, so the
-// doubled diagonal adds Abar(C[p], C[p]) L_C(p, :) here.  A warp per column.
+// doubled diagonal adds Abar(C[p], C[p]) L_C(p, :) here.  A warp per column,
+// grid (tiles, kPullY): a tile's columns one after the other on 8 warps were
+// a chain of loads (38 us at 128 columns).
+constexpr int kPullY = 4;
 __global__ void __launch_bounds__(256) k_fadj_pull_tc(const AdjDesc *__restrict__ ad,
                                                       const Item *__restrict__ items, int nitems) {
     grid_dep_wait();
@@ -723,7 +732,7 @@ __global__ void __launch_bounds__(256) k_fadj_pull_tc(const AdjDesc *__restrict_
     double *Lb = A.Lb + off + s;
     double *part = A.partial + A.part_off[J] + (int64_t)it.tile * s * s;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int k = warp; k < s; k += 8) {
+    for (int k = blockIdx.y * 8 + warp; k < s; k += 8 * kPullY) {
         double v = 0.0;
         for (int pl = lane; pl < pm; pl += 32) {
             const int64_t e = (int64_t)k * ld + p0 + pl;
@@ -737,7 +746,7 @@ __global__ void __launch_bounds__(256) k_fadj_pull_tc(const AdjDesc *__restrict_
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(&A.counter[J], 1) == it.ntiles - 1);
+    if (threadIdx.x == 0) s_last = (atomicAdd(&A.counter[J], 1) == it.ntiles * kPullY - 1);
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -786,6 +795,12 @@ __global__ void __launch_bounds__(kThreads) k_fadj_trsm(const AdjDesc *__restric
         for (int k = j; k < s; k++) v = fma(Br[pl * TN + k], Li[(int64_t)j * s + k], v);
         Ar[pl * TN + j] = v;
         if (pl < pm) Ab[(int64_t)j * ld + p0 + pl] = v;
+        if (A.colexp) {   // (a warp holds one column)
+            int x = pl < pm ? bexp(v) : 0;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+            if (threadIdx.x % 32 == 0) atomicMax(&A.colexp[fc + j], x);
+        }
     }
     __syncthreads();
     const int64_t ss = (int64_t)s * s;
@@ -812,6 +827,16 @@ __global__ void k_gather_vals(const int64_t *__restrict__ pos, const double *__r
 // spread over many CTAs.  Scratch per supernode J: 4 s x s slots at
 // 4 * linv_off[J] (selinv: Mbar, W, T1; factorization: P, P M, G, Ubar).
 // ---------------------------------------------------------------------------
+// The factorization's part is the reverse of the dense LDL^T of J's diagonal
+// block in closed form.  U = D L^T (A_C = L_C U) gives Dbar_i += sum_{j>=i}
+// Ubar(i,j) L(j,i) and Lbar(j,i) += Ubar(i,j) D_i, j > i.  With X = L^{-1} dA
+// L^{-T} one has dD = diag(X) and dL = L stril(X) D^{-1}, so dloss = <P, X> with
+//   P = stril(L^T Lbar D^{-1}) + diag(Dbar)                         (T3)
+// and the full-matrix gradient is G = L^{-T} P L^{-1} = M^T P M (M = L_JJ^{-1};
+// G1, G2).  The stored lower entries of the symmetric block get G(i,j) + G(j,i)
+// below the diagonal, G(i,i) on it.  Ubar's updates ride in T3's operand and
+// the fold in G2 (two products per lower tile): as kernels of their own they
+// took 20 and 14 us of a top level's 300.
 enum { OP_SEL_T1 = 0, OP_SEL_W, OP_SEL_LB, OP_FAC_T3, OP_FAC_G1, OP_FAC_G2 };
 constexpr int kAdjTop = 8;        // most supernodes of a level of the adjoint's last group
 constexpr int kFinChunk = 1024;   // entries of an s x s block per item of the partial sums
@@ -835,11 +860,13 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
     if (w >= nitems) return;
     const AdjDesc &A = *ad;
     const int J = items[w].x;
-    const int s = A.super_ptr[J + 1] - A.super_ptr[J];
+    const int fc = A.super_ptr[J];
+    const int s = A.super_ptr[J + 1] - fc;
     const int nt = (s + kGT - 1) / kGT;
     const int i0 = (items[w].y / nt) * kGT + (Q == 1 ? 0 : (qd / 2) * GT);
     const int j0 = (items[w].y % nt) * kGT + (Q == 1 ? 0 : (qd % 2) * GT);
     if (i0 >= s || j0 >= s) return;
+    if (op >= OP_FAC_T3 && i0 < j0) return;   // P and P M are lower triangular, and so is what G2 stores
     const int64_t ss = (int64_t)s * s;
     const int64_t ld = A.rowptr[J + 1] - A.rowptr[J];
     const double *M = A.Linv + A.linv_off[J];             // M(i, k) = M[k*s + i]
@@ -862,7 +889,8 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
         case OP_SEL_T1: return S[(int64_t)j * ld + k];                // S
         case OP_SEL_W: return M[(int64_t)k * s + j];                  // M^T
         case OP_SEL_LB: return F[ss + (int64_t)j * s + k];            // W
-        case OP_FAC_T3: return k > j ? LbJ[(int64_t)j * ld + k] : 0.0;  // Lbar_JJ, strictly lower
+        case OP_FAC_T3:                                               // Lbar_JJ + Ubar^T D, strictly lower
+            return k > j ? fma(F[3 * ss + (int64_t)k * s + j], A.D[fc + j], LbJ[(int64_t)j * ld + k]) : 0.0;
         case OP_FAC_G1: return M[(int64_t)j * s + k];                 // M
         default: return F[ss + (int64_t)j * s + k];                   // P M
         }
@@ -880,31 +908,56 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
     case OP_SEL_W: khi = min(s, j0 + GT); break;    // M(j, k): k <= j
     case OP_SEL_LB: klo = i0; break;                // M(k, i): k >= i
     case OP_FAC_T3: klo = i0; break;                // L_JJ(k, i): k >= i
-    case OP_FAC_G1: klo = j0; break;                // M(k, j): k >= j
-    default: klo = i0; break;                       // M(k, i): k >= i
+    case OP_FAC_G1: klo = j0; khi = min(s, i0 + GT); break;   // M(k, j): k >= j; P(i, k): k <= i
+    default: klo = i0; break;                       // G2: M(k, i), k >= i
     }
-    double acc = 0.0;
-    for (int k0 = klo; k0 < khi; k0 += kGK) {
-        const int kn = khi - k0 < kGK ? khi - k0 : kGK;
-        __syncthreads();
+    double acc = 0.0, acc2 = 0.0;
+    auto product = [&](auto &&fa, auto &&fb) {
+        double r1 = 0.0, r2 = 0.0;   // two chains: half the FMA latency per k
+        for (int k0 = klo; k0 < khi; k0 += kGK) {
+            const int kn = khi - k0 < kGK ? khi - k0 : kGK;
+            __syncthreads();
 #pragma unroll 4
-        for (int e = threadIdx.x; e < GT * kn; e += NT) {
-            const int r = e % GT, q = e / GT;
-            As[r][q] = i0 + r < s ? a_at(i0 + r, k0 + q) : 0.0;
-            Bs[q][r] = j0 + r < s ? b_at(k0 + q, j0 + r) : 0.0;
-        }
-        __syncthreads();
-        if (wact) {
-            double a2 = 0.0;   // two chains: half the FMA latency per k
-            int q = 0;
-#pragma unroll 4
-            for (; q + 1 < kn; q += 2) {
-                acc = fma(As[ty][q], Bs[q][tx], acc);
-                a2 = fma(As[ty][q + 1], Bs[q + 1][tx], a2);
+            for (int e = threadIdx.x; e < GT * kn; e += NT) {
+                const int r = e % GT, q = e / GT;
+                As[r][q] = i0 + r < s ? fa(i0 + r, k0 + q) : 0.0;
+                Bs[q][r] = j0 + r < s ? fb(k0 + q, j0 + r) : 0.0;
             }
-            if (q < kn) acc = fma(As[ty][q], Bs[q][tx], acc);
-            acc += a2;
+            __syncthreads();
+            if (wact) {
+                int q = 0;
+#pragma unroll 4
+                for (; q + 1 < kn; q += 2) {
+                    r1 = fma(As[ty][q], Bs[q][tx], r1);
+                    r2 = fma(As[ty][q + 1], Bs[q + 1][tx], r2);
+                }
+                if (q < kn) r1 = fma(As[ty][q], Bs[q][tx], r1);
+            }
         }
+        return r1 + r2;
+    };
+    acc = product(a_at, b_at);
+    if (op == OP_FAC_G2) {
+        // the entry (j, i) of G for the mirrored sum: M(k, j) (P M)(k, i), k >= i
+        acc2 = product([&](int i, int k) { return F[ss + (int64_t)i * s + k]; },
+                       [&](int k, int j) { return M[(int64_t)j * s + k]; });
+    }
+    if (op == OP_FAC_T3 && i0 == j0) {
+        // the diagonal of L_JJ^T Ubar^T, which Dbar takes: the lanes of row ty
+        // share its sum over k >= j (unit diagonal of L)
+        for (int k0 = klo; k0 < khi; k0 += kGK) {
+            const int kn = khi - k0 < kGK ? khi - k0 : kGK;
+            __syncthreads();
+            for (int e = threadIdx.x; e < GT * kn; e += NT) {
+                const int r = e % GT, q = e / GT, i = i0 + r, k = k0 + q;
+                As[r][q] = i < s ? a_at(i, k) : 0.0;
+                Bs[q][r] = i < s && k >= i ? F[3 * ss + (int64_t)k * s + i] : 0.0;
+            }
+            __syncthreads();
+            for (int q = tx; q < kn; q += GT) acc2 = fma(As[ty][q], Bs[q][ty], acc2);
+        }
+#pragma unroll
+        for (int o = 1; o < GT; o <<= 1) acc2 += __shfl_xor_sync(0xffffffffu, acc2, o);
     }
     double *Lb = A.Lb + A.panel_off[J];
     const int i = i0 + ty, j = j0 + tx;
@@ -915,10 +968,16 @@ __global__ void __launch_bounds__(256) k_adj_gemm(const AdjDesc *__restrict__ ad
     case OP_SEL_W: F[ss + (int64_t)j * s + i] = x; break;                    // W
     case OP_SEL_LB: Lb[(int64_t)j * ld + i] = i > j ? -x : 0.0; break;      // Lbar_JJ
     case OP_FAC_T3:                                                          // P
-        F[(int64_t)j * s + i] = i > j ? x / A.D[A.super_ptr[J] + j] : (i == j ? A.Db[A.super_ptr[J] + i] : 0.0);
+        F[(int64_t)j * s + i] = i > j ? x / A.D[fc + j] : (i == j ? A.Db[fc + i] + acc2 : 0.0);
         break;
     case OP_FAC_G1: F[ss + (int64_t)j * s + i] = x; break;                   // P M
-    default: F[2 * ss + (int64_t)j * s + i] = x; break;                      // G = M^T P M
+    default:                                                                 // G = M^T P M, folded
+        if (i >= j) {
+            const double g = i > j ? x + acc2 : x;
+            A.Ab[A.panel_off[J] + (int64_t)j * ld + i] = g;
+            if (A.colexp) atomicMax(&A.colexp[fc + j], bexp(g));
+        }
+        break;
     }
 }
 
@@ -1094,73 +1153,6 @@ __global__ void __launch_bounds__(256) k_fadj_usum(const AdjDesc *__restrict__ a
     }
 }
 
-// factorization adjoint: U = D L^T gives Dbar_i += sum_{j>=i} Ubar(i,j) L(j,i),
-// Lbar(j,i) += Ubar(i,j) D_i (j > i); grid (supernodes, kFinY), the sums as
-// in k_adj_sel_dbar
-__global__ void __launch_bounds__(256) k_fadj_ubar(const AdjDesc *__restrict__ ad,
-                                                   const int *__restrict__ js, int nj) {
-    grid_dep_wait();
-    __shared__ double red[8][33];
-    const int w = blockIdx.x;
-    if (w >= nj) return;
-    const AdjDesc &A = *ad;
-    const int J = js[w];
-    const int fc = A.super_ptr[J];
-    const int s = A.super_ptr[J + 1] - fc;
-    const int64_t ss = (int64_t)s * s;
-    const int64_t ld = A.rowptr[J + 1] - A.rowptr[J];
-    const double *__restrict__ U = A.fin + 4 * A.linv_off[J] + 3 * ss;
-    const double *__restrict__ L = A.L + A.panel_off[J];
-    double *__restrict__ Lb = A.Lb + A.panel_off[J];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int ib = blockIdx.y; ib * 32 < s; ib += gridDim.y) {
-        const int i = ib * 32 + lane;
-        double v = 0.0;
-        if (i < s)
-            for (int j = i + 1 + warp; j < s; j += 8) v = fma(U[(int64_t)j * s + i], L[(int64_t)i * ld + j], v);
-        red[warp][lane] = v;
-        __syncthreads();
-        if (warp == 0 && i < s) {
-            double t = U[(int64_t)i * s + i];
-#pragma unroll
-            for (int q = 0; q < 8; q++) t += red[q][lane];
-            A.Db[fc + i] += t;
-        }
-        __syncthreads();
-    }
-    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < ss; e += (int64_t)gridDim.y * blockDim.x) {
-        const int j = (int)(e % s), i = (int)(e / s);
-        if (j > i) Lb[(int64_t)i * ld + j] += U[(int64_t)j * s + i] * A.D[fc + i];
-    }
-}
-
-// factorization adjoint: reverse of the dense LDL^T of J's diagonal block in
-// closed form.  With X = L^{-1} dA L^{-T} one has dD = diag(X) and
-// dL = L stril(X) D^{-1}, so dloss = <P, X> with
-//   P = stril(L^T Lbar D^{-1}) + diag(Dbar),
-// and the full-matrix gradient is G = L^{-T} P L^{-1} = M^T P M (M = L_JJ^{-1};
-// three s x s products in k_adj_gemm).  The stored lower entries of the
-// symmetric block get G(i,j) + G(j,i) below the diagonal, G(i,i) on it.
-// Grid (supernodes, kFinY).
-__global__ void __launch_bounds__(256) k_fadj_fold(const AdjDesc *__restrict__ ad,
-                                                   const int *__restrict__ js, int nj) {
-    grid_dep_wait();
-    const int w = blockIdx.x;
-    if (w >= nj) return;
-    const AdjDesc &A = *ad;
-    const int J = js[w];
-    const int s = A.super_ptr[J + 1] - A.super_ptr[J];
-    const int64_t ld = A.rowptr[J + 1] - A.rowptr[J];
-    const int64_t ss = (int64_t)s * s;
-    const double *__restrict__ G = A.fin + 4 * A.linv_off[J] + 2 * ss;
-    double *__restrict__ Ab = A.Ab + A.panel_off[J];
-    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < ss; e += (int64_t)gridDim.y * blockDim.x) {
-        const int i = (int)(e % s), k = (int)(e / s);
-        Ab[(int64_t)k * ld + i] = i > k ? G[(int64_t)k * s + i] + G[(int64_t)i * s + k]
-                                        : (i == k ? G[(int64_t)k * s + i] : 0.0);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -1283,7 +1275,7 @@ static int adj_build(selinv_plan_s *plan) {
             a->lvl_bucket_ptr.push_back((int)a->items.size());
         }
     }
-    a->g_lptr.assign(1, 0); a->c_lptr.assign(1, 0); a->j_lptr.assign(1, 0); a->cz_lptr.assign(1, 0);
+    a->g_lptr.assign(1, 0); a->c_lptr.assign(1, 0); a->j_lptr.assign(1, 0);
     a->v_lptr.assign(1, 0);
     for (int l = p.nlevels - 1; l >= 0; l--) {      // deepest first, like every list here
         for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
@@ -1300,7 +1292,6 @@ static int adj_build(selinv_plan_s *plan) {
             for (int ti = 0; ti < nvt; ti++)
                 for (int tj = 0; tj <= ti; tj++) a->vitems.push_back(make_int4(J, ti, tj, 0));
         }
-        a->cz_lptr.push_back((int64_t)a->cz_work.size());
         a->v_lptr.push_back((int64_t)a->vitems.size());
         a->g_lptr.push_back((int64_t)a->gitems.size());
         a->c_lptr.push_back((int64_t)a->citems.size());
@@ -1365,6 +1356,7 @@ static AdjDesc make_adesc(selinv_plan_s *plan, const double *L, const double *D,
     h.chpos = f->d_chpos;
     h.V = a->V;
     h.G = static_cast<double *>(w.work);
+    h.colexp = nullptr;
     return h;
 }
 
@@ -1826,9 +1818,10 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
     cudaMemsetAsync(a->Ab, 0, bytes, st);
     AdjDesc h = make_adesc(plan, static_cast<const double *>(L), static_cast<const double *>(D), nullptr,
                            a->Lbw, a->YB);
-    cudaMemcpyAsync(a->d_desc, &h, sizeof(h), cudaMemcpyHostToDevice, st);
     Workspace &w = plan->ws[0];
     const bool tc = !a->dig_work.empty();
+    if (tc) h.colexp = w.colexpZ;
+    cudaMemcpyAsync(a->d_desc, &h, sizeof(h), cudaMemcpyHostToDevice, st);
     if (tc) {
         // tcgen05 gather-GEMM of the wide supernodes: A^{-1}(C,C) -> the
         // finished Abar of the ancestors, B = L_C (digit planes of L, once),
@@ -1850,6 +1843,7 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
     }
     const int nl = p.nlevels;
     auto levels = [&](cudaStream_t st) {
+        if (tc) cudaMemsetAsync(w.colexpZ, 0, sizeof(int) * (size_t)p.n, st);
         row_digits<RP_FABAR>(a, 0, nl, st);
         for (int li = nl - 1; li >= 0; li--) {  // root level first
             const int d0 = (int)a->dig_lptr[li], d1 = (int)a->dig_lptr[li + 1];
@@ -1863,7 +1857,7 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
                 launch_bucket(1, b, a->d_desc, a->d_sm + b0, b1 - b0, st);
             }
             const int w0 = (int)a->wd_lptr[li], w1 = (int)a->wd_lptr[li + 1];
-            if (w1 > w0) { k_fadj_pull_tc<<<w1 - w0, 256, 0, st>>>(a->d_desc, a->d_wd + w0, w1 - w0); note_launch(); }
+            if (w1 > w0) { k_fadj_pull_tc<<<dim3(w1 - w0, kPullY), 256, 0, st>>>(a->d_desc, a->d_wd + w0, w1 - w0); note_launch(); }
             for (int b = 0; b < kNumBuckets; b++) {
                 const int b0 = a->sm_bptr[li * kNumBuckets + b], b1 = a->sm_bptr[li * kNumBuckets + b + 1];
                 launch_bucket(2, b, a->d_desc, a->d_sm + b0, b1 - b0, st);
@@ -1875,24 +1869,10 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
                 note_launch();
             }
             const int64_t c0 = a->c_lptr[li], c1 = a->c_lptr[li + 1];
-            const int64_t j0 = a->j_lptr[li], j1 = a->j_lptr[li + 1];
             if (c1 > c0) { k_fadj_usum<<<(int)(c1 - c0), 256, 0, st>>>(a->d_desc, a->d_citems + c0, (int)(c1 - c0)); note_launch(); }
-            if (j1 > j0) {
-                k_fadj_ubar<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0));
-                note_launch();
-            }
             launch_gemm(a, OP_FAC_T3, li, li + 1, st);
             launch_gemm(a, OP_FAC_G1, li, li + 1, st);
             launch_gemm(a, OP_FAC_G2, li, li + 1, st);
-            if (j1 > j0) {
-                k_fadj_fold<<<dim3((int)(j1 - j0), kFinY), 256, 0, st>>>(a->d_desc, a->d_js + j0, (int)(j1 - j0));
-                note_launch();
-                const int z0 = (int)a->cz_lptr[li], z1 = (int)a->cz_lptr[li + 1];
-                if (tc && li > 0 && z1 > z0) {
-                    k_adj_colexpz<<<z1 - z0, 256, 0, st>>>(a->d_desc, a->Ab, w.colexpZ, a->d_cz + z0, z1 - z0);
-                    note_launch();
-                }
-            }
         }
     };
     if ((rc = a->g_fac.run(a->gen, w.colexpZ, st, levels))) return rc;
