@@ -18,6 +18,11 @@
 //   and their exact sum is added into a 96-bit word per entry in shared
 //   memory (an int64 high part and a 32-bit low part, carried after every
 //   chunk).
+// A k16 step takes 1400 clocks of the tensor pipe and an eighth of a chunk's
+// read-back 700, during which the products wait (the groups fill tensor
+// memory).  Shared memory bounds the former: the step's 10 MMAs read 96 KB of
+// operands, its copies write 28 KB, the producers 14 KB and the sums move
+// 24 KB, 1300 clocks at 128 bytes each, where the products alone would take 900.
 // Operand rings: 3 stages for the Lhat^T copies, 3 for the gathered digits.
 // The copies are issued by a thread of their own, so that the thread issuing
 // the products never waits for products to finish: it waits only for its
@@ -65,7 +70,7 @@ struct TwCfg {
     static constexpr size_t SMEM = sizeof(uint16_t) * (size_t)(kTwAS * A_STAGE + kTwBS * B_STAGE) +
                                    (sizeof(long long) + sizeof(uint32_t)) * (size_t)kTwN * kTwHS + sizeof(int) * kTwN;
 };
-static_assert(TwCfg::SMEM + 2048 <= 232448, "dynamic + static shared memory within the opt-in limit");
+static_assert(TwCfg::SMEM + 3072 <= 232448, "dynamic + static shared memory within the opt-in limit");
 
 // One chunk's group sums (g weighted 256^(6 - g)), exact, added into the
 // entry's 96-bit sum hi 2^32 + lo (0 <= lo < 2^32): the chunk's value is
@@ -147,7 +152,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
     __shared__ uint32_t s_tmem;
     __shared__ int s_pre;
     __shared__ volatile int s_abort;
-    __shared__ int ymax[kTcM];
+    __shared__ int ymax[kTcM], colE[kTcM];   // colE: exponents of the rows of A
     __shared__ int ksh[BAL ? kTcM : 1];   // shift of the exponents of B's column k
 
     const int w = blockIdx.x;
@@ -282,7 +287,11 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             Hi[e] = 0;
             Lo[e] = 0;
         }
-    for (int e = tid; e < kTcM; e += kTwThreads) ymax[e] = 0;
+    for (int e = tid; e < kTcM; e += kTwThreads) {
+        ymax[e] = 0;
+        const int jr = m0 + e, j = CPLX && jr >= s ? jr - s : jr;
+        colE[e] = jr < mrows ? (SYRK ? P.linvexp[pos0 + jr] : (LHAT ? P.linvexp[fc + j] : P.colexp[fc + j])) : 0;
+    }
     if (warp == kTwMmaWarp) {
         umma::tmem_alloc(&s_tmem, Cfg::TCOLS);
         umma::tmem_relinquish();
@@ -311,28 +320,33 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         // 4 kq .. 4 kq + 3 of each 16-k step; a warp holds 16 rows x 2
         // quarters, so that its stores of a plane fill two 128-byte core
         // matrices.  Complex: the 4 k-values are (Re, Im) of the entries
-        // q = 8 step + 2 kq and + 1.  The gather runs three steps ahead in
-        // registers, every load a whole step before its use: column data
-        // (step i + 3), relative rows (i + 2), values (i + 1).
+        // q = 8 step + 2 kq and + 1.  The gather runs four steps ahead in
+        // registers: column data (step i + 4) and relative rows (i + 3) a whole
+        // step before their use, values (i + 2) two, for the ancestors' panels
+        // lie anywhere in L2 or memory; nothing touches a value before then
+        // (40^3: 5.32 ms with one step, 5.20 with two; a sheet of 32 x 32
+        // blocks of 16: 7.89 and 7.80).
         const TcGather g{P.colbase + pos0, P.relbase + pos0, P.relidx, tile_cb, tile_rb, p0, c, gather_check(P)};
         const int r = (warp % 4) * 16 + (lane >> 1), kq = (warp / 4) * 2 + (lane & 1);
         const int E = rowE[r];
         constexpr int NV = CPLX ? 2 : 4;        // entries of A^{-1}_{C,C} per thread and step
         constexpr int QS = CPLX ? 8 : 16;       // entries per step
-        double v[4];
+        double v0[4], v1[4];                    // values of the even and the odd steps
+        bool neg0[NV], neg1[NV];                // Hermitian: imaginary parts to be negated
         int64_t ab[NV], cb[NV], rb[NV];
         int32_t ar[NV];
         bool up[NV];
         // Hermitian: an entry above the diagonal is the conjugate of the stored one
         const bool herm = CPLX && P.herm;
-        auto load = [&]() {
+        auto load = [&](double (&v)[4], bool (&neg)[NV]) {
             if (CPLX) {
                 const double2 *Zc = static_cast<const double2 *>(P.Z);
 #pragma unroll
                 for (int u = 0; u < NV; u++) {
                     const double2 z = ab[u] >= 0 ? Zc[ab[u] + ar[u]] : make_double2(0.0, 0.0);
                     v[2 * u] = z.x;
-                    v[2 * u + 1] = herm && up[u] ? -z.y : z.y;
+                    v[2 * u + 1] = z.y;
+                    neg[u] = herm && up[u];
                 }
             } else {
                 const double *Zg = static_cast<const double *>(P.Z);
@@ -353,7 +367,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         const double *Zc2 = static_cast<const double *>(P.Z) + P.panel_off[K] + s + p0 + r;  // PAIR: k >= s
         const bool rok = p0 + r < c;
         const double2 *Lz = static_cast<const double2 *>(P.L) + P.panel_off[K] + s + p0 + r;   // complex X(p0 + r, q)
-        auto load_dense = [&](int i_) {
+        auto load_dense = [&](int i_, double (&v)[4]) {
             if (CPLX) {
 #pragma unroll
                 for (int u = 0; u < 2; u++) {
@@ -383,21 +397,25 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                     if (ab[u] >= 0 && !g.chk.ok(ab[u] + ar[u])) ab[u] = -1;
         };
         if (DENSE) {
-            if (n > 0) load_dense(0);
-        } else if (n > 0) {
+            load_dense(0, v0);
+            load_dense(1, v1);
+        } else {
             cols(0);
             parts(0);
-            load();
+            load(v0, neg0);
             cols(1);
             parts(1);
+            load(v1, neg1);
             cols(2);
+            parts(2);
+            cols(3);
         }
-        for (int i_ = 0; i_ < n; i_++) {
+        auto step = [&](int i_, double (&v)[4], bool (&neg)[NV]) -> bool {
             const int stage = i_ % kTwBS, use = i_ / kTwBS;
             uint16_t *Bb = Bs + stage * Cfg::B_STAGE;
             if (i_ >= kTwBS && !umma::mbar_wait(&bempty[stage], (uint32_t)((use - 1) & 1), mlim)) {
                 s_abort = 1;
-                break;
+                return false;
             }
             {
                 uint32_t lo[4], hi[4];
@@ -408,7 +426,9 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                         const int k = (st0 + i_) * 16 + kq * 4 + u;
                         add = k < kw ? ksh[BAL ? (CPLX ? k >> 1 : k) : 0] : 0;
                     }
-                    const unsigned long long wv = (unsigned long long)(fixed54<BAL>(v[u], E, add) + 0x80808080808080ll);
+                    long long x = fixed54<BAL>(v[u], E, add);
+                    if (CPLX && !DENSE && (u & 1) && neg[u >> 1]) x = -x;
+                    const unsigned long long wv = (unsigned long long)(x + 0x80808080808080ll);
                     lo[u] = (uint32_t)wv;
                     hi[u] = (uint32_t)(wv >> 32);
                 }
@@ -427,13 +447,17 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             __syncwarp();
             if (lane == 0) umma::mbar_arrive(&full[stage]);
             if (DENSE) {
-                load_dense(i_ + 1);
+                load_dense(i_ + 2, v);
             } else {
-                load();            // values of step i + 1
-                parts(i_ + 2);     // relative rows of step i + 2
-                cols(i_ + 3);      // column data of step i + 3
+                load(v, neg);      // values of step i + 2
+                parts(i_ + 3);     // relative rows of step i + 3
+                cols(i_ + 4);      // column data of step i + 4
             }
-            if (s_abort) break;
+            return !s_abort;
+        };
+        for (int i_ = 0; i_ < n; i_ += 2) {
+            if (!step(i_, v0, neg0)) break;
+            if (i_ + 1 < n && !step(i_ + 1, v1, neg1)) break;
         }
     } else if (warp == kTwMmaWarp) {
         // ---- one thread issues the products once both operands of a step
@@ -553,7 +577,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             for (int u = 0; u < NV; u++) {
                 const int e = e0 + u * kTwThreads, mm = e % kTcM, p = e / kTcM, p1 = m0 + mm, p2 = p0 + p;
                 if (e >= kTwN * kTcM || p1 >= c || p1 < p2) continue;
-                const int e1 = P.linvexp[pos0 + p1], e2 = rowE[p];
+                const int e1 = colE[mm], e2 = rowE[p];
                 const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0) - (BAL ? 2 * kBalBias : 0);
                 const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
                 V[(int64_t)p2 * c + p1] = SYRK == 2 && max(e1, e2) >= kBalBad ? __longlong_as_double(0x7FF8000000000000ll) : old[u] - y;
@@ -570,7 +594,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 const int p = e % kTwN, mm = e / kTwN, jr = m0 + mm;
                 if (p0 + p >= c || jr >= mrows) continue;
                 const int j = jr >= s ? jr - s : jr;
-                const int e1 = rowE[p], e2 = P.linvexp[fc + j];
+                const int e1 = rowE[p], e2 = colE[mm];
                 const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], e1 - 1022 + e2 - 1022 - 13 - 2 * kBalBias);
                 // an infinity or a NaN in the row or the column: NaN, as FP64 products give
                 Lz[2 * ((int64_t)j * ld + s + p0 + p) + (jr >= s ? 1 : 0)] =
@@ -582,7 +606,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         for (int e = tid; e < kTwN * kTcM; e += kTwThreads) {
             const int p = e % kTwN, j = e / kTwN;
             if (p0 + p >= c || j >= s) continue;
-            const int sc = (rowE[p] - 1022) + (P.linvexp[fc + j] - 1022) - 13;
+            const int sc = (rowE[p] - 1022) + (colE[j] - 1022) - 13;
             const double y = fixed_to_double(Hi[p * kTwHS + j], (long long)Lo[p * kTwHS + j], sc);
             const int64_t at = (int64_t)j * ld + s + p0 + p;
             if (op == 0) Lh[at] = y;
@@ -597,7 +621,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             const int p = e % kTwN, mm = e / kTwN, jr = m0 + mm;   // a warp shares mm
             if (p0 + p >= c || jr >= mrows) continue;
             const int j = CPLX && jr >= s ? jr - s : jr;
-            const int sc = (rowE[p] - 1022) + (P.colexp[fc + j] - 1022) - 13;
+            const int sc = (rowE[p] - 1022) + (colE[mm] - 1022) - 13;
             const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
             const int64_t at = (int64_t)j * ld + s + p0 + p;
             if (CPLX) Zk[2 * at + (jr >= s ? 1 : 0)] = -y;
