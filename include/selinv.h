@@ -344,8 +344,8 @@ int selinv_pole_sum(int nitems, const selinv_dtype *dtypes, const void *const *A
  * launch with CUDA events on the stream, and synchronizes.  kernel_ms[k] and
  * kernel_launches[k] (arrays of SELINV_PROFILE_KINDS entries) receive the
  * summed device time in ms and the launch count of each kernel kind:
- *   0 L_KK^{-1} and Dinv (DFMA)        1 Lhat (DFMA)
- *   2 gather-GEMM + diagonal (DFMA)    3 digit planes of Lhat
+ *   0 L_KK^{-1} (and Dinv up to 32 columns; DFMA)   1 Lhat (DFMA)
+ *   2 gather-GEMM and diagonal block (DFMA)         3 digit planes of Lhat
  *   4 gather-GEMM on tensor cores      5 diagonal block after it
  *   6 digit planes of L_KK^{-1}        7 Lhat on tensor cores
  *   8 the persistent traversal          9 gather-GEMM on tcgen05
@@ -353,9 +353,9 @@ int selinv_pole_sum(int nitems, const selinv_dtype *dtypes, const void *const *A
  *  11 diagonal block from the tensor-core sums (finisher)
  *  12 push schedule: diagonal block from the pushed A^{-1}_{C,K}
  *  13 push schedule: outer- and inner-product updates of the descendants
- *  14 Dinv_K of the supernodes wider than 32 columns (32 x 32 tiles)
+ *  14 Dinv_K of the supernodes wider than 32 columns (16 x 16 tiles)
  *  15 diagonal block on tcgen05 (exact sums of Lhat^T A^{-1}_{C,K})
- *  16 the whole step for supernodes of <= 8 columns and <= 64 rows, a warp each
+ *  16 the whole step for narrow supernodes (<= 16 columns), a CTA or a cluster each
  * For measurement only. */
 #define SELINV_PROFILE_KINDS 17
 int selinv_numeric_profile(selinv_plan plan, selinv_dtype dtype, const void *L_dev,

@@ -21,10 +21,10 @@
 // Factorization adjoint, root -> leaves (reverse of k_fupdate / k_fdiag / k_ftrsm):
 //   Lbar_CJ -= (Abar(C,C) L_CJ) o D, the gathered Abar with its diagonal
 //   doubled; Dbar_k -= 1/2 (L_CJ^T Abar(C,C) L_CJ)_kk          [k_fadj_pull]
-//   Abar_CJ = Lbar_CJ D^{-1} L_JJ^{-1}; Nbar = A_CJ^T Lbar_CJ   [k_fadj_trsm]
-//   Ubar = -N^T Nbar N^T with N = L_JJ^{-T} D^{-1}  [k_fadj_nbar, k_adj_gemm, k_fadj_ubar]
+//   Abar_CJ = Lbar_CJ D^{-1} L_JJ^{-1}; Ubar = -L_CJ^T Abar_CJ (U = D L_JJ^T)
+//                                                   [k_fadj_trsm, k_fadj_usum]
 //   then the reverse of the dense LDL^T of the diagonal block in closed form
-//                                                   [k_adj_gemm, k_fadj_fold]
+//                                                                [k_adj_gemm]
 #include <cuda_runtime.h>
 
 #include <algorithm>
