@@ -93,4 +93,40 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
     return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | (q & 0xFFFFFFFFFFFFFull)));
 }
 
+// The same for a low word of 32 bits (96-bit sums): three 32-bit words, half the
+// instructions.  Issue slots bound the conversions at the end of a tensor-core
+// tile (18 warps, 8192 of them).
+__device__ __forceinline__ double fixed96_to_double(long long hi, uint32_t lo, int sc) {
+    const bool neg = hi < 0;
+    uint32_t w0 = neg ? 0u - lo : lo;
+    const unsigned long long h = neg ? ~(unsigned long long)hi + (lo == 0u ? 1ull : 0ull) : (unsigned long long)hi;
+    uint32_t w2 = (uint32_t)(h >> 32), w1 = (uint32_t)h;
+    int be = sc - 48 + 95 + 1023;                       // biased exponent of bit 95
+    if (w2 == 0u) {
+        w2 = w1;
+        w1 = w0;
+        w0 = 0u;
+        be -= 32;
+        if (w2 == 0u) {
+            w2 = w1;
+            w1 = 0u;
+            be -= 32;
+            if (w2 == 0u) return 0.0;
+        }
+    }
+    const int lz = __clz((int)w2);                      // leading bit to bit 31 of w2
+    w2 = __funnelshift_l(w1, w2, lz);
+    w1 = __funnelshift_l(w0, w1, lz);
+    w0 <<= lz;
+    be -= lz;
+    if (be <= 0 || be >= 2046) return fixed_to_double(hi, (long long)lo, sc);   // outside the normal range, or next to it
+    // the top 53 bits; the bit below with all that follows rounds them, and a
+    // carry out of the mantissa is one more in the exponent
+    const uint32_t cut = w1 & 0x7FFu;
+    unsigned long long q = ((unsigned long long)w2 << 21) | (w1 >> 11);
+    q += cut > 0x400u || (cut == 0x400u && (w0 != 0u || (q & 1ull))) ? 1ull : 0ull;
+    q += (unsigned long long)(uint32_t)(be - 1) << 52;
+    return __longlong_as_double((long long)(q | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
 }  // namespace selinv

@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 if (e >= kTwN * kTcM || p1 >= c || p1 < p2) continue;
                 const int e1 = colE[mm], e2 = rowE[p];
                 const int sc = (e2 - 1022) + (e1 - 1022) - 13 - (PAIR && p1 == p2 ? 1 : 0) - (BAL ? 2 * kBalBias : 0);
-                const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
+                const double y = fixed96_to_double(Hi[p * kTwHS + mm], Lo[p * kTwHS + mm], sc);
                 V[(int64_t)p2 * c + p1] = SYRK == 2 && max(e1, e2) >= kBalBad ? __longlong_as_double(0x7FF8000000000000ll) : old[u] - y;
             }
         }
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                 if (p0 + p >= c || jr >= mrows) continue;
                 const int j = jr >= s ? jr - s : jr;
                 const int e1 = rowE[p], e2 = colE[mm];
-                const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], e1 - 1022 + e2 - 1022 - 13 - 2 * kBalBias);
+                const double y = fixed96_to_double(Hi[p * kTwHS + mm], Lo[p * kTwHS + mm], e1 - 1022 + e2 - 1022 - 13 - 2 * kBalBias);
                 // an infinity or a NaN in the row or the column: NaN, as FP64 products give
                 Lz[2 * ((int64_t)j * ld + s + p0 + p) + (jr >= s ? 1 : 0)] =
                     max(e1, e2) >= kBalBad ? __longlong_as_double(0x7FF8000000000000ll) : y;
@@ -607,7 +607,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             const int p = e % kTwN, j = e / kTwN;
             if (p0 + p >= c || j >= s) continue;
             const int sc = (rowE[p] - 1022) + (colE[j] - 1022) - 13;
-            const double y = fixed_to_double(Hi[p * kTwHS + j], (long long)Lo[p * kTwHS + j], sc);
+            const double y = fixed96_to_double(Hi[p * kTwHS + j], Lo[p * kTwHS + j], sc);
             const int64_t at = (int64_t)j * ld + s + p0 + p;
             if (op == 0) Lh[at] = y;
             else if (op == 1) Lh[at] -= y;
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
             if (p0 + p >= c || jr >= mrows) continue;
             const int j = CPLX && jr >= s ? jr - s : jr;
             const int sc = (rowE[p] - 1022) + (colE[mm] - 1022) - 13;
-            const double y = fixed_to_double(Hi[p * kTwHS + mm], (long long)Lo[p * kTwHS + mm], sc);
+            const double y = fixed96_to_double(Hi[p * kTwHS + mm], Lo[p * kTwHS + mm], sc);
             const int64_t at = (int64_t)j * ld + s + p0 + p;
             if (CPLX) Zk[2 * at + (jr >= s ? 1 : 0)] = -y;
             else Zk[at] = -y;
