@@ -370,6 +370,8 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const FactorDesc *__restri
 // zeros above the diagonal).  The FP64 pipe bounds it, so a warp packs four
 // rows of its share into its lanes, then two, then one (tri_rows), and the row
 // tiles are made small enough that every SM gets one.
+// 40^3: the panel solves of all levels 3.95 ms with one row to a lane block of
+// 32 columns, 3.53 so.
 // items {J, first row of C, rows}
 // ---------------------------------------------------------------------------
 constexpr int kFtThreads = kTriThreads;
