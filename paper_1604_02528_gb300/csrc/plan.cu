@@ -1596,7 +1596,11 @@ static cudaError_t issue(Schedule &S, cudaStream_t st, bool count, const IssueHo
         }
         if ((e = marks(i)) != cudaSuccess) return e;
         if (forked && (int)i == S.join_at) {
-            if (S.join_at2 < 0) e = join();   // (two phases: the side stream's whole work)
+            // the side stream's whole work where it has no second phase: two
+            // phases, or a selection without supernodes in the third (ev_mid,
+            // recorded when the side stream enters that, would not hold this
+            // call's work)
+            if (S.join_at2 < 0 || side_phase < 2) e = join();
             else e = cudaStreamWaitEvent(st, S.ev_mid, 0);
             if (e != cudaSuccess) return e;
         }

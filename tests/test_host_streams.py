@@ -1,0 +1,144 @@
+"""What the host side issues, without a GPU: the library runs on a CUDA runtime
+that executes nothing and logs launches, their order over streams and the
+addresses that they are given (fake_cudart.cpp)."""
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+import oracle
+import synth
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes as ct, json, os, sys
+sys.path.insert(0, {root!r})
+import numpy as np
+import synth
+from paper_1604_02528_gb300 import _native as N
+LIB, RT = N.LIB, ct.CDLL(None)
+def mem(count):
+    p = ct.c_void_p()
+    assert RT.cudaMalloc(ct.byref(p), ct.c_size_t(16 * count)) == 0
+    return p
+class Ctx:
+    def __init__(self, p, **opts):
+        self.p, sn = p, p.supernodes
+        a = N.selinv_analyse(p.n, p.colptr, p.rowind, 1 if sn["kind"] == "relaxed" else 0, sn["cap"], sn["fill"])
+        o = N.selinv_default_opts()
+        for k, v in opts.items():
+            setattr(o, k, v)
+        self.plan = N.selinv_symbolic(p.n, a["nsuper"], a["super_ptr"], a["sparent"], a["rowptr"], a["rows"], o)
+        self.h, self.opts = self.plan.handle, o
+        nnz = self.plan.nnz
+        self.L, self.D, self.Z, self.Zu, self.Lb, self.Db = (mem(x) for x in (nnz, p.n, nnz, nnz, nnz, p.n))
+        self.A = mem(p.colptr[-1])
+        N.selinv_plan_set_matrix(self.plan, p.n, p.colptr, p.rowind)
+    def set(self, **opts):
+        for k, v in opts.items():
+            setattr(self.opts, k, v)
+        N.selinv_plan_set_opts(self.plan, self.opts)
+    def selinv(self, dtype=0, stream=None):
+        return LIB.selinv_numeric(self.h, dtype, self.L, self.D, self.Z, stream)
+    def lu(self, dtype=0, stream=None):
+        return LIB.selinv_numeric_lu(self.h, dtype, self.L, self.Lb, self.Z, self.Zu, stream)
+    def factor(self, dtype=0, stream=None):
+        return LIB.selinv_factor(self.h, dtype, self.A, self.L, self.D, stream)
+    def adjoint(self, stream=None):
+        return LIB.selinv_adjoint(self.h, 0, self.L, self.D, self.Z, self.Zu, self.Lb, self.Db, stream)
+    def factor_adjoint(self, stream=None):
+        return LIB.selinv_factor_adjoint(self.h, 0, self.L, self.D, self.Lb, self.Db, self.A, stream)
+def batched(ctxs, dtypes):
+    n = len(ctxs)
+    arr = lambda xs: (ct.c_void_p * n)(*[x.value for x in xs])
+    return LIB.selinv_numeric_batched(n, (ct.c_void_p * n)(*[c.h.value for c in ctxs]), (ct.c_int * n)(*dtypes),
+                                      arr([c.L for c in ctxs]), arr([c.D for c in ctxs]), arr([c.Z for c in ctxs]), None)
+def mark(name):      # a line of its own in the log
+    with open(os.environ["FAKE_CUDART_LOG"], "a") as f:
+        f.write("# " + name + "\\n")
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(native, tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "fake_cudart.so")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-w", "-o", so, os.path.join(HERE, "fake_cudart.cpp"),
+                    "-I" + os.path.join(cuda, "include"), "-I" + os.path.join(ROOT, "include"),
+                    "-I" + os.path.join(ROOT, "paper_1604_02528_gb300", "csrc")], check=True)
+    return so
+
+
+def run(fake, tmp_path, script):
+    """The log of a script: [(mark, [line, ...])] in order, and what it printed (JSON)."""
+    log = str(tmp_path / "log")
+    env = dict(os.environ, LD_PRELOAD=fake, FAKE_CUDART_LOG=log)
+    r = subprocess.run([sys.executable, "-c", PRELUDE.format(root=ROOT) + script], env=env, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr[-3000:]
+    parts = [("", [])]
+    for line in open(log):
+        if line.startswith("# "):
+            parts.append((line[2:].strip(), []))
+        else:
+            parts[-1][1].append(line.split())
+    return parts, (json.loads(r.stdout) if r.stdout.strip() else None)
+
+
+class Launch:
+    def __init__(self, f):
+        self.stream, self.index, self.stale, self.yacc, self.name = int(f[1]), int(f[2]), int(f[4]), int(f[5]), f[6]
+        self.clock = [int(x) for x in f[3].split(",")]
+        self.ks = {int(x) for x in f[7:]}
+
+    def after(self, other):
+        return other.stream < len(self.clock) and self.clock[other.stream] >= other.index
+
+
+def launches(lines):
+    return [Launch(f) for f in lines if f[0] == "L"]
+
+
+def _ordered(sym, got):
+    """Launches that touch one supernode come one after the other, and a
+    traversal launch of a supernode after everything that touches its parent."""
+    by = {}
+    for x in got:
+        for K in x.ks:
+            for y in by.setdefault(K, []):
+                assert x.after(y), (K, y.name, x.name)
+            by[K].append(x)
+    norm = ("k_linv", "k_dinv", "k_lhat", "k_fma_lhat", "digits", "k_selinv_tcw<false,_true", "k_selinv_tcw<true,_true")
+    for K, own in by.items():
+        J = int(sym.sparent[K])
+        for x in own:
+            if J >= 0 and not any(n in x.name for n in norm):
+                for y in by[J]:
+                    assert x.after(y), (K, J, y.name, x.name)
+    return set(by)
+
+
+# every branch, the side stream's phases, and a selection that needs the first
+# of them only (the second then has no launch)
+@pytest.mark.parametrize("picked", ["all", "top", "middle", "leaf"])
+@pytest.mark.parametrize("make,dtype", [("laplacian_3d(12, 4)", 0), ("laplacian_2d(31, 19)", 0), ("magnetic_laplacian_3d(10, 4)", 2),
+                                        ("random_sparse_spd(900, 0.002, 2, supernodes=synth.problems.RELAXED_128)", 0)])
+def test_launches_of_dependent_supernodes_are_ordered(fake, tmp_path, make, dtype, picked):
+    parts, active = run(fake, tmp_path, f"""
+c = Ctx(synth.{make}, use_graph=0)
+level, lptr, lst = (N.selinv_plan_get(c.plan, x) for x in ("level", "level_ptr", "level_list"))
+a = N.selinv_analyse(c.p.n, c.p.colptr, c.p.rowind, 1 if c.p.supernodes["kind"] == "relaxed" else 0, c.p.supernodes["cap"], c.p.supernodes["fill"])
+at = {{"top": np.searchsorted(lptr, 16, "right") - 2, "middle": np.searchsorted(lptr, 256, "right") - 2, "leaf": len(lptr) - 2}}.get({picked!r})
+if at is not None:
+    cols = a["super_ptr"][lst[lptr[at]:lptr[at + 1]]]
+    N.selinv_plan_select(c.plan, cols, cols)
+mark("run")
+assert c.selinv({dtype}) == 0
+print(json.dumps(N.selinv_plan_get(c.plan, "active").tolist()))
+""")
+    sym = oracle.symbolic_for(eval("synth." + make))
+    assert _ordered(sym, launches(parts[-1][1])) == {K for K in range(sym.nsuper) if active[K]}
