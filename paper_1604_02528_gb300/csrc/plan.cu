@@ -56,6 +56,7 @@ void Workspace::release() {
     partial_all = nullptr;
     colexpZ = tcount = nullptr;
     yacc = nullptr;
+    yacc_words = 0;
     lhs = nullptr;
     lhsu = nullptr;
     colexp = colexpY = nullptr;
@@ -79,7 +80,17 @@ template <typename X> static bool wget(Workspace &w, X **ptr, size_t bytes) {
 
 int Workspace::ensure(const PlanData &p, int dtype) {
     const size_t es = elem_size(dtype);
-    if (LD && bytes_elem >= es) return SELINV_OK;
+    const size_t ny = (dtype == SELINV_F64 && p.lhs_total > 0) ? 2 * (size_t)p.nnz : 2;   // words of yacc
+    if (LD && bytes_elem >= es) {
+        if (yacc_words >= ny) return SELINV_OK;
+        // real values in a workspace made for complex ones, which have no such sums
+        DeviceGuard g(device);
+        if (!wget(*this, &yacc, sizeof(long long) * ny)) return SELINV_ERR_OOM;
+        if (cudaMemset(yacc, 0, sizeof(long long) * ny) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+            return SELINV_ERR_CUDA;
+        yacc_words = ny;
+        return SELINV_OK;
+    }
     release();
     DeviceGuard g(p.device);
     device = p.device;
@@ -107,7 +118,6 @@ int Workspace::ensure(const PlanData &p, int dtype) {
     if (!wget(*this, &linvd, sizeof(uint16_t) * (size_t)nlinvd)) return SELINV_ERR_OOM;
     cudaMemset(linvd, 0, sizeof(uint16_t) * (size_t)nlinvd);   // padding rows stay zero
     cudaMemset(colexpZ, 0, sizeof(int) * (size_t)std::max(p.n, 1));
-    const size_t ny = (dtype == SELINV_F64 && p.lhs_total > 0) ? 2 * (size_t)p.nnz : 2;
     if (!wget(*this, &yacc, sizeof(long long) * ny)) return SELINV_ERR_OOM;
     if (!wget(*this, &tcount, sizeof(int) * (size_t)std::max<int64_t>(p.tile_total, 1)))
         return SELINV_ERR_OOM;
@@ -123,6 +133,7 @@ int Workspace::ensure(const PlanData &p, int dtype) {
     // see the buffers (reused ones hold a previous plan's data)
     if (cudaDeviceSynchronize() != cudaSuccess) return SELINV_ERR_CUDA;
     bytes_elem = es;
+    yacc_words = ny;
     return SELINV_OK;
 }
 

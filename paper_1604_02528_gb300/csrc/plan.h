@@ -101,7 +101,8 @@ struct Workspace {
     int *ticket = nullptr;     // work-item ticket of the persistent schedule
     uint16_t *linvd = nullptr; // digit planes of L_KK^{-1}
     int *linvexp = nullptr;    // [n]
-    long long *yacc = nullptr; // [2 * nnz] (real problems with tensor-core supernodes), zero between calls
+    long long *yacc = nullptr; // [yacc_words] 2 * nnz (real problems with tensor-core supernodes), zero between calls
+    size_t yacc_words = 0;
     int *tcount = nullptr;     // [tile_total], zero between calls
     void *LDu = nullptr;       // LU form: Uhat^T panels
     void *Vt = nullptr;        // LU form: (U_KK^T)^{-1} blocks

@@ -142,3 +142,19 @@ print(json.dumps(N.selinv_plan_get(c.plan, "active").tolist()))
 """)
     sym = oracle.symbolic_for(eval("synth." + make))
     assert _ordered(sym, launches(parts[-1][1])) == {K for K in range(sym.nsuper) if active[K]}
+
+
+@pytest.mark.parametrize("call", ["c.selinv({0})", "batched([c], [{0}])"])
+def test_real_sums_have_room_beside_a_complex_workspace(fake, tmp_path, call):
+    """The mma.sync engine adds split contractions of real values into two
+    words per panel entry, whatever type the plan's workspace was made for."""
+    parts, nnz = run(fake, tmp_path, f"""
+c = Ctx(synth.laplacian_3d(12, 4), use_graph=0)
+assert {call.format(1)} == 0
+c.set(fast_contraction=2)
+mark("run")
+assert {call.format(0)} == 0
+print(c.plan.nnz)
+""")
+    got = [x.yacc for x in launches(parts[-1][1]) if "k_selinv_oz" in x.name]
+    assert got and min(got) >= 16 * nnz
