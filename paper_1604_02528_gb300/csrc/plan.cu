@@ -67,6 +67,7 @@ void Workspace::release() {
     counter = done = nullptr;
     work = nullptr;
     bytes_elem = 0;
+    gen = 0;
 }
 
 // a workspace buffer of `bytes`, recorded for release
@@ -77,6 +78,10 @@ template <typename X> static bool wget(Workspace &w, X **ptr, size_t bytes) {
     *ptr = static_cast<X *>(v);
     return true;
 }
+
+// every set of buffers has a number of its own: a schedule keeps the number of
+// the set that its descriptors point into
+static std::atomic<int64_t> g_workspaces{0};
 
 int Workspace::ensure(const PlanData &p, int dtype) {
     const size_t es = elem_size(dtype);
@@ -89,6 +94,7 @@ int Workspace::ensure(const PlanData &p, int dtype) {
         if (cudaMemset(yacc, 0, sizeof(long long) * ny) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
             return SELINV_ERR_CUDA;
         yacc_words = ny;
+        gen = ++g_workspaces;
         return SELINV_OK;
     }
     release();
@@ -134,6 +140,7 @@ int Workspace::ensure(const PlanData &p, int dtype) {
     if (cudaDeviceSynchronize() != cudaSuccess) return SELINV_ERR_CUDA;
     bytes_elem = es;
     yacc_words = ny;
+    gen = ++g_workspaces;
     return SELINV_OK;
 }
 
@@ -2048,7 +2055,7 @@ static int numeric_prepare(selinv_plan plan, selinv_dtype dtype, const void *L, 
     const bool capturing = st != nullptr && st != cudaStreamLegacy &&
                            (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
     cudaGetLastError();
-    if (S.valid && S.key_dtype == dtype && S.mode == mode && !capturing &&
+    if (S.valid && S.key_dtype == dtype && S.mode == mode && S.key_ws == plan->ws[0].gen && !capturing &&
         (S.key_L != L || S.key_D != D || S.key_Z != Z)) {
         // only the caller's buffers changed: every kernel of the schedule
         // reads them through the device descriptors, so those are rewritten
@@ -2059,7 +2066,7 @@ static int numeric_prepare(selinv_plan plan, selinv_dtype dtype, const void *L, 
         S.key_L = L; S.key_D = D; S.key_Z = Z;
     }
     if (!S.valid || S.key_L != L || S.key_D != D || S.key_Z != Z || S.key_dtype != dtype ||
-        S.mode != mode) {
+        S.mode != mode || S.key_ws != plan->ws[0].gen) {
         std::vector<const PlanData *> plans{&p};
         const bool persist = mode == SELINV_SCHED_PERSISTENT;
         if (persist && (rc = plan->ws[0].ensure_persistent(p))) return rc;
@@ -2075,7 +2082,7 @@ static int numeric_prepare(selinv_plan plan, selinv_dtype dtype, const void *L, 
             S.reset_bytes = {sizeof(int) * (size_t)(p.ns + 1), sizeof(int)};
         }
         S.valid = true;
-        S.key_L = L; S.key_D = D; S.key_Z = Z; S.key_dtype = dtype; S.mode = mode;
+        S.key_L = L; S.key_D = D; S.key_Z = Z; S.key_dtype = dtype; S.mode = mode; S.key_ws = plan->ws[0].gen;
     }
     plan->last_stream = st;
     if (p.opts.debug_checks & 1) {
@@ -2308,7 +2315,7 @@ extern "C" int selinv_numeric_lu(selinv_plan plan, selinv_dtype dtype, const voi
     Schedule &S = plan->lu;
     const int mode = p.opts.schedule == SELINV_SCHED_PLAIN ? SELINV_SCHED_PLAIN : SELINV_SCHED_LEVEL;
     if (!S.valid || S.key_L != L || S.key_D != Ut || S.key_Z != Zl || S.key_Z2 != Zu || S.key_dtype != dtype ||
-        S.mode != mode) {
+        S.mode != mode || S.key_ws != w.gen) {
         ProbDesc d = make_desc(p, w, dtype, L, nullptr, Zl, false);
         d.lu = 1;
         d.symmetrize = 0;
@@ -2323,6 +2330,7 @@ extern "C" int selinv_numeric_lu(selinv_plan plan, selinv_dtype dtype, const voi
         S.spin_limit = p.opts.spin_limit;
         S.valid = true;
         S.key_L = L; S.key_D = Ut; S.key_Z = Zl; S.key_Z2 = Zu; S.key_dtype = dtype; S.mode = mode;
+        S.key_ws = w.gen;
     }
     plan->last_stream = st;
     return run_schedule(S, st, p.opts.use_graph != 0);
@@ -2389,7 +2397,8 @@ extern "C" int selinv_numeric_batched(int nitems, const selinv_plan *plans, cons
         bool same = true;
         for (int i = 0; i < nitems && same; i++)
             same = b.plans[i] == plans[i] && b.dtypes[i] == dtypes[i] && b.L[i] == L[i] &&
-                   b.D[i] == D[i] && b.Z[i] == Z[i] && b.sel_version[i] == plans[i]->data.sel_version;
+                   b.D[i] == D[i] && b.Z[i] == Z[i] && b.sel_version[i] == plans[i]->data.sel_version &&
+                   b.ws_gen[i] == owner->ws[i + 1].gen;
         if (same) { hit = &b; break; }
     }
     for (int i = 0; i < nitems; i++) {
@@ -2422,7 +2431,10 @@ extern "C" int selinv_numeric_batched(int nitems, const selinv_plan *plans, cons
         b.L.assign(L, L + nitems);
         b.D.assign(D, D + nitems);
         b.Z.assign(Z, Z + nitems);
-        for (int i = 0; i < nitems; i++) b.sel_version.push_back(plans[i]->data.sel_version);
+        for (int i = 0; i < nitems; i++) {
+            b.sel_version.push_back(plans[i]->data.sel_version);
+            b.ws_gen.push_back(owner->ws[i + 1].gen);
+        }
         int rc = build_schedule(b.sched, pds, descs, mode);
         if (rc) {
             b.sched.release();

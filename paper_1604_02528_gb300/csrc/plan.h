@@ -107,6 +107,7 @@ struct Workspace {
     void *LDu = nullptr;       // LU form: Uhat^T panels
     void *Vt = nullptr;        // LU form: (U_KK^T)^{-1} blocks
     size_t bytes_elem = 0;
+    int64_t gen = 0;           // number of this set of buffers (0: none)
     std::vector<std::pair<void *, size_t>> owned;   // every buffer above, with its size
     int ensure(const PlanData &p, int dtype);
     int ensure_lu(const PlanData &p);
@@ -169,6 +170,7 @@ struct Schedule {
     int mode = -1;
     const void *key_L = nullptr, *key_D = nullptr, *key_Z = nullptr, *key_Z2 = nullptr;
     int key_dtype = -1;
+    int64_t key_ws = 0;             // Workspace::gen of the buffers in its descriptors
     std::vector<ProbDesc> h_descs;
     std::vector<Item> h_items;
     std::vector<int2> h_work;
@@ -222,6 +224,7 @@ struct BatchEntry {
     std::vector<int> dtypes;
     std::vector<const void *> L, D;
     std::vector<void *> Z;
+    std::vector<int64_t> ws_gen;        // Workspace::gen of each item's
     std::vector<int64_t> sel_version;   // each plan's selection when the schedule was built
     Schedule sched;
 };

@@ -158,3 +158,20 @@ print(c.plan.nnz)
 """)
     got = [x.yacc for x in launches(parts[-1][1]) if "k_selinv_oz" in x.name]
     assert got and min(got) >= 16 * nnz
+
+
+@pytest.mark.parametrize("first,widen", [("c.selinv(0)", "c.lu(1)"), ("c.lu(0)", "c.selinv(1)"), ("c.lu(0)", "c.selinv(2)"),
+                                         ("batched([c, c], [0, 0])", "batched([c, c], [1, 0])")])
+def test_schedules_follow_their_workspace(fake, tmp_path, first, widen):
+    """A workspace made again for a wider type: a schedule kept from before
+    must not run on the buffers that were given back."""
+    parts, _ = run(fake, tmp_path, f"""
+c = Ctx(synth.laplacian_3d(9, 4))
+for call in ({first!r}, {first!r}, {widen!r}):
+    assert eval(call) == 0
+N.selinv_release_cached_memory()
+mark("run")
+assert eval({first!r}) == 0 and eval({first!r}) == 0
+""")
+    got = launches(parts[-1][1])
+    assert got and not any(x.stale for x in got)
