@@ -67,6 +67,7 @@ void Workspace::release() {
     counter = done = nullptr;
     work = nullptr;
     bytes_elem = 0;
+    shape = 0;
     gen = 0;
 }
 
@@ -86,7 +87,7 @@ static std::atomic<int64_t> g_workspaces{0};
 int Workspace::ensure(const PlanData &p, int dtype) {
     const size_t es = elem_size(dtype);
     const size_t ny = (dtype == SELINV_F64 && p.lhs_total > 0) ? 2 * (size_t)p.nnz : 2;   // words of yacc
-    if (LD && bytes_elem >= es) {
+    if (LD && bytes_elem >= es && shape == p.shape) {
         if (yacc_words >= ny) return SELINV_OK;
         // real values in a workspace made for complex ones, which have no such sums
         DeviceGuard g(device);
@@ -140,6 +141,7 @@ int Workspace::ensure(const PlanData &p, int dtype) {
     if (cudaDeviceSynchronize() != cudaSuccess) return SELINV_ERR_CUDA;
     bytes_elem = es;
     yacc_words = ny;
+    shape = p.shape;
     gen = ++g_workspaces;
     return SELINV_OK;
 }
@@ -383,6 +385,15 @@ static int build_plan(PlanData &p, int32_t n, int32_t ns, const int32_t *super_p
         p.part_all += (int64_t)p.ntiles[K] * s * s;
     }
     p.part_all = std::max<int64_t>(p.part_all, 1);
+    // what the sizes and the layouts of a workspace follow from: the widths and
+    // row counts of the supernodes (FNV-1a over 64-bit words, never 0)
+    uint64_t h = 14695981039346656037ull;
+    auto word = [&](uint64_t x) { h = (h ^ x) * 1099511628211ull; };
+    for (int32_t K = 0; K <= ns; K++) {
+        word((uint64_t)super_ptr[K]);
+        word((uint64_t)rowptr[K]);
+    }
+    p.shape = h | 1;
     return SELINV_OK;
 }
 

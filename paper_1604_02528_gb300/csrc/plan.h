@@ -54,6 +54,7 @@ struct PlanData {
     int64_t sel_version = 0;
     int64_t *d_sel_pos = nullptr;
     int nlevels = 0;
+    uint64_t shape = 0;   // hash of the supernodes' widths and row counts
     int64_t nnz = 0, linv_total = 0, part_max = 1, part_all = 1, lhs_total = 0, lhsu_total = 0, tile_total = 0, linvd_total = 0,
             lhsuz_total = 0, linvdz_total = 0;
     // device copies
@@ -108,6 +109,7 @@ struct Workspace {
     void *Vt = nullptr;        // LU form: (U_KK^T)^{-1} blocks
     size_t bytes_elem = 0;
     int64_t gen = 0;           // number of this set of buffers (0: none)
+    uint64_t shape = 0;        // PlanData::shape of the plan that they fit
     std::vector<std::pair<void *, size_t>> owned;   // every buffer above, with its size
     int ensure(const PlanData &p, int dtype);
     int ensure_lu(const PlanData &p);

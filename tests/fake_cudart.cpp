@@ -2,11 +2,12 @@
 // preloaded in front of libcudart, keeps device memory in host memory, runs no
 // kernel and writes one line per call of interest to the file FAKE_CUDART_LOG:
 //
-//   L stream index clock stale yacc name K...   a kernel launch: the stream and its
-//        launch count, the launches of every stream that come before it
+//   L stream index clock stale yacc panels name K...   a kernel launch: the stream and
+//        its launch count, the launches of every stream that come before it
 //        (comma-separated counts), whether its descriptors hold an address of
-//        freed memory, the bytes behind their yacc, the kernel's name and the
-//        supernodes of its work list
+//        freed memory, the bytes behind the first one's yacc and behind the LD
+//        panels of each (comma-separated), the kernel's name and the supernodes
+//        of its work list
 //   G / B / I / T       graph launch, begin of capture, instantiation, record of a timing event
 //
 // A captured launch is logged like an issued one.  fake_fail(what, n) makes the
@@ -69,21 +70,28 @@ cudaError_t launch(const void *fun, void **args, cudaStream_t st) {
     const char *descs = *static_cast<const char **>(args[0]);
     int stale = 0;
     long long yacc = -1;
+    std::string panels = "-";
     if (auto *a = find(descs)) {
         const char *end = a->first + std::min<size_t>(a->second.bytes, 1 << 20);
         for (const char *w = a->first; w + 8 <= end; w += 8) {
             auto *t = find(*reinterpret_cast<void *const *>(w));
             stale |= t && !t->second.live;
         }
+        const auto *d = reinterpret_cast<const selinv::ProbDesc *>(descs);
         if (has("k_selinv_oz")) {
-            auto *t = find(reinterpret_cast<const selinv::ProbDesc *>(descs)->yacc);
+            auto *t = find(d->yacc);
             yacc = t ? (long long)t->second.bytes : 0;
         }
+        if (a->second.bytes % sizeof(*d) == 0)
+            for (size_t i = 0; i < a->second.bytes / sizeof(*d); i++) {
+                auto *t = find(d[i].LD);
+                panels += "," + std::to_string(t ? t->second.bytes : 0);
+            }
     }
     std::fprintf(out(), "L %d %d ", s, ++c[s]);
     for (size_t i = 0; i < before.size(); i++) std::fprintf(out(), "%s%d", i ? "," : "", before[i]);
     if (before.empty()) std::fprintf(out(), "0");
-    std::fprintf(out(), " %d %lld %s", stale, yacc, name.c_str());
+    std::fprintf(out(), " %d %lld %s %s", stale, yacc, panels.c_str(), name.c_str());
     // work lists: (problem, K), (problem, K << 8 | part), Item
     const bool k = has("k_linv<"), k8 = has("k_linv_cols") || has("k_dinv") || has("_digits");
     const bool item = !k && !k8 && !has("reduce") && (has("k_fma_") || has("k_lhat") || has("k_selinv") || has("k_diag"));

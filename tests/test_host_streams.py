@@ -91,9 +91,10 @@ def run(fake, tmp_path, script):
 
 class Launch:
     def __init__(self, f):
-        self.stream, self.index, self.stale, self.yacc, self.name = int(f[1]), int(f[2]), int(f[4]), int(f[5]), f[6]
+        self.stream, self.index, self.stale, self.yacc, self.name = int(f[1]), int(f[2]), int(f[4]), int(f[5]), f[7]
+        self.panels = [int(x) for x in f[6].split(",")[1:]]
         self.clock = [int(x) for x in f[3].split(",")]
-        self.ks = {int(x) for x in f[7:]}
+        self.ks = {int(x) for x in f[8:]}
 
     def after(self, other):
         return other.stream < len(self.clock) and self.clock[other.stream] >= other.index
@@ -175,3 +176,26 @@ assert eval({first!r}) == 0 and eval({first!r}) == 0
 """)
     got = launches(parts[-1][1])
     assert got and not any(x.stale for x in got)
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_batch_workspaces_fit_their_plans(fake, tmp_path, dtype):
+    """An item's place in a batch is taken by a larger problem than before:
+    its workspace has to grow (digit planes, panels, the exact sums)."""
+    parts, sizes = run(fake, tmp_path, f"""
+a, b, c = Ctx(synth.laplacian_3d(7, 4)), Ctx(synth.laplacian_3d(7, 4)), Ctx(synth.laplacian_3d(12, 4))
+for x in (a, b, c):
+    x.set(fast_contraction=2, use_graph=0)
+assert batched([a, b], [{dtype}, {dtype}]) == 0
+mark("run")
+assert batched([a, c], [{dtype}, {dtype}]) == 0
+mark("back")
+assert batched([a, b], [{dtype}, {dtype}]) == 0
+print([x.plan.nnz for x in (a, b, c)])
+""")
+    for lines, want in ((parts[-2][1], [sizes[0], sizes[2]]), (parts[-1][1], sizes[:2])):
+        got = launches(lines)
+        assert got and not any(x.stale for x in got)
+        for x in got:
+            for have, nnz in zip(x.panels, want):
+                assert have >= (16 if dtype else 8) * nnz
