@@ -26,6 +26,11 @@ namespace selinv {
 static std::atomic<int64_t> g_launches{0};
 void note_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+int64_t next_plan_version() {
+    static std::atomic<int64_t> last{0};
+    return ++last;
+}
+
 size_t elem_size(int dtype) { return dtype == SELINV_F64 ? 8 : 16; }
 
 template <typename X, typename A>
@@ -2408,7 +2413,7 @@ extern "C" int selinv_numeric_batched(int nitems, const selinv_plan *plans, cons
         bool same = true;
         for (int i = 0; i < nitems && same; i++)
             same = b.plans[i] == plans[i] && b.dtypes[i] == dtypes[i] && b.L[i] == L[i] &&
-                   b.D[i] == D[i] && b.Z[i] == Z[i] && b.sel_version[i] == plans[i]->data.sel_version &&
+                   b.D[i] == D[i] && b.Z[i] == Z[i] && b.version[i] == plans[i]->data.version &&
                    b.ws_gen[i] == owner->ws[i + 1].gen;
         if (same) { hit = &b; break; }
     }
@@ -2443,7 +2448,7 @@ extern "C" int selinv_numeric_batched(int nitems, const selinv_plan *plans, cons
         b.D.assign(D, D + nitems);
         b.Z.assign(Z, Z + nitems);
         for (int i = 0; i < nitems; i++) {
-            b.sel_version.push_back(plans[i]->data.sel_version);
+            b.version.push_back(plans[i]->data.version);
             b.ws_gen.push_back(owner->ws[i + 1].gen);
         }
         int rc = build_schedule(b.sched, pds, descs, mode);

@@ -29,6 +29,8 @@ template <typename T> struct UninitAlloc : std::allocator<T> {
 };
 template <typename T> using fill_vector = std::vector<T, UninitAlloc<T>>;
 
+int64_t next_plan_version();
+
 struct PlanData {
     int32_t n = 0, ns = 0;
     int device = -1;   // CUDA device of the plan's device arrays (set by ensure_device)
@@ -51,7 +53,7 @@ struct PlanData {
     // positions of the selected entries
     std::vector<uint8_t> active;
     std::vector<int64_t> sel_pos;
-    int64_t sel_version = 0;
+    int64_t version = next_plan_version();   // of this plan and its selection: no two plans ever share one
     int64_t *d_sel_pos = nullptr;
     int nlevels = 0;
     uint64_t shape = 0;   // hash of the supernodes' widths and row counts
@@ -227,7 +229,7 @@ struct BatchEntry {
     std::vector<const void *> L, D;
     std::vector<void *> Z;
     std::vector<int64_t> ws_gen;        // Workspace::gen of each item's
-    std::vector<int64_t> sel_version;   // each plan's selection when the schedule was built
+    std::vector<int64_t> version;       // PlanData::version of each when the schedule was built
     Schedule sched;
 };
 

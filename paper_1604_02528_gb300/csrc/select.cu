@@ -98,7 +98,7 @@ extern "C" int selinv_plan_select(selinv_plan plan, int64_t nsel, const int32_t 
     if (pos_out && nsel > 0) std::memcpy(pos_out, pos.data(), sizeof(int64_t) * (size_t)nsel);
     p.active.swap(active);
     p.sel_pos.swap(pos);
-    p.sel_version++;
+    p.version = next_plan_version();
     if (p.d_sel_pos) cudaFree(p.d_sel_pos);
     p.d_sel_pos = nullptr;
     // schedules built for the previous selection are stale

@@ -199,3 +199,27 @@ print([x.plan.nnz for x in (a, b, c)])
         for x in got:
             for have, nnz in zip(x.panels, want):
                 assert have >= (16 if dtype else 8) * nnz
+
+
+def test_batch_of_a_plan_at_a_destroyed_plans_address(fake, tmp_path):
+    """A batch is recognized by its plans: a new plan whose handle has the
+    address of a destroyed one is another plan."""
+    parts, same = run(fake, tmp_path, """
+a, b = Ctx(synth.laplacian_3d(7, 4)), Ctx(synth.laplacian_3d(7, 4))
+s = N.selinv_analyse(b.p.n, b.p.colptr, b.p.rowind, 1, b.p.supernodes["cap"], b.p.supernodes["fill"])
+args = (b.p.n, s["nsuper"], s["super_ptr"], s["sparent"], s["rowptr"], s["rows"], b.opts)
+assert batched([a, b], [0, 0]) == 0
+old, plans = b.h.value, []
+LIB.selinv_plan_destroy(b.plan.handle)
+b.plan.handle = None
+while len(plans) < 4000 and not (plans and plans[-1].handle.value == old):
+    plans.append(N.selinv_symbolic(*args))
+b.h = plans[-1].handle
+mark("run")
+assert batched([a, b], [0, 0]) == 0
+print(int(b.h.value == old))
+""")
+    got = launches(parts[-1][1])
+    if not same:
+        pytest.skip("the allocator did not hand the address out again")
+    assert got and not any(x.stale for x in got)
