@@ -1951,8 +1951,11 @@ extern "C" int selinv_plan_set_opts(selinv_plan plan, const selinv_opts *opts) {
     if (!plan || !opts || !opts_valid(opts)) return SELINV_ERR_INVALID_ARG;
     plan->data.opts = *opts;
     plan->data.tuned[0] = plan->data.tuned[1] = false;
+    plan->data.version = next_plan_version();   // batches of other owners read this plan's options too
     plan->single.release();
     plan->single.valid = false;
+    plan->lu.release();
+    plan->lu.valid = false;
     for (auto &b : plan->batch_cache) b.sched.release();
     plan->batch_cache.clear();
     return SELINV_OK;

@@ -53,7 +53,7 @@ struct PlanData {
     // positions of the selected entries
     std::vector<uint8_t> active;
     std::vector<int64_t> sel_pos;
-    int64_t version = next_plan_version();   // of this plan and its selection: no two plans ever share one
+    int64_t version = next_plan_version();   // of this plan, its options and its selection: no two plans ever share one
     int64_t *d_sel_pos = nullptr;
     int nlevels = 0;
     uint64_t shape = 0;   // hash of the supernodes' widths and row counts

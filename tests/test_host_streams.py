@@ -223,3 +223,31 @@ print(int(b.h.value == old))
     if not same:
         pytest.skip("the allocator did not hand the address out again")
     assert got and not any(x.stale for x in got)
+
+
+def test_options_of_every_plan_reach_a_batch(fake, tmp_path):
+    parts, _ = run(fake, tmp_path, """
+a, b = Ctx(synth.laplacian_3d(12, 4), fast_contraction=0), Ctx(synth.laplacian_3d(12, 5))
+assert batched([a, b], [0, 0]) == 0
+b.set(fast_contraction=0)
+mark("run")
+assert batched([a, b], [0, 0]) == 0
+""")
+    tensor = [sum("k_selinv_tc" in x.name for x in launches(lines)) for _, lines in parts]
+    assert tensor[0] > 0 and tensor[1] == 0
+
+
+def test_options_reach_the_lu_form(fake, tmp_path):
+    """debug_checks bit 2 sits in the descriptors of a kept schedule."""
+    parts, _ = run(fake, tmp_path, """
+c = Ctx(synth.laplacian_3d(7, 4))
+for _ in range(3):
+    assert c.lu() == 0
+mark("replay")
+assert c.lu() == 0
+c.set(debug_checks=4)
+mark("checked")
+assert c.lu() == 0
+""")
+    assert not launches(parts[1][1])
+    assert launches(parts[2][1])
