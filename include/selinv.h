@@ -100,7 +100,9 @@ typedef struct {
                               the results are then invalid); default 0                 */
     long long spin_limit;  /* polls (about 256 ns each) of every device spin-wait before
                               it gives up and latches SELINV_ERR_TIMEOUT; default 1<<22 */
-    int use_graph;         /* 1: capture the level schedule in a CUDA graph; default 1  */
+    int use_graph;         /* 1: replay the level schedule and the level loops of the
+                              factorization and the adjoints as CUDA graphs; 0: issue
+                              every launch of every call; default 1                     */
     int fast_contraction;  /* contraction of the supernodes with s >= oz_min_s: FP64-exact
                               on fp16 tensor cores (error-free slicing into 8-bit digits,
                               exact integer accumulation) -- 1: tcgen05 with tensor-memory

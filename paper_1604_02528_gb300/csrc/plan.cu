@@ -1727,14 +1727,14 @@ cudaError_t programmatic_edges(cudaGraph_t g) {
     return cudaSuccess;
 }
 
-int CapturedLoop::run(long long want_key, const void *want_ws, cudaStream_t st,
+int CapturedLoop::run(long long want_key, const void *want_ws, cudaStream_t st, bool use_graph,
                       const std::function<void(cudaStream_t)> &body) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool legacy = st == nullptr || st == cudaStreamLegacy;
     const bool capturing = !legacy && (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
     const bool known = key == want_key && ws == want_ws;
-    if (capturing || !known) {
-        if (!capturing) {
+    if (capturing || !use_graph || !known) {
+        if (!capturing && use_graph) {
             if (exec) cudaGraphExecDestroy(exec);
             exec = nullptr;
             key = want_key;

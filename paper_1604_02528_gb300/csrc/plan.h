@@ -251,14 +251,16 @@ cudaError_t programmatic_edges(cudaGraph_t g);
 // only the plan's own device buffers as arguments (the caller's pointers reach
 // the kernels through descriptors uploaded before), so one capture serves
 // every call until the lists (key) or the workspace (ws) change.  A stream
-// that the caller is capturing gets the launches themselves.
+// that the caller is capturing gets the launches themselves, and so does every
+// call with use_graph off.
 struct CapturedLoop {
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap = nullptr;
     int nlaunch = 0;
     long long key = -1;
     const void *ws = nullptr;
-    int run(long long want_key, const void *want_ws, cudaStream_t st, const std::function<void(cudaStream_t)> &body);
+    int run(long long want_key, const void *want_ws, cudaStream_t st, bool use_graph,
+            const std::function<void(cudaStream_t)> &body);
     void release();
 };
 cudaError_t launch_with(const Schedule &S, const Launch &L, const ProbDesc *d, cudaStream_t st);

@@ -251,3 +251,23 @@ assert c.lu() == 0
 """)
     assert not launches(parts[1][1])
     assert launches(parts[2][1])
+
+
+LOOPS = ["c.factor()", "c.adjoint()", "c.factor_adjoint()"]
+
+
+@pytest.mark.parametrize("call", ["c.selinv()", "c.lu()"] + LOOPS)
+@pytest.mark.parametrize("stream", [None, 0x1000000])
+def test_use_graph_0_keeps_every_call_off_graphs(fake, tmp_path, call, stream):
+    parts, _ = run(fake, tmp_path, f"""
+st = {stream}
+c = Ctx(synth.laplacian_3d(9, 4))
+for graph in (1, 0):
+    c.set(use_graph=graph)
+    for _ in range(3):
+        mark(str(graph))
+        assert {call.replace("()", "(stream=st)")} == 0
+""")
+    kinds = [{f[0] for f in lines} for _, lines in parts[1:]]
+    assert "G" in kinds[2]                                   # replayed
+    assert all(k == {"L"} for k in kinds[3:])
