@@ -1791,7 +1791,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
             rest(g, st);
         }
     };
-    return a->g_sel.run(a->gen, w.colexpZ, st, p.opts.use_graph != 0, levels);
+    return a->g_sel.run({a->gen, p.opts.spin_limit}, w.colexpZ, st, p.opts.use_graph != 0, levels);
 }
 
 extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const void *L, const void *D,
@@ -1875,7 +1875,7 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
             launch_gemm(a, OP_FAC_G2, li, li + 1, st);
         }
     };
-    if ((rc = a->g_fac.run(a->gen, w.colexpZ, st, p.opts.use_graph != 0, levels))) return rc;
+    if ((rc = a->g_fac.run({a->gen, p.opts.spin_limit}, w.colexpZ, st, p.opts.use_graph != 0, levels))) return rc;
     if (f->nnzA > 0) {
         const int blocks = (int)std::min<int64_t>((f->nnzA + 255) / 256, 152 * 8);
         k_gather_vals<<<blocks, 256, 0, st>>>(f->d_a_pos, a->Ab, f->nnzA, static_cast<double *>(Abar_vals));

@@ -838,7 +838,7 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         }
     };
     if (cudaGetLastError() != cudaSuccess) return SELINV_ERR_CUDA;
-    return f->loop[sizeof(T) > 8].run(2 * p.opts.spin_limit + tc, f->d_js, st, p.opts.use_graph != 0, levels);
+    return f->loop[sizeof(T) > 8].run({(long long)tc, p.opts.spin_limit}, f->d_js, st, p.opts.use_graph != 0, levels);
 }
 
 }  // namespace selinv

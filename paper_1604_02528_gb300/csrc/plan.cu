@@ -1727,7 +1727,7 @@ cudaError_t programmatic_edges(cudaGraph_t g) {
     return cudaSuccess;
 }
 
-int CapturedLoop::run(long long want_key, const void *want_ws, cudaStream_t st, bool use_graph,
+int CapturedLoop::run(const Key &want_key, const void *want_ws, cudaStream_t st, bool use_graph,
                       const std::function<void(cudaStream_t)> &body) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool legacy = st == nullptr || st == cudaStreamLegacy;
@@ -1769,7 +1769,7 @@ void CapturedLoop::release() {
     if (cap) cudaStreamDestroy(cap);
     exec = nullptr;
     cap = nullptr;
-    key = -1;
+    key = Key{-1, -1};
     ws = nullptr;
 }
 

@@ -254,12 +254,13 @@ cudaError_t programmatic_edges(cudaGraph_t g);
 // that the caller is capturing gets the launches themselves, and so does every
 // call with use_graph off.
 struct CapturedLoop {
+    using Key = std::array<long long, 2>;   // the launch lists; what else the launches take from the options
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap = nullptr;
     int nlaunch = 0;
-    long long key = -1;
+    Key key{-1, -1};
     const void *ws = nullptr;
-    int run(long long want_key, const void *want_ws, cudaStream_t st, bool use_graph,
+    int run(const Key &want_key, const void *want_ws, cudaStream_t st, bool use_graph,
             const std::function<void(cudaStream_t)> &body);
     void release();
 };

@@ -271,3 +271,18 @@ for graph in (1, 0):
     kinds = [{f[0] for f in lines} for _, lines in parts[1:]]
     assert "G" in kinds[2]                                   # replayed
     assert all(k == {"L"} for k in kinds[3:])
+
+
+@pytest.mark.parametrize("call", LOOPS)
+def test_a_new_spin_limit_reaches_every_loop(fake, tmp_path, call):
+    """The bound of the device waits is an argument of the captured launches:
+    a call after it has changed cannot replay them."""
+    parts, _ = run(fake, tmp_path, f"""
+c = Ctx(synth.laplacian_3d(9, 4))
+for limit in (1 << 22, 1 << 23, (1 << 62) + 1):
+    c.set(spin_limit=limit)
+    for _ in range(3):
+        mark(str(limit))
+        assert {call} == 0
+""")
+    assert ["G" in [f[0] for f in lines] for _, lines in parts[1:]] == [False, True, True] * 3
