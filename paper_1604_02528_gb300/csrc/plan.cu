@@ -1749,7 +1749,9 @@ int CapturedLoop::run(const Key &want_key, const void *want_ws, cudaStream_t st,
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
         body(cap);
+        const cudaError_t eb = cudaGetLastError();   // a launch that failed is not in the graph
         cudaError_t e = cudaStreamEndCapture(cap, &g);
+        if (e == cudaSuccess) e = eb;
         nlaunch = (int)(selinv_launch_count() - n0);
         note_launch(-nlaunch);   // captured, not yet issued
         if (e == cudaSuccess && g) e = programmatic_edges(g);

@@ -11,7 +11,8 @@
 //   G / B / I / T       graph launch, begin of capture, instantiation, record of a timing event
 //
 // A captured launch is logged like an issued one.  fake_fail(what, n) makes the
-// next n begins of capture (1) or instantiations (2) fail.
+// next n begins of capture (1), instantiations (2) or cluster launches and
+// launches of k_adj_gemm (3) fail.
 #include <cuda_runtime.h>
 #include <cxxabi.h>
 
@@ -36,7 +37,8 @@ std::map<cudaStream_t, int> g_id;
 std::vector<std::vector<int>> g_clock;      // per stream: launches known to come before its next one
 std::map<cudaEvent_t, std::vector<int>> g_event;
 std::set<cudaEvent_t> g_timing;
-int g_fail[3];
+int g_fail[4];
+cudaError_t g_last = cudaSuccess;            // as cudaGetLastError returns it
 uintptr_t g_next = 0x1000;
 
 FILE *out() {
@@ -60,13 +62,20 @@ void merge(std::vector<int> &a, const std::vector<int> &b) {
     for (size_t i = 0; i < b.size(); i++) a[i] = std::max(a[i], b[i]);
 }
 
-cudaError_t launch(const void *fun, void **args, cudaStream_t st) {
+cudaError_t fails(int what) {
+    if (g_fail[what] <= 0) return cudaSuccess;
+    g_fail[what]--;
+    return g_last = cudaErrorUnknown;
+}
+
+cudaError_t launch(const void *fun, void **args, cudaStream_t st, bool cluster) {
     const int s = id(st);
     std::vector<int> &c = g_clock[s];
     if ((int)c.size() <= s) c.resize(s + 1);
     const std::vector<int> before = c;
     const std::string &name = g_name[fun];
     auto has = [&](const char *x) { return name.find(x) != std::string::npos; };
+    if ((cluster || has("k_adj_gemm")) && fails(3) != cudaSuccess) return cudaErrorUnknown;
     const char *descs = *static_cast<const char **>(args[0]);
     int stale = 0;
     long long yacc = -1;
@@ -107,11 +116,6 @@ cudaError_t launch(const void *fun, void **args, cudaStream_t st) {
     std::fflush(out());
     return cudaSuccess;
 }
-cudaError_t fails(int what) {
-    if (g_fail[what] <= 0) return cudaSuccess;
-    g_fail[what]--;
-    return cudaErrorUnknown;
-}
 void note(const char *what) {
     std::fprintf(out(), "%s\n", what);
     std::fflush(out());
@@ -143,8 +147,8 @@ cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *sh, void *st) {
     *g = g_grid; *b = g_block; *sh = g_shared; *static_cast<void **>(st) = g_stream;
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t, cudaStream_t st) { return launch((const void *)k, args, st); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *cfg, const void *fun, void **args) { return launch(fun, args, cfg->stream); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t, cudaStream_t st) { return launch((const void *)k, args, st, false); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *cfg, const void *fun, void **args) { return launch(fun, args, cfg->stream, true); }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
     if (posix_memalign(p, 256, n ? n : 1)) return cudaErrorMemoryAllocation;
@@ -170,7 +174,7 @@ cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() { const cudaError_t e = g_last; g_last = cudaSuccess; return e; }
 cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) { *n = 1; return cudaSuccess; }
 

@@ -286,3 +286,17 @@ for limit in (1 << 22, 1 << 23, (1 << 62) + 1):
         assert {call} == 0
 """)
     assert ["G" in [f[0] for f in lines] for _, lines in parts[1:]] == [False, True, True] * 3
+
+
+@pytest.mark.parametrize("call", LOOPS)
+def test_a_launch_that_fails_under_capture_is_reported(fake, tmp_path, call):
+    """A kernel that cannot be launched must not drop out of the graph unnoticed."""
+    _, rc = run(fake, tmp_path, f"""
+c = Ctx(synth.laplacian_3d(9, 4))
+assert {call} == 0
+RT.fake_fail(3, 1 << 30)
+rc = [{call}, {call}]
+RT.fake_fail(3, 0)
+print(rc + [{call}, {call}])
+""")
+    assert rc == [-7, -7, 0, 0]
