@@ -1727,40 +1727,50 @@ cudaError_t programmatic_edges(cudaGraph_t g) {
     return cudaSuccess;
 }
 
+// body(cs) captured on the stream cs and instantiated; nothing is left behind
+// where it cannot be
+static cudaError_t capture(cudaStream_t cs, cudaGraphExec_t *exec, const std::function<cudaError_t(cudaStream_t)> &body) {
+    *exec = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    cudaGraph_t g = nullptr;
+    const cudaError_t eb = body(cs);
+    e = cudaStreamEndCapture(cs, &g);
+    if (eb != cudaSuccess) e = eb;
+    if (e == cudaSuccess) e = g ? programmatic_edges(g) : cudaErrorUnknown;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) *exec = nullptr;
+    return e;
+}
+
 int CapturedLoop::run(const Key &want_key, const void *want_ws, cudaStream_t st, bool use_graph,
                       const std::function<void(cudaStream_t)> &body) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool legacy = st == nullptr || st == cudaStreamLegacy;
     const bool capturing = !legacy && (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
     const bool known = key == want_key && ws == want_ws;
-    if (capturing || !use_graph || !known) {
-        if (!capturing && use_graph) {
-            if (exec) cudaGraphExecDestroy(exec);
-            exec = nullptr;
-            key = want_key;
-            ws = want_ws;
-        }
-        body(st);
-        return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
+    if (!capturing && use_graph && !known) {
+        if (exec) cudaGraphExecDestroy(exec);
+        exec = nullptr;
+        key = want_key;
+        ws = want_ws;
     }
-    if (!exec) {
-        if (!cap && cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return SELINV_ERR_CUDA;
+    if (!capturing && use_graph && known && !exec) {
         const int64_t n0 = selinv_launch_count();
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
-        body(cap);
-        const cudaError_t eb = cudaGetLastError();   // a launch that failed is not in the graph
-        cudaError_t e = cudaStreamEndCapture(cap, &g);
-        if (e == cudaSuccess) e = eb;
+        cudaError_t e = cap ? cudaSuccess : cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+        if (e == cudaSuccess)
+            e = capture(cap, &exec, [&](cudaStream_t c) {
+                body(c);
+                return cudaGetLastError();   // a launch that failed is not in the graph
+            });
         nlaunch = (int)(selinv_launch_count() - n0);
         note_launch(-nlaunch);   // captured, not yet issued
-        if (e == cudaSuccess && g) e = programmatic_edges(g);
-        if (e == cudaSuccess && g) e = cudaGraphInstantiate(&exec, g, 0);
-        if (g) cudaGraphDestroy(g);
-        if (e != cudaSuccess || !g) {
-            exec = nullptr;
-            return SELINV_ERR_CUDA;
-        }
+        if (e != cudaSuccess) cudaGetLastError();
+    }
+    if (capturing || !use_graph || !known || !exec) {   // (no graph could be made: the launches themselves)
+        body(st);
+        return cudaGetLastError() == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
     }
     note_launch(nlaunch);
     return cudaGraphLaunch(exec, st) == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
@@ -1782,30 +1792,16 @@ int run_schedule(Schedule &S, cudaStream_t st, bool use_graph) {
     const bool legacy = st == nullptr || st == cudaStreamLegacy;
     const bool first = !S.issued;
     S.issued = true;
-    if (use_graph && (S.graph || !legacy || !first)) {
-        if (!S.graph) {
-            cudaGraph_t g = nullptr;
-            if (legacy && !S.cap && cudaStreamCreateWithFlags(&S.cap, cudaStreamNonBlocking) != cudaSuccess)
-                return SELINV_ERR_CUDA;
-            cudaStream_t cs = legacy ? S.cap : st;
-            if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SELINV_ERR_CUDA;
-            cudaError_t e = issue(S, cs, false);
-            cudaError_t e2 = cudaStreamEndCapture(cs, &g);
-            if (e != cudaSuccess || e2 != cudaSuccess) {
-                if (g) cudaGraphDestroy(g);
-                return SELINV_ERR_CUDA;
-            }
-            if (programmatic_edges(g) != cudaSuccess) {
-                cudaGraphDestroy(g);
-                return SELINV_ERR_CUDA;
-            }
-            e = cudaGraphInstantiate(&S.graph, g, 0);
-            cudaGraphDestroy(g);
-            if (e != cudaSuccess) {
-                S.graph = nullptr;
-                return SELINV_ERR_CUDA;
-            }
+    if (use_graph && !S.graph && (!legacy || !first)) {
+        cudaError_t e = cudaSuccess;
+        if (legacy && !S.cap) e = cudaStreamCreateWithFlags(&S.cap, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = capture(legacy ? S.cap : st, &S.graph, [&](cudaStream_t c) { return issue(S, c, false); });
+        if (e != cudaSuccess) {
+            if (!legacy) return SELINV_ERR_CUDA;
+            cudaGetLastError();   // the default stream needs no graph: the launches themselves
         }
+    }
+    if (use_graph && S.graph) {
         note_launch((int)S.launches.size());
         return cudaGraphLaunch(S.graph, st) == cudaSuccess ? SELINV_OK : SELINV_ERR_CUDA;
     }

@@ -300,3 +300,29 @@ RT.fake_fail(3, 0)
 print(rc + [{call}, {call}])
 """)
     assert rc == [-7, -7, 0, 0]
+@pytest.mark.parametrize("what", [1, 2])
+@pytest.mark.parametrize("call", ["c.selinv()", "c.lu()", "batched([c], [0])"] + LOOPS)
+def test_default_stream_runs_without_a_graph_where_none_can_be_made(fake, tmp_path, call, what):
+    """No capture (1) or no instantiation (2): the launches themselves go out,
+    once, and are counted."""
+    parts, n = run(fake, tmp_path, f"""
+c = Ctx(synth.laplacian_3d(9, 4))
+count = []
+for k in range(4):
+    RT.fake_fail({what}, 1 if k == 1 else 0)
+    before = LIB.selinv_launch_count()
+    mark(str(k))
+    assert {call} == 0
+    count.append(LIB.selinv_launch_count() - before)
+print(count)
+""")
+    want = [x.name for x in launches(parts[1][1])]
+    lines = parts[2][1]                                       # the call that cannot capture
+    kinds = [f[0] for f in lines]
+    begin, end = kinds.index("B"), kinds.index("I") if what == 2 else kinds.index("B")
+    names = lambda part: [x.name for x in launches(part)]     # noqa: E731
+    assert names(lines[:begin]) + names(lines[end:]) == want and "G" not in kinds
+    assert all("G" in [f[0] for f in p[1]] for p in parts[3:])
+    assert len(set(n)) == 1
+
+
