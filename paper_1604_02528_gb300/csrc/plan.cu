@@ -1967,7 +1967,7 @@ static int numeric_run(selinv_plan plan, selinv_dtype dtype, const void *L, cons
 // Autotuner: coordinate search over the tensor engine, the k-split of narrow
 // levels and the narrowest tensor-core supernode, each candidate timed with
 // CUDA events on the caller's stream and data (best of two runs after a
-// warm-up that builds its schedule); the fastest options stay with the plan.
+// warm-up that builds its schedule and its graph); the fastest options stay with the plan.
 static int autotune(selinv_plan plan, selinv_dtype dtype, const void *L, const void *D, void *Z,
                     cudaStream_t st) {
     PlanData &p = plan->data;
@@ -1980,6 +1980,8 @@ static int autotune(selinv_plan plan, selinv_dtype dtype, const void *L, const v
         plan->single.release();
         plan->single.valid = false;
         int rc = numeric_run(plan, dtype, L, D, Z, st);
+        // (the default stream's graph is made by the second call)
+        if (!rc && o.use_graph && !plan->single.graph) rc = numeric_run(plan, dtype, L, D, Z, st);
         if (rc) return rc;
         float best = 1e30f;
         for (int r = 0; r < 2; r++) {

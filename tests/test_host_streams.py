@@ -326,3 +326,20 @@ print(count)
     assert len(set(n)) == 1
 
 
+
+
+@pytest.mark.parametrize("stream", [None, 0x1000000])
+def test_autotuner_times_replays_only(fake, tmp_path, stream):
+    """What a candidate's timed runs contain is what later calls will do: no
+    capture and no instantiation between the two events of a run."""
+    parts, _ = run(fake, tmp_path, f"""
+c = Ctx(synth.laplacian_3d(7, 4), autotune=1)
+assert c.selinv(stream={stream}) == 0
+""")
+    kinds = [f[0] for f in parts[0][1]]
+    timed, inside = 0, False
+    for k in kinds:
+        if k == "T":
+            inside, timed = not inside, timed + 1
+        assert not (inside and k in "BIL")
+    assert timed >= 4 and not inside
