@@ -770,7 +770,7 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         f->U_bytes = ubytes;
     }
     // real updates on the tensor cores unless the plan asks for FP64 FMA
-    const bool tc = sizeof(T) == 8 && p.opts.fast_contraction == 1 && f->dig_total > 0;
+    const bool tc = sizeof(T) == 8 && p.asked.fast_contraction == 1 && f->dig_total > 0;
     if (tc && !f->digits) {
         if (cudaMalloc(&f->digexp, sizeof(int) * (size_t)p.rowptr[p.ns]) != cudaSuccess) return SELINV_ERR_OOM;
         if (cudaMalloc(&f->digits, sizeof(uint16_t) * (size_t)f->dig_total) != cudaSuccess) return SELINV_ERR_OOM;

@@ -1856,6 +1856,7 @@ extern "C" int selinv_symbolic(int32_t n, int32_t nsuper, const int32_t *super_p
     } else {
         selinv_default_opts(&pl->data.opts);
     }
+    pl->data.asked = pl->data.opts;
     int rc;
     try {
         rc = build_plan(pl->data, n, nsuper, super_ptr, sparent, rowptr, rowind);
@@ -1947,7 +1948,7 @@ extern "C" int selinv_plan_get_opts(selinv_plan plan, selinv_opts *opts) {
 
 extern "C" int selinv_plan_set_opts(selinv_plan plan, const selinv_opts *opts) {
     if (!plan || !opts || !opts_valid(opts)) return SELINV_ERR_INVALID_ARG;
-    plan->data.opts = *opts;
+    plan->data.opts = plan->data.asked = *opts;
     plan->data.tuned[0] = plan->data.tuned[1] = false;
     plan->data.version = next_plan_version();   // batches of other owners read this plan's options too
     plan->single.release();

@@ -35,6 +35,7 @@ struct PlanData {
     int32_t n = 0, ns = 0;
     int device = -1;   // CUDA device of the plan's device arrays (set by ensure_device)
     selinv_opts opts{};
+    selinv_opts asked{};   // as the caller gave them: the autotuner changes opts, by the inversion's times
     bool tuned[3] = {false, false, false};   // autotuning done, per selinv_dtype
     // host arrays (kept for inspection and schedule building)
     std::vector<int32_t> super_ptr, sparent, rows, level, level_list;

@@ -12,7 +12,8 @@
 //
 // A captured launch is logged like an issued one.  fake_fail(what, n) makes the
 // next n begins of capture (1), instantiations (2) or cluster launches and
-// launches of k_adj_gemm (3) fail.
+// launches of k_adj_gemm (3) fail; every timed run takes 1 ms, those of the
+// autotuner's next fake_slow(n) candidates 2.
 #include <cuda_runtime.h>
 #include <cxxabi.h>
 
@@ -124,6 +125,8 @@ void note(const char *what) {
 
 extern "C" {
 void fake_fail(int what, int n) { g_fail[what] = n; }
+static int g_slow;
+void fake_slow(int candidates) { g_slow = 2 * candidates; }   // two timed runs each
 
 void **__cudaRegisterFatBinary(void *) { static void *h; return &h; }
 void __cudaRegisterFatBinaryEnd(void **) {}
@@ -193,7 +196,7 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
     return cudaSuccess;
 }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 1.0f; return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = g_slow-- > 0 ? 2.0f : 1.0f; return cudaSuccess; }
 
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { note("B"); return fails(1); }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) { *g = handle<cudaGraph_t>(); return cudaSuccess; }

@@ -343,3 +343,30 @@ assert c.selinv(stream={stream}) == 0
             inside, timed = not inside, timed + 1
         assert not (inside and k in "BIL")
     assert timed >= 4 and not inside
+
+
+def _syrk(lines):
+    return set().union(*([set()] + [x.ks for x in launches(lines) if x.name.endswith("k_selinv_tcw<false,_false,_2>")]))
+
+
+def test_factorization_keeps_the_callers_engine(fake, tmp_path):
+    """What the autotuner settles on by timing the inversion must not change
+    the arithmetic of the factorization."""
+    parts, tuned = run(fake, tmp_path, """
+out = []
+for engine in (1, 0):
+    c = Ctx(synth.laplacian_3d(12, 4), autotune=1, fast_contraction=engine, use_graph=0)
+    mark("before")
+    assert c.factor() == 0
+    mark("tuning")
+    RT.fake_slow(1 if engine else 0)
+    assert c.selinv() == 0
+    out.append(N.selinv_plan_get_opts(c.plan).fast_contraction)
+    mark("after")
+    assert c.factor() == 0
+print(out)
+""")
+    on, off = (parts[1][1], parts[3][1]), (parts[4][1], parts[6][1])
+    assert tuned == [2, 1]
+    assert _syrk(on[0]) and _syrk(on[0]) == _syrk(on[1])
+    assert not _syrk(off[0]) and not _syrk(off[1])
