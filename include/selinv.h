@@ -113,7 +113,9 @@ typedef struct {
     int split_min_steps;   /* smallest k-range of a split item, in 16-row steps (8..64,
                               a multiple of 8); default 16                              */
     int oz_min_s;          /* narrowest supernode (columns) that uses the tensor-core
-                              contraction (1..128); default 16                          */
+                              contraction (1..128); default 16.  This and
+                              fast_contraction also choose the arithmetic of
+                              selinv_factor's real updates (see there)                  */
 } selinv_opts;
 
 /* Fills *opts with the defaults listed above. */
@@ -251,6 +253,17 @@ int selinv_numeric_batched(int nitems, const selinv_plan *plans, const selinv_dt
  * given to selinv_analyse (host arrays, copied).  A_vals_dev holds the values
  * of that CSC on the device.  Writes L (panels) and D.  A zero pivot latches
  * SELINV_ERR_ZERO_PIVOT in the status word (the factors are then invalid).
+ * Real updates of supernodes of max(17, oz_min_s) columns or more with 96 rows
+ * or more below them run on the tensor cores when the caller's
+ * fast_contraction is 1 (the options as given to selinv_symbolic or
+ * selinv_plan_set_opts: autotuning does not change them here), everything
+ * else in FP64 FMA.  Both keep |A - L D L^T|_ij within a modest multiple of
+ * n 2^-53 sqrt(S_ii S_jj), S_ii = sum_k |L_ik|^2 |D_k|, definite or not.  FMA's
+ * error is also small against the single products of an entry,
+ * sum_k |L_ik D_k L_jk|; the tensor-core form rounds each row of L sqrt(|D|)
+ * to 53 bits below its largest entry, so an entry whose products lie far below
+ * sqrt(S_ii S_jj) can lose relative accuracy.  A caller that needs those
+ * entries sets fast_contraction = 0 (or oz_min_s = 128).
  * ------------------------------------------------------------------------- */
 int selinv_plan_set_matrix(selinv_plan plan, int32_t n, const int64_t *colptr,
                            const int32_t *rowind);

@@ -35,7 +35,8 @@ namespace cg = cooperative_groups;
 
 constexpr int kFSmallS = 16;        // widest supernode of k_fsmall
 constexpr int kFSmallElems = 3400;  // ... and its largest panel (both copies of a complex one in 109 KB)
-// narrowest supernode and shortest C of the tcgen05 update: one of its
+// narrowest supernode (with the caller's oz_min_s, if that is wider) and
+// shortest C of the tcgen05 update: one of its
 // CTAs takes about as long as the FP64 pipe of an SM needs for 16 columns of
 // a 128 x 64 tile, and below 96 rows most of that tile is padding
 constexpr int kFTcS = 17, kFTcC = 96;
@@ -521,13 +522,20 @@ __global__ void __launch_bounds__(kFsThreads) k_fsmall(const FactorDesc *__restr
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
+void FactorLists::release() {
+    for (void *q : {(void *)d_tiles, (void *)d_js, (void *)d_uitems, (void *)d_tcitems, (void *)d_tcwork, (void *)d_digoff})
+        if (q) cudaFree(q);
+}
+
 void factor_release(selinv_plan_s *plan) {
     FactorData *f = plan->factor;
     if (!f) return;
     auto fr = [](void *p) { if (p) cudaFree(p); };
-    fr(f->d_a_pos); fr(f->d_tiles); fr(f->d_js); fr(f->d_desc);
-    fr(f->d_asm); fr(f->d_uitems); fr(f->d_uoff); fr(f->d_chpos); fr(f->U);
-    fr(f->d_tcitems); fr(f->d_tcwork); fr(f->d_digoff); fr(f->digits); fr(f->digexp);
+    fr(f->d_a_pos); fr(f->d_desc);
+    fr(f->d_asm); fr(f->d_uoff); fr(f->d_chpos); fr(f->U);
+    fr(f->digits); fr(f->digexp);
+    for (auto &l : f->lists)
+        if (l.second) l.second->release();
     for (CapturedLoop &g : f->loop) g.release();
     adjoint_release(f->adj);
     delete f;
@@ -543,17 +551,22 @@ static int up(X **d, const std::vector<X> &h) {
     return SELINV_OK;
 }
 
-// launch lists and update-matrix tables, shared by the factorization and
-// the selected-inversion adjoint
-int factor_tables(selinv_plan_s *plan) {
+// the factorization's launch lists for the narrowest tensor-core supernode tc_s:
+// made once for each value that the caller sets, and kept (a caller's own
+// graph may hold their addresses)
+static int factor_lists(selinv_plan_s *plan, int tc_s, FactorLists **out) {
     FactorData *f = plan->factor;
-    if (f->d_desc) return SELINV_OK;
     const PlanData &p = plan->data;
-    int rc = ensure_device(plan->data);
-    if (rc) return rc;
+    std::unique_ptr<FactorLists> &slot = f->lists[tc_s];
+    if (slot) {
+        *out = slot.get();
+        return SELINV_OK;
+    }
+    std::unique_ptr<FactorLists> made(new FactorLists());
+    FactorLists *q = made.get();
+    int64_t dig_total = 0;   // of every supernode that some tc_s takes
     // per-level launch lists, leaves first: the narrow supernodes, then the
     // others' diagonal blocks and row tiles
-    f->lev.clear();
     std::vector<int> js;
     std::vector<int4> tiles, uitems;
     std::vector<Item> tcitems;
@@ -615,7 +628,7 @@ int factor_tables(selinv_plan_s *plan) {
         v.tile1 = (int64_t)tiles.size();
         // update tiles: the side (64, 32, 16) whose waves over the SMs multiply
         // least, for all of them and for those that the tcgen05 form leaves
-        auto tc = [&](int32_t J) { return width(J) >= kFTcS && below(J) >= kFTcC; };
+        auto tc = [&](int32_t J) { return width(J) >= tc_s && below(J) >= kFTcC; };
         for (int part = 0; part < 2; part++) {
             FactorLevel::Upd &u = v.upd[part];
             int64_t best = INT64_MAX;
@@ -645,20 +658,44 @@ int factor_tables(selinv_plan_s *plan) {
         v.tc0 = (int64_t)tcitems.size();
         v.tw0 = (int64_t)tcwork.size();
         int64_t dig = 0;
+        int64_t any = 0;
         for (int32_t J : wide) {
+            const int64_t planes = (int64_t)((below(J) + 127) / 128) * 7 * 128 * ((width(J) + 15) / 16 * 16);
+            if (width(J) >= kFTcS && below(J) >= kFTcC) any += planes;
             if (!tc(J)) continue;
             const int c = below(J), n2 = (c + 63) / 64;
             for (int m = 0; m < (c + 127) / 128; m++)
                 for (int t = 0; t < n2 && 64 * t <= 128 * m + 127; t++) tcitems.push_back(Item{0, J, m * n2 + t, 1});
             for (int b = 0; b < (c + 31) / 32; b++) tcwork.push_back(make_int2(J, b));
             digoff[J] = dig;
-            dig += (int64_t)((c + 127) / 128) * 7 * 128 * ((width(J) + 15) / 16 * 16);
+            dig += planes;
         }
         v.tc1 = (int64_t)tcitems.size();
+        q->tc = q->tc || v.tc1 > v.tc0;
         v.tw1 = (int64_t)tcwork.size();
-        f->dig_total = std::max(f->dig_total, dig);
-        f->lev.push_back(v);
+        dig_total = std::max(dig_total, any);
+        q->lev.push_back(v);
     }
+    int rc;
+    if ((rc = up(&q->d_tiles, tiles)) || (rc = up(&q->d_js, js)) || (rc = up(&q->d_uitems, uitems)) ||
+        (rc = up(&q->d_tcitems, tcitems)) || (rc = up(&q->d_tcwork, tcwork)) || (rc = up(&q->d_digoff, digoff))) {
+        q->release();
+        return rc;
+    }
+    f->dig_total = dig_total;
+    slot = std::move(made);
+    *out = q;
+    return SELINV_OK;
+}
+
+// update-matrix tables, shared by the factorization and the selected-inversion
+// adjoint
+int factor_tables(selinv_plan_s *plan) {
+    FactorData *f = plan->factor;
+    if (f->d_desc) return SELINV_OK;
+    const PlanData &p = plan->data;
+    int rc = ensure_device(plan->data);
+    if (rc) return rc;
     // update matrices: offsets; the position of every C_K entry in its
     // parent's row list (closure: C_K lies inside rows(parent)); children by rank
     f->u_off.assign(p.ns + 1, 0);
@@ -702,20 +739,14 @@ int factor_tables(selinv_plan_s *plan) {
             f->asm_lptr.push_back((int64_t)f->asm_items.size());
         }
     }
-    if ((rc = up(&f->d_tiles, tiles))) return rc;
-    if ((rc = up(&f->d_js, js))) return rc;
     if ((rc = up(&f->d_asm, f->asm_items))) return rc;
-    if ((rc = up(&f->d_uitems, uitems))) return rc;
-    if ((rc = up(&f->d_tcitems, tcitems))) return rc;
-    if ((rc = up(&f->d_tcwork, tcwork))) return rc;
-    if ((rc = up(&f->d_digoff, digoff))) return rc;
     if ((rc = up(&f->d_uoff, f->u_off))) return rc;
     if ((rc = up(&f->d_chpos, f->chpos))) return rc;
     if (cudaMalloc((void **)&f->d_desc, sizeof(FactorDesc)) != cudaSuccess) return SELINV_ERR_OOM;
     return SELINV_OK;
 }
 
-FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, int herm) {
+static FactorDesc *factor_desc(selinv_plan_s *plan, const FactorLists *q, void *L, void *D, cudaStream_t st, int herm) {
     FactorData *f = plan->factor;
     const PlanData &p = plan->data;
     FactorDesc h = {};
@@ -726,7 +757,7 @@ FactorDesc *factor_desc(selinv_plan_s *plan, void *L, void *D, cudaStream_t st, 
     h.up.L = L;
     h.up.D = D;
     h.up.linvd = f->digits;
-    h.up.linvd_off = f->d_digoff;
+    h.up.linvd_off = q->d_digoff;
     h.up.linvexp = f->digexp;
     h.up.Yout = f->U;
     h.up.part_off = f->d_uoff;
@@ -760,6 +791,9 @@ template <typename T> static cudaError_t configure_factor_kernels() {
 template <typename T>
 static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaStream_t st, int herm) {
     FactorData *f = plan->factor;
+    const int tc_s = std::max(kFTcS, plan->data.asked.oz_min_s);
+    FactorLists *q = nullptr;
+    if (const int rc = factor_lists(plan, tc_s, &q)) return rc;
     const PlanData &p = plan->data;
     const size_t ubytes = sizeof(T) * (size_t)std::max<int64_t>(f->u_off[p.ns], 1);
     if (f->U_bytes < ubytes) {
@@ -770,12 +804,12 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         f->U_bytes = ubytes;
     }
     // real updates on the tensor cores unless the plan asks for FP64 FMA
-    const bool tc = sizeof(T) == 8 && p.asked.fast_contraction == 1 && f->dig_total > 0;
+    const bool tc = sizeof(T) == 8 && p.asked.fast_contraction == 1 && q->tc;
     if (tc && !f->digits) {
         if (cudaMalloc(&f->digexp, sizeof(int) * (size_t)p.rowptr[p.ns]) != cudaSuccess) return SELINV_ERR_OOM;
         if (cudaMalloc(&f->digits, sizeof(uint16_t) * (size_t)f->dig_total) != cudaSuccess) return SELINV_ERR_OOM;
     }
-    FactorDesc *fd = factor_desc(plan, L, D, st, herm);
+    FactorDesc *fd = factor_desc(plan, q, L, D, st, herm);
     if (cudaMemsetAsync(L, 0, sizeof(T) * (size_t)p.nnz, st) != cudaSuccess) return SELINV_ERR_CUDA;
     if (cudaMemsetAsync(f->U, 0, ubytes, st) != cudaSuccess) return SELINV_ERR_CUDA;
     if (f->nnzA > 0) {
@@ -788,16 +822,16 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         f->configured[sizeof(T) > 8] = true;
     }
     auto levels = [&](cudaStream_t st) {
-        for (size_t l = 0; l < f->lev.size(); l++) {
+        for (size_t l = 0; l < q->lev.size(); l++) {
             // the children's update matrices complete J's panel and start U_J
             for (int r = 0; r < f->npass; r++) {
                 const int64_t x0 = f->asm_lptr[l * f->npass + r], x1 = f->asm_lptr[l * f->npass + r + 1];
                 if (x1 > x0) { k_fasm<T><<<(int)(x1 - x0), 256, 0, st>>>(fd, f->d_asm + x0, (int)(x1 - x0)); note_launch(); }
             }
-            const FactorLevel &v = f->lev[l];
+            const FactorLevel &v = q->lev[l];
             if (v.wide0 > v.small0) {
                 k_fsmall<T><<<(int)(v.wide0 - v.small0), kFsThreads, 2 * sizeof(T) * (size_t)v.small_elems, st>>>(
-                    fd, f->d_js + v.small0, (int)(v.wide0 - v.small0));
+                    fd, q->d_js + v.small0, (int)(v.wide0 - v.small0));
                 note_launch();
             }
             if (v.wide1 > v.wide0) {
@@ -812,33 +846,33 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
                 at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
                 cfg.attrs = at;
                 cfg.numAttrs = 1;
-                cudaLaunchKernelEx(&cfg, k_fdiag<T>, (const FactorDesc *)fd, (const int *)(f->d_js + v.wide0),
+                cudaLaunchKernelEx(&cfg, k_fdiag<T>, (const FactorDesc *)fd, (const int *)(q->d_js + v.wide0),
                                    (int)(v.wide1 - v.wide0));   // (an error stays for cudaGetLastError)
                 note_launch();
             }
             if (v.tile1 > v.tile0) {
                 k_ftrsm<T><<<(int)(v.tile1 - v.tile0), kFtThreads, sizeof(T) * (size_t)tri_store_elems(v.wide_s), st>>>(
-                    fd, f->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
+                    fd, q->d_tiles + v.tile0, (int)(v.tile1 - v.tile0));
                 note_launch();
             }
             const FactorLevel::Upd &u = v.upd[tc];
             if (u.i1 > u.i0) {
                 const int nu = (int)(u.i1 - u.i0);
-                if (u.b == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
-                else if (u.b == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
-                else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, f->d_uitems + u.i0, nu);
+                if (u.b == 64) k_fupd<T, 64><<<nu, 256, 0, st>>>(fd, q->d_uitems + u.i0, nu);
+                else if (u.b == 32) k_fupd<T, 32><<<nu, 256, 0, st>>>(fd, q->d_uitems + u.i0, nu);
+                else k_fupd<T, 16><<<nu, 256, 0, st>>>(fd, q->d_uitems + u.i0, nu);
                 note_launch();
             }
             if (tc && v.tc1 > v.tc0) {
                 const int nw = (int)(v.tw1 - v.tw0);
-                k_fupd_digits<<<nw, 256, 0, st>>>(fd, f->d_tcwork + v.tw0, nw);
-                launch_syrk_tcw(2, &fd->up, f->d_tcitems + v.tc0, (int)(v.tc1 - v.tc0), p.opts.spin_limit, st);
+                k_fupd_digits<<<nw, 256, 0, st>>>(fd, q->d_tcwork + v.tw0, nw);
+                launch_syrk_tcw(2, &fd->up, q->d_tcitems + v.tc0, (int)(v.tc1 - v.tc0), p.opts.spin_limit, st);
                 note_launch(2);
             }
         }
     };
     if (cudaGetLastError() != cudaSuccess) return SELINV_ERR_CUDA;
-    return f->loop[sizeof(T) > 8].run({(long long)tc, p.opts.spin_limit}, f->d_js, st, p.opts.use_graph != 0, levels);
+    return f->loop[sizeof(T) > 8].run({2 * tc_s + tc, p.opts.spin_limit}, f, st, p.opts.use_graph != 0, levels);
 }
 
 }  // namespace selinv

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <array>
 #include <functional>
+#include <map>
 #include <memory>
 #include <utility>
 #include <vector>
@@ -296,16 +297,26 @@ struct FactorLevel {
     int cl = 1;                                 // CTAs per diagonal block
 };
 
+// The factorization's launch lists, leaves first.
+struct FactorLists {
+    std::vector<FactorLevel> lev;
+    bool tc = false;                  // some level has tcgen05 updates
+    int4 *d_tiles = nullptr;          // (J, first row of C, rows)
+    int *d_js = nullptr;
+    int4 *d_uitems = nullptr;         // (K, row tile, column tile) of the lower c x c
+    Item *d_tcitems = nullptr;        // tcgen05 form of the update
+    int2 *d_tcwork = nullptr;         // (K, 32-row block) of its digit planes
+    int64_t *d_digoff = nullptr;      // [ns] where K's digit planes start (per level, one buffer)
+    void release();
+};
+
 struct FactorData {
     int32_t n = -1;
     int64_t nnzA = 0;
     std::vector<int64_t> a_pos;       // panel position of every stored entry of A
     int64_t *d_a_pos = nullptr;
-    // launch lists, leaves first
-    std::vector<FactorLevel> lev;
+    std::map<int, std::unique_ptr<FactorLists>> lists;   // by the narrowest supernode of the tcgen05 updates
     bool configured[2] = {false, false};   // kernel attributes set (real, complex)
-    int4 *d_tiles = nullptr;          // (J, first row of C, rows)
-    int *d_js = nullptr;
     // update matrices (multifrontal hand-off from child to parent; shared
     // with the selected-inversion adjoint)
     std::vector<int64_t> u_off;
@@ -314,11 +325,7 @@ struct FactorData {
     std::vector<int64_t> asm_lptr;    // [level * npass + rank]
     int npass = 1;
     int2 *d_asm = nullptr;
-    int4 *d_uitems = nullptr;         // (K, row tile, column tile) of the lower c x c
-    Item *d_tcitems = nullptr;        // tcgen05 form of the update
-    int2 *d_tcwork = nullptr;         // (K, 32-row block) of its digit planes
-    int64_t *d_digoff = nullptr;      // [ns] where K's digit planes start (per level, one buffer)
-    int64_t dig_total = 0;
+    int64_t dig_total = 0;            // elements of the tcgen05 updates' digit planes
     uint16_t *digits = nullptr;
     int *digexp = nullptr;            // row exponents, by row-list position
     int64_t *d_uoff = nullptr;

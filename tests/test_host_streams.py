@@ -370,3 +370,26 @@ print(out)
     assert tuned == [2, 1]
     assert _syrk(on[0]) and _syrk(on[0]) == _syrk(on[1])
     assert not _syrk(off[0]) and not _syrk(off[1])
+
+
+def test_factorization_follows_oz_min_s(fake, tmp_path):
+    """Narrower supernodes than the caller's oz_min_s keep FP64 updates; the
+    lists follow a later change, under replay too."""
+    parts, _ = run(fake, tmp_path, """
+c = Ctx(synth.laplacian_3d(12, 4))
+for ozm in (16, 40, 128, 16):
+    c.set(oz_min_s=ozm)
+    for k in range(3):
+        mark(str(ozm))
+        assert c.factor() == 0
+""")
+    sym = oracle.symbolic_for(synth.laplacian_3d(12, 4))
+    s = sym.super_ptr[1:] - sym.super_ptr[:-1]
+    c = (sym.rowptr[1:] - sym.rowptr[:-1]) - s
+    for i, ozm in enumerate((16, 40, 128, 16)):
+        want = set((((s >= max(17, ozm)) & (c >= 96)).nonzero()[0]).tolist())
+        first, second, third = (p[1] for p in parts[1 + 3 * i:4 + 3 * i])
+        assert _syrk(first) == want and _syrk(second) == want            # issued, captured
+        assert "G" in [f[0] for f in third] and not any("k_fupd" in x.name for x in launches(third))
+        updated = lambda n: sum("k_fupd<" in x.name for x in launches(n))     # noqa: E731
+        assert bool(updated(first)) and not any(x.stale for x in launches(first) + launches(second))
