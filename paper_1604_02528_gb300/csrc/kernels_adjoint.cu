@@ -34,6 +34,7 @@
 #include "launch.h"
 #include "nvtx.h"
 #include "plan.h"
+#include "put.cuh"
 #include "digit_rows.cuh"
 #include "fixedpoint.cuh"
 #include "tile_gemm.cuh"
@@ -1364,7 +1365,7 @@ static AdjDesc make_adesc(selinv_plan_s *plan, const double *L, const double *D,
 static int adj_normalize(selinv_plan_s *plan, const void *L, const void *D, cudaStream_t st) {
     AdjData *a = static_cast<AdjData *>(plan->factor->adj);
     ProbDesc pd = make_desc(plan->data, plan->ws[0], SELINV_F64, L, D, nullptr, false);
-    cudaMemcpyAsync(a->d_pdesc, &pd, sizeof(pd), cudaMemcpyHostToDevice, st);
+    put(a->d_pdesc, &pd, 1, st);
     if (!a->tcn.launches.empty()) {
         // the forward's own normalization launches (Lhat of the wide supernodes on the tensor cores)
         for (const Launch &Ln : a->tcn.launches)
@@ -1665,7 +1666,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
     AdjDesc h = make_adesc(plan, static_cast<const double *>(L), static_cast<const double *>(D),
                            static_cast<const double *>(Z), static_cast<double *>(Lbar),
                            static_cast<double *>(Dbar));
-    cudaMemcpyAsync(a->d_desc, &h, sizeof(h), cudaMemcpyHostToDevice, st);
+    put(a->d_desc, &h, 1, st);
     k_adj_fold<<<dim3(p.ns, kFinY), 256, 0, st>>>(a->d_desc, p.ns);
     note_launch();
     FactorData *f = plan->factor;
@@ -1678,7 +1679,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
         pd.LD = a->YB;
         pd.Yout = w.work;
         pd.colexpY = a->cy;
-        cudaMemcpyAsync(a->d_tcdesc, &pd, sizeof(pd), cudaMemcpyHostToDevice, st);
+        put(a->d_tcdesc, &pd, 1, st);
         // the row products: Ybar = Zbar_{C,K} - Lhat S, G -= Y S (G becomes
         // Lhat_bar), Lbar_{C,K} = Lhat_bar M^T
         ProbDesc base = make_desc(p, w, SELINV_F64, L, D, const_cast<void *>(Z), false);
@@ -1689,7 +1690,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
         pdp[0].L = w.LD; pdp[0].LD = a->YB; pdp[0].Yout = a->Zb; pdp[0].prod_op = 2;
         pdp[1].L = Z; pdp[1].LD = w.work; pdp[1].prod_op = 1;
         pdp[2].L = w.work; pdp[2].LD = Lbar; pdp[2].prod_op = 0;
-        cudaMemcpyAsync(a->d_pdp, pdp, sizeof(pdp), cudaMemcpyHostToDevice, st);
+        put(a->d_pdp, pdp, 3, st);
         // the update V_K -= sym(Ybar Lhat^T): B = [Lhat, Ybar] from the panels
         // LD and YB, A = the digit planes of [Ybar, Lhat], out V (offsets u_off)
         ProbDesc sy = base;
@@ -1700,7 +1701,7 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
         sy.linvd = a->sy;
         sy.linvd_off = a->d_sy_off;
         sy.linvexp = a->syexp;
-        cudaMemcpyAsync(a->d_sydesc, &sy, sizeof(sy), cudaMemcpyHostToDevice, st);
+        put(a->d_sydesc, &sy, 1, st);
         const int ncz = (int)a->cz_work.size();
         k_adj_colexpz<<<ncz, 256, 0, st>>>(a->d_desc, static_cast<const double *>(Z), w.colexpZ, a->d_cz, ncz);
         note_launch();
@@ -1821,7 +1822,7 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
     Workspace &w = plan->ws[0];
     const bool tc = !a->dig_work.empty();
     if (tc) h.colexp = w.colexpZ;
-    cudaMemcpyAsync(a->d_desc, &h, sizeof(h), cudaMemcpyHostToDevice, st);
+    put(a->d_desc, &h, 1, st);
     if (tc) {
         // tcgen05 gather-GEMM of the wide supernodes: A^{-1}(C,C) -> the
         // finished Abar of the ancestors, B = L_C (digit planes of L, once),
@@ -1830,14 +1831,14 @@ extern "C" int selinv_factor_adjoint(selinv_plan plan, selinv_dtype dtype, const
         pd.LD = const_cast<void *>(L);   // read only: the digit kernel takes B from LD
         pd.Yout = w.work;
         pd.colexpY = a->cy;
-        cudaMemcpyAsync(a->d_tcdesc, &pd, sizeof(pd), cudaMemcpyHostToDevice, st);
+        put(a->d_tcdesc, &pd, 1, st);
         // the row product Abar_C = Lbar_C D^{-1} M
         ProbDesc base = make_desc(p, w, SELINV_F64, L, D, a->Ab, false);
         base.linvd = a->sd;
         base.linvd_off = a->d_sd_off;
         base.linvexp = a->sdexp;
         base.L = a->Lbw; base.LD = a->Ab; base.prod_op = 0;
-        cudaMemcpyAsync(a->d_pdp + 3, &base, sizeof(base), cudaMemcpyHostToDevice, st);
+        put(a->d_pdp + 3, &base, 1, st);
         launch_lhat_digits(a->d_tcdesc, a->d_dig, (int)a->dig_work.size(), st);
         note_launch();
     }

@@ -26,6 +26,7 @@
 #include "launch.h"
 #include "nvtx.h"
 #include "plan.h"
+#include "put.cuh"
 #include "seg_update.cuh"
 #include "tri_rows.cuh"
 
@@ -774,7 +775,7 @@ static FactorDesc *factor_desc(selinv_plan_s *plan, const FactorLists *q, void *
     h.D = D;
     h.status = p.d_status;
     h.herm = herm;
-    cudaMemcpyAsync(f->d_desc, &h, sizeof(h), cudaMemcpyHostToDevice, st);
+    put(f->d_desc, &h, 1, st);
     return f->d_desc;
 }
 

@@ -9,11 +9,13 @@
 //        panels of each (comma-separated), the kernel's name and the supernodes
 //        of its work list
 //   G / B / I / T       graph launch, begin of capture, instantiation, record of a timing event
+//   H                   copy from host memory on a stream that the caller captures
 //
 // A captured launch is logged like an issued one.  fake_fail(what, n) makes the
 // next n begins of capture (1), instantiations (2) or cluster launches and
 // launches of k_adj_gemm (3) fail; every timed run takes 1 ms, those of the
-// autotuner's next fake_slow(n) candidates 2.
+// autotuner's next fake_slow(n) candidates 2.  fake_capturing(st): the stream
+// that the caller captures.
 #include <cuda_runtime.h>
 #include <cxxabi.h>
 
@@ -23,6 +25,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <set>
 #include <string>
 #include <vector>
@@ -123,9 +126,30 @@ void note(const char *what) {
 }
 }  // namespace
 
+// A handle (the library makes them with the nothrow form) gets the address of the
+// last one of its size that was given back.
+static std::map<void *, size_t> g_handles;
+static std::multimap<size_t, void *> g_given_back;
+void *operator new(size_t n, const std::nothrow_t &) noexcept {
+    auto it = g_given_back.find(n);
+    void *p = it != g_given_back.end() ? it->second : std::malloc(n);
+    if (it != g_given_back.end()) g_given_back.erase(it);
+    g_handles[p] = n;
+    return p;
+}
+void operator delete(void *p) noexcept {
+    auto it = p ? g_handles.find(p) : g_handles.end();
+    if (it == g_handles.end()) return std::free(p);
+    g_given_back.emplace(it->second, p);
+    g_handles.erase(it);
+}
+void operator delete(void *p, size_t) noexcept { operator delete(p); }
+
 extern "C" {
 void fake_fail(int what, int n) { g_fail[what] = n; }
 static int g_slow;
+static cudaStream_t g_capturing;
+void fake_capturing(cudaStream_t st) { g_capturing = st; }
 void fake_slow(int candidates) { g_slow = 2 * candidates; }   // two timed runs each
 
 void **__cudaRegisterFatBinary(void *) { static void *h; return &h; }
@@ -164,7 +188,11 @@ cudaError_t cudaFree(void *p) {                  // (the address stays taken: a 
     return cudaSuccess;
 }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind k, cudaStream_t st) {
+    if (k == cudaMemcpyHostToDevice && st && st == g_capturing) note("H");
+    std::memcpy(d, s, n);
+    return cudaSuccess;
+}
 cudaError_t cudaMemset(void *p, int v, size_t n) { if (n <= 64) std::memset(p, v, n); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void *, int, size_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
@@ -184,7 +212,10 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = handle<cudaStream_t>(); return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) { *s = cudaStreamCaptureStatusNone; return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus *s) {
+    *s = st && st == g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) { const int i = id(s); merge(g_clock[i], g_event[e]); return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t *e) { g_timing.insert(*e = handle<cudaEvent_t>()); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { *e = handle<cudaEvent_t>(); return cudaSuccess; }
