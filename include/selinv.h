@@ -43,6 +43,16 @@
  *    void*; NULL = legacy default stream).  Errors found on the device
  *    (timeouts of bounded waits, zero pivots, non-finite values) are latched
  *    in a per-plan status word read by selinv_status() after synchronizing.
+ *  - A caller may capture selinv_factor and the adjoints into a CUDA graph of
+ *    its own, and selinv_numeric, selinv_numeric_lu and
+ *    selinv_numeric_batched with use_graph = 0 (otherwise they launch graphs
+ *    themselves, and return SELINV_ERR_CUDA), after one call each with the
+ *    same plan, options and element type outside the capture (that call
+ *    allocates).  Such a graph holds addresses of the plan's tables: it is
+ *    valid until the plan's options or selection change, a wider element type
+ *    is used on the plan, or the plan is destroyed; the LU form's and a
+ *    batch's, which need the buffers of the call before, only until such a
+ *    call with other buffers.
  *  - Every call returns SELINV_OK (0) or a negative error code.
  */
 #ifndef SELINV_H

@@ -20,6 +20,7 @@
 #include "launch.h"
 #include "nvtx.h"
 #include "plan.h"
+#include "put.cuh"
 
 namespace selinv {
 
@@ -514,6 +515,7 @@ void Schedule::release() {
     if (cap) cudaStreamDestroy(cap);
     cap = nullptr;
     issued = false;
+    lent = false;
     if (graph_host) cudaGraphExecDestroy(graph_host);
     graph_host = nullptr;
     host_key.fill(nullptr);
@@ -2075,14 +2077,16 @@ static int numeric_prepare(selinv_plan plan, selinv_dtype dtype, const void *L, 
     const bool capturing = st != nullptr && st != cudaStreamLegacy &&
                            (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone);
     cudaGetLastError();
-    if (S.valid && S.key_dtype == dtype && S.mode == mode && S.key_ws == plan->ws[0].gen && !capturing &&
-        (S.key_L != L || S.key_D != D || S.key_Z != Z)) {
+    if (S.valid && S.key_dtype == dtype && S.mode == mode && S.key_ws == plan->ws[0].gen &&
+        (S.key_L != L || S.key_D != D || S.key_Z != Z || capturing || S.lent)) {
         // only the caller's buffers changed: every kernel of the schedule
         // reads them through the device descriptors, so those are rewritten
-        // in stream order and the schedule (and its graph) stays
+        // in stream order and the schedule (and its graph) stays.  A graph that
+        // the caller captures writes its own at every launch; from then on
+        // nothing is known of what they hold.
+        S.lent = S.lent || capturing;
         S.h_descs.assign(1, make_desc(p, plan->ws[0], dtype, L, D, Z, mode == SELINV_SCHED_PERSISTENT));
-        if (cudaMemcpyAsync(S.d_descs, S.h_descs.data(), sizeof(ProbDesc), cudaMemcpyHostToDevice, st) != cudaSuccess)
-            return SELINV_ERR_CUDA;
+        if (put(S.d_descs, S.h_descs.data(), 1, st) != cudaSuccess) return SELINV_ERR_CUDA;
         S.key_L = L; S.key_D = D; S.key_Z = Z;
     }
     if (!S.valid || S.key_L != L || S.key_D != D || S.key_Z != Z || S.key_dtype != dtype ||

@@ -202,6 +202,7 @@ struct Schedule {
     // launch by launch, so that a single inversion does not pay for a graph)
     cudaStream_t cap = nullptr;
     bool issued = false;
+    bool lent = false;           // a graph of the caller's may rewrite d_descs
     // selinv_numeric_host's captured call and the buffers it was captured for
     cudaGraphExec_t graph_host = nullptr;
     std::array<const void *, 6> host_key{};
