@@ -389,7 +389,7 @@ __device__ __forceinline__ void ftrsm_group(const T *Ls, const T *rD, T *P, int6
         const int k = c + W * t;
         a[t] = row < end && k < s ? P[(int64_t)k * ld + row] : Sc<T>::zero();
     }
-    tri_rows<T, W, NC, false>(a, Ls, nullptr, (s + W - 1) / W, 0, herm);
+    tri_rows<T, W, NC, false>(a, Ls, nullptr, (s + W - 1) / W, 0, 0, herm);
 #pragma unroll
     for (int t = 0; t < NT; t++) {
         const int k = c + W * t;

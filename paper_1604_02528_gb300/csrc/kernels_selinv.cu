@@ -257,9 +257,11 @@ __global__ void __launch_bounds__(256) k_dinv(const ProbDesc *__restrict__ descs
             Bs[q][rr] = (k < s && j0 + rr < s) ? X[(int64_t)(j0 + rr) * s + k] : Sc<T>::zero();
         }
         __syncthreads();
+        // from max(i, j) on: a zero above the diagonal times an infinite or
+        // undefined entry is no term of the sum
         const int kk = s - k0 < 32 ? s - k0 : 32;
 #pragma unroll 8
-        for (int q = 0; q < kk; q++) madd(acc, As[q][ty], Bs[q][tx]);
+        for (int q = max(0, max(i0 + ty, j0 + tx) - k0); q < kk; q++) madd(acc, As[q][ty], Bs[q][tx]);
     }
     const int i = i0 + ty, j = j0 + tx;
     if (i >= s || j >= s || (!lu && i < j)) return;

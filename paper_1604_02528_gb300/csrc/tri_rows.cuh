@@ -50,10 +50,12 @@ __device__ __forceinline__ void tri_store(T *dst, const T *L, int64_t ld, int s,
 // y L^T = a for the warp's 32 / W rows a (unit lower L; conj(L) in place of L
 // when herm) of nt blocks of W columns, from column j0 on: y_j, final after step
 // j - 1, is taken from every later column k as y_j L(k, j).  Finished columns
-// are not touched.  SCALED: L has the diagonal 1 / rd: y_j = a_j rd[j] is what
+// are not touched, and a row takes the steps from its own on (the columns of an
+// inverse: what lies before is zero, which an infinite or undefined entry of L
+// would not keep so).  SCALED: L has the diagonal 1 / rd: y_j = a_j rd[j] is what
 // the later columns lose, and what is left in a is the undivided a_j.
 template <typename T, int W, int NC, bool SCALED>
-__device__ __forceinline__ void tri_rows(T (&a)[NC * 32 / W], const T *Ls, const T *rd, int nt, int j0, bool herm) {
+__device__ __forceinline__ void tri_rows(T (&a)[NC * 32 / W], const T *Ls, const T *rd, int nt, int j0, int own, bool herm) {
     constexpr int NT = NC * 32 / W;
     const int c = threadIdx.x % W;
 #pragma unroll
@@ -69,7 +71,7 @@ __device__ __forceinline__ void tri_rows(T (&a)[NC * 32 / W], const T *Ls, const
             const T *l = Lb + jj * 32 * (NC - q);
 #pragma unroll
             for (int t = b; t < NT; t++)
-                if ((t > b || c > jj) && (t <= NT - 32 / W || t < nt)) msub(a[t], y, cjif(l[W * t], herm));
+                if (W * b + jj >= own && (t > b || c > jj) && (t <= NT - 32 / W || t < nt)) msub(a[t], y, cjif(l[W * t], herm));
         }
     }
 }
@@ -91,14 +93,14 @@ __device__ __forceinline__ void tri_inverse_cols(const T *Ls, const T *rd, T *X,
     T a[NT];
 #pragma unroll
     for (int t = 0; t < NT; t++) a[t] = c0 + c + W * t == col ? Sc<T>::one() : Sc<T>::zero();
-    tri_rows<T, W, NC, SCALED>(a, Ls, SCALED ? rd + c0 : rd, (s - c0 + W - 1) / W, j - c0, false);
+    tri_rows<T, W, NC, SCALED>(a, Ls, SCALED ? rd + c0 : rd, (s - c0 + W - 1) / W, j - c0, col - c0, false);
     if (col >= s) return;
     T *x = X + (int64_t)col * ldx;
     for (int i = c; i < c0; i += W) x[i] = Sc<T>::zero();
 #pragma unroll
     for (int t = 0; t < NT; t++) {
         const int i = c0 + c + W * t;
-        if (i < s) x[i] = SCALED ? mul(a[t], rd[i]) : a[t];
+        if (i < s) x[i] = i < col ? Sc<T>::zero() : (SCALED ? mul(a[t], rd[i]) : a[t]);
     }
 }
 

@@ -71,3 +71,13 @@ def test_terms_are_quotients(native, cuda_device):
         got = _call(native, np.array([[1.0, 0.0], [l, 1.0]]), np.array([np.inf, d]))
         with np.errstate(all="ignore"):
             assert got[0, 0] == (-l / d) * -l
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("s,i,j", [(2, 1, 0), (17, 9, 4), (33, 32, 0), (40, 36, 34), (96, 50, 10), (96, 95, 62), (128, 127, 126), (128, 65, 64)])
+def test_an_entry_of_l_reaches_its_own_columns_only(native, cuda_device, s, i, j, bad):
+    """L(i, j) is in the columns of X up to j; those after it never meet it,
+    although they share a warp with column j."""
+    L, D = _block(s, 7 * s + j)
+    L[i, j] = bad
+    _agree(_call(native, L, D), _reference(L, D))
