@@ -155,10 +155,12 @@ constexpr int kFdLd = kFdNB + 1;   // row stride of the exchanged rows
 constexpr int kFdSlots = (kFdNB * (kFdNB + 1) / 2 + kFdChain - 1) / kFdChain;   // entries per chain thread
 
 // 1 / d: the hardware's approximate reciprocal r0 (relative error below
-// 2^-19), then one step of the third-order iteration r0 (1 + e + e^2),
-// e = 1 - d r0: three dependent FP64 operations (240 clocks with the seed)
-// where the division takes 385.  Magnitudes near the ends of the exponent
-// range (and zero, infinities, NaN) go through the division.
+// 2^-19), then one step r0 (1 + e + e^2), e = 1 - d r0, of the hyperpower
+// iteration of third order (M. Altman, Pacific J. Math. 10, 1960): e^3 < 2^-57
+// beside the last rounding, 0.5625 units in the last place where the division
+// has 0.5.  Three dependent FP64 operations, 240 clocks with the seed, where
+// the division takes 385.  Magnitudes near the ends of the exponent range (and
+// zero, infinities, NaN) go through the division.
 // The division is a call: inlined, its own FP64 operations would run beside
 // the others in every lane.
 __device__ __noinline__ double full_recip(double d) { return 1.0 / d; }

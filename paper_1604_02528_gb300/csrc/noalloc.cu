@@ -50,8 +50,8 @@ __global__ void __launch_bounds__(kTriThreads) k_noalloc_linv(int s, const doubl
 // of X above the diagonal times an infinite or undefined 1 / D_k is no term.
 // A quotient is the product with the rounded reciprocal and one correction by
 // its residual, which rounds correctly (P. Markstein, IBM J. Res. Dev. 34,
-// 1990; 34.8 us at s = 96, where six divisions
-// a thread took 36.9 and products with the reciprocal 32.8).  Magnitudes near the ends of the range are divided.
+// 1990; 34.8 us at s = 96, where six divisions a thread took 36.9 and products
+// with the reciprocal 32.8).  Magnitudes near the ends of the range are divided.
 constexpr int kMidLo = 1023 - 400, kMidHi = 1023 + 400;   // biased exponents
 __device__ __forceinline__ bool mid(double v) {
     const int e = (int)((__double_as_longlong(v) >> 52) & 0x7FF);

@@ -131,3 +131,130 @@ def test_graph_of_the_caller(native, cuda_device, make, use_graph):
         for call in replay:
             call()
         t.check(b, t.want(v, W))
+
+
+@pytest.mark.parametrize("stream", [False, True])
+@pytest.mark.parametrize("make", list(MAKE))
+def test_training_step(native, cuda_device, make, stream):
+    """Issued, captured, replayed, and then on buffers of its own in every pass."""
+    import torch
+    t = Training(MAKE[make]())
+    st = torch.cuda.Stream() if stream else None
+    kept = t.buffers()
+    for k in range(5):
+        b = kept if k < 3 else t.buffers()
+        v, W = t.values(k)
+        for name in b:
+            b[name].fill_(float("nan"))
+        b["A"].copy_(torch.from_numpy(v))
+        b["W"].copy_(torch.from_numpy(W))
+        torch.cuda.synchronize()
+        t.step(native, b, st)
+        t.check(b, t.want(v, W))
+
+
+def _dense(n, cap, kind, seed):
+    """One dense diagonally dominant matrix in supernodes of `cap` columns."""
+    rng = np.random.default_rng(seed)
+    g = rng.standard_normal((n, n)) + (1j * rng.standard_normal((n, n)) if kind != "f64" else 0)
+    a = (g + (g.conj().T if kind == "c128h" else g.T)) / 2
+    np.fill_diagonal(a, np.abs(a).sum(axis=1) + 1.0)
+    colptr = np.concatenate([[0], np.cumsum(np.arange(n, 0, -1))]).astype(np.int64)
+    rowind = np.concatenate([np.arange(j, n) for j in range(n)]).astype(np.int32)
+    return synth.Problem("dense", n, colptr, rowind, np.concatenate([a[j:, j] for j in range(n)]), np.arange(n),
+                         {"kind": "fundamental", "cap": cap, "fill": 0.0}, {"hermitian": kind == "c128h"})
+
+
+class Pattern:
+    """One plan for matrices of any type and values on a dense pattern."""
+
+    def __init__(self, native, n, cap):
+        from paper_1604_02528_gb300.api import SelInvContext
+        self.native, self.n, self.cap = native, n, cap
+        p = _dense(n, cap, "f64", 0)
+        self.sym, self.ctx = oracle.symbolic_for(p), SelInvContext.from_problem(p)
+        self.ctx.attach_matrix()
+        r, c, _ = oracle.panel_entries(self.sym)
+        self.lower, self.diag = r > c, r == c
+
+    def check(self, kind, seed, stream=None, keep=None):
+        """Factorization and inversion of one matrix, on fresh buffers or on `keep`."""
+        import torch
+        N = self.native
+        p = _dense(self.n, self.cap, kind, seed)
+        L0, D0 = oracle.ldlt(p, self.sym)
+        Z0 = oracle.selinv(self.sym, L0, D0, hermitian=p.hermitian)
+        new = lambda m: torch.full((m,), float("nan"), dtype=torch.from_numpy(L0).dtype, device="cuda")   # noqa: E731
+        L, D, Z = keep if keep else (new(self.ctx.nnz), new(self.n), new(self.ctx.nnz))
+        for x in (L, D, Z):
+            x.fill_(float("nan"))
+        A, dt = torch.from_numpy(p.values).cuda(), {"f64": N.SELINV_F64, "c128": N.SELINV_C128, "c128h": N.SELINV_C128H}[kind]
+        torch.cuda.synchronize()
+        N.selinv_factor(self.ctx.plan, dt, A, L, D, stream)
+        N.selinv_numeric(self.ctx.plan, dt, L, D, Z, stream)
+        torch.cuda.synchronize()
+        assert self.ctx.status() == 0
+        Lg = L.cpu().numpy()
+        assert np.abs(D.cpu().numpy() - D0).max() <= 1e-12 * np.abs(D0).max()
+        assert np.abs(np.where(self.lower, Lg - L0, 0)).max() <= 1e-12
+        assert np.all(Lg[self.diag] == 1) and np.all(Lg[~self.lower & ~self.diag] == 0)
+        assert oracle.block_errors(self.sym, Z.cpu().numpy(), Z0).max() <= 1e-11
+        return L, D, Z
+
+
+# narrow and wide kernels, one and several blocks of 32 columns, the shortest C
+# of the tensor-core update and several tiles of it
+@pytest.mark.parametrize("stream", [False, True])
+@pytest.mark.parametrize("kind", ["f64", "c128", "c128h"])
+@pytest.mark.parametrize("cap,n", [(9, 30), (16, 60), (17, 113), (33, 180), (65, 150), (128, 290)])
+def test_factor_and_inverse(native, cuda_device, cap, n, kind, stream):
+    import torch
+    t, st, keep = Pattern(native, n, cap), torch.cuda.Stream() if stream else None, None
+    for k in range(4):
+        keep = t.check(kind, 10 * n + k, st, keep if k < 3 else None)
+
+
+def test_types_alternate_on_one_plan(native, cuda_device):
+    """Real, complex symmetric and Hermitian values, each issued, captured and
+    replayed between the others; the workspace is widened on the way."""
+    t = Pattern(native, 200, 40)
+    for k, kind in enumerate(["f64"] * 3 + ["c128"] * 3 + ["c128h"] * 2 + ["c128", "f64", "c128h", "f64", "c128"]):
+        t.check(kind, k)
+
+
+@pytest.mark.parametrize("stream", [False, True])
+def test_options_change_between_replays(native, cuda_device, stream):
+    import torch
+    t, st = Pattern(native, 290, 64), torch.cuda.Stream() if stream else None
+    bits = {}
+    for k, (fast, ozm, graph) in enumerate([(1, 16, 1), (0, 16, 1), (1, 16, 1), (1, 65, 1), (1, 16, 0), (2, 16, 1), (1, 16, 1)]):
+        t.ctx.set_options(fast_contraction=fast, oz_min_s=ozm, use_graph=graph)
+        keep = None
+        for _ in range(3):
+            keep = t.check("f64", 5, st, keep)
+            L = keep[0].cpu().numpy()
+            engine = "tensor" if fast == 1 and ozm <= 64 else "fma"
+            assert np.array_equal(bits.setdefault(engine, L), L)      # the engine decides, and nothing else
+    assert not np.array_equal(bits["tensor"], bits["fma"])
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("cap,n", [(8, 50), (16, 110), (33, 120), (64, 200), (128, 300)])
+def test_lu_form(native, cuda_device, cap, n, cplx):
+    import torch
+    p = synth.random_sparse_nonsym(n, 1.0, n, complex_values=cplx, supernodes={"kind": "fundamental", "cap": cap, "fill": 0.0})
+    sym = oracle.symbolic_for(p)
+    L, Ut = oracle.lu(p, sym)
+    Zl0, Zu0 = oracle.selinv_lu(sym, L, Ut)
+    low = oracle.lower_mask(sym)
+    plan = native.selinv_symbolic(sym.n, sym.nsuper, sym.super_ptr, sym.sparent, sym.rowptr, sym.rows)
+    Lt, Ut_t = torch.from_numpy(L).cuda(), torch.from_numpy(Ut).cuda()
+    Zl, Zu = torch.empty_like(Lt), torch.empty_like(Lt)
+    for _ in range(3):
+        Zl.fill_(float("nan"))
+        Zu.fill_(float("nan"))
+        native.selinv_numeric_lu(plan, native.SELINV_C128 if cplx else native.SELINV_F64, Lt, Ut_t, Zl, Zu)
+        torch.cuda.synchronize()
+        assert native.selinv_status(plan) == 0
+        assert oracle.block_errors(sym, Zl.cpu().numpy(), Zl0).max() <= 1e-12
+        assert oracle.block_errors(sym, np.where(low, Zu.cpu().numpy(), 0), np.where(low, Zu0, 0)).max() <= 1e-12
