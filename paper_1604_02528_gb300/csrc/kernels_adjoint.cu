@@ -1706,7 +1706,6 @@ extern "C" int selinv_adjoint(selinv_plan plan, selinv_dtype dtype, const void *
         k_adj_colexpz<<<ncz, 256, 0, st>>>(a->d_desc, static_cast<const double *>(Z), w.colexpZ, a->d_cz, ncz);
         note_launch();
     }
-    const int nl = p.nlevels;
     // Only Ybar and the update matrices V climb the tree; what each supernode
     // makes of them (Lhat_bar, Lbar, Dbar) meets no other supernode and has
     // storage of its own, so it runs for whole groups of levels at once, on a

@@ -587,11 +587,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_diag_oz(const ProbDesc *__res
     const int pm = c - p0 < kTM ? c - p0 : kTM;
     const int s16 = (s + 15) & ~15;
     double *Zk = static_cast<double *>(P.Z) + P.panel_off[K];
-    const double *LDk = static_cast<const double *>(P.LD) + P.panel_off[K];
     const double *Y = Zk + s;                                       // Y(p, j) = Y[j*ld + p]
     const uint16_t *Ag = P.lhs + P.lhs_off[K];
     const int64_t aplane = (int64_t)s * c16;
-    const int64_t ss = (int64_t)s * s;
     long long *acc64 = P.dacc + 2 * P.linv_off[K];            // [s*s] x (hi, lo)
 
     if (pm > 0) {

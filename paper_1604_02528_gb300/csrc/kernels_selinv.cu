@@ -76,11 +76,10 @@ __device__ void linv_lu(const ProbDesc &P, int K, int s, int64_t ld, const T *L,
     }
 }
 
-// with_dinv = 0: only L_KK^{-1} (k_dinv forms Dinv_K afterwards, spread over tiles)
 template <typename T>
 __global__ void __launch_bounds__(kLinvThreads) k_linv(const ProbDesc *__restrict__ descs,
                                                        const int2 *__restrict__ work, int nwork,
-                                                       size_t smem_cap, int with_dinv) {
+                                                       size_t smem_cap) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int w = blockIdx.x;
@@ -150,7 +149,6 @@ __global__ void __launch_bounds__(kLinvThreads) k_linv(const ProbDesc *__restric
     }
     if (in_smem)
         for (int e = threadIdx.x; e < s * s; e += kLinvThreads) Li[e] = X[(e / s) * lx + e % s];
-    if (!with_dinv) return;
     const bool h = P.herm != 0;
     for (int e = threadIdx.x; e < s * s; e += kLinvThreads) {
         const int i = e % s, j = e / s;
@@ -606,20 +604,18 @@ cudaError_t launch_check_finite(const void *x, int64_t n, int *status, cudaStrea
 }
 
 template <typename T>
-static cudaError_t launch_linv_t(const ProbDesc *d, const int2 *work, int nwork, int large, int with_dinv,
-                                 cudaStream_t st) {
+static cudaError_t launch_linv_t(const ProbDesc *d, const int2 *work, int nwork, int large, cudaStream_t st) {
     if (nwork <= 0) return cudaSuccess;
     // small blocks (s <= 32) need at most 33 KB (X and a staged block of L);
     // large ones get room for s = 128 (real)
     const size_t cap = large ? kLinvSmemMax : (32 * 33 + 32 + 64 * 32) * sizeof(T);
-    k_linv<T><<<nwork, kLinvThreads, cap, st>>>(d, work, nwork, cap, with_dinv);
+    k_linv<T><<<nwork, kLinvThreads, cap, st>>>(d, work, nwork, cap);
     return cudaGetLastError();
 }
 
-cudaError_t launch_linv(int dtype, const ProbDesc *d, const int2 *work, int nwork, int large, cudaStream_t st,
-                        int with_dinv) {
-    return dtype == SELINV_C128 ? launch_linv_t<zd>(d, work, nwork, large, with_dinv, st)
-                                : launch_linv_t<double>(d, work, nwork, large, with_dinv, st);
+cudaError_t launch_linv(int dtype, const ProbDesc *d, const int2 *work, int nwork, int large, cudaStream_t st) {
+    return dtype == SELINV_C128 ? launch_linv_t<zd>(d, work, nwork, large, st)
+                                : launch_linv_t<double>(d, work, nwork, large, st);
 }
 
 cudaError_t launch_linv_cols(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st) {

@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
         const bool rok = p0 + r < c;
         const double2 *Lz = static_cast<const double2 *>(P.L) + P.panel_off[K] + s + p0 + r;   // complex X(p0 + r, q)
         auto load_dense = [&](int i_, double (&v)[4]) {
-            if (CPLX) {
+            if constexpr (CPLX) {
 #pragma unroll
                 for (int u = 0; u < 2; u++) {
                     const int q = (st0 + i_) * 8 + kq * 2 + u;
@@ -376,12 +376,12 @@ __global__ void __launch_bounds__(kTwThreads, 1) k_selinv_tcw(const ProbDesc *__
                     v[2 * u] = z.x;
                     v[2 * u + 1] = z.y;
                 }
-                return;
-            }
+            } else {
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int k = (st0 + i_) * 16 + kq * 4 + u;
-                v[u] = (rok && i_ < n && k < kw) ? (PAIR && k >= s ? Zc2[(int64_t)(k - s) * ld] : Lc[(int64_t)k * ld]) : 0.0;
+                for (int u = 0; u < 4; u++) {
+                    const int k = (st0 + i_) * 16 + kq * 4 + u;
+                    v[u] = (rok && i_ < n && k < kw) ? (PAIR && k >= s ? Zc2[(int64_t)(k - s) * ld] : Lc[(int64_t)k * ld]) : 0.0;
+                }
             }
         };
         auto parts = [&](int i_) {

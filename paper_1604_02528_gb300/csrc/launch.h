@@ -11,9 +11,10 @@ namespace selinv {
 void note_launch(int n = 1);
 
 cudaError_t configure_selinv_kernels();
-// L_KK^{-1} (and Dinv_K) by one CTA per supernode; large = 1: any width (128 KB of shared memory), 0: s <= 32
-cudaError_t launch_linv(int dtype, const ProbDesc *d, const int2 *work, int nwork, int large, cudaStream_t st,
-                        int with_dinv = 1);
+// L_KK^{-1} and Dinv_K by one CTA per supernode of at most 32 columns; large = 1:
+// of any width (real, 194 KB of shared memory): the adjoints' one launch for all
+// supernodes when none of them is on the tensor cores
+cudaError_t launch_linv(int dtype, const ProbDesc *d, const int2 *work, int nwork, int large, cudaStream_t st);
 // L_KK^{-1} of supernodes wider than 32 columns, kLinvCols columns per work entry
 constexpr int kLinvCols = 8;
 cudaError_t launch_linv_cols(int dtype, const ProbDesc *d, const int2 *work, int nwork, cudaStream_t st);

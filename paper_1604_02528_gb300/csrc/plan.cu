@@ -1416,7 +1416,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
             put(g_wide, 0, 0);
             if (!b64) put(g_64, 0, 0);
             if (!bsm) put(g_small, 0, b64 ? 1u << 1 : 0);
-            put(g_diag, 0, b64 && bsm ? 1u << 1 : (b64 ? 1u << 1 : 0));
+            put(g_diag, 0, b64 ? 1u << 1 : 0);
             put(g_fin, 0, (b64 ? 1u << 1 : 0) | (bsm ? 1u << 2 : 0));
             if (z_main && some(g_z)) {
                 // complex: after the contraction and its sums, the diagonal blocks of
