@@ -1304,16 +1304,16 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
                 // 8 rows of C (shorter ones lose more to the cluster's barriers than
                 // the split saves; so do clusters on more than the 152 SMs for levels
                 // whose largest supernode is far above the average: up to 304, 608 or
-                // 1216 CTAs the 12 poles took 12.16, 12.46 and 12.46 ms against 11.88,
-                // a batch of 24 matrices 3.59, 3.74 and 3.88 against 3.51); the
-                // supernodes in order of their work, longest first, where the SMs hold
-                // few of them (longer levels even out by themselves)
+                // 1216 CTAs factoring, inverting and summing 4 poles of 16 x 17 x 15
+                // took 12.16, 12.46 and 12.46 ms against 11.88, a batch of 8 matrices
+                // 3.59, 3.74 and 3.88 against 3.51); the supernodes in order of their
+                // work, longest first (that batch 3.31 ms, 3.40 unsorted; single
+                // inversions from 63^2 to 40^3 within 1 % either way)
                 int cl = 8;
                 while (cl > 1 && ((int64_t)list.size() * cl > 152 || cmax < 8 * cl)) cl /= 2;
-                if (list.size() <= 512)
-                    std::stable_sort(list.begin(), list.end(), [](const std::pair<int64_t, Item> &a, const std::pair<int64_t, Item> &b) {
-                        return a.first > b.first;
-                    });
+                std::stable_sort(list.begin(), list.end(), [](const std::pair<int64_t, Item> &a, const std::pair<int64_t, Item> &b) {
+                    return a.first > b.first;
+                });
                 int smem = 0;
                 const bool lu_any = descs[list[0].second.prob].lu != 0;   // (an LU schedule holds one problem)
                 for (const auto &x : list) {
