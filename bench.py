@@ -379,6 +379,17 @@ def variant_adjoint(dev, stream, flush, N):
             "forward_gflops": round(F / t_fwd / 1e6, 2)}
 
 
+def kernel_classes(s, c, cplx, opts):
+    """Which supernodes (s columns, c rows below) the inversion takes to the
+    tensor cores, and which to the kernel of narrow ones (level schedule: at
+    most 16 columns, gather and operands within 110 KB of shared memory)."""
+    engine = opts.fast_contraction == 1 if cplx else opts.fast_contraction != 0
+    oz = (s >= max(1, opts.oz_min_s)) & engine
+    words = c * (c + 1) / 2 + 2 * c * s + s * s
+    narrow = ~oz & (s <= 16) & (c <= 256) & (words * (16 if cplx else 8) <= 110 * 1024) & (opts.schedule == 1)
+    return oz, narrow
+
+
 def sample_kmin(sym, flops_target):
     """Smallest K such that the root-side supernodes K..N carry ~flops_target."""
     s, c = sym.sizes()
@@ -541,12 +552,12 @@ def main():
     s_ = np.diff(sp).astype(np.float64)
     c_ = np.diff(rp).astype(np.float64) - s_
     mult = 1.0 if dt == N.SELINV_F64 else 4.0
-    oz = (s_ >= max(16, topts.oz_min_s)) & (dt == N.SELINV_F64) & bool(topts.fast_contraction)
+    oz, narrow = kernel_classes(s_, c_, dt != N.SELINV_F64, topts)
     peaks = measured_peaks()
     dom = int(np.argmax(kms))
     name = N.PROFILE_KINDS[dom]
     # algorithmic flops of the supernodes each kernel kind processes
-    f_of = {"k_selinv": mult * float(((2 * c_ * c_ * s_ + 2 * c_ * s_ * s_) * ~oz).sum()),
+    f_of = {"k_selinv": mult * float(((2 * c_ * c_ * s_ + 2 * c_ * s_ * s_) * ~(oz | narrow)).sum()),
             "k_selinv_oz": mult * float((2 * c_ * c_ * s_ * oz).sum()),
             "k_selinv_tc": mult * float((2 * c_ * c_ * s_ * oz).sum()),
             "k_selinv_persist": mult * float((2 * c_ * c_ * s_ + 2 * c_ * s_ * s_).sum()),
@@ -562,7 +573,7 @@ def main():
             "k_push_diag": mult * float((2 * c_ * s_ * s_).sum()),
             "k_push": mult * float((2 * c_ * c_ * s_).sum()),
             "k_diag_tc": mult * float((2 * c_ * s_ * s_ * oz).sum()),
-            "k_selinv_tiny": mult * float(((2 * c_ * c_ * s_ + 2 * c_ * s_ * s_) * ~oz * (s_ <= 16) * (c_ <= 256)).sum())}
+            "k_selinv_tiny": mult * float(((2 * c_ * c_ * s_ + 2 * c_ * s_ * s_) * narrow).sum())}
     f_dom = f_of[name]
     achieved = f_dom / (kms[dom] * 1e-3) / 1e9 if kms[dom] > 0 else None
     traffic = ncu_traffic(name, options_tag(topts))

@@ -405,3 +405,32 @@ assert {call.replace("()", "(stream=st)")} == 0
 """)
     kinds = [f[0] for f in parts[1][1]]
     assert "L" in kinds and "H" not in kinds and "G" not in kinds
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("cap,n,ozm,schedule", [(1, 240, 128, 1), (16, 240, 128, 1), (16, 240, 8, 1), (40, 200, 16, 1), (16, 120, 16, 0)])
+def test_bench_counts_the_kernels_supernodes(fake, tmp_path, cap, n, ozm, schedule, dtype):
+    """bench.py's roofline divides the operations of a kernel's supernodes by its
+    time: its classes are those of the launches."""
+    import bench
+    from paper_1604_02528_gb300 import _native as N
+    parts, _ = run(fake, tmp_path, f"""
+p = synth.random_sparse_spd({n}, 1.0, 1, supernodes={{"kind": "fundamental", "cap": {cap}, "fill": 0.0}})
+c = Ctx(p, oz_min_s={ozm}, schedule={schedule}, use_graph=0)
+mark("run")
+assert c.selinv({dtype}) == 0
+""")
+    sym = oracle.symbolic_for(synth.random_sparse_spd(n, 1.0, 1, supernodes={"kind": "fundamental", "cap": cap, "fill": 0.0}))
+    opts = N.selinv_default_opts()
+    opts.oz_min_s, opts.schedule = ozm, schedule
+    s = (sym.super_ptr[1:] - sym.super_ptr[:-1]).astype(float)
+    c = (sym.rowptr[1:] - sym.rowptr[:-1]) - s
+    oz, narrow = bench.kernel_classes(s, c, dtype != 0, opts)
+    got = {"narrow": set(), "oz": set()}
+    for x in launches(parts[-1][1]):
+        if "k_selinv_narrow" in x.name:
+            got["narrow"] |= x.ks
+        if "k_selinv_tc" in x.name and "_true" not in x.name.split(",")[1:2]:
+            got["oz"] |= x.ks
+    assert got["narrow"] == set(narrow.nonzero()[0].tolist())
+    assert got["oz"] == set((oz & (c > 0)).nonzero()[0].tolist())
