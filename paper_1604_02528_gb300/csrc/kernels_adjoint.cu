@@ -1518,9 +1518,10 @@ static int adj_split(selinv_plan_s *plan) {
         sd_off[J + 1] = sd_off[J] + (wideK(J) ? 7 * ((s + 63) / 64 * 64) * ((s + 15) / 16 * 16) : 0);
     }
     // two groups: the last levels, of at most kAdjTop supernodes each, leave most
-    // SMs to the first group's products (24^3: a training step takes 14.1 ms with
-    // one group, 13.5 so; cuts at 4 to 22 levels 13.5 to 14.1, three to six
-    // groups 13.5 to 14.0)
+    // SMs to the first group's products.  Training steps with one group, with
+    // cuts at 2, 4, 8, 16 and 32 supernodes: 24^3 13.3 ms, 12.9, 12.8, 12.7, 12.9
+    // and 13.0; 16^3 4.91, 4.83, 4.76, 4.74, 4.78 and 4.86; 8^3 2.46 to 2.50
+    // (three to six groups on 24^3: no gain)
     int top = p.nlevels;
     while (top > 0 && p.level_ptr[p.nlevels - top + 1] - p.level_ptr[p.nlevels - top] <= kAdjTop) top--;
     a->grp.assign(1, 0);

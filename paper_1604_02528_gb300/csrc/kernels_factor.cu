@@ -583,7 +583,10 @@ static int factor_lists(selinv_plan_s *plan, int tc_s, FactorLists **out) {
         v.small0 = (int64_t)js.size();
         // one CTA for a whole supernode while its update's c^2 s / 2 products take
         // under 10 us of an SM (c = 64, s = 16), or up to twice that where the
-        // level has supernodes for two CTAs on every SM
+        // level has supernodes for two CTAs on every SM.  Limits of 16384, 65536
+        // and 400000 on the shorter levels: 40^3 11.42, 11.42 and 11.50 ms, 16^3
+        // 0.92 each, 20^3 Hermitian 4.36, 4.41 and 4.70, 240^2 2.38, 2.78 and
+        // 2.91; on the longer ones 32768 to 400000 differ by under 2 % anywhere
         const int64_t small_prod = p.level_ptr[l + 1] - p.level_ptr[l] >= 304 ? 150000 : 65536;
         for (int64_t e = p.level_ptr[l]; e < p.level_ptr[l + 1]; e++) {
             const int32_t J = p.level_list[e];
@@ -612,7 +615,12 @@ static int factor_lists(selinv_plan_s *plan, int tc_s, FactorLists **out) {
         // rows per tile: the number whose tiles, dealt to the SMs, take least --
         // a warp's groups of four, two and one row cost about 34, 18 and 10 us
         // of an SM sub-partition at 128 columns, a tile's L_JJ 5 us more for
-        // each of the two CTAs in flight
+        // each of the two CTAs in flight; the ratios serve every width (weights
+        // scaled to the level's widest supernode choose no better: 24^3 2.93
+        // against 2.89 ms).  Tiles of 4, 8, 16 and 64 rows throughout: 40^3 12.35,
+        // 11.53, 11.72 and 15.26 ms against 11.42, 16^3 0.93, 0.94, 1.01 and 1.45
+        // against 0.92, 20^3 Hermitian 4.57, 4.55, 4.96 and 8.21 against 4.41,
+        // 24^3 2.80, 2.81, 3.04 and 4.85 against 2.89
         int rt = 4;
         int64_t least = INT64_MAX;
         for (int t = 4; t <= 64; t += 4) {

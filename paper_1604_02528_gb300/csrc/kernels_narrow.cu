@@ -20,8 +20,10 @@
 // so a sum is split over neighbouring lanes where that fills the last pass;
 // levels of up to a CTA per SM take 512 threads and an SM each, longer ones 256
 // threads and, alone on their rows, the stored triangle instead of the square.
-// 40^3: 6.06 ms without the three, 5.38 with; a batch of 24 matrices 4.78 and
-// 3.53; a 2-D grid of 63^2 0.46 and 0.43; the 12 poles 12.5 and 11.9.  Every stored entry of A^{-1}_{C,C} is read once, down the columns of
+// 40^3: 6.06 ms without the three, 5.38 with; a batch of 8 matrices (6 poles of
+// 18 x 19 x 17 and two real meshes) 4.78 and 3.53; a 2-D grid of 63^2 0.46 and
+// 0.43; factoring, inverting and summing 4 poles of 16 x 17 x 15 12.5 and 11.9.
+// Every stored entry of A^{-1}_{C,C} is read once, down the columns of
 // its panel (contiguous runs of rows), and serves both (p, q) and (q, p).
 //
 // LU form (nonsymmetric values): entries above the diagonal come from the

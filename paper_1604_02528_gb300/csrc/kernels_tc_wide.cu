@@ -66,7 +66,7 @@ struct TwCfg {
     static constexpr int B_PLANE = kTwN * 16;    // ... of one gathered digit plane
     static constexpr int A_STAGE = kTcDig * A_PLANE;
     static constexpr int B_STAGE = kTcDig * B_PLANE;
-    static constexpr uint32_t TCOLS = 512;       // 7 groups x 64 columns
+    static constexpr uint32_t TCOLS = 512;       // 7 groups x 64 columns, 8 where NG is 8
     static constexpr size_t SMEM = sizeof(uint16_t) * (size_t)(kTwAS * A_STAGE + kTwBS * B_STAGE) +
                                    (sizeof(long long) + sizeof(uint32_t)) * (size_t)kTwN * kTwHS + sizeof(int) * kTwN;
 };
