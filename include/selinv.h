@@ -335,9 +335,9 @@ int selinv_numeric_lu(selinv_plan plan, selinv_dtype dtype, const void *L_dev, c
  *     matrix (host arrays, copied; an upper entry is taken as its symmetric
  *     lower one).  Every entry must lie on the pattern of L + L^T, else
  *     BAD_PATTERN and the plan is unchanged; indices out of range give
- *     INVALID_ARG.  Later selinv_numeric / selinv_numeric_batched calls on
- *     this plan run only the needed supernodes: the panels of the others are
- *     not written.  nsel = 0 restores the full inversion.  pos_out (host,
+ *     INVALID_ARG.  Later selinv_numeric / selinv_numeric_batched /
+ *     selinv_numeric_lu calls on this plan run only the needed supernodes: the
+ *     panels of the others are not written.  nsel = 0 restores the full inversion.  pos_out (host,
  *     nsel entries, may be NULL) receives each entry's panel position.
  *     selinv_adjoint needs every block of A^{-1} and returns UNSUPPORTED
  *     while a selection is set.

@@ -104,6 +104,8 @@ extern "C" int selinv_plan_select(selinv_plan plan, int64_t nsel, const int32_t 
     // schedules built for the previous selection are stale
     plan->single.release();
     plan->single.valid = false;
+    plan->lu.release();
+    plan->lu.valid = false;
     for (auto &b : plan->batch_cache) b.sched.release();
     plan->batch_cache.clear();
     return SELINV_OK;

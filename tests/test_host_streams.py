@@ -434,3 +434,20 @@ assert c.selinv({dtype}) == 0
             got["oz"] |= x.ks
     assert got["narrow"] == set(narrow.nonzero()[0].tolist())
     assert got["oz"] == set((oz & (c > 0)).nonzero()[0].tolist())
+
+
+def test_lu_form_follows_the_selection(fake, tmp_path):
+    """Its schedule is built for the supernodes of the current selection."""
+    parts, active = run(fake, tmp_path, """
+c = Ctx(synth.laplacian_3d(9, 4), use_graph=0)
+top = np.array([c.p.n - 1], np.int32)
+out = []
+for cols in (top[:0], top, top[:0]):
+    N.selinv_plan_select(c.plan, cols, cols)
+    mark("lu")
+    assert c.lu() == 0
+    out.append(N.selinv_plan_get(c.plan, "active").tolist())
+print(json.dumps(out))
+""")
+    for (_, lines), a in zip(parts[1:], active):
+        assert set().union(*(x.ks for x in launches(lines))) == {K for K, on in enumerate(a) if on}
