@@ -56,6 +56,12 @@ int device_of(const void *ptr) {
 }
 }  // namespace
 
+cudaError_t dev_malloc(void **ptr, size_t bytes) {
+    const cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e != cudaSuccess) cudaGetLastError();   // reported by this call: a later one must not find it
+    return e;
+}
+
 cudaError_t dev_alloc(void **ptr, size_t bytes) {
     const int dev = current_device();
     {
@@ -68,14 +74,13 @@ cudaError_t dev_alloc(void **ptr, size_t bytes) {
             return cudaSuccess;
         }
     }
-    cudaError_t e = cudaMalloc(ptr, bytes);
+    cudaError_t e = dev_malloc(ptr, bytes);
     if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();   // the failed allocation is not sticky
         {
             std::lock_guard<std::mutex> lk(g_mu);
             trim_locked();
         }
-        e = cudaMalloc(ptr, bytes);
+        e = dev_malloc(ptr, bytes);
     }
     if (e != cudaSuccess) *ptr = nullptr;
     return e;

@@ -1250,7 +1250,7 @@ void adjoint_release(void *p) {
 template <typename X>
 static int upl(X **d, const std::vector<X> &h) {
     *d = nullptr;
-    if (cudaMalloc((void **)d, sizeof(X) * std::max<size_t>(1, h.size())) != cudaSuccess) return SELINV_ERR_OOM;
+    if (dev_malloc((void **)d, sizeof(X) * std::max<size_t>(1, h.size())) != cudaSuccess) return SELINV_ERR_OOM;
     if (!h.empty() && cudaMemcpy(*d, h.data(), sizeof(X) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return SELINV_ERR_CUDA;
     return SELINV_OK;
@@ -1311,7 +1311,7 @@ static int adj_build(selinv_plan_s *plan) {
         }
         a->lhat_bptr.push_back((int)a->lhat_items.size());
     }
-    if (cudaMalloc((void **)&a->V, 8 * (size_t)std::max<int64_t>(f->u_off[p.ns], 1)) != cudaSuccess) {
+    if (dev_malloc((void **)&a->V, 8 * (size_t)std::max<int64_t>(f->u_off[p.ns], 1)) != cudaSuccess) {
         adjoint_release(a);
         return SELINV_ERR_OOM;
     }
@@ -1323,11 +1323,11 @@ static int adj_build(selinv_plan_s *plan) {
         return rc;
     }
     const size_t nz = (size_t)std::max<int64_t>(p.nnz, 1);
-    if (cudaMalloc((void **)&a->YB, 8 * nz) || cudaMalloc((void **)&a->Zb, 8 * nz) ||
-        cudaMalloc((void **)&a->Lbw, 8 * nz) || cudaMalloc((void **)&a->Ab, 8 * nz) ||
-        cudaMalloc((void **)&a->part, 8 * (size_t)std::max<int64_t>(p.part_all, 1)) ||
-        cudaMalloc((void **)&a->fin, 8 * (size_t)std::max<int64_t>(4 * p.linv_total, 1)) ||
-        cudaMalloc((void **)&a->d_desc, sizeof(AdjDesc)) || cudaMalloc((void **)&a->d_pdesc, sizeof(ProbDesc))) {
+    if (dev_malloc((void **)&a->YB, 8 * nz) || dev_malloc((void **)&a->Zb, 8 * nz) ||
+        dev_malloc((void **)&a->Lbw, 8 * nz) || dev_malloc((void **)&a->Ab, 8 * nz) ||
+        dev_malloc((void **)&a->part, 8 * (size_t)std::max<int64_t>(p.part_all, 1)) ||
+        dev_malloc((void **)&a->fin, 8 * (size_t)std::max<int64_t>(4 * p.linv_total, 1)) ||
+        dev_malloc((void **)&a->d_desc, sizeof(AdjDesc)) || dev_malloc((void **)&a->d_pdesc, sizeof(ProbDesc))) {
         adjoint_release(a);
         return SELINV_ERR_OOM;
     }
@@ -1544,16 +1544,16 @@ static int adj_split(selinv_plan_s *plan) {
         (rc = upl(&a->d_syw, a->sy_work)) || (rc = upl(&a->d_sy, a->sy_items)) || (rc = upl(&a->d_vn, a->vn_items)) ||
         (rc = upl(&a->d_sy_off, sy_off)))
         return rc;
-    if (sy_max > 0 && cudaMalloc((void **)&a->sy, sizeof(uint16_t) * (size_t)sy_max) != cudaSuccess)
+    if (sy_max > 0 && dev_malloc((void **)&a->sy, sizeof(uint16_t) * (size_t)sy_max) != cudaSuccess)
         return SELINV_ERR_OOM;
-    if (!a->syexp && cudaMalloc((void **)&a->syexp, sizeof(int) * (size_t)std::max<int64_t>(p.rowptr[p.ns], 1)) != cudaSuccess)
+    if (!a->syexp && dev_malloc((void **)&a->syexp, sizeof(int) * (size_t)std::max<int64_t>(p.rowptr[p.ns], 1)) != cudaSuccess)
         return SELINV_ERR_OOM;
-    if (!a->d_sydesc && cudaMalloc((void **)&a->d_sydesc, sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
-    if (sd_off[p.ns] > 0 && cudaMalloc((void **)&a->sd, sizeof(uint16_t) * (size_t)sd_off[p.ns]) != cudaSuccess)
+    if (!a->d_sydesc && dev_malloc((void **)&a->d_sydesc, sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
+    if (sd_off[p.ns] > 0 && dev_malloc((void **)&a->sd, sizeof(uint16_t) * (size_t)sd_off[p.ns]) != cudaSuccess)
         return SELINV_ERR_OOM;
-    if (!a->sdexp && cudaMalloc((void **)&a->sdexp, sizeof(int) * (size_t)std::max(p.n, 1)) != cudaSuccess)
+    if (!a->sdexp && dev_malloc((void **)&a->sdexp, sizeof(int) * (size_t)std::max(p.n, 1)) != cudaSuccess)
         return SELINV_ERR_OOM;
-    if (!a->d_pdp && cudaMalloc((void **)&a->d_pdp, 4 * sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
+    if (!a->d_pdp && dev_malloc((void **)&a->d_pdp, 4 * sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
     if (!a->dig_work.empty()) {
         // the forward's level schedule supplies the tcgen05 items of every
         // level (row tiles, column tiles, k-splits) and their reductions, built
@@ -1582,8 +1582,8 @@ static int adj_split(selinv_plan_s *plan) {
                 a->tc_launch[p.nlevels - 1 - L.level].push_back(e);
         }
     }
-    if (!a->d_tcdesc && cudaMalloc((void **)&a->d_tcdesc, sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
-    if (!a->cy && cudaMalloc((void **)&a->cy, sizeof(int) * (size_t)std::max(p.n, 1)) != cudaSuccess)
+    if (!a->d_tcdesc && dev_malloc((void **)&a->d_tcdesc, sizeof(ProbDesc)) != cudaSuccess) return SELINV_ERR_OOM;
+    if (!a->cy && dev_malloc((void **)&a->cy, sizeof(int) * (size_t)std::max(p.n, 1)) != cudaSuccess)
         return SELINV_ERR_OOM;
     a->split_key = key;
     a->gen++;

@@ -548,7 +548,7 @@ void factor_release(selinv_plan_s *plan) {
 template <typename X>
 static int up(X **d, const std::vector<X> &h) {
     *d = nullptr;
-    if (cudaMalloc((void **)d, sizeof(X) * std::max<size_t>(1, h.size())) != cudaSuccess) return SELINV_ERR_OOM;
+    if (dev_malloc((void **)d, sizeof(X) * std::max<size_t>(1, h.size())) != cudaSuccess) return SELINV_ERR_OOM;
     if (!h.empty() && cudaMemcpy(*d, h.data(), sizeof(X) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return SELINV_ERR_CUDA;
     return SELINV_OK;
@@ -753,7 +753,7 @@ int factor_tables(selinv_plan_s *plan) {
     if ((rc = up(&f->d_asm, f->asm_items))) return rc;
     if ((rc = up(&f->d_uoff, f->u_off))) return rc;
     if ((rc = up(&f->d_chpos, f->chpos))) return rc;
-    if (cudaMalloc((void **)&f->d_desc, sizeof(FactorDesc)) != cudaSuccess) return SELINV_ERR_OOM;
+    if (dev_malloc((void **)&f->d_desc, sizeof(FactorDesc)) != cudaSuccess) return SELINV_ERR_OOM;
     return SELINV_OK;
 }
 
@@ -811,14 +811,14 @@ static int factor_t(selinv_plan_s *plan, const void *A, void *L, void *D, cudaSt
         if (f->U) cudaFree(f->U);
         f->U = nullptr;
         f->U_bytes = 0;
-        if (cudaMalloc(&f->U, ubytes) != cudaSuccess) return SELINV_ERR_OOM;
+        if (dev_malloc((void **)&f->U, ubytes) != cudaSuccess) return SELINV_ERR_OOM;
         f->U_bytes = ubytes;
     }
     // real updates on the tensor cores unless the plan asks for FP64 FMA
     const bool tc = sizeof(T) == 8 && p.asked.fast_contraction == 1 && q->tc;
     if (tc && !f->digits) {
-        if (cudaMalloc(&f->digexp, sizeof(int) * (size_t)p.rowptr[p.ns]) != cudaSuccess) return SELINV_ERR_OOM;
-        if (cudaMalloc(&f->digits, sizeof(uint16_t) * (size_t)f->dig_total) != cudaSuccess) return SELINV_ERR_OOM;
+        if (!f->digexp && dev_malloc((void **)&f->digexp, sizeof(int) * (size_t)p.rowptr[p.ns]) != cudaSuccess) return SELINV_ERR_OOM;
+        if (dev_malloc((void **)&f->digits, sizeof(uint16_t) * (size_t)f->dig_total) != cudaSuccess) return SELINV_ERR_OOM;
     }
     FactorDesc *fd = factor_desc(plan, q, L, D, st, herm);
     if (cudaMemsetAsync(L, 0, sizeof(T) * (size_t)p.nnz, st) != cudaSuccess) return SELINV_ERR_CUDA;

@@ -38,7 +38,7 @@ template <typename X, typename A>
 static int upload(X **dptr, const std::vector<X, A> &h) {
     *dptr = nullptr;
     size_t bytes = sizeof(X) * (h.empty() ? 1 : h.size());
-    if (cudaMalloc((void **)dptr, bytes) != cudaSuccess) return SELINV_ERR_OOM;
+    if (dev_malloc((void **)dptr, bytes) != cudaSuccess) return SELINV_ERR_OOM;
     if (!h.empty() && cudaMemcpy(*dptr, h.data(), sizeof(X) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return SELINV_ERR_CUDA;
     return SELINV_OK;
@@ -438,7 +438,7 @@ int ensure_device(PlanData &p) {
     if ((rc = upload(&p.d_seg_ptr, p.seg_ptr))) return rc;
     if ((rc = upload(&p.d_seg_start, p.seg_start))) return rc;
     int *st = nullptr;
-    if (cudaMalloc((void **)&st, sizeof(int)) != cudaSuccess) return SELINV_ERR_OOM;
+    if (dev_malloc((void **)&st, sizeof(int)) != cudaSuccess) return SELINV_ERR_OOM;
     if (cudaMemset(st, 0, sizeof(int)) != cudaSuccess) return SELINV_ERR_CUDA;
     p.d_status = st;
     return SELINV_OK;
@@ -1499,7 +1499,7 @@ int build_schedule(Schedule &S, const std::vector<const PlanData *> &plans,
         }
     // one partial (hi, lo) tile of 128 x 64 per CTA of a level's k-split tcgen05 launches
     if (slab_slots > 0 &&
-        cudaMalloc((void **)&S.tcslab, sizeof(long long) * (size_t)kTcSlotWords * (size_t)slab_slots) != cudaSuccess)
+        dev_malloc((void **)&S.tcslab, sizeof(long long) * (size_t)kTcSlotWords * (size_t)slab_slots) != cudaSuccess)
         return SELINV_ERR_OOM;
 
     if (!S.h_red.empty() && (rc = upload(&S.d_red, S.h_red))) return rc;

@@ -125,6 +125,8 @@ struct Workspace {
 // dev_alloc hands out a cached buffer of exactly `bytes` or allocates one;
 // dev_release caches the buffer (the caller has synchronized the device).
 cudaError_t dev_alloc(void **ptr, size_t bytes);
+// cudaMalloc whose failure leaves no error behind for cudaGetLastError
+cudaError_t dev_malloc(void **ptr, size_t bytes);
 void dev_release(void *ptr, size_t bytes);
 
 // launch kinds

@@ -129,7 +129,7 @@ extern "C" int selinv_gather(selinv_plan plan, selinv_dtype dtype, const void *A
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!p.d_sel_pos) {
-        if (cudaMalloc((void **)&p.d_sel_pos, sizeof(int64_t) * (size_t)n) != cudaSuccess) return SELINV_ERR_OOM;
+        if (dev_malloc((void **)&p.d_sel_pos, sizeof(int64_t) * (size_t)n) != cudaSuccess) return SELINV_ERR_OOM;
         if (cudaMemcpy(p.d_sel_pos, p.sel_pos.data(), sizeof(int64_t) * (size_t)n, cudaMemcpyHostToDevice) !=
             cudaSuccess)
             return SELINV_ERR_CUDA;

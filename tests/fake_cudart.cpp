@@ -4,8 +4,8 @@
 //
 //   L stream index clock stale yacc panels name K...   a kernel launch: the stream and
 //        its launch count, the launches of every stream that come before it
-//        (comma-separated counts), whether its descriptors hold an address of
-//        freed memory, the bytes behind the first one's yacc and behind the LD
+//        (comma-separated counts), whether its descriptors or its work list are
+//        freed memory or missing, the bytes behind the first one's yacc and behind the LD
 //        panels of each (comma-separated), the kernel's name and the supernodes
 //        of its work list
 //   G / B / I / T       graph launch, begin of capture, instantiation, record of a timing event
@@ -13,7 +13,8 @@
 //
 // A captured launch is logged like an issued one.  fake_fail(what, n) makes the
 // next n begins of capture (1), instantiations (2) or cluster launches and
-// launches of k_adj_gemm (3) fail; every timed run takes 1 ms, those of the
+// launches of k_adj_gemm (3) fail, (4) the n-th allocation from
+// now on; every timed run takes 1 ms, those of the
 // autotuner's next fake_slow(n) candidates 2.  fake_capturing(st): the stream
 // that the caller captures.
 #include <cuda_runtime.h>
@@ -41,7 +42,7 @@ std::map<cudaStream_t, int> g_id;
 std::vector<std::vector<int>> g_clock;      // per stream: launches known to come before its next one
 std::map<cudaEvent_t, std::vector<int>> g_event;
 std::set<cudaEvent_t> g_timing;
-int g_fail[4];
+int g_fail[5];
 cudaError_t g_last = cudaSuccess;            // as cudaGetLastError returns it
 uintptr_t g_next = 0x1000;
 
@@ -91,6 +92,10 @@ cudaError_t launch(const void *fun, void **args, cudaStream_t st, bool cluster) 
             stale |= t && !t->second.live;
         }
         const auto *d = reinterpret_cast<const selinv::ProbDesc *>(descs);
+        const void *list = *static_cast<void *const *>(args[1]);
+        auto *t = find(list);
+        stale |= !list || (t && !t->second.live);
+        if (a->second.bytes % sizeof(*d) == 0 && d->lu) stale |= !d->LDu || !d->Vt || !d->Zu || !d->Ut;
         if (has("k_selinv_oz")) {
             auto *t = find(d->yacc);
             yacc = t ? (long long)t->second.bytes : 0;
@@ -146,8 +151,8 @@ void operator delete(void *p) noexcept {
 void operator delete(void *p, size_t) noexcept { operator delete(p); }
 
 extern "C" {
-void fake_fail(int what, int n) { g_fail[what] = n; }
-static int g_slow;
+static int g_slow, g_refused;
+void fake_fail(int what, int n) { g_fail[what] = n; g_refused = 0; }
 static cudaStream_t g_capturing;
 void fake_capturing(cudaStream_t st) { g_capturing = st; }
 void fake_slow(int candidates) { g_slow = 2 * candidates; }   // two timed runs each
@@ -178,6 +183,11 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t, 
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *cfg, const void *fun, void **args) { return launch(fun, args, cfg->stream, true); }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
+    if (g_fail[4] > 0 && --g_fail[4] == 0) {
+        g_fail[4] = 1;                           // (and the retry after the caches have been emptied)
+        if (++g_refused == 2) g_fail[4] = g_refused = 0;
+        return g_last = cudaErrorMemoryAllocation;
+    }
     if (posix_memalign(p, 256, n ? n : 1)) return cudaErrorMemoryAllocation;
     g_mem[(char *)*p] = {n ? n : 1, true};
     return cudaSuccess;

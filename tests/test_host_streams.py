@@ -451,3 +451,30 @@ print(json.dumps(out))
 """)
     for (_, lines), a in zip(parts[1:], active):
         assert set().union(*(x.ks for x in launches(lines))) == {K for K, on in enumerate(a) if on}
+
+
+CALLS_THAT_ALLOCATE = ["c.selinv()", "c.factor()", "batched([c, c], [0, 1])"]
+
+
+@pytest.mark.parametrize("call", CALLS_THAT_ALLOCATE)
+def test_calls_after_a_failed_allocation(fake, tmp_path, call):
+    """Whichever allocation of a first call fails, that call says so, and the
+    next ones are complete."""
+    parts, rc = run(fake, tmp_path, f"""
+rc = []
+for n in range(1, 41):
+    c = Ctx(synth.laplacian_3d(6, 4), use_graph=0)
+    mark("first")
+    RT.fake_fail(4, n)
+    r = [{call}]
+    RT.fake_fail(4, 0)
+    for _ in range(2):
+        mark("later")
+        r.append({call})
+    rc.append(r)
+print(json.dumps(rc))
+""")
+    assert all(r[0] in (0, -6) and r[1:] == [0, 0] for r in rc) and [-6, 0, 0] in rc and [0, 0, 0] in rc
+    later = [launches(lines) for name, lines in parts if name == "later"]
+    assert len({tuple(x.name for x in got) for got in later}) == 1
+    assert not any(x.stale for got in later for x in got)
