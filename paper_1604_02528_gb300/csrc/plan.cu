@@ -154,10 +154,9 @@ int Workspace::ensure(const PlanData &p, int dtype) {
 
 // the LU form's extra scratch (element size of the current workspace)
 int Workspace::ensure_lu(const PlanData &p) {
-    if (LDu) return SELINV_OK;
     DeviceGuard g(device);
-    if (!wget(*this, &LDu, bytes_elem * (size_t)std::max<int64_t>(p.nnz, 1))) return SELINV_ERR_OOM;
-    if (!wget(*this, &Vt, bytes_elem * (size_t)std::max<int64_t>(p.linv_total, 1))) return SELINV_ERR_OOM;
+    if (!LDu && !wget(*this, &LDu, bytes_elem * (size_t)std::max<int64_t>(p.nnz, 1))) return SELINV_ERR_OOM;
+    if (!Vt && !wget(*this, &Vt, bytes_elem * (size_t)std::max<int64_t>(p.linv_total, 1))) return SELINV_ERR_OOM;
     return SELINV_OK;
 }
 

@@ -453,7 +453,7 @@ print(json.dumps(out))
         assert set().union(*(x.ks for x in launches(lines))) == {K for K, on in enumerate(a) if on}
 
 
-CALLS_THAT_ALLOCATE = ["c.selinv()", "c.factor()", "batched([c, c], [0, 1])"]
+CALLS_THAT_ALLOCATE = ["c.selinv()", "c.lu()", "c.factor()", "batched([c, c], [0, 1])"]
 
 
 @pytest.mark.parametrize("call", CALLS_THAT_ALLOCATE)
