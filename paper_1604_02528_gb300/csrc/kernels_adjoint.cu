@@ -1401,6 +1401,7 @@ static int adj_split(selinv_plan_s *plan) {
     // here: the reverse passes have no mma.sync variant.
     const int key = o.fast_contraction != 0 ? std::max(8, o.oz_min_s) : 0;
     if (key == a->split_key) return SELINV_OK;
+    a->split_key = -1;   // (no lists until they are complete: an allocation may fail)
     auto fr = [](void *q) { if (q) cudaFree(q); };
     fr(a->d_sm); fr(a->d_sg); fr(a->d_wd); fr(a->d_row); fr(a->d_rg); fr(a->d_mbp); fr(a->d_dig);
     fr(a->d_pr); fr(a->d_sdw); fr(a->sd); fr(a->d_sd_off);

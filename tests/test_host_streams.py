@@ -478,3 +478,31 @@ print(json.dumps(rc))
     later = [launches(lines) for name, lines in parts if name == "later"]
     assert len({tuple(x.name for x in got) for got in later}) == 1
     assert not any(x.stale for got in later for x in got)
+
+
+def test_adjoint_lists_after_a_failed_allocation(fake, tmp_path):
+    """Lists that could not be rebuilt for a new option are rebuilt by the next
+    call, also under the old option: nothing is launched on freed or missing ones."""
+    parts, rc = run(fake, tmp_path, """
+rc = []
+for n in range(1, 41):
+    c = Ctx(synth.laplacian_3d(9, 4), use_graph=0)
+    r = [c.adjoint()]
+    mark("under 16")
+    r.append(c.adjoint())
+    c.set(oz_min_s=8)
+    mark("fails")
+    RT.fake_fail(4, n)
+    r.append(c.adjoint())
+    RT.fake_fail(4, 0)
+    c.set(oz_min_s=16)
+    mark("under 16")
+    r.append(c.adjoint())
+    mark("done")
+    rc.append(r)
+print(json.dumps(rc))
+""")
+    assert all(r[:2] == [0, 0] and r[2] in (0, -6) and r[3] == 0 for r in rc) and [0, 0, -6, 0] in rc
+    same = [launches(lines) for name, lines in parts if name == "under 16"]
+    assert len({tuple(x.name for x in got) for got in same}) == 1
+    assert not any(x.stale for got in same for x in got)
