@@ -463,6 +463,8 @@ def test_calls_after_a_failed_allocation(fake, tmp_path, call):
     parts, rc = run(fake, tmp_path, f"""
 rc = []
 for n in range(1, 41):
+    c = None
+    N.selinv_release_cached_memory()     # (every buffer of this call is an allocation)
     c = Ctx(synth.laplacian_3d(6, 4), use_graph=0)
     mark("first")
     RT.fake_fail(4, n)
