@@ -48,36 +48,45 @@ __global__ void __launch_bounds__(kTriThreads) k_noalloc_linv(int s, const doubl
 // The terms are quotients: a product with 1 / D_k rounds twice, and 1 / D_k
 // overflows where the quotient does not.  Each sum starts at its own k: a zero
 // of X above the diagonal times an infinite or undefined 1 / D_k is no term.
-// A quotient is the product with the rounded reciprocal and one correction by
-// its residual, which rounds correctly (P. Markstein, IBM J. Res. Dev. 34,
-// 1990; 34.8 us at s = 96, where six divisions a thread took 36.9 and products
-// with the reciprocal 32.8).  Magnitudes near the ends of the range are divided.
+// A quotient is x r + x r', r the rounded reciprocal and r' its residual over D_k:
+// one rounding, to within 2^-100 of the product.  Both kernels: 34.8 us at s = 96
+// and 51.2 at 128 (with divisions 36.9 and 55.2; products with r alone 32.8 and
+// 49.2).  Where a magnitude is near the ends of the range, the CTA divides.
 constexpr int kMidLo = 1023 - 400, kMidHi = 1023 + 400;   // biased exponents
 __device__ __forceinline__ bool mid(double v) {
     const int e = (int)((__double_as_longlong(v) >> 52) & 0x7FF);
     return e >= kMidLo && e <= kMidHi;
 }
-__device__ __forceinline__ double quotient(double x, double d, double r) {   // r = 1 / d, or 0: divide
-    if (r == 0.0 || !(mid(x) || x == 0.0)) return x / d;
-    const double q = x * r;
-    return fma(fma(-q, d, x), r, q);
-}
 
 __global__ void __launch_bounds__(256) k_noalloc_dinv(int s, const double *__restrict__ X, const double *__restrict__ D,
                                                       double *__restrict__ Dinv, int64_t ldo) {
     grid_dep_wait();
-    __shared__ double As[128][17], Bs[128][17], rd[128];
+    __shared__ double As[128][17], Bs[128][17], rd[128], rl[128];
     int ti = 0, tj = blockIdx.x;
     while (tj > ti) { tj -= ti + 1; ti++; }
     const int i0 = ti * 16, j0 = tj * 16, n = s - i0;
-    for (int q = threadIdx.x; q < n; q += 256) rd[q] = mid(D[i0 + q]) ? 1.0 / D[i0 + q] : 0.0;
+    bool far = false;
+    for (int q = threadIdx.x; q < n; q += 256) {
+        const double d = D[i0 + q], r = 1.0 / d;
+        far = !mid(d);
+        rd[q] = r;
+        rl[q] = fma(-d, r, 1.0) * r;
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < 16 * n; e += 256) {
         const int q = e % n, r = e / n, k = i0 + q;   // k fastest: contiguous in X's columns
-        As[q][r] = r <= q ? quotient(X[(int64_t)(i0 + r) * s + k], D[k], rd[q]) : 0.0;
+        const double x = r <= q ? X[(int64_t)(i0 + r) * s + k] : 0.0;
+        far = far || !(mid(x) || x == 0.0);
+        As[q][r] = fma(x, rd[q], x * rl[q]);
         Bs[q][r] = j0 + r < s ? X[(int64_t)(j0 + r) * s + k] : 0.0;
     }
-    __syncthreads();
+    if (__syncthreads_or(far)) {
+        for (int e = threadIdx.x; e < 16 * n; e += 256) {
+            const int q = e % n, r = e / n, k = i0 + q;
+            if (r <= q) As[q][r] = X[(int64_t)(i0 + r) * s + k] / D[k];
+        }
+        __syncthreads();
+    }
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, i = i0 + ty, j = j0 + tx;
     if (i >= s || i < j) return;
     double acc = 0.0;

@@ -50,9 +50,9 @@ __device__ __forceinline__ void tri_store(T *dst, const T *L, int64_t ld, int s,
 // y L^T = a for the warp's 32 / W rows a (unit lower L; conj(L) in place of L
 // when herm) of nt blocks of W columns, from column j0 on: y_j, final after step
 // j - 1, is taken from every later column k as y_j L(k, j).  Finished columns
-// are not touched, and a row takes the steps from its own on (the columns of an
-// inverse: what lies before is zero, which an infinite or undefined entry of L
-// would not keep so).  SCALED: L has the diagonal 1 / rd: y_j = a_j rd[j] is what
+// are not touched, and a row takes the steps from `own` on, which is among the
+// warp's first 32 / W (the columns of an inverse: what lies before is zero, which
+// an infinite or undefined entry of L would not keep so).  SCALED: L has the diagonal 1 / rd: y_j = a_j rd[j] is what
 // the later columns lose, and what is left in a is the undivided a_j.
 template <typename T, int W, int NC, bool SCALED>
 __device__ __forceinline__ void tri_rows(T (&a)[NC * 32 / W], const T *Ls, const T *rd, int nt, int j0, int own, bool herm) {
@@ -64,15 +64,18 @@ __device__ __forceinline__ void tri_rows(T (&a)[NC * 32 / W], const T *Ls, const
         if (W * (b + 1) <= j0) continue;
         const int q = b * W / 32;                       // the store's block of 32 columns
         const T *Lb = Ls + 32 * 32 * (q * NC - q * (q - 1) / 2) + b * W % 32 * 32 * (NC - q) + c - 32 * q;
-#pragma unroll 2
-        for (int jj = max(0, j0 - W * b); jj < W; jj++) {
+        auto step = [&](int jj, bool on) {
             T y = shfl_elem<W>(a[b], jj);
             if (SCALED) y = mul(y, rd[W * b + jj]);
             const T *l = Lb + jj * 32 * (NC - q);
 #pragma unroll
             for (int t = b; t < NT; t++)
-                if (W * b + jj >= own && (t > b || c > jj) && (t <= NT - 32 / W || t < nt)) msub(a[t], y, cjif(l[W * t], herm));
-        }
+                if (on && (t > b || c > jj) && (t <= NT - 32 / W || t < nt)) msub(a[t], y, cjif(l[W * t], herm));
+        };
+        int jj = max(0, j0 - W * b);
+        for (; jj < W && W * b + jj < j0 + 32 / W - 1; jj++) step(jj, W * b + jj >= own);   // up to the warp's last own step
+#pragma unroll 2
+        for (; jj < W; jj++) step(jj, true);
     }
 }
 
