@@ -607,9 +607,11 @@ static int factor_lists(selinv_plan_s *plan, int tc_s, FactorLists **out) {
             v.wide_s = std::max(v.wide_s, width(J));
             rows += below(J);
         }
-        // a cluster of 8 CTAs per diagonal block while all of them find an SM
-        // (one 128-column block: 54 us on 8 SMs, 127 on one); wide levels
-        // have blocks enough by themselves
+        // a cluster of 8 CTAs per diagonal block while all of them find an SM;
+        // wide levels have blocks enough by themselves.  At most 8, 4, 2 and 1
+        // CTAs: 40^3 11.3, 11.6, 12.3 and 14.0 ms, 20^3 Hermitian 4.4, 4.7, 5.4 and
+        // 6.8, 16^3 complex 2.05, 2.24, 2.68 and 3.54 (one 128-column block of 40^3
+        // takes 105 us on 8 SMs, cold caches)
         const int64_t nw = (int64_t)wide.size();
         v.cl = v.wide_s <= 32 ? 1 : (nw * 8 <= 152 ? 8 : (nw * 4 <= 152 ? 4 : (nw * 2 <= 152 ? 2 : 1)));
         // rows per tile: the number whose tiles, dealt to the SMs, take least --
