@@ -94,8 +94,9 @@ int Workspace::ensure(const PlanData &p, int dtype) {
     const size_t es = elem_size(dtype);
     const size_t ny = (dtype == SELINV_F64 && p.lhs_total > 0) ? 2 * (size_t)p.nnz : 2;   // words of yacc
     if (LD && bytes_elem >= es && shape == p.shape) {
-        if (yacc_words >= ny) return SELINV_OK;
-        // real values in a workspace made for complex ones, which have no such sums
+        // real values in a workspace made for complex ones, which have no such
+        // sums: only the mma.sync engine adds into them
+        if (yacc_words >= ny || p.opts.fast_contraction != 2) return SELINV_OK;
         DeviceGuard g(device);
         if (!wget(*this, &yacc, sizeof(long long) * ny)) return SELINV_ERR_OOM;
         if (cudaMemset(yacc, 0, sizeof(long long) * ny) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
